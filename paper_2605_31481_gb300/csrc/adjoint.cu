@@ -301,13 +301,28 @@ __global__ void __launch_bounds__(256) crba_vjp_kernel(ModelView mv, int64_t B, 
   }
 }
 
-// out[p] = sum over blocks b (in order) of partial[b * P + p]
-__global__ void partial_reduce_kernel(const float* __restrict__ partial, int nblk, int P, float* __restrict__ out) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
+// out[p] = sum over blocks b of partial[b * P + p]. A block sums 32 columns;
+// its 32 warps take every 32nd row each, eight loads in flight, and the warps'
+// sums are added in warp order: the order is fixed, so the result is the same
+// run to run. (One thread per column read nblk rows one after the other: 5.0 us
+// for 256 rows of 71 values.)
+__global__ void __launch_bounds__(1024) partial_reduce_kernel(const float* __restrict__ partial, int nblk, int P,
+                                                              float* __restrict__ out) {
+  __shared__ float part[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int b = 0; b < nblk; ++b) s += partial[(int64_t)b * P + p];
-  out[p] = s;
+  if (p < P) {
+#pragma unroll 8
+    for (int b = w; b < nblk; b += 32) s += partial[(int64_t)b * P + p];
+  }
+  part[w][lane] = s;
+  __syncthreads();
+  if (w) return;
+  s = 0.f;
+#pragma unroll
+  for (int k = 0; k < 32; ++k) s += part[k][lane];
+  if (p < P) out[p] = s;
 }
 
 // Largest power-of-two block (<= the default, >= 32) whose shared memory
@@ -319,7 +334,7 @@ int fit_block(int64_t B, int n, int rows, bool theta) {
 }
 
 cudaError_t reduce(const float* partial, int nblk, int P, float* out, cudaStream_t s) {
-  partial_reduce_kernel<<<(P + 127) / 128, 128, 0, s>>>(partial, nblk, P, out);
+  partial_reduce_kernel<<<(P + 31) / 32, 1024, 0, s>>>(partial, nblk, P, out);
   return cudaGetLastError();
 }
 
