@@ -1,0 +1,476 @@
+// Dynamics in body-origin frames whose axes are aligned with the root.
+//
+// Every spatial quantity of body i is expressed with the axes of its tree's
+// root (the world for a fixed base, body 0 for a floating one) and about
+// body i's own origin. Moving a vector between a body and its parent is then
+// a shift by r_i (the body's origin seen from the parent's), one cross
+// product, instead of a rotation and a shift, and the quantities keep the
+// magnitudes they have in body coordinates: no moment arm to a far root
+// enters, so nothing cancels that does not cancel there.
+//
+// What that buys is a short chain. The only serial recursions left are the
+// rotations and velocities down the tree and plain sums (with a shift) up it;
+// joint transforms, inertias, forces and every derivative below are per-body
+// work that all warps of a block share between two barriers.
+//
+// Derivatives. With psi_j the motion subspace of degree of freedom j in this
+// form, v, a the velocity and acceleration (gravity included) of j's parent
+// at j's origin,
+//     psid_j = v x psi_j,   psidd_j = a x psi_j + v x psid_j,
+//     eta_j  = 2 psid_j     (a free root: psid = 0, eta_j = v_0 x psi_j),
+// and for body k  f_k = I a_k + v_k x* I v_k  and the velocity operator
+//     2 B_k x = v_k x* (I x) - I (v_k x x) + x x* (I v_k).
+// Displacing q_j moves j's subtree rigidly; the difference to moving the
+// whole world is a velocity psid_j and an acceleration psidd_j + psid_j x v_k
+// added to the subtree, so the force of the subtree changes by
+//     psi_j x* f + I psidd_j + 2 B psid_j        (f, I, B summed over it),
+// and adding to qd_j changes it by  I eta_j + 2 B psi_j.  Projected on
+// psi_i this gives every entry of d tau / d q and d tau / d qd as dot products
+// along the support paths (the analytic form of the derivatives that the
+// paper names as the step after autograd, Sec. 3.5), and summed against a
+// cotangent it gives the adjoint. Expanding 2 B for a rigid body (mass m,
+// first moment h, inertia I_o about the origin, S = tr(I_o)/2 1 - I_o) shows
+// that it acts on the angular part only:
+//     2 B (w, u) = 2 (P w, p x w),
+//     P = -[omega] S + (h . nu) 1 - nu h^T,   p = h x omega - m nu
+// with v_k = (omega, nu), so a subtree's B is 12 numbers.
+#pragma once
+
+#include "level.cuh"
+
+namespace fst {
+
+// motion about the parent's origin -> about the child's, r = child - parent
+__device__ __forceinline__ SV shift_motion(SV m, f3 r) { return SV{m.w, m.v + cross(m.w, r)}; }
+// force about the child's origin -> about the parent's
+__device__ __forceinline__ SV shift_force(SV f, f3 r) { return SV{f.w + cross(r, f.v), f.v}; }
+
+// A rigid-body inertia's axes rotated by R (no shift).
+__device__ __forceinline__ In10 in_rotate(const float* R, const In10& I) {
+  In10 o;
+  o.m = I.m;
+  o.h = Rmul(R, I.h);
+  sym_rot(R, I.I, o.I);
+  return o;
+}
+
+// The same body about the parent's origin, r = child - parent (parallel axes).
+__device__ __forceinline__ In10 in_shift(const In10& I, f3 r) {
+  In10 o;
+  o.m = I.m;
+  o.h = I.h + I.m * r;
+  const float d = fmaf(2.0f, dot(I.h, r), I.m * dot(r, r));
+  const f3 z = I.h + (0.5f * I.m) * r;  // h r^T + r h^T + m r r^T = z r^T + r z^T
+  o.I[0] = I.I[0] + (d - 2.0f * z.x * r.x);
+  o.I[1] = I.I[1] - fmaf(z.x, r.y, r.x * z.y);
+  o.I[2] = I.I[2] + (d - 2.0f * z.y * r.y);
+  o.I[3] = I.I[3] - fmaf(z.x, r.z, r.x * z.z);
+  o.I[4] = I.I[4] - fmaf(z.y, r.z, r.y * z.z);
+  o.I[5] = I.I[5] + (d - 2.0f * z.z * r.z);
+  return o;
+}
+
+// The velocity operator of a body or subtree (see above).
+struct BOp {
+  float P[9];
+  f3 p;
+};
+
+__device__ __forceinline__ BOp b_of(const In10& I, SV v, SV hv) {
+  BOp b;
+  const float ht = 0.5f * (I.I[0] + I.I[2] + I.I[5]);
+  // columns of -[omega] S: S column c crossed with omega
+  const f3 s0 = f3{ht - I.I[0], -I.I[1], -I.I[3]};
+  const f3 s1 = f3{-I.I[1], ht - I.I[2], -I.I[4]};
+  const f3 s2 = f3{-I.I[3], -I.I[4], ht - I.I[5]};
+  const f3 c0 = cross(s0, v.w), c1 = cross(s1, v.w), c2 = cross(s2, v.w);
+  const float hn = dot(I.h, v.v);
+  b.P[0] = c0.x + fmaf(-v.v.x, I.h.x, hn);
+  b.P[1] = fmaf(-v.v.x, I.h.y, c1.x);
+  b.P[2] = fmaf(-v.v.x, I.h.z, c2.x);
+  b.P[3] = fmaf(-v.v.y, I.h.x, c0.y);
+  b.P[4] = c1.y + fmaf(-v.v.y, I.h.y, hn);
+  b.P[5] = fmaf(-v.v.y, I.h.z, c2.y);
+  b.P[6] = fmaf(-v.v.z, I.h.x, c0.z);
+  b.P[7] = fmaf(-v.v.z, I.h.y, c1.z);
+  b.P[8] = c2.z + fmaf(-v.v.z, I.h.z, hn);
+  b.p = -hv.v;
+  return b;
+}
+
+// a += the child's operator b moved to the parent's origin
+__device__ __forceinline__ void b_add_shifted(BOp& a, const BOp& b, f3 r) {
+  const float rp = dot(r, b.p);
+  a.P[0] += b.P[0] + fmaf(b.p.x, r.x, -rp);
+  a.P[1] += fmaf(b.p.x, r.y, b.P[1]);
+  a.P[2] += fmaf(b.p.x, r.z, b.P[2]);
+  a.P[3] += fmaf(b.p.y, r.x, b.P[3]);
+  a.P[4] += b.P[4] + fmaf(b.p.y, r.y, -rp);
+  a.P[5] += fmaf(b.p.y, r.z, b.P[5]);
+  a.P[6] += fmaf(b.p.z, r.x, b.P[6]);
+  a.P[7] += fmaf(b.p.z, r.y, b.P[7]);
+  a.P[8] += b.P[8] + fmaf(b.p.z, r.z, -rp);
+  a.p = a.p + b.p;
+}
+
+// 2 B (w, .) as a force
+__device__ __forceinline__ SV b_mul2(const BOp& b, f3 w) {
+  return SV{2.f * Rmul(b.P, w), 2.f * cross(b.p, w)};
+}
+// The functional x -> psi . 2 B x, which only sees x's angular part
+__device__ __forceinline__ f3 b_row2(const BOp& b, SV psi) {
+  return 2.f * (RTmul(b.P, psi.w) + cross(psi.v, b.p));
+}
+
+// psi of a 1-DOF joint: its body-coordinate subspace with the axes rotated
+__device__ __forceinline__ SV psi_of(const BodyC& c, const float* R) {
+  const SV s = S_of(c);
+  return SV{Rmul(R, s.w), Rmul(R, s.v)};
+}
+
+__device__ __forceinline__ bool one_dof(const BodyI& b) {
+  return b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC;
+}
+
+// ---- dense derivatives of inverse dynamics ------------------------------------
+// Floats of shared state per body and environment: psi 6 | psid 6 | psidd 6 |
+// r 3 | then R 9, v 6, a 6 while the kinematics run down the tree, replaced
+// in place by the body's (then its subtree's) I 10, f 6, P 9, p 3
+// (kDerivState = 49).
+
+// The mass matrix keeps only entries of related degrees of freedom: row c
+// holds M_cc, then c's ancestors from the nearest to the root (DofLists), in
+// shared memory as [entry][lane].
+struct TreeMat {
+  float* base;
+  const int* off;   // first entry of each row
+  const int* dep;   // entries of each row (the diagonal included)
+  const int* anc;   // degree of freedom of each entry
+  __device__ __forceinline__ float* at(int entry) const { return base + (entry << 5) + (threadIdx.x & 31); }
+};
+
+// d tau / d q and d tau / d qd, [nv][nv][B] each (either may be null), and
+// with MASS the mass matrix into H, of one tile of 32 environments. The caller
+// has staged q, qd and qdd.
+template <bool MASS>
+__device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, const Col& q, const Col& qd,
+                                                    const Col& qdd, int nv, const LaneState& S, const TreeMat& H,
+                                                    float* __restrict__ dq, float* __restrict__ dqd, int64_t B,
+                                                    int64_t e, bool act) {
+  const int W = n_warps(), w = warp_id(), n = tp.n();
+  enum { PSI = 0, PSD = 6, PSDD = 12, RR = 18, R_ = 21, V_ = 30, A_ = 36, I_ = 21, F_ = 31, P_ = 37, p_ = 46 };
+  // structural zeros: entries of unrelated degrees of freedom
+  const int64_t e0 = e - (threadIdx.x & 31);
+  if (dq) m_clear_tile(dq, (int64_t)nv * nv, B, e0, W, w);
+  if (dqd) m_clear_tile(dqd, (int64_t)nv * nv, B, e0, W, w);
+  // joint transforms, all bodies at once
+  for (int i = w; i < n; i += W) {
+    const BodyI bi = tp.I(i);
+    S.putX(i, R_, joint_X(tp.C(i), bi, q));  // R 9, t 3 (t in the V slot until the level pass reads it)
+  }
+  __syncthreads();
+  // down the tree: rotations, velocities, accelerations, subspaces
+  for (int l = 0; l < tp.depth(); ++l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const Xf X = S.X(i, R_);
+      if (bi.type == FST_JOINT_FREE) {  // the root frame is this body's own
+        const SV v0 = S_times(tp.C(i), bi, qd);
+        const SV g{f3{0.f, 0.f, 0.f}, RTmul(X.R, a0.v)};
+        const float Id[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
+        S.put_n(i, R_, Id, 9);
+        S.put(i, V_, v0);
+        S.put(i, A_, S_times(tp.C(i), bi, qdd) + g);
+        S.put(i, PSI, v0);   // what its columns need later: v_0 and the gravity term
+        S.put(i, PSD, g);
+        continue;
+      }
+      float R[9];
+      f3 r;
+      SV vl = sv_zero(), al = a0;
+      if (bi.parent < 0) {
+#pragma unroll
+        for (int c = 0; c < 9; ++c) R[c] = X.R[c];
+        r = tvec(X);
+      } else {
+        float Rp[9];
+        S.get_n(bi.parent, R_, Rp, 9);
+        const float zero[3] = {0.f, 0.f, 0.f};
+        float rr[3];
+        compose(Rp, zero, X, R, rr);
+        r = f3{rr[0], rr[1], rr[2]};
+        vl = shift_motion(S.sv(bi.parent, V_), r);
+        al = shift_motion(S.sv(bi.parent, A_), r);
+      }
+      const float rv[3] = {r.x, r.y, r.z};
+      S.put_n(i, RR, rv, 3);
+      S.put_n(i, R_, R, 9);
+      if (one_dof(bi)) {
+        const SV psi = psi_of(tp.C(i), R);
+        const SV psd = crm(vl, psi);
+        S.put(i, PSI, psi);
+        S.put(i, PSD, psd);
+        S.put(i, PSDD, crm(al, psi) + crm(vl, psd));
+        vl = vl + qd[bi.vi] * psi;
+        al = al + (qdd[bi.vi] * psi + qd[bi.vi] * psd);
+      }
+      S.put(i, V_, vl);
+      S.put(i, A_, al);
+    }
+    __syncthreads();
+  }
+  // inertias, forces and velocity operators, all bodies at once
+  for (int i = w; i < n; i += W) {
+    float R[9];
+    S.get_n(i, R_, R, 9);
+    const SV v = S.sv(i, V_), a = S.sv(i, A_);
+    const In10 I = in_rotate(R, in_load(tp.theta(i)));
+    const SV hv = in_mul(I, v);
+    const BOp b = b_of(I, v, hv);
+    S.putin(i, I_, I);
+    S.put(i, F_, in_mul(I, a) + crf(v, hv));
+    S.put_n(i, P_, b.P, 9);
+    const float pv[3] = {b.p.x, b.p.y, b.p.z};
+    S.put_n(i, p_, pv, 3);
+  }
+  __syncthreads();
+  // up the tree: sums over subtrees (the deepest level has no children)
+  for (int l = tp.depth() - 2; l >= 0; --l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const int c0 = tp.child_begin(i), c1 = tp.child_begin(i + 1);
+      if (c0 == c1) continue;
+      In10 I = S.in10(i, I_);
+      SV f = S.sv(i, F_);
+      BOp b;
+      float t3[3];
+      S.get_n(i, P_, b.P, 9);
+      S.get_n(i, p_, t3, 3);
+      b.p = f3{t3[0], t3[1], t3[2]};
+      for (int ch = c0; ch < c1; ++ch) {
+        const int c = tp.child(ch);
+        S.get_n(c, RR, t3, 3);
+        const f3 r = f3{t3[0], t3[1], t3[2]};
+        in_add(I, in_shift(S.in10(c, I_), r));
+        f = f + shift_force(S.sv(c, F_), r);
+        BOp bc;
+        S.get_n(c, P_, bc.P, 9);
+        S.get_n(c, p_, t3, 3);
+        bc.p = f3{t3[0], t3[1], t3[2]};
+        b_add_shifted(b, bc, r);
+      }
+      S.putin(i, I_, I);
+      S.put(i, F_, f);
+      S.put_n(i, P_, b.P, 9);
+      const float pv[3] = {b.p.x, b.p.y, b.p.z};
+      S.put_n(i, p_, pv, 3);
+    }
+    __syncthreads();
+  }
+  // every pair of related degrees of freedom, from the deeper one up its
+  // support path (deepest bodies first: they have the longest paths)
+  float* const Q = dq && act ? dq + e : nullptr;
+  float* const D = dqd && act ? dqd + e : nullptr;
+  for (int it = w; it < n; it += W) {
+    const int i = tp.level_body(n - 1 - it);
+    const BodyI bi = tp.I(i);
+    if (nv_of(bi.type) == 0) continue;
+    const In10 I = S.in10(i, I_);
+    BOp b;
+    float t3[3];
+    S.get_n(i, P_, b.P, 9);
+    S.get_n(i, p_, t3, 3);
+    b.p = f3{t3[0], t3[1], t3[2]};
+    auto at = [&](int r, int c) { return ((int64_t)r * nv + c) * B; };
+    if (bi.type == FST_JOINT_FREE) {  // the root's own 6 x 6 blocks, rows and columns [v; w]
+      const SV v0 = S.sv(i, PSI), g = S.sv(i, PSD);
+#pragma unroll 1
+      for (int j = 0; j < 6; ++j) {
+        SV psi = sv_zero();
+        if (j < 3)
+          (j == 0 ? psi.v.x : j == 1 ? psi.v.y : psi.v.z) = 1.f;
+        else
+          (j == 3 ? psi.w.x : j == 4 ? psi.w.y : psi.w.z) = 1.f;
+        const SV cq = in_mul(I, crm(g, psi));
+        const SV cd = in_mul(I, crm(v0, psi)) + b_mul2(b, psi.w);
+        const SV cm = in_mul(I, psi);
+        const float xq[6] = {cq.v.x, cq.v.y, cq.v.z, cq.w.x, cq.w.y, cq.w.z};
+        const float xd[6] = {cd.v.x, cd.v.y, cd.v.z, cd.w.x, cd.w.y, cd.w.z};
+        const float xm[6] = {cm.v.x, cm.v.y, cm.v.z, cm.w.x, cm.w.y, cm.w.z};
+        if (MASS)  // row vi + j: the diagonal, then columns j - 1 .. 0
+#pragma unroll
+          for (int r = 0; r < 6; ++r)
+            if (r <= j) *H.at(H.off[bi.vi + j] + j - r) = xm[r];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+          const int64_t o = at(bi.vi + r, bi.vi + j);
+          if (Q) Q[o] = xq[r];
+          if (D) D[o] = xd[r];
+        }
+      }
+      continue;
+    }
+    const int c = bi.vi;
+    const SV psi = S.sv(i, PSI), psd = S.sv(i, PSD);
+    SV t = in_mul(I, psi);
+    SV uq = in_mul(I, S.sv(i, PSDD)) + b_mul2(b, psd.w);
+    SV ud = 2.f * in_mul(I, psd) + b_mul2(b, psi.w);
+    const f3 rw = b_row2(b, psi);
+    if (Q) Q[at(c, c)] = dot(psi, uq);
+    if (D) D[at(c, c)] = dot(psi, ud);
+    float* hrow = MASS ? H.at(H.off[c]) : nullptr;  // the row's next entry
+    if (MASS) {
+      *hrow = dot(psi, t);
+      hrow += 32;
+    }
+    uq = uq + crf(psi, S.sv(i, F_));
+    int kk = i;
+    for (int j = bi.parent; j >= 0; j = tp.I(j).parent) {
+      S.get_n(kk, RR, t3, 3);
+      const f3 r = f3{t3[0], t3[1], t3[2]};
+      kk = j;
+      t = shift_force(t, r);
+      uq = shift_force(uq, r);
+      ud = shift_force(ud, r);
+      const BodyI bj = tp.I(j);
+      if (one_dof(bj)) {
+        const SV pj = S.sv(j, PSI), pdj = S.sv(j, PSD);
+        if (Q) {
+          Q[at(bj.vi, c)] = dot(pj, uq);
+          Q[at(c, bj.vi)] = dot(t, S.sv(j, PSDD)) + dot(rw, pdj.w);
+        }
+        if (D) {
+          D[at(bj.vi, c)] = dot(pj, ud);
+          D[at(c, bj.vi)] = fmaf(2.f, dot(t, pdj), dot(rw, pj.w));
+        }
+        if (MASS) {
+          *hrow = dot(pj, t);
+          hrow += 32;
+        }
+      } else if (bj.type == FST_JOINT_FREE) {
+        const SV v0 = S.sv(j, PSI), g = S.sv(j, PSD);
+        const f3 z = cross(t.v, g.v);        // t . psidd of the angular directions
+        const SV y = crf(v0, t);             // t . eta = -psi . (v0 x* t)
+        const float uqr[6] = {uq.v.x, uq.v.y, uq.v.z, uq.w.x, uq.w.y, uq.w.z};
+        const float udr[6] = {ud.v.x, ud.v.y, ud.v.z, ud.w.x, ud.w.y, ud.w.z};
+        const float tr[6] = {t.v.x, t.v.y, t.v.z, t.w.x, t.w.y, t.w.z};
+        const float zq[6] = {0.f, 0.f, 0.f, z.x, z.y, z.z};
+        const float yd[6] = {-y.v.x, -y.v.y, -y.v.z, rw.x - y.w.x, rw.y - y.w.y, rw.z - y.w.z};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const int64_t up = at(bj.vi + k, c), left = at(c, bj.vi + k);
+          if (Q) {
+            Q[up] = uqr[k];
+            Q[left] = zq[k];
+          }
+          if (D) {
+            D[up] = udr[k];
+            D[left] = yd[k];
+          }
+          if (MASS) hrow[(5 - k) * 32] = tr[k];  // the nearest ancestor is the root's last coordinate
+        }
+      }
+    }
+  }
+}
+
+// ---- forward-dynamics derivatives: the tree-sparse factorisation ----------------
+// M = L^T D L with L unit lower triangular and as sparse as the tree: an
+// elimination from the leaves to the roots fills no entry of unrelated degrees
+// of freedom (Featherstone, Rigid Body Dynamics Algorithms, Sec. 6.5). Rows of
+// one depth are independent; a row's updates all come from one warp (row mod
+// W), so the block needs one barrier per depth. On return H holds L below the
+// diagonal and 1 / D on it.
+__device__ __forceinline__ void axpy_rows(float x, const float* src, float* dst, int n) {
+  // dst += x src, four rows at a time: src and dst never overlap, which the
+  // compiler cannot know, so the loads are issued ahead of the stores by hand
+  int b = 0;
+  for (; b + 4 <= n; b += 4, src += 128, dst += 128) {
+    const float s0 = src[0], s1 = src[32], s2 = src[64], s3 = src[96];
+    const float d0 = dst[0], d1 = dst[32], d2 = dst[64], d3 = dst[96];
+    dst[0] = fmaf(x, s0, d0);
+    dst[32] = fmaf(x, s1, d1);
+    dst[64] = fmaf(x, s2, d2);
+    dst[96] = fmaf(x, s3, d3);
+  }
+  for (; b < n; ++b, src += 32, dst += 32) *dst = fmaf(x, *src, *dst);
+}
+
+__device__ __forceinline__ void tree_factor(const TreeMat& H, const int* order, const int* level, int dof_depth) {
+  const int W = n_warps(), w = warp_id();
+  for (int l = dof_depth - 1; l >= 0; --l) {
+    for (int s = level[l]; s < level[l + 1]; ++s) {
+      const int k = order[s], o = H.off[k], d = H.dep[k];
+      const float inv = 1.0f / fmaxf(*H.at(o), 1e-30f);
+      for (int a = 1; a < d; ++a) {
+        const int i = H.anc[o + a];
+        if (i % W != w) continue;
+        const float x = *H.at(o + a) * inv;
+        axpy_rows(-x, H.at(o + a), H.at(H.off[i]), d - a);
+      }
+    }
+    __syncthreads();
+    // scale the finished rows (every warp has read them)
+    for (int s = level[l] + w; s < level[l + 1]; s += W) {
+      const int k = order[s], o = H.off[k], d = H.dep[k];
+      const float inv = 1.0f / fmaxf(*H.at(o), 1e-30f);
+      *H.at(o) = inv;
+      for (int a = 1; a < d; ++a) *H.at(o + a) *= inv;
+    }
+  }
+  __syncthreads();
+}
+
+// x := M^-1 x for NC columns held as [nv][32] in shared memory, one after the
+// other `ld` floats apart (this lane's element of row i at x[i * 32]).
+// Children have larger indices than their ancestors.
+template <int NC>
+__device__ __forceinline__ void tree_solve(const TreeMat& H, int nv, float* x, int ld) {
+  for (int i = nv - 1; i >= 0; --i) {  // L^T y = x, from the leaves
+    const int o = H.off[i], d = H.dep[i];
+    float xi[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) xi[c] = x[c * ld + (i << 5)];
+    int a = 1;
+    for (; a + 4 <= d; a += 4) {  // distinct ancestors: all loads ahead of the stores
+      int j[4];
+      float l[4], t[4][NC];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        j[u] = H.anc[o + a + u] << 5;
+        l[u] = *H.at(o + a + u);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) t[u][c] = x[c * ld + j[u]];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) x[c * ld + j[u]] = fmaf(-l[u], xi[c], t[u][c]);
+    }
+    for (; a < d; ++a) {
+      const int j = H.anc[o + a] << 5;
+      const float l = *H.at(o + a);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) x[c * ld + j] = fmaf(-l, xi[c], x[c * ld + j]);
+    }
+  }
+  for (int i = 0; i < nv; ++i) {  // D, then L x = y, from the roots
+    const int o = H.off[i], d = H.dep[i];
+    const float inv = *H.at(o);
+    float s[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) s[c] = x[c * ld + (i << 5)] * inv;
+#pragma unroll 4
+    for (int a = 1; a < d; ++a) {
+      const int j = H.anc[o + a] << 5;
+      const float l = *H.at(o + a);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) s[c] = fmaf(-l, x[c * ld + j], s[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) x[c * ld + (i << 5)] = s[c];
+  }
+}
+
+}  // namespace fst

@@ -92,6 +92,15 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
          level_smem_needed(view_of(m, nullptr), level_kind, level_tiles(m, kind)) <= kLevelSmemLimit;
 }
 
+// Whether a call of this kind runs its aligned-frame kernel (aligned.cu): the
+// default unless the kind is pinned to another variant or the tree's state
+// does not fit in shared memory (`need` bytes; about 33 bodies). There is no
+// line in B: the aligned kernels were the faster ones at every size measured,
+// against the generic and the specialised kernels: derivatives 3 to 20 times.
+bool aligned_fits(const fst_model* m, int kind, size_t need) {
+  return m->variant[kind] == FST_VARIANT_AUTO && need + 1024 <= kLevelSmemLimit;  // 1 KB: static shared memory
+}
+
 // The path-parallel kernel slot a call of this kind runs (0: none): 1 for
 // FST_VARIANT_PATH (a lane per path), 2 for FST_VARIANT_PATH_WARP (a warp
 // per path).
@@ -206,8 +215,9 @@ fst_status fst_model_create(const fst_body_desc* bodies, int32_t n_bodies, const
   if (err == cudaSuccess) err = cudaMalloc((void**)&m->di, sizeof(BodyI) * m->n);
   if (err == cudaSuccess) err = cudaMemcpy(m->dc, m->hc.data(), sizeof(BodyC) * m->n, cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMemcpy(m->di, m->hi.data(), sizeof(BodyI) * m->n, cudaMemcpyHostToDevice);
-  if (err == cudaSuccess) err = cudaMalloc((void**)&m->dt, sizeof(TopoLists));
+  if (err == cudaSuccess) err = cudaMalloc((void**)&m->dt, sizeof(TopoLists) + sizeof(DofLists));
   if (err == cudaSuccess) err = cudaMemcpy(m->dt, &m->ht, sizeof(TopoLists), cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = cudaMemcpy(m->dt + 1, &m->hd, sizeof(DofLists), cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = cudaMalloc((void**)&m->dpin, sizeof(int) * (kPinTableSize + 2 * kPinRegion));
   if (err == cudaSuccess) err = cudaMemset(m->dpin, 0xff, sizeof(int) * kPinTableSize);  // no roles: -1
   for (int i = 0; i < kPinTableSize; ++i) m->pin_table[i] = FST_ROLE_NONE;
@@ -861,6 +871,9 @@ fst_status fst_rnea_derivatives(const fst_model* m, int64_t B, const float* q, c
   FST_CHECK(need(fn, qd, "qd"));
   FST_CHECK(need(fn, qdd, "qdd"));
   const ModelView mv = view_of(m, theta);
+  if (aligned_fits(m, JK_RNEA_DERIVS, rnea_derivs_aligned_smem(mv)))
+    return finish(fn, launch_rnea_derivs_aligned(mv, B, q, qd, qdd, dtau_dq, dtau_dqd, m->block[JK_RNEA_DERIVS],
+                                                 (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_DERIVS))
     return finish(fn, jit_go(m, JK_RNEA_DERIVS, B, m->nq + 2 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              qd, qdd, dtau_dq, dtau_dqd));
@@ -879,6 +892,10 @@ fst_status fst_aba_derivatives(const fst_model* m, int64_t B, const float* q, co
   FST_CHECK(need(fn, tau, "tau"));
   FST_CHECK(need(fn, Minv, "Minv"));
   const ModelView mv = view_of(m, theta);
+  if (aligned_fits(m, JK_ABA_DERIVS, aba_derivs_aligned_smem(mv, m->max_width, m->dof_entries)))
+    return finish(fn, launch_aba_derivs_aligned(mv, B, q, qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv, m->max_width,
+                                                m->dof_entries, m->dof_depth, m->block[JK_ABA_DERIVS],
+                                                (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_DERIVS))
     return finish(fn, jit_go(m, JK_ABA_DERIVS, B, m->nq + 3 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv));

@@ -27,7 +27,10 @@ struct fst_model {
   fst::BodyC* dc = nullptr;
   fst::BodyI* di = nullptr;
   fst::TopoLists ht{};               // level and child lists (host copy)
-  fst::TopoLists* dt = nullptr;      // device copy
+  fst::TopoLists* dt = nullptr;      // device copy, followed by the device copy of hd
+  fst::DofLists hd{};                // the tree of the degrees of freedom (host copy)
+  int dof_depth = 0;                 // its depth
+  int dof_entries = 0;               // entries of a tree-sparse matrix (hd.anc)
   int* dpin = nullptr;               // SM-pinned launches: role table, then the counter regions
   int pin_table[256] = {};           // host copy of the role table (FST_ROLE_*, -1 none)
   std::vector<int> sm_ids;           // the device's SM ids (probed when the role table is set)

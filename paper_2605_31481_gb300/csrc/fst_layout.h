@@ -62,6 +62,23 @@ struct TopoLists {
   int child[FST_MAX_BODIES];
 };
 
+// The tree of the degrees of freedom (a free joint's six form a chain, a
+// fixed joint's body passes its parent's on): row c of a tree-sparse matrix
+// holds its diagonal, then c's ancestors from the nearest to the root, at
+// entries off[c] .. off[c] + dep[c] - 1; anc names each entry's column. order
+// lists the degrees of freedom by depth: those of depth l + 1 are
+// order[level[l]] .. order[level[l + 1] - 1]. Stored behind the TopoLists on
+// the device.
+constexpr int kMaxDof = FST_MAX_BODIES + 5;
+constexpr int kMaxTreeEntries = kMaxDof * (kMaxDof + 1) / 2;
+struct DofLists {
+  int off[kMaxDof];
+  int dep[kMaxDof];
+  int order[kMaxDof];
+  int level[kMaxDof + 1];
+  int anc[kMaxTreeEntries];
+};
+
 // Everything a kernel needs to find the model; passed by value.
 struct ModelView {
   const BodyC* c;        // device, n entries
@@ -101,6 +118,10 @@ constexpr int kAbaLeanRingFloats = 27;
 // the composite-inertia contribution to the parent (10).
 constexpr int kCrbaLeanBodyFloats = 18;
 constexpr int kCrbaLeanRingFloats = 10;
+
+// Shared state per body and environment of the dense derivatives in aligned
+// frames (aligned.cuh).
+constexpr int kDerivState = 49;
 
 // Operators of the fused evaluation kernel, in launch order (longest first,
 // so the slowest role's blocks are dispatched first).

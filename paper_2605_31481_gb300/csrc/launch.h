@@ -147,6 +147,17 @@ cudaError_t launch_jac_vjp(const ModelView& mv, int64_t B, const float* q, const
                            float* qbar, cudaStream_t s);
 cudaError_t launch_crba_vjp(const ModelView& mv, int64_t B, const float* q, const float* Mbar, float* qbar,
                             float* thbar, float* scratch, cudaStream_t s);
+// Aligned-frame kernels (aligned.cu), one tile of 32 environments per block
+// (block = 0: built-in choice). The *_smem functions give the shared memory a
+// launch needs: above kLevelSmemLimit the kernel cannot run. maxw = bodies of
+// the widest tree level; entries, dof_depth: see fst_model.
+size_t rnea_derivs_aligned_smem(const ModelView& mv);
+size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries);
+cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
+                                       const float* qdd, float* dq, float* dqd, int block, cudaStream_t s);
+cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
+                                      const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int maxw,
+                                      int entries, int dof_depth, int block, cudaStream_t s);
 cudaError_t launch_aba_level_pinned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                     const float* tau, float* qdd, int block, const PinArgs& p, cudaStream_t s);
 cudaError_t launch_aba_vjp(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,

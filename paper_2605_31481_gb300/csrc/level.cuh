@@ -576,7 +576,8 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
 template <class TP>
 __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& tau,
                                                const LaneState& S, const LaneState& R, int maxw,
-                                               float* __restrict__ qdd, int64_t B, int64_t e, bool act) {
+                                               float* __restrict__ qdd, int64_t B, int64_t e, bool act,
+                                               float* qdd_col = nullptr) {
   const int W = n_warps(), w = warp_id();
   enum { VU_ = 0, C_ = 6, ID_ = 12, u_ = 13 };  // per body
   enum { RI_ = 0, RP_ = 21 };                      // per ring slot
@@ -658,17 +659,19 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
       SV ai = X_motion(joint_X(tp.C(i), bi, q), ap) + S.sv(i, C_);
       if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
         const float qi = (*S.at(i, u_) - dot(S.sv(i, VU_), ai)) * *S.at(i, ID_);
-        if (act) qdd[(int64_t)bi.vi * B + e] = qi;
+        if (act && qdd) qdd[(int64_t)bi.vi * B + e] = qi;
+        if (qdd_col) qdd_col[bi.vi << 5] = qi;
         ai = ai + qi * S_of(tp.C(i));
       } else if (bi.type == FST_JOINT_FREE) {
         const int slot = k - tp.level_begin(l);  // level 0: ring parity 0
         const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};
         const SV anew = sym6_solve(R.sym(slot, RI_), tf - R.sv(slot, RP_));
         const SV x = anew - ai;
-        if (act) {
-          const float xo[6] = {x.v.x, x.v.y, x.v.z, x.w.x, x.w.y, x.w.z};
+        const float xo[6] = {x.v.x, x.v.y, x.v.z, x.w.x, x.w.y, x.w.z};
 #pragma unroll
-          for (int r = 0; r < 6; ++r) qdd[(int64_t)(bi.vi + r) * B + e] = xo[r];
+        for (int r = 0; r < 6; ++r) {
+          if (act && qdd) qdd[(int64_t)(bi.vi + r) * B + e] = xo[r];
+          if (qdd_col) qdd_col[(bi.vi + r) << 5] = xo[r];
         }
         ai = anew;
       }

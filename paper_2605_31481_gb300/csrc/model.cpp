@@ -237,6 +237,32 @@ fst_status build_model_host(const fst_body_desc* bodies, int32_t n, const double
       if (bodies[j].parent == i) T.child[k++] = j;
   }
   T.child_start[n] = k;
+  // the tree of the degrees of freedom
+  DofLists& D = m->hd;
+  std::vector<int> par(nv, -1), last(n, -1);  // parent of each; the last one on each body's support path
+  for (int i = 0; i < n; ++i) {
+    const int p = m->hi[i].parent;
+    last[i] = p < 0 ? -1 : last[p];
+    const int ni = m->hi[i].type == FST_JOINT_FREE ? 6 : (m->hi[i].type == FST_JOINT_FIXED ? 0 : 1);
+    for (int j = 0; j < ni; ++j) {
+      par[m->hi[i].vi + j] = last[i];
+      last[i] = m->hi[i].vi + j;
+    }
+  }
+  m->dof_depth = m->dof_entries = 0;
+  for (int c = 0; c < nv; ++c) {
+    D.off[c] = m->dof_entries;
+    for (int a = c; a >= 0; a = par[a]) D.anc[m->dof_entries++] = a;
+    D.dep[c] = m->dof_entries - D.off[c];
+    m->dof_depth = std::max(m->dof_depth, D.dep[c]);
+  }
+  k = 0;
+  for (int l = 0; l < m->dof_depth; ++l) {
+    D.level[l] = k;
+    for (int c = 0; c < nv; ++c)
+      if (D.dep[c] == l + 1) D.order[k++] = c;
+  }
+  D.level[m->dof_depth] = k;
   return FST_OK;
 }
 
