@@ -116,6 +116,78 @@ __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, i
   }
 }
 
+// The adjoint of inverse dynamics and the identification loss with its
+// gradient. Bound by latency: shared memory holds one tile of the humanoid
+// (172 KB) or two of the quadruped per SM. The one-thread-per-environment
+// kernel ran all sweeps in series with their state in local memory and 50
+// shuffles per body for the parameter gradient: humanoid, B = 65536: 310 ->
+// 160 us; arm, B = 8192, loss and gradient: 16.0 -> 12.0 us (the specialised
+// kernel against this one).
+template <int MODE>
+__global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                               const float* __restrict__ qd,
+                                                               const float* __restrict__ qdd, const float* tb,
+                                                               float* qbar, float* qdbar, float* qddbar,
+                                                               float* partial) {
+  FST_TILE;
+  const int nv = mv.nv, P = mv.n * 10 + (MODE == VJP_LOSS ? 1 : 0);
+  stage_block_rows(tile, q, mv.nq, B, e);
+  stage_block_rows(tile + mv.nq * kLaneEnvs, qd, nv, B, e);
+  stage_block_rows(tile + (mv.nq + nv) * kLaneEnvs, qdd, nv, B, e);
+  stage_block_rows(tile + (mv.nq + 2 * nv) * kLaneEnvs, tb, nv, B, e);
+  const SmemModel sm = stage_model(mv, smem);
+  const LaneState S{tile + (mv.nq + 3 * nv) * kLaneEnvs, kVjpState};
+  float* const th = partial ? partial + (int64_t)blockIdx.x * P : nullptr;
+  const VjpAligned o{nullptr, qbar, qdbar, qddbar, th, 1.f};
+  float loss = rnea_vjp_aligned<MODE>(sm, world_accel(mv), tile_col(tile, 0), tile_col(tile, mv.nq),
+                                      tile_col(tile, mv.nq + nv), tile + (mv.nq + 2 * nv) * kLaneEnvs + lane, S, o, B,
+                                      e, act);
+  if (MODE == VJP_LOSS) {
+    __shared__ float wsum[16];
+    loss = act ? loss : 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, off);
+    if (lane == 0) wsum[warp_id()] = loss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float s = 0.f;
+      for (int k = 0; k < n_warps(); ++k) s += wsum[k];
+      th[P - 1] = s;
+    }
+  }
+}
+
+// The ABA adjoint in one launch: lambda = M^-1 qddbar by the lean
+// level-parallel ABA at rest and without gravity, then minus the adjoint of
+// inverse dynamics at (q, qd, qdd) for the cotangent lambda. Quadruped,
+// B = 5001: 20.2 us, the specialised one-thread-per-environment kernel 41.9.
+__global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                              const float* __restrict__ qd,
+                                                              const float* __restrict__ qdd,
+                                                              const float* __restrict__ qddbar, float* qbar,
+                                                              float* qdbar, float* taubar, float* partial, int maxw) {
+  FST_TILE;
+  const int nv = mv.nv;
+  // rows: q | qd | qdd | qddbar | lambda | one row of zeros
+  stage_block_rows(tile, q, mv.nq, B, e);
+  stage_block_rows(tile + mv.nq * kLaneEnvs, qd, nv, B, e);
+  stage_block_rows(tile + (mv.nq + nv) * kLaneEnvs, qdd, nv, B, e);
+  stage_block_rows(tile + (mv.nq + 2 * nv) * kLaneEnvs, qddbar, nv, B, e);
+  const int rows = mv.nq + 4 * nv + 1;
+  float* const zero = tile + (rows - 1) * kLaneEnvs + lane;
+  if (threadIdx.x < 32) *zero = 0.f;
+  const SmemModel sm = stage_model(mv, smem);
+  float* const state = tile + rows * kLaneEnvs;
+  float* const lam = tile + (mv.nq + 3 * nv) * kLaneEnvs + lane;
+  const Col cq = tile_col(tile, 0);
+  aba_level_lean(sm, sv_zero(), cq, Col{zero, 0}, tile_col(tile, mv.nq + 2 * nv), LaneState{state, kAbaLeanBodyFloats},
+                 LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, taubar, B, e, act,
+                 lam);
+  const VjpAligned o{nullptr, qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
+  rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, tile_col(tile, mv.nq), tile_col(tile, mv.nq + nv), lam,
+                              LaneState{state, kVjpState}, o, B, e, act);
+}
+
 size_t floats32(size_t f) { return f * kLaneEnvs * sizeof(float); }
 
 // Per-body state that also holds the lean ABA's (run before it in the same space).
@@ -136,6 +208,14 @@ int aligned_block(int set, int n, int64_t tiles) {
 
 size_t rnea_derivs_aligned_smem(const ModelView& mv) {
   return smem_bytes(mv.n) + floats32((size_t)mv.nq + 2 * mv.nv + (size_t)kDerivState * mv.n);
+}
+
+size_t rnea_vjp_aligned_smem(const ModelView& mv) {
+  return smem_bytes(mv.n) + floats32((size_t)mv.nq + 3 * mv.nv + (size_t)kVjpState * mv.n);
+}
+
+size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw) {
+  return smem_bytes(mv.n) + floats32((size_t)mv.nq + 4 * mv.nv + 1 + state_with_aba(mv.n, maxw, kVjpState));
 }
 
 // The forward-dynamics derivatives' solve phase keeps two columns per warp in
@@ -172,6 +252,45 @@ cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const floa
   aba_derivs_aligned_kernel<<<tiles, aba_derivs_threads(mv, maxw, block, tiles), sh, s>>>(
       mv, B, q, qd, tau, qdd, dq, dqd, Minv, maxw, entries, dof_depth, (int)state_with_aba(mv.n, maxw, kDerivState));
   return cudaGetLastError();
+}
+
+cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                    const float* tbar, float* qbar, float* qdbar, float* qddbar, float* thbar,
+                                    float* scratch, int block, cudaStream_t s) {
+  const size_t sh = rnea_vjp_aligned_smem(mv);
+  const unsigned tiles = grid_for(B, kLaneEnvs);
+  prepare(rnea_vjp_aligned_kernel<VJP_GIVEN>, sh);
+  rnea_vjp_aligned_kernel<VJP_GIVEN><<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(
+      mv, B, q, qd, qdd, tbar, qbar, qdbar, qddbar, thbar ? scratch : nullptr);
+  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
+  return err;
+}
+
+cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                     const float* tau_meas, float* loss_theta, float* qbar, float* qdbar,
+                                     float* scratch, int block, cudaStream_t s) {
+  const size_t sh = rnea_vjp_aligned_smem(mv);
+  const unsigned tiles = grid_for(B, kLaneEnvs);
+  prepare(rnea_vjp_aligned_kernel<VJP_LOSS>, sh);
+  rnea_vjp_aligned_kernel<VJP_LOSS><<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(
+      mv, B, q, qd, qdd, tau_meas, qbar, qdbar, nullptr, scratch);
+  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10 + 1, loss_theta, s);
+  return err;
+}
+
+cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                   const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
+                                   float* scratch, int maxw, int block, cudaStream_t s) {
+  const size_t sh = aba_vjp_aligned_smem(mv, maxw);
+  const unsigned tiles = grid_for(B, kLaneEnvs);
+  prepare(aba_vjp_aligned_kernel, sh);
+  aba_vjp_aligned_kernel<<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(mv, B, q, qd, qdd, qddbar, qbar, qdbar,
+                                                                             taubar, thbar ? scratch : nullptr, maxw);
+  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
+  return err;
 }
 
 }  // namespace fst

@@ -36,6 +36,7 @@
 // with v_k = (omega, nu), so a subtree's B is 12 numbers.
 #pragma once
 
+#include "adjoint.cuh"
 #include "level.cuh"
 
 namespace fst {
@@ -68,6 +69,12 @@ __device__ __forceinline__ In10 in_shift(const In10& I, f3 r) {
   o.I[4] = I.I[4] - fmaf(z.y, r.z, r.y * z.z);
   o.I[5] = I.I[5] + (d - 2.0f * z.z * r.z);
   return o;
+}
+
+// S x with S = tr(I_o)/2 1 - I_o
+__device__ __forceinline__ f3 second_moment_mul(const In10& I, f3 x) {
+  const float ht = 0.5f * (I.I[0] + I.I[2] + I.I[5]);
+  return ht * x - sym_mul(I.I, x);
 }
 
 // The velocity operator of a body or subtree (see above).
@@ -373,6 +380,317 @@ __device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, 
       }
     }
   }
+}
+
+// ---- the adjoint of inverse dynamics ------------------------------------------
+// For the cotangent tbar of tau let w_k be the velocity that tbar would give
+// body k as a joint velocity. Then L = sum_k w_k . f_k, and with f, A = I w and
+// H = 2 B^T w (angular only, 3 numbers) summed over j's subtree
+//     qbar_j   = (w x psi_j) . f + psidd_j . A + psid_j . H   (w of the parent)
+//     qdbar_j  = eta_j . A + psi_j . H
+//     qddbar_j = psi_j . A,
+// so the reverse sweep is one sum of 15 numbers up the tree. The gradient in
+// the inertial parameters is local to a body: the contraction of (w, a) and
+// (w x v, v), turned back to body axes.
+// Floats of shared state per body and environment (kVjpState = 51):
+// psi 6 | R 9 | r 3 | v 6 | a 6 | w 6 | f 6 | A 6 | H 3.
+
+// Where the cotangent comes from.
+enum VjpMode {
+  VJP_GIVEN = 0,  // staged in tb
+  VJP_LOSS,       // tb holds measured torques; the cotangent is 2 (tau - tb) and *loss their squared norm
+  VJP_TAU         // the cotangent is tau itself
+};
+
+struct VjpAligned {
+  float* tau;      // [nv][B] or null (VJP_LOSS, VJP_TAU)
+  float* qbar;     // [nq][B] or null
+  float* qdbar;    // [nv][B] or null
+  float* qddbar;   // [nv][B] or null
+  float* thbar;    // this tile's [n][10] partial sums in global memory, or null
+  float sign;      // multiplies every cotangent
+};
+
+// Sums each of 10 values over the warp: halving the set of values a lane
+// still carries at every step takes 16 shuffles instead of 50. The sum of
+// value k ends in lanes whose bits 4, 3, 2, 1 spell k.
+__device__ __forceinline__ void warp_sum10_store(const float* g, float* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  float v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = k < 10 ? g[k] : 0.f;
+#pragma unroll
+  for (int half = 8; half >= 1; half >>= 1) {
+    const bool hi = lane & (2 * half);
+#pragma unroll
+    for (int k = 0; k < half; ++k) {
+      const float send = hi ? v[k] : v[k + half];
+      v[k] = (hi ? v[k + half] : v[k]) + __shfl_xor_sync(0xffffffffu, send, 2 * half);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  const int k = lane >> 1;
+  if ((lane & 1) == 0 && k < 10) out[k] = v[0];
+}
+
+// d/dtheta of y . (I x), accumulated in g in the order of the 10 parameters,
+// for vectors in the axes of the caller (theta_contract's formulas).
+__device__ __forceinline__ void inertia_contract(SV y, SV x, float* g) {
+  g[0] += dot(y.v, x.v);
+  const f3 dh = cross(x.v, y.w) - cross(x.w, y.v);
+  g[1] += dh.x;
+  g[2] += dh.y;
+  g[3] += dh.z;
+  g[4] = fmaf(y.w.x, x.w.x, g[4]);
+  g[5] = fmaf(y.w.x, x.w.y, fmaf(y.w.y, x.w.x, g[5]));
+  g[6] = fmaf(y.w.y, x.w.y, g[6]);
+  g[7] = fmaf(y.w.x, x.w.z, fmaf(y.w.z, x.w.x, g[7]));
+  g[8] = fmaf(y.w.y, x.w.z, fmaf(y.w.z, x.w.y, g[8]));
+  g[9] = fmaf(y.w.z, x.w.z, g[9]);
+}
+
+// The same gradient for the parameters in axes turned by R (in = R body).
+__device__ __forceinline__ void inertia_grad_to_body(const float* R, float* g) {
+  const f3 h = RTmul(R, f3{g[1], g[2], g[3]});
+  g[1] = h.x;
+  g[2] = h.y;
+  g[3] = h.z;
+  const float G[6] = {g[4], 0.5f * g[5], g[6], 0.5f * g[7], 0.5f * g[8], g[9]};
+  const float Rt[9] = {R[0], R[3], R[6], R[1], R[4], R[7], R[2], R[5], R[8]};
+  float o[6];
+  sym_rot(Rt, G, o);
+  g[4] = o[0];
+  g[5] = 2.f * o[1];
+  g[6] = o[2];
+  g[7] = 2.f * o[3];
+  g[8] = 2.f * o[4];
+  g[9] = o[5];
+}
+
+// One tile of 32 environments. The caller has staged q, qd, qdd and, for
+// VJP_GIVEN and VJP_LOSS, tb ([nv] rows of 32; VJP_TAU and VJP_LOSS write the
+// cotangent there). Returns this thread's share of the loss (VJP_LOSS).
+template <int MODE>
+__device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, const Col& q, const Col& qd,
+                                                  const Col& qdd, float* tbcol, const LaneState& S,
+                                                  const VjpAligned& o, int64_t B, int64_t e, bool act) {
+  const int W = n_warps(), w = warp_id(), n = tp.n();
+  enum { PSI = 0, R_ = 6, RR = 15, V_ = 18, A_ = 24, W_ = 30, F_ = 36, AS_ = 42, H_ = 48 };
+  const Col tb{tbcol, kLaneEnvs};
+  float loss = 0.f;
+  for (int i = w; i < n; i += W) S.putX(i, R_, joint_X(tp.C(i), tp.I(i), q));  // R 9 | r 3
+  __syncthreads();
+  // down the tree: rotations, velocities, accelerations (and w when tb is known)
+  for (int l = 0; l < tp.depth(); ++l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const Xf X = S.X(i, R_);
+      if (bi.type == FST_JOINT_FREE) {  // the root frame is this body's own
+        const float Id[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
+        S.put_n(i, R_, Id, 9);
+        S.put(i, V_, S_times(tp.C(i), bi, qd));
+        S.put(i, A_, S_times(tp.C(i), bi, qdd) + SV{f3{0.f, 0.f, 0.f}, RTmul(X.R, a0.v)});
+        if (MODE == VJP_GIVEN) S.put(i, W_, S_times(tp.C(i), bi, tb));
+        continue;
+      }
+      SV vl = sv_zero(), al = a0, wl = sv_zero();
+      float R[9];
+      if (bi.parent < 0) {
+#pragma unroll
+        for (int c = 0; c < 9; ++c) R[c] = X.R[c];
+      } else {
+        float Rp[9], rr[3];
+        S.get_n(bi.parent, R_, Rp, 9);
+        const float zero[3] = {0.f, 0.f, 0.f};
+        compose(Rp, zero, X, R, rr);
+        const f3 r = f3{rr[0], rr[1], rr[2]};
+        S.put_n(i, RR, rr, 3);
+        S.put_n(i, R_, R, 9);
+        vl = shift_motion(S.sv(bi.parent, V_), r);
+        al = shift_motion(S.sv(bi.parent, A_), r);
+        if (MODE == VJP_GIVEN) wl = shift_motion(S.sv(bi.parent, W_), r);
+      }
+      if (one_dof(bi)) {
+        const SV psi = psi_of(tp.C(i), R);
+        S.put(i, PSI, psi);
+        const SV psd = crm(vl, psi);
+        vl = vl + qd[bi.vi] * psi;
+        al = al + (qdd[bi.vi] * psi + qd[bi.vi] * psd);
+        if (MODE == VJP_GIVEN) wl = wl + tb[bi.vi] * psi;
+      }
+      S.put(i, V_, vl);
+      S.put(i, A_, al);
+      if (MODE == VJP_GIVEN) S.put(i, W_, wl);
+    }
+    __syncthreads();
+  }
+  // the cotangent's velocity, force functionals and parameter gradient of a body
+  auto local_adjoint = [&](int i, const float* R, const In10& I, SV v, SV a, SV hv) {
+    const SV wv = S.sv(i, W_);
+    S.put(i, AS_, in_mul(I, wv));
+    const f3 H = 2.f * (second_moment_mul(I, cross(v.w, wv.w)) +
+                        (dot(I.h, v.v) * wv.w - dot(v.v, wv.w) * I.h) - cross(wv.v, hv.v));
+    const float Hn[3] = {H.x, H.y, H.z};
+    S.put_n(i, H_, Hn, 3);
+    if (o.thbar) {
+      float g[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+      inertia_contract(wv, a, g);
+      inertia_contract(crm(wv, v), v, g);
+      inertia_grad_to_body(R, g);
+#pragma unroll
+      for (int c = 0; c < 10; ++c) g[c] = act ? o.sign * g[c] : 0.f;
+      warp_sum10_store(g, o.thbar + 10 * i);
+    }
+  };
+  for (int i = w; i < n; i += W) {
+    float R[9];
+    S.get_n(i, R_, R, 9);
+    const SV v = S.sv(i, V_), a = S.sv(i, A_);
+    const In10 I = in_rotate(R, in_load(tp.theta(i)));
+    const SV hv = in_mul(I, v);
+    S.put(i, F_, in_mul(I, a) + crf(v, hv));
+    if (MODE == VJP_GIVEN) local_adjoint(i, R, I, v, a, hv);
+  }
+  __syncthreads();
+  if (MODE != VJP_GIVEN) {
+    // forces up the tree, tau and the cotangent, then its velocity down the tree
+    for (int l = tp.depth() - 1; l >= 0; --l) {
+      FST_FOR_MY_BODIES(tp, l, k) {
+        const int i = tp.level_body(k);
+        const BodyI bi = tp.I(i);
+        SV f = S.sv(i, F_);
+        for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
+          const int c = tp.child(ch);
+          float t3[3];
+          S.get_n(c, RR, t3, 3);
+          f = f + shift_force(S.sv(c, F_), f3{t3[0], t3[1], t3[2]});
+        }
+        S.put(i, F_, f);
+        const int ni = nv_of(bi.type);
+        float tau[6];
+        if (ni == 1) {
+          tau[0] = dot(S.sv(i, PSI), f);
+        } else {
+          tau[0] = f.v.x, tau[1] = f.v.y, tau[2] = f.v.z;
+          tau[3] = f.w.x, tau[4] = f.w.y, tau[5] = f.w.z;
+        }
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+          if (r >= ni) break;
+          float* tr = tbcol + (bi.vi + r) * kLaneEnvs;
+          if (o.tau && act) o.tau[(int64_t)(bi.vi + r) * B + e] = tau[r];
+          if (MODE == VJP_LOSS) {
+            const float res = tau[r] - *tr;
+            loss = fmaf(res, res, loss);
+            *tr = 2.f * res;
+          } else {
+            *tr = tau[r];
+          }
+        }
+      }
+      __syncthreads();
+    }
+    for (int l = 0; l < tp.depth(); ++l) {
+      FST_FOR_MY_BODIES(tp, l, k) {
+        const int i = tp.level_body(k);
+        const BodyI bi = tp.I(i);
+        SV wl = sv_zero();
+        if (bi.type == FST_JOINT_FREE) {
+          wl = S_times(tp.C(i), bi, tb);
+        } else {
+          if (bi.parent >= 0) {
+            float t3[3];
+            S.get_n(i, RR, t3, 3);
+            wl = shift_motion(S.sv(bi.parent, W_), f3{t3[0], t3[1], t3[2]});
+          }
+          if (one_dof(bi)) wl = wl + tb[bi.vi] * S.sv(i, PSI);
+        }
+        S.put(i, W_, wl);
+      }
+      __syncthreads();
+    }
+    for (int i = w; i < n; i += W) {
+      float R[9];
+      S.get_n(i, R_, R, 9);
+      const SV v = S.sv(i, V_);
+      const In10 I = in_rotate(R, in_load(tp.theta(i)));
+      local_adjoint(i, R, I, v, S.sv(i, A_), in_mul(I, v));
+    }
+    __syncthreads();
+  }
+  if (!o.qbar && !o.qdbar && !o.qddbar) return loss;  // block-uniform: only the parameters were asked for
+  // up the tree: A and H (and f where it has not been summed yet)
+  for (int l = tp.depth() - 2; l >= 0; --l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const int c0 = tp.child_begin(i), c1 = tp.child_begin(i + 1);
+      if (c0 == c1) continue;
+      SV f = S.sv(i, F_), A = S.sv(i, AS_);
+      float H[3], t3[3];
+      S.get_n(i, H_, H, 3);
+      for (int ch = c0; ch < c1; ++ch) {
+        const int c = tp.child(ch);
+        S.get_n(c, RR, t3, 3);
+        const f3 r = f3{t3[0], t3[1], t3[2]};
+        A = A + shift_force(S.sv(c, AS_), r);
+        if (MODE == VJP_GIVEN) f = f + shift_force(S.sv(c, F_), r);
+        S.get_n(c, H_, t3, 3);
+        H[0] += t3[0];
+        H[1] += t3[1];
+        H[2] += t3[2];
+      }
+      S.put(i, AS_, A);
+      S.put_n(i, H_, H, 3);
+      if (MODE == VJP_GIVEN) S.put(i, F_, f);
+    }
+    __syncthreads();
+  }
+  if (!act) return loss;
+  for (int i = w; i < n; i += W) {
+    const BodyI bi = tp.I(i);
+    if (nv_of(bi.type) == 0) continue;
+    const SV A = S.sv(i, AS_);
+    float t3[3];
+    S.get_n(i, H_, t3, 3);
+    const f3 H = f3{t3[0], t3[1], t3[2]};
+    if (bi.type == FST_JOINT_FREE) {
+      // v = S qd, a = X a0 + S qdd: q enters through gravity only
+      const SV y = crf(S.sv(i, V_), A);  // eta . A = -psi . (v_0 x* A)
+      const f3 g1 = RTmul(tp.C(i).R0, a0.v);
+      const float G[9] = {g1.x * A.v.x, g1.x * A.v.y, g1.x * A.v.z, g1.y * A.v.x, g1.y * A.v.y,
+                          g1.y * A.v.z, g1.z * A.v.x, g1.z * A.v.y, g1.z * A.v.z};
+      float gq[4];
+      quat_grad(q[bi.qi + 3], q[bi.qi + 4], q[bi.qi + 5], q[bi.qi + 6], G, gq);
+      const float qo[7] = {0.f, 0.f, 0.f, gq[0], gq[1], gq[2], gq[3]};
+      const float vo[6] = {-y.v.x, -y.v.y, -y.v.z, H.x - y.w.x, H.y - y.w.y, H.z - y.w.z};
+      const float ao[6] = {A.v.x, A.v.y, A.v.z, A.w.x, A.w.y, A.w.z};
+#pragma unroll
+      for (int r = 0; r < 7; ++r) store_if(o.qbar, bi.qi + r, B, e, o.sign * qo[r], true);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        store_if(o.qdbar, bi.vi + r, B, e, o.sign * vo[r], true);
+        store_if(o.qddbar, bi.vi + r, B, e, o.sign * ao[r], true);
+      }
+      continue;
+    }
+    SV vl = sv_zero(), al = a0, wl = sv_zero();
+    if (bi.parent >= 0) {
+      S.get_n(i, RR, t3, 3);
+      const f3 r = f3{t3[0], t3[1], t3[2]};
+      vl = shift_motion(S.sv(bi.parent, V_), r);
+      al = shift_motion(S.sv(bi.parent, A_), r);
+      wl = shift_motion(S.sv(bi.parent, W_), r);
+    }
+    const SV psi = S.sv(i, PSI);
+    const SV psd = crm(vl, psi);
+    const SV psdd = crm(al, psi) + crm(vl, psd);
+    store_if(o.qbar, bi.qi, B, e,
+             o.sign * (dot(crm(wl, psi), S.sv(i, F_)) + dot(psdd, A) + dot(psd.w, H)), true);
+    store_if(o.qdbar, bi.vi, B, e, o.sign * fmaf(2.f, dot(psd, A), dot(psi.w, H)), true);
+    store_if(o.qddbar, bi.vi, B, e, o.sign * dot(psi, A), true);
+  }
+  return loss;
 }
 
 // ---- forward-dynamics derivatives: the tree-sparse factorisation ----------------

@@ -96,7 +96,9 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 // default unless the kind is pinned to another variant or the tree's state
 // does not fit in shared memory (`need` bytes; about 33 bodies). There is no
 // line in B: the aligned kernels were the faster ones at every size measured,
-// against the generic and the specialised kernels: derivatives 3 to 20 times.
+// against the generic and the specialised kernels (us): arm7 RNEA adjoint
+// B = 32768 27 / 26-40, quadruped B = 16384 25 / 43, humanoid B = 512 14 / 66;
+// derivatives 3 to 20 times faster everywhere.
 bool aligned_fits(const fst_model* m, int kind, size_t need) {
   return m->variant[kind] == FST_VARIANT_AUTO && need + 1024 <= kLevelSmemLimit;  // 1 KB: static shared memory
 }
@@ -750,6 +752,9 @@ fst_status fst_rnea_vjp(const fst_model* m, int64_t B, const float* q, const flo
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, tau_bar, "tau_bar"));
   const ModelView mv = view_of(m, theta);
+  if (aligned_fits(m, JK_RNEA_VJP, rnea_vjp_aligned_smem(mv)))
+    return finish(fn, launch_rnea_vjp_aligned(mv, B, q, qd, qdd, tau_bar, q_bar, qd_bar, qdd_bar, theta_bar,
+                                              (float*)scratch, m->block[JK_RNEA_VJP], (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_VJP)) {
     unsigned nblk = 0;
     float* partial = theta_bar ? (float*)scratch : nullptr;
@@ -918,6 +923,10 @@ fst_status fst_aba_vjp(const fst_model* m, int64_t B, const float* q, const floa
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, qdd_bar, "qdd_bar"));
   const ModelView mv = view_of(m, theta);
+  if (aligned_fits(m, JK_ABA_VJP, aba_vjp_aligned_smem(mv, m->max_width)))
+    return finish(fn, launch_aba_vjp_aligned(mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
+                                             (float*)scratch, m->max_width, m->block[JK_ABA_VJP],
+                                             (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_VJP)) {
     unsigned nblk = 0;
     float* partial = theta_bar ? (float*)scratch : nullptr;
@@ -947,6 +956,9 @@ fst_status fst_rnea_loss_grad(const fst_model* m, int64_t B, const float* q, con
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, tau_meas, "tau_meas"));
   const ModelView mv = view_of(m, theta);
+  if (aligned_fits(m, JK_LOSS_GRAD, rnea_vjp_aligned_smem(mv)))
+    return finish(fn, launch_loss_grad_aligned(mv, B, q, qd, qdd, tau_meas, loss_theta_bar, q_bar, qd_bar,
+                                               (float*)scratch, m->block[JK_LOSS_GRAD], (cudaStream_t)stream));
   if (use_jit(m, JK_LOSS_GRAD)) {
     unsigned nblk = 0;
     const int P = m->n * 10 + 1;

@@ -119,9 +119,10 @@ constexpr int kAbaLeanRingFloats = 27;
 constexpr int kCrbaLeanBodyFloats = 18;
 constexpr int kCrbaLeanRingFloats = 10;
 
-// Shared state per body and environment of the dense derivatives in aligned
-// frames (aligned.cuh).
+// Shared state per body and environment of the dense derivatives and of the
+// adjoint in aligned frames (aligned.cuh).
 constexpr int kDerivState = 49;
+constexpr int kVjpState = 51;
 
 // Operators of the fused evaluation kernel, in launch order (longest first,
 // so the slowest role's blocks are dispatched first).

@@ -153,11 +153,22 @@ cudaError_t launch_crba_vjp(const ModelView& mv, int64_t B, const float* q, cons
 // the widest tree level; entries, dof_depth: see fst_model.
 size_t rnea_derivs_aligned_smem(const ModelView& mv);
 size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries);
+size_t rnea_vjp_aligned_smem(const ModelView& mv);
+size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw);
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                        const float* qdd, float* dq, float* dqd, int block, cudaStream_t s);
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                       const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int maxw,
                                       int entries, int dof_depth, int block, cudaStream_t s);
+cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                    const float* tbar, float* qbar, float* qdbar, float* qddbar, float* thbar,
+                                    float* scratch, int block, cudaStream_t s);
+cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                     const float* tau_meas, float* loss_theta, float* qbar, float* qdbar,
+                                     float* scratch, int block, cudaStream_t s);
+cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                   const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
+                                   float* scratch, int maxw, int block, cudaStream_t s);
 cudaError_t launch_aba_level_pinned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                     const float* tau, float* qdd, int block, const PinArgs& p, cudaStream_t s);
 cudaError_t launch_aba_vjp(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
