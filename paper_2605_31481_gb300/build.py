@@ -34,6 +34,11 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found: the CUDA toolkit is required to build libfst.so")
 
 
+# The tile kernels (level.cuh, aligned.cuh) are instantiated in several units and
+# entry points that must agree bit for bit: products and sums are fused only
+# where the source says fmaf, so the surrounding code cannot change a rounding.
+UNIT_FLAGS = {f: ["-fmad=false"] for f in ("aligned.cu", "level.cu", "multi_level.cu")}
+
 # Device headers embedded into the library for run-time specialisation
 # (NVRTC compiles them again for one fixed tree; see csrc/jit.cpp).
 JIT_HEADERS = ["fst_layout.h", "fst_device.cuh", "ops.cuh", "adjoint.cuh", "derivs.cuh", "level.cuh", "pathpar.cuh", "jit_kernels.cuh"]
@@ -76,6 +81,7 @@ def _headers_digest() -> str:
 
 def _compile(nvcc, src, flags, hdr, force):
     path = os.path.join(BUILD if src == EMBED else CSRC, src)
+    flags = flags + UNIT_FLAGS.get(src, [])
     obj = os.path.join(BUILD, src + ".o")
     stamp = obj + ".stamp"
     with open(path, "rb") as fh:

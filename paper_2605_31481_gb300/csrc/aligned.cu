@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int
   const SmemModel sm = stage_model(mv, smem);
   const LaneState S{tile + (mv.nq + 3 * nv) * kLaneEnvs, kVjpState};
   float* const th = partial ? partial + (int64_t)blockIdx.x * P : nullptr;
-  const VjpAligned o{nullptr, qbar, qdbar, qddbar, th, 1.f};
+  const VjpAligned o{qbar, qdbar, qddbar, th, 1.f};
   float loss = rnea_vjp_aligned<MODE>(sm, world_accel(mv), tile_col(tile, 0), tile_col(tile, mv.nq),
                                       tile_col(tile, mv.nq + nv), tile + (mv.nq + 2 * nv) * kLaneEnvs + lane, S, o, B,
                                       e, act);
@@ -183,9 +183,74 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
   aba_level_lean(sm, sv_zero(), cq, Col{zero, 0}, tile_col(tile, mv.nq + 2 * nv), LaneState{state, kAbaLeanBodyFloats},
                  LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, taubar, B, e, act,
                  lam);
-  const VjpAligned o{nullptr, qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
+  const VjpAligned o{qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
   rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, tile_col(tile, mv.nq), tile_col(tile, mv.nq + nv), lam,
                               LaneState{state, kVjpState}, o, B, e, act);
+}
+
+// The store variant's forward: RNEA that also leaves its state on the tape.
+__global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                              const float* __restrict__ qd,
+                                                              const float* __restrict__ qdd, float* __restrict__ tau,
+                                                              float* tape) {
+  FST_TILE;
+  stage_block_rows(tile, q, mv.nq, B, e);
+  stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
+  stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
+  const SmemModel sm = stage_model(mv, smem);
+  rnea_level(sm, world_accel(mv), tile_col(tile, 0), tile_col(tile, mv.nq), tile_col(tile, mv.nq + mv.nv),
+             LaneState{tile + (mv.nq + 2 * mv.nv) * kLaneEnvs, kRneaState}, tau, B, e, act, nullptr, tape);
+}
+
+// ---- fused evaluation ----------------------------------------------------------
+// blockIdx.y picks the operator of a block, blockIdx.x its tile; the bodies
+// are those of the per-operator kernels, so the results are theirs bit for
+// bit. Blocks of the heaviest operator come first. EXT (a kernel of its own,
+// so that the plain one keeps its registers): the RNEA adjoint beside tau, and
+// M and J in the packed layouts.
+template <bool EXT>
+__global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B, EvalArgs a, int maxw) {
+  FST_TILE;
+  const int role = a.roles[blockIdx.y], nv = mv.nv;
+  const bool vjp = EXT && role == ROLE_RNEA && (a.rnea_flags & EVAL_RNEA_VJP);
+  stage_block_rows(tile, a.q, mv.nq, B, e);
+  int rows = mv.nq;
+  if (role == ROLE_RNEA || role == ROLE_ABA) {
+    stage_block_rows(tile + rows * kLaneEnvs, a.qd, nv, B, e);
+    stage_block_rows(tile + (rows + nv) * kLaneEnvs, role == ROLE_ABA ? a.tau : a.qdd, nv, B, e);
+    if (vjp && !(a.rnea_flags & EVAL_TBAR_IS_TAU))
+      stage_block_rows(tile + (rows + 2 * nv) * kLaneEnvs, a.tau_bar, nv, B, e);
+    rows += (vjp ? 3 : 2) * nv;
+  }
+  const SmemModel sm = stage_model(mv, smem);
+  float* const state = tile + rows * kLaneEnvs;
+  const Col cq = tile_col(tile, 0), c1 = tile_col(tile, mv.nq), c2 = tile_col(tile, mv.nq + nv);
+  switch (role) {
+    case ROLE_ABA:
+      aba_level_lean(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
+                     LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, a.qdd_out, B,
+                     e, act);
+      break;
+    case ROLE_CRBA:
+      if (EXT && a.packed)
+        crba_level<true>(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
+      else
+        crba_level(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
+      break;
+    case ROLE_RNEA:
+      if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
+        rnea_level(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaState}, a.tau_out, B, e, act,
+                   vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
+      if (vjp)  // rnea_level ends with a barrier: the cotangent is complete and the state free
+        rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, c1, c2, tile + (mv.nq + 2 * nv) * kLaneEnvs + lane,
+                                    LaneState{state, kVjpState}, VjpAligned{a.qbar, a.qdbar, a.qddbar, nullptr, 1.f},
+                                    B, e, act);
+      break;
+    default:
+      kin_level(sm, cq, nv, a.links, LaneState{state, kFkState}, a.poses, a.J, B, e, act,
+                EXT && a.packed ? &a.pj : nullptr);
+      break;
+  }
 }
 
 size_t floats32(size_t f) { return f * kLaneEnvs * sizeof(float); }
@@ -232,6 +297,40 @@ size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries) {
   return smem_bytes(mv.n) +
          floats32((size_t)mv.nq + 3 * mv.nv + state_with_aba(mv.n, maxw, kDerivState) + entries) +
          ((size_t)4 * mv.nv + 1 + entries) * sizeof(int);
+}
+
+size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw) {
+  size_t f = mv.nq;
+  if (role == ROLE_ABA)
+    f += 2 * (size_t)mv.nv + (size_t)kAbaLeanBodyFloats * mv.n + (size_t)2 * kAbaLeanRingFloats * maxw;
+  else if (role == ROLE_CRBA)
+    f += (size_t)kCrbaState * mv.n;
+  else if (role == ROLE_RNEA)
+    f += (vjp ? 3 : 2) * (size_t)mv.nv + (size_t)(vjp ? kVjpState : kRneaState) * mv.n;
+  else
+    f += (size_t)kFkState * mv.n;
+  return smem_bytes(mv.n) + floats32(f);
+}
+
+cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                   float* tau, float* tape, int block, cudaStream_t s) {
+  const size_t sh = level_smem_needed(mv, LEVEL_RNEA);
+  prepare(rnea_store_tile_kernel, sh);
+  rnea_store_tile_kernel<<<grid_for(B, kLaneEnvs), block, sh, s>>>(mv, B, q, qd, qdd, tau, tape);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, size_t smem, int maxw, int block,
+                             cudaStream_t s) {
+  const dim3 grid(grid_for(B, kLaneEnvs), a.n_roles);
+  if (a.rnea_flags || a.packed) {
+    prepare(eval_tile_kernel<true>, smem);
+    eval_tile_kernel<true><<<grid, block, smem, s>>>(mv, B, a, maxw);
+  } else {
+    prepare(eval_tile_kernel<false>, smem);
+    eval_tile_kernel<false><<<grid, block, smem, s>>>(mv, B, a, maxw);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,

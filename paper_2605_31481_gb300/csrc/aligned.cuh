@@ -41,9 +41,8 @@
 
 namespace fst {
 
-// motion about the parent's origin -> about the child's, r = child - parent
+// motion about the parent's origin -> about the child's, and force back; r = child - parent
 __device__ __forceinline__ SV shift_motion(SV m, f3 r) { return SV{m.w, m.v + cross(m.w, r)}; }
-// force about the child's origin -> about the parent's
 __device__ __forceinline__ SV shift_force(SV f, f3 r) { return SV{f.w + cross(r, f.v), f.v}; }
 
 // A rigid-body inertia's axes rotated by R (no shift).
@@ -59,16 +58,27 @@ __device__ __forceinline__ In10 in_rotate(const float* R, const In10& I) {
 __device__ __forceinline__ In10 in_shift(const In10& I, f3 r) {
   In10 o;
   o.m = I.m;
-  o.h = I.h + I.m * r;
+  o.h = f3{fmaf(I.m, r.x, I.h.x), fmaf(I.m, r.y, I.h.y), fmaf(I.m, r.z, I.h.z)};
   const float d = fmaf(2.0f, dot(I.h, r), I.m * dot(r, r));
-  const f3 z = I.h + (0.5f * I.m) * r;  // h r^T + r h^T + m r r^T = z r^T + r z^T
-  o.I[0] = I.I[0] + (d - 2.0f * z.x * r.x);
+  const float hm = 0.5f * I.m;  // h r^T + r h^T + m r r^T = z r^T + r z^T
+  const f3 z = f3{fmaf(hm, r.x, I.h.x), fmaf(hm, r.y, I.h.y), fmaf(hm, r.z, I.h.z)};
+  o.I[0] = I.I[0] + fmaf(-2.0f * z.x, r.x, d);
   o.I[1] = I.I[1] - fmaf(z.x, r.y, r.x * z.y);
-  o.I[2] = I.I[2] + (d - 2.0f * z.y * r.y);
+  o.I[2] = I.I[2] + fmaf(-2.0f * z.y, r.y, d);
   o.I[3] = I.I[3] - fmaf(z.x, r.z, r.x * z.z);
   o.I[4] = I.I[4] - fmaf(z.y, r.z, r.y * z.z);
-  o.I[5] = I.I[5] + (d - 2.0f * z.z * r.z);
+  o.I[5] = I.I[5] + fmaf(-2.0f * z.z, r.z, d);
   return o;
+}
+
+// The motion subspace of a 1-DOF joint with its axes rotated
+__device__ __forceinline__ SV psi_of(const BodyC& c, const float* R) {
+  const SV s = S_of(c);
+  return SV{Rmul(R, s.w), Rmul(R, s.v)};
+}
+
+__device__ __forceinline__ bool one_dof(const BodyI& b) {
+  return b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC;
 }
 
 // S x with S = tr(I_o)/2 1 - I_o
@@ -127,16 +137,6 @@ __device__ __forceinline__ SV b_mul2(const BOp& b, f3 w) {
 // The functional x -> psi . 2 B x, which only sees x's angular part
 __device__ __forceinline__ f3 b_row2(const BOp& b, SV psi) {
   return 2.f * (RTmul(b.P, psi.w) + cross(psi.v, b.p));
-}
-
-// psi of a 1-DOF joint: its body-coordinate subspace with the axes rotated
-__device__ __forceinline__ SV psi_of(const BodyC& c, const float* R) {
-  const SV s = S_of(c);
-  return SV{Rmul(R, s.w), Rmul(R, s.v)};
-}
-
-__device__ __forceinline__ bool one_dof(const BodyI& b) {
-  return b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC;
 }
 
 // ---- dense derivatives of inverse dynamics ------------------------------------
@@ -219,8 +219,8 @@ __device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, 
         S.put(i, PSI, psi);
         S.put(i, PSD, psd);
         S.put(i, PSDD, crm(al, psi) + crm(vl, psd));
-        vl = vl + qd[bi.vi] * psi;
-        al = al + (qdd[bi.vi] * psi + qd[bi.vi] * psd);
+        al = sv_fma(qdd[bi.vi], psi, sv_fma(qd[bi.vi], psd, al));
+        vl = sv_fma(qd[bi.vi], psi, vl);
       }
       S.put(i, V_, vl);
       S.put(i, A_, al);
@@ -398,12 +398,10 @@ __device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, 
 // Where the cotangent comes from.
 enum VjpMode {
   VJP_GIVEN = 0,  // staged in tb
-  VJP_LOSS,       // tb holds measured torques; the cotangent is 2 (tau - tb) and *loss their squared norm
-  VJP_TAU         // the cotangent is tau itself
+  VJP_LOSS        // tb holds measured torques; the cotangent is 2 (tau - tb), the loss their squared difference
 };
 
 struct VjpAligned {
-  float* tau;      // [nv][B] or null (VJP_LOSS, VJP_TAU)
   float* qbar;     // [nq][B] or null
   float* qdbar;    // [nv][B] or null
   float* qddbar;   // [nv][B] or null
@@ -467,9 +465,8 @@ __device__ __forceinline__ void inertia_grad_to_body(const float* R, float* g) {
   g[9] = o[5];
 }
 
-// One tile of 32 environments. The caller has staged q, qd, qdd and, for
-// VJP_GIVEN and VJP_LOSS, tb ([nv] rows of 32; VJP_TAU and VJP_LOSS write the
-// cotangent there). Returns this thread's share of the loss (VJP_LOSS).
+// One tile of 32 environments. The caller has staged q, qd, qdd and
+// tb ([nv] rows of 32; VJP_LOSS writes the cotangent there). Returns this thread's share of the loss (VJP_LOSS).
 template <int MODE>
 __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, const Col& q, const Col& qd,
                                                   const Col& qdd, float* tbcol, const LaneState& S,
@@ -515,9 +512,9 @@ __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, co
         const SV psi = psi_of(tp.C(i), R);
         S.put(i, PSI, psi);
         const SV psd = crm(vl, psi);
-        vl = vl + qd[bi.vi] * psi;
-        al = al + (qdd[bi.vi] * psi + qd[bi.vi] * psd);
-        if (MODE == VJP_GIVEN) wl = wl + tb[bi.vi] * psi;
+        al = sv_fma(qdd[bi.vi], psi, sv_fma(qd[bi.vi], psd, al));
+        vl = sv_fma(qd[bi.vi], psi, vl);
+        if (MODE == VJP_GIVEN) wl = sv_fma(tb[bi.vi], psi, wl);
       }
       S.put(i, V_, vl);
       S.put(i, A_, al);
@@ -579,14 +576,9 @@ __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, co
         for (int r = 0; r < 6; ++r) {
           if (r >= ni) break;
           float* tr = tbcol + (bi.vi + r) * kLaneEnvs;
-          if (o.tau && act) o.tau[(int64_t)(bi.vi + r) * B + e] = tau[r];
-          if (MODE == VJP_LOSS) {
-            const float res = tau[r] - *tr;
-            loss = fmaf(res, res, loss);
-            *tr = 2.f * res;
-          } else {
-            *tr = tau[r];
-          }
+          const float res = tau[r] - *tr;
+          loss = fmaf(res, res, loss);
+          *tr = 2.f * res;
         }
       }
       __syncthreads();
@@ -604,7 +596,7 @@ __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, co
             S.get_n(i, RR, t3, 3);
             wl = shift_motion(S.sv(bi.parent, W_), f3{t3[0], t3[1], t3[2]});
           }
-          if (one_dof(bi)) wl = wl + tb[bi.vi] * S.sv(i, PSI);
+          if (one_dof(bi)) wl = sv_fma(tb[bi.vi], S.sv(i, PSI), wl);
         }
         S.put(i, W_, wl);
       }

@@ -1,6 +1,7 @@
 // C ABI of libfst.so: argument validation, device checks, launches.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <climits>
 #include <cstring>
@@ -101,6 +102,27 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 // derivatives 3 to 20 times faster everywhere.
 bool aligned_fits(const fst_model* m, int kind, size_t need) {
   return m->variant[kind] == FST_VARIANT_AUTO && need + 1024 <= kLevelSmemLimit;  // 1 KB: static shared memory
+}
+
+// Whether calls that keep the default variant run as tiles of 32 environments
+// whose warps share the bodies (level.cuh, aligned.cuh), for this model and
+// batch. The rule does not look at the operator, so every entry point that
+// computes one gives the same bits.
+bool tile_default(const fst_model* m, int64_t B) {
+  (void)m;
+  (void)B;
+  return true;
+}
+
+bool use_tile(const fst_model* m, int kind, int64_t B, size_t need) {
+  return m->variant[kind] == FST_VARIANT_AUTO && need <= kLevelSmemLimit && tile_default(m, B);
+}
+
+constexpr int kMultiTileBlock = 256;  // threads per block of the mixed-tree launch in tiles
+
+int tile_block(const fst_model* m, int kind) {
+  if (m->block[kind]) return m->block[kind];
+  return 256;
 }
 
 // The path-parallel kernel slot a call of this kind runs (0: none): 1 for
@@ -376,6 +398,8 @@ fst_status fst_fk(const fst_model* m, int64_t B, const float* q, float* poses, v
   if (use_level(m, JK_FK, LEVEL_FK))
     return finish(fn, launch_fk_level(mv, B, q, poses, level_block(m, JK_FK), level_tiles(m, JK_FK),
                         (cudaStream_t)stream));
+  if (use_tile(m, JK_FK, B, level_smem_needed(mv, LEVEL_FK)))
+    return finish(fn, launch_fk_level(mv, B, q, poses, tile_block(m, JK_FK), 1, (cudaStream_t)stream));
   if (use_path(m, JK_FK))
     return finish(fn, path_go(m, JK_FK, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, poses));
   if (use_jit(m, JK_FK))
@@ -404,6 +428,8 @@ fst_status fst_jacobian(const fst_model* m, int64_t B, const float* q, const int
   if (use_level(m, JK_JACOBIAN, LEVEL_JAC))
     return finish(fn, launch_jac_level(mv, B, q, L, J, level_block(m, JK_JACOBIAN), level_tiles(m, JK_JACOBIAN),
                         (cudaStream_t)stream));
+  if (use_tile(m, JK_JACOBIAN, B, level_smem_needed(mv, LEVEL_JAC)))
+    return finish(fn, launch_jac_level(mv, B, q, L, J, tile_block(m, JK_JACOBIAN), 1, (cudaStream_t)stream));
   if (use_path(m, JK_JACOBIAN))
     return finish(fn, path_go(m, JK_JACOBIAN, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, L, J));
   if (use_jit(m, JK_JACOBIAN))
@@ -425,6 +451,8 @@ fst_status fst_rnea(const fst_model* m, int64_t B, const float* q, const float* 
   if (use_level(m, JK_RNEA, LEVEL_RNEA))
     return finish(fn, launch_rnea_level(mv, B, q, qd, qdd, tau, level_block(m, JK_RNEA), level_tiles(m, JK_RNEA),
                         (cudaStream_t)stream));
+  if (use_tile(m, JK_RNEA, B, level_smem_needed(mv, LEVEL_RNEA)))
+    return finish(fn, launch_rnea_level(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA), 1, (cudaStream_t)stream));
   if (use_path(m, JK_RNEA))
     return finish(fn, path_go(m, JK_RNEA, B, m->nq + 2 * m->nv, 1, (cudaStream_t)stream, mv, B, q, qd, qdd, tau));
   if (use_jit(m, JK_RNEA))
@@ -447,6 +475,8 @@ fst_status fst_crba(const fst_model* m, int64_t B, const float* q, const float* 
   if (m->variant[JK_CRBA] == FST_VARIANT_LEVEL_LEAN && crba_lean_smem_needed(mv, m->max_width) <= kLevelSmemLimit)
     return finish(fn, launch_crba_level_lean(mv, B, q, M, level_block(m, JK_CRBA), m->max_width,
                                              (cudaStream_t)stream));
+  if (use_tile(m, JK_CRBA, B, level_smem_needed(mv, LEVEL_CRBA)))
+    return finish(fn, launch_crba_level(mv, B, q, M, tile_block(m, JK_CRBA), 1, (cudaStream_t)stream));
   if (use_path(m, JK_CRBA))
     return finish(fn, path_go(m, JK_CRBA, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, M));
   if (use_jit(m, JK_CRBA))
@@ -479,6 +509,9 @@ fst_status fst_aba(const fst_model* m, int64_t B, const float* q, const float* q
                                     PinArgs{m->dpin, counters}, (cudaStream_t)stream);
     return finish(fn, err);
   }
+  if (use_tile(m, JK_ABA, B, aba_lean_smem_needed(mv, m->max_width)))
+    return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, tile_block(m, JK_ABA), m->max_width,
+                                            (cudaStream_t)stream));
   if (use_path(m, JK_ABA))
     return finish(fn, path_go(m, JK_ABA, B, m->nq + 2 * m->nv, 1, (cudaStream_t)stream, mv, B, q, qd, tau, qdd));
   if (use_jit(m, JK_ABA))
@@ -635,6 +668,20 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
   if (skip || a.n_roles == 0) return FST_OK;
   if (m->nq) FST_CHECK(need(fn, io->q, "q"));
   const ModelView mv = view_of(m, theta);
+  if (m->variant[JK_EVAL] == FST_VARIANT_AUTO && tile_default(m, B)) {
+    EvalArgs t = a;  // the kinematics run in blocks of their own
+    if (t.rnea_flags & EVAL_KIN_IN_RNEA) {
+      t.rnea_flags &= ~EVAL_KIN_IN_RNEA;
+      t.roles[t.n_roles++] = ROLE_KIN;
+    }
+    size_t sh = 0;
+    for (int r = 0; r < t.n_roles; ++r) {
+      const size_t role = eval_tile_smem(mv, t.roles[r], vjp, m->max_width);
+      if (role > sh) sh = role;
+    }
+    if (sh <= kLevelSmemLimit)
+      return finish(fn, launch_eval_tile(mv, B, t, sh, m->max_width, tile_block(m, JK_EVAL), (cudaStream_t)stream));
+  }
   if (a.rnea_flags || a.packed) {
     // the shared sweep and the packed layouts live in the one-environment-
     // per-thread fused kernels
@@ -790,6 +837,9 @@ fst_status fst_rnea_store(const fst_model* m, int64_t B, const float* q, const f
     FST_CHECK(need(fn, qdd, "qdd"));
   }
   const ModelView mv = view_of(m, theta);
+  if (use_tile(m, JK_RNEA_STORE, B, level_smem_needed(mv, LEVEL_RNEA)))
+    return finish(fn, launch_rnea_store_tile(mv, B, q, qd, qdd, tau, tape, tile_block(m, JK_RNEA_STORE),
+                                             (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_STORE))
     return finish(fn, jit_go(m, JK_RNEA_STORE, B, m->nq + 2 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              qd, qdd, tau, tape));
@@ -1034,9 +1084,30 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
   for (int k = 0; k < n; ++k) order[k] = k;
   for (int i = 1; i < n; ++i)
     for (int j = i; j > 0 && g->models[order[j]]->n > g->models[order[j - 1]]->n; --j) std::swap(order[j], order[j - 1]);
-  const bool level = g->variant == FST_VARIANT_LEVEL;
-  const int T = level ? 32 : g->block;  // environments per item
-  size_t state_bytes = 0;               // level: per-body state of the largest (tree, operator) pair
+  // the default form is the one that the single-tree calls take: tiles of 32
+  // environments if every tree's calls do and their state fits
+  auto state_of = [&](int k, int r) {  // level: bytes of per-body state of a (tree, operator) pair
+    const fst_model* m = g->models[k];
+    const size_t floats = r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + 2 * kAbaLeanRingFloats * m->max_width
+                          : (size_t)(r == ROLE_CRBA ? kCrbaStateFloats
+                                     : r == ROLE_RNEA ? kRneaStateFloats : kFkStateFloats) * m->n;
+    return floats * 32 * sizeof(float);
+  };
+  a.model_bytes = (size_t)max_n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;
+  a.model_bytes = (a.model_bytes + 15) / 16 * 16;
+  bool level = g->variant == FST_VARIANT_LEVEL;
+  if (g->variant == FST_VARIANT_AUTO) {
+    level = true;
+    size_t most = 0;
+    for (int k = 0; k < n; ++k) {
+      level = level && (io[k].B == 0 || tile_default(g->models[k], io[k].B));
+      for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) most = std::max(most, state_of(k, r));
+    }
+    level = level && a.model_bytes + (size_t)a.max_rows * 32 * sizeof(float) + most <= kLevelSmemLimit;
+  }
+  const int block = g->variant == FST_VARIANT_AUTO && level ? kMultiTileBlock : g->block;
+  const int T = level ? 32 : block;  // environments per item
+  size_t state_bytes = 0;            // level: per-body state of the largest (tree, operator) pair
   // every block of the persistent grid draws one item past the last, so the
   // int work counter reaches n_items + grid: keep ample headroom below 2^31
   const int64_t kMaxItems = (int64_t)INT32_MAX - (1 << 24);
@@ -1050,14 +1121,7 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
                        : r == ROLE_CRBA ? (const void*)x.M
                        : r == ROLE_RNEA ? (const void*)x.tau_out : (const void*)x.poses;
       if (!outp || x.B == 0) continue;
-      if (level) {
-        const fst_model* m = g->models[k];
-        const size_t floats = r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + 2 * kAbaLeanRingFloats * m->max_width
-                              : (size_t)(r == ROLE_CRBA ? kCrbaStateFloats
-                                         : r == ROLE_RNEA ? kRneaStateFloats : kFkStateFloats) * m->n;
-        const size_t need = floats * 32 * sizeof(float);
-        if (need > state_bytes) state_bytes = need;
-      }
+      if (level) state_bytes = std::max(state_bytes, state_of(k, r));
       a.seg_start[seg] = (int)items;  // within kMaxItems: checked below on every addition
       a.seg_model[seg] = (unsigned char)k;
       a.seg_op[seg] = (unsigned char)r;
@@ -1068,15 +1132,13 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
     }
   a.seg_start[seg] = (int)items;
   a.n_items = (int)items;
-  a.model_bytes = (size_t)max_n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;
-  a.model_bytes = (a.model_bytes + 15) / 16 * 16;
   if (items == 0) return FST_OK;
   if (level) {
     const size_t sh = a.model_bytes + (size_t)a.max_rows * 32 * sizeof(float) + state_bytes;
     if (sh > kLevelSmemLimit)
       return set_error(FST_ERR_INVALID_ARG, std::string(fn) + ": the level-parallel state of the largest tree "
                                                               "does not fit in shared memory");
-    return finish(fn, launch_multi_level(a, state_bytes, g->block, (cudaStream_t)stream));
+    return finish(fn, launch_multi_level(a, state_bytes, block, (cudaStream_t)stream));
   }
   return finish(fn, launch_multi(a, max_n, T, (cudaStream_t)stream));
 }

@@ -51,6 +51,11 @@ struct SV {
 __device__ __forceinline__ SV operator+(SV a, SV b) { return SV{a.w + b.w, a.v + b.v}; }
 __device__ __forceinline__ SV operator-(SV a, SV b) { return SV{a.w - b.w, a.v - b.v}; }
 __device__ __forceinline__ SV operator*(float s, SV a) { return SV{s * a.w, s * a.v}; }
+// s a + b
+__device__ __forceinline__ SV sv_fma(float s, SV a, SV b) {
+  return SV{f3{fmaf(s, a.w.x, b.w.x), fmaf(s, a.w.y, b.w.y), fmaf(s, a.w.z, b.w.z)},
+            f3{fmaf(s, a.v.x, b.v.x), fmaf(s, a.v.y, b.v.y), fmaf(s, a.v.z, b.v.z)}};
+}
 __device__ __forceinline__ float dot(SV a, SV b) { return dot(a.w, b.w) + dot(a.v, b.v); }
 __device__ __forceinline__ SV sv_zero() { return SV{f3{0, 0, 0}, f3{0, 0, 0}}; }
 __device__ __forceinline__ f3 tvec(const Xf& X) { return f3{X.t[0], X.t[1], X.t[2]}; }
@@ -88,7 +93,9 @@ __device__ __forceinline__ f3 sym_mul(const float* I, f3 w) {
 }
 // I * (w, v) = (I_o w + h x v, m v - h x w)
 __device__ __forceinline__ SV in_mul(const In10& I, SV m) {
-  return SV{sym_mul(I.I, m.w) + cross(I.h, m.v), I.m * m.v - cross(I.h, m.w)};
+  const f3 c = cross(I.h, m.w);
+  return SV{sym_mul(I.I, m.w) + cross(I.h, m.v),
+            f3{fmaf(I.m, m.v.x, -c.x), fmaf(I.m, m.v.y, -c.y), fmaf(I.m, m.v.z, -c.z)}};
 }
 __device__ __forceinline__ In10 in_load(const float* th) {
   In10 I;
@@ -134,16 +141,17 @@ __device__ __forceinline__ In10 in_to_parent(const Xf& X, const In10& I) {
   o.m = I.m;
   f3 y = Rmul(X.R, I.h);
   f3 t = tvec(X);
-  o.h = y + I.m * t;
+  o.h = f3{fmaf(I.m, t.x, y.x), fmaf(I.m, t.y, y.y), fmaf(I.m, t.z, y.z)};
   sym_rot(X.R, I.I, o.I);
   float d = fmaf(2.0f, dot(y, t), I.m * dot(t, t));
-  f3 z = y + (0.5f * I.m) * t;  // y t^T + t y^T + m t t^T = z t^T + t z^T
-  o.I[0] += d - 2.0f * z.x * t.x;
+  const float hm = 0.5f * I.m;
+  const f3 z = f3{fmaf(hm, t.x, y.x), fmaf(hm, t.y, y.y), fmaf(hm, t.z, y.z)};  // y t^T + t y^T + m t t^T = z t^T + t z^T
+  o.I[0] += fmaf(-2.0f * z.x, t.x, d);
   o.I[1] -= fmaf(z.x, t.y, t.x * z.y);
-  o.I[2] += d - 2.0f * z.y * t.y;
+  o.I[2] += fmaf(-2.0f * z.y, t.y, d);
   o.I[3] -= fmaf(z.x, t.z, t.x * z.z);
   o.I[4] -= fmaf(z.y, t.z, t.y * z.z);
-  o.I[5] += d - 2.0f * z.z * t.z;
+  o.I[5] += fmaf(-2.0f * z.z, t.z, d);
   return o;
 }
 
@@ -197,27 +205,27 @@ __device__ __forceinline__ void sym6_add(Sym6& a, const Sym6& b) {
 __device__ __forceinline__ void sym6_rank1_sub(Sym6& s, SV U, float invD) {
   f3 n = U.w, f = U.v;
   f3 ns = invD * n, fs = invD * f;
-  s.A[0] -= ns.x * n.x;
-  s.A[1] -= ns.x * n.y;
-  s.A[2] -= ns.y * n.y;
-  s.A[3] -= ns.x * n.z;
-  s.A[4] -= ns.y * n.z;
-  s.A[5] -= ns.z * n.z;
-  s.C[0] -= fs.x * f.x;
-  s.C[1] -= fs.x * f.y;
-  s.C[2] -= fs.y * f.y;
-  s.C[3] -= fs.x * f.z;
-  s.C[4] -= fs.y * f.z;
-  s.C[5] -= fs.z * f.z;
-  s.Bk[0] -= ns.x * f.x;
-  s.Bk[1] -= ns.x * f.y;
-  s.Bk[2] -= ns.x * f.z;
-  s.Bk[3] -= ns.y * f.x;
-  s.Bk[4] -= ns.y * f.y;
-  s.Bk[5] -= ns.y * f.z;
-  s.Bk[6] -= ns.z * f.x;
-  s.Bk[7] -= ns.z * f.y;
-  s.Bk[8] -= ns.z * f.z;
+  s.A[0] = fmaf(-ns.x, n.x, s.A[0]);
+  s.A[1] = fmaf(-ns.x, n.y, s.A[1]);
+  s.A[2] = fmaf(-ns.y, n.y, s.A[2]);
+  s.A[3] = fmaf(-ns.x, n.z, s.A[3]);
+  s.A[4] = fmaf(-ns.y, n.z, s.A[4]);
+  s.A[5] = fmaf(-ns.z, n.z, s.A[5]);
+  s.C[0] = fmaf(-fs.x, f.x, s.C[0]);
+  s.C[1] = fmaf(-fs.x, f.y, s.C[1]);
+  s.C[2] = fmaf(-fs.y, f.y, s.C[2]);
+  s.C[3] = fmaf(-fs.x, f.z, s.C[3]);
+  s.C[4] = fmaf(-fs.y, f.z, s.C[4]);
+  s.C[5] = fmaf(-fs.z, f.z, s.C[5]);
+  s.Bk[0] = fmaf(-ns.x, f.x, s.Bk[0]);
+  s.Bk[1] = fmaf(-ns.x, f.y, s.Bk[1]);
+  s.Bk[2] = fmaf(-ns.x, f.z, s.Bk[2]);
+  s.Bk[3] = fmaf(-ns.y, f.x, s.Bk[3]);
+  s.Bk[4] = fmaf(-ns.y, f.y, s.Bk[4]);
+  s.Bk[5] = fmaf(-ns.y, f.z, s.Bk[5]);
+  s.Bk[6] = fmaf(-ns.z, f.x, s.Bk[6]);
+  s.Bk[7] = fmaf(-ns.z, f.y, s.Bk[7]);
+  s.Bk[8] = fmaf(-ns.z, f.z, s.Bk[8]);
 }
 
 // R M R^T for a full 3x3 M
@@ -267,12 +275,12 @@ __device__ __forceinline__ Sym6 sym6_to_parent(const Xf& X, const Sym6& s) {
     Y[3 * r + 1] = fmaf(-Z[3 * r + 0], tz, Z[3 * r + 2] * tx);
     Y[3 * r + 2] = fmaf(Z[3 * r + 0], ty, -Z[3 * r + 1] * tx);
   }
-  o.A[0] -= 2.0f * Y[0];
+  o.A[0] = fmaf(-2.0f, Y[0], o.A[0]);
   o.A[1] -= Y[1] + Y[3];
-  o.A[2] -= 2.0f * Y[4];
+  o.A[2] = fmaf(-2.0f, Y[4], o.A[2]);
   o.A[3] -= Y[2] + Y[6];
   o.A[4] -= Y[5] + Y[7];
-  o.A[5] -= 2.0f * Y[8];
+  o.A[5] = fmaf(-2.0f, Y[8], o.A[5]);
   return o;
 }
 

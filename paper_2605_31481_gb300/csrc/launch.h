@@ -155,6 +155,14 @@ size_t rnea_derivs_aligned_smem(const ModelView& mv);
 size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries);
 size_t rnea_vjp_aligned_smem(const ModelView& mv);
 size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw);
+// The fused evaluation with these bodies; smem: the largest eval_tile_smem of
+// its roles. The RNEA role may carry the adjoint (a.rnea_flags), M and J the
+// packed layouts; EVAL_KIN_IN_RNEA does not apply.
+size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw);
+cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                                   float* tau, float* tape, int block, cudaStream_t s);
+cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, size_t smem, int maxw, int block,
+                             cudaStream_t s);
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                        const float* qdd, float* dq, float* dqd, int block, cudaStream_t s);
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,

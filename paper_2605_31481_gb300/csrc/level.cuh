@@ -176,50 +176,29 @@ __device__ __forceinline__ void fk_level(const TP& tp, const Col& q, const LaneS
 // tile's rows first and writing only the support-path columns, as
 // crba_level does for M, was measured slower here: the columns are cheap to
 // write, and the clear adds L2 writes.)
+// Packed (PK non-null, see PackedJ): only the columns on the support path.
 template <class TP>
 __device__ __forceinline__ void jac_columns(const TP& tp, int nv, const LinkList& links, const LaneState& S,
-                                           float* __restrict__ J, int64_t B, int64_t e, bool act) {
+                                           float* __restrict__ J, int64_t B, int64_t e, bool act,
+                                           const PackedJ* PK = nullptr) {
   const int W = n_warps(), w = warp_id();
   const int n = tp.n();
   for (int item = w; item < links.n * n; item += W) {
     const int l = item / n, k = item % n;
     const BodyI bk = tp.I(k);
-    const int nvk = nv_of(bk.type);
-    if (nvk == 0 || !act) continue;
+    if (nv_of(bk.type) == 0 || !act) continue;
     const bool on_path = (tp.C(links.idx[l]).anc >> k) & 1ull;
-    float* Jl = J + (int64_t)l * 6 * nv * B + e;
-    const Xf P = S.X(k, 0);
-    const f3 p = tvec(P);
-    if (nvk == 1) {
-      float col[6] = {0, 0, 0, 0, 0, 0};
-      if (on_path) {
-        const SV s = S_of(tp.C(k));
-        const f3 wv = Rmul(P.R, s.w);
-        const f3 v = Rmul(P.R, s.v) + cross(p, wv);
-        col[0] = v.x; col[1] = v.y; col[2] = v.z;
-        col[3] = wv.x; col[4] = wv.y; col[5] = wv.z;
-      }
-#pragma unroll
-      for (int r = 0; r < 6; ++r) Jl[((int64_t)r * nv + bk.vi) * B] = col[r];
-    } else {
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        float col[6] = {0, 0, 0, 0, 0, 0};
-        if (on_path) {
-          const int a = j % 3;
-          const f3 Re = f3{P.R[a], P.R[3 + a], P.R[6 + a]};
-          if (j < 3) {
-            col[0] = Re.x; col[1] = Re.y; col[2] = Re.z;
-          } else {
-            const f3 v = cross(p, Re);
-            col[0] = v.x; col[1] = v.y; col[2] = v.z;
-            col[3] = Re.x; col[4] = Re.y; col[5] = Re.z;
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < 6; ++r) Jl[((int64_t)r * nv + bk.vi + j) * B] = col[r];
-      }
+    int64_t first = (int64_t)l * 6 * nv;
+    int stride = nv, col = bk.vi;
+    if (PK) {
+      if (!on_path) continue;
+      first = PK->off[l];
+      stride = PK->cols[l];
+      col = 0;
+      for (int j = bk.parent; j >= 0; j = tp.I(j).parent) col += nv_of(tp.I(j).type);
     }
+    const Xf P = S.X(k, 0);
+    jac_column(tp, k, P.R, P.t, on_path, stride, col, J + first * B + e, B);
   }
 }
 
@@ -227,16 +206,20 @@ __device__ __forceinline__ void jac_columns(const TP& tp, int nv, const LinkList
 template <class TP>
 __device__ __forceinline__ void kin_level(const TP& tp, const Col& q, int nv, const LinkList& links,
                                           const LaneState& S, float* __restrict__ poses, float* __restrict__ J,
-                                          int64_t B, int64_t e, bool act) {
+                                          int64_t B, int64_t e, bool act, const PackedJ* PK = nullptr) {
   fk_level(tp, q, S, poses, B, e, act);
-  if (J) jac_columns(tp, nv, links, S, J, B, e, act);
+  if (J) jac_columns(tp, nv, links, S, J, B, e, act, PK);
 }
 
 // ---- RNEA -----------------------------------------------------------------------
+// tau goes to global memory (may be null) and, if tau_col is not null, also to
+// that shared-memory column (rows of 32). With a tape, the forward state of
+// every body is left there for the store variant of the adjoint (tape_store's
+// layout).
 template <class TP>
 __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& qdd,
                                            const LaneState& S, float* __restrict__ tau, int64_t B, int64_t e,
-                                           bool act) {
+                                           bool act, float* tau_col = nullptr, float* tape = nullptr) {
   const int W = n_warps(), w = warp_id();
   enum { X_ = 0, V_ = 12, A_ = 18, F_ = 24 };
   FST_UNROLL
@@ -261,6 +244,14 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
       S.put(i, V_, vi);
       S.put(i, A_, ai);
       S.put(i, F_, in_mul(I, ai) + crf(vi, in_mul(I, vi)));
+      if (tape && act) {
+        float* p = tape + (int64_t)i * 30 * B + e;
+        const float r[24] = {X.R[0], X.R[1], X.R[2], X.R[3], X.R[4], X.R[5], X.R[6], X.R[7],
+                             X.R[8], X.t[0], X.t[1], X.t[2], vi.w.x, vi.w.y, vi.w.z, vi.v.x,
+                             vi.v.y, vi.v.z, ai.w.x, ai.w.y, ai.w.z, ai.v.x, ai.v.y, ai.v.z};
+#pragma unroll
+        for (int c = 0; c < 24; ++c) p[(int64_t)c * B] = r[c];
+      }
     }
     __syncthreads();
   }
@@ -272,6 +263,13 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
       SV F = S.sv(i, F_);
       for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) F = F + S.sv(tp.child(ch), F_);
       if (act && tau) ST_store(tp.C(i), bi, F, tau, B, e);
+      if (tau_col) ST_store(tp.C(i), bi, F, tau_col, kLaneEnvs, 0);
+      if (tape && act) {
+        float* p = tape + ((int64_t)i * 30 + 24) * B + e;
+        const float r[6] = {F.w.x, F.w.y, F.w.z, F.v.x, F.v.y, F.v.z};
+#pragma unroll
+        for (int c = 0; c < 6; ++c) p[(int64_t)c * B] = r[c];
+      }
       if (bi.parent >= 0) S.put(i, F_, XT_force(S.X(i, X_), F));
     }
     __syncthreads();
@@ -300,7 +298,7 @@ __device__ __forceinline__ void m_clear_tile(float* __restrict__ M, int64_t rows
   for (int64_t r = t >> 5; r < rows; r += W, p += (int64_t)W * B) *p = 0.f;
 }
 
-template <class TP>
+template <bool PACKED = false, class TP>
 __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, const LaneState& S,
                                            float* __restrict__ M, int64_t B, int64_t e, bool act) {
   const int W = n_warps(), w = warp_id();
@@ -310,7 +308,7 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
   // The block barriers of the composite pass order the two sets of stores.
   // Nothing is read back, so DRAM sees each line once; the clear costs L2
   // writes, not a per-entry ancestry test.
-  if (tp.depth() > 0) m_clear_tile(M, (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
+  if (tp.depth() > 0) m_clear_tile(M, PACKED ? (int64_t)nv * (nv + 1) / 2 : (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
   FST_UNROLL
   for (int l = tp.depth() - 1; l >= 0; --l) {
     FST_FOR_MY_BODIES(tp, l, k) {
@@ -326,13 +324,13 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
     __syncthreads();
   }
   if (!act) return;
-  float* Me = M + e;
+  const MOut<PACKED> Me{M + e, nv, B};
   for (int i = w; i < tp.n(); i += W) {
     const BodyI bi = tp.I(i);
     if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
       const In10 Ic = S.in10(i, IC_);
       SV F = in_mul(Ic, S_of(tp.C(i)));
-      Me[((int64_t)bi.vi * nv + bi.vi) * B] = dot(S_of(tp.C(i)), F);
+      Me.one(bi.vi, bi.vi, dot(S_of(tp.C(i)), F));
       // up the support path, parent by parent (parents precede children)
       int kk = i;
       for (int j = bi.parent; j >= 0; j = tp.I(j).parent) {
@@ -340,16 +338,11 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
         kk = j;
         const BodyI bj = tp.I(j);
         if (bj.type == FST_JOINT_REVOLUTE || bj.type == FST_JOINT_PRISMATIC) {
-          const float mij = dot(S_of(tp.C(j)), F);
-          Me[((int64_t)bi.vi * nv + bj.vi) * B] = mij;
-          Me[((int64_t)bj.vi * nv + bi.vi) * B] = mij;
+          Me.sym(bi.vi, bj.vi, dot(S_of(tp.C(j)), F));
         } else if (bj.type == FST_JOINT_FREE) {
           const float col[6] = {F.v.x, F.v.y, F.v.z, F.w.x, F.w.y, F.w.z};
 #pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            Me[((int64_t)(bj.vi + r) * nv + bi.vi) * B] = col[r];
-            Me[((int64_t)bi.vi * nv + bj.vi + r) * B] = col[r];
-          }
+          for (int r = 0; r < 6; ++r) Me.sym(bj.vi + r, bi.vi, col[r]);
         }
       }
     } else if (bi.type == FST_JOINT_FREE) {
@@ -365,7 +358,7 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
 #pragma unroll
       for (int r = 0; r < 6; ++r)
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) Me[((int64_t)(bi.vi + r) * nv + bi.vi + cc) * B] = blk[r][cc];
+        for (int cc = 0; cc < 6; ++cc) Me.one(bi.vi + r, bi.vi + cc, blk[r][cc]);
     }
   }
 }
@@ -523,7 +516,7 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
         *S.at(i, u_) = ui;
         if (bi.parent < 0) continue;
         sym6_rank1_sub(Ia, Ui, iD);
-        pa = pa + sym6_mul(Ia, S.sv(i, C_)) + (ui * iD) * Ui;
+        pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, S.sv(i, C_)));
       } else {
         if (bi.parent < 0) continue;
         pa = pa + sym6_mul(Ia, S.sv(i, C_));
@@ -545,7 +538,7 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
       if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
         const float qi = (*S.at(i, u_) - dot(S.sv(i, U_), ai)) * *S.at(i, ID_);
         if (act) qdd[(int64_t)bi.vi * B + e] = qi;
-        ai = ai + qi * S_of(tp.C(i));
+        ai = sv_fma(qi, S_of(tp.C(i)), ai);
       } else if (bi.type == FST_JOINT_FREE) {
         const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};
         const SV anew = sym6_solve(S.sym(i, IA_), tf - S.sv(i, PA_));
@@ -637,7 +630,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         *S.at(i, u_) = ui;
         if (bi.parent < 0) continue;
         sym6_rank1_sub(Ia, Ui, iD);
-        pa = pa + sym6_mul(Ia, S.sv(i, C_)) + (ui * iD) * Ui;
+        pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, S.sv(i, C_)));
       } else {
         if (bi.parent < 0) continue;
         pa = pa + sym6_mul(Ia, S.sv(i, C_));
@@ -661,7 +654,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         const float qi = (*S.at(i, u_) - dot(S.sv(i, VU_), ai)) * *S.at(i, ID_);
         if (act && qdd) qdd[(int64_t)bi.vi * B + e] = qi;
         if (qdd_col) qdd_col[bi.vi << 5] = qi;
-        ai = ai + qi * S_of(tp.C(i));
+        ai = sv_fma(qi, S_of(tp.C(i)), ai);
       } else if (bi.type == FST_JOINT_FREE) {
         const int slot = k - tp.level_begin(l);  // level 0: ring parity 0
         const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};

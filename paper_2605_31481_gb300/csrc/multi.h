@@ -35,6 +35,18 @@ struct MultiArgs {
   int* counter;          // device work counter (reset before each launch)
 };
 
+// Grid = resident blocks per SM x SMs (from the occupancy calculator), but
+// never more blocks than items.
+template <typename K>
+inline int persistent_grid(K* kernel, int block, size_t smem, int n_items) {
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
+  const int g = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+  return g < n_items ? g : n_items;
+}
+
 // Environments per item: `block` for the generic kernel (one environment per
 // thread), 32 for the level-parallel one.
 cudaError_t launch_multi(const MultiArgs& a, int max_n, int block, cudaStream_t s);
@@ -49,5 +61,5 @@ struct fst_multi {
   int* counter = nullptr;
   int device = -1;
   int block = 64;
-  int variant = FST_VARIANT_GENERIC;  // or FST_VARIANT_LEVEL
+  int variant = FST_VARIANT_AUTO;  // or FST_VARIANT_GENERIC, FST_VARIANT_LEVEL
 };
