@@ -22,12 +22,24 @@ from . import _ffi
 from ._ffi import check
 
 
+# The calls below are short (a launch takes the host 2.7 us), so the checks in
+# front of it are kept to attribute reads: device pointers travel as plain
+# integers, and the current stream comes from the raw accessor (0.1 us; building
+# a torch.cuda.Stream object for it took 3.1 us).
+_f32 = torch.float32
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current device's current stream, as an integer handle."""
+    if _raw_stream is not None and _raw_device is not None:
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def soa(x: torch.Tensor) -> torch.Tensor:
@@ -145,6 +157,11 @@ def set_smem_carveout(percent: int):
 
 
 def _check_in(x, rows, name, model):
+    if isinstance(x, torch.Tensor):
+        shape = x.shape
+        if (len(shape) == 2 and shape[0] == rows and x.dtype is _f32 and x.device == model.device
+                and x.is_contiguous()):
+            return shape[1]
     if not isinstance(x, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if x.dtype != torch.float32 or x.device != model.device:
@@ -177,7 +194,9 @@ def _out(out, shape, model):
     """An output tensor: on the model's device, or pinned host memory the
     device addresses directly (the kernels then write to the host)."""
     if out is None:
-        return torch.empty(shape, dtype=torch.float32, device=model.device)
+        return torch.empty(shape, dtype=_f32, device=model.device)
+    if (out.shape == shape and out.dtype is _f32 and out.device == model.device and out.is_contiguous()):
+        return out
     if out.shape != torch.Size(shape) or out.dtype != torch.float32 or not out.is_contiguous() or \
             (out.device != model.device and not _host_out_ok(out)):
         raise ValueError(f"out must be a contiguous float32 {shape} tensor on {model.device} "
@@ -526,7 +545,9 @@ def rnea_loss_grad(model: Model, q, qd, qdd, tau_meas, theta=None, *, q_bar=Fals
     sp, sb = _scratch(model, B, scratch)
     check(_ffi.lib().fst_rnea_loss_grad(model.handle, B, _ptr(q), _ptr(qd), _ptr(qdd), _ptr(_theta(theta, model)),
                                         _ptr(tau_meas), _ptr(buf), _ptr(qb), _ptr(qdb), sp, sb, _stream()))
-    return buf[-1], buf[:-1].view(model.n_bodies, 10), qb, qdb
+    # the same views as buf[-1] and buf[:-1].view(n_b, 10), at a third of the cost of indexing
+    o = buf.storage_offset()
+    return buf.as_strided((), (), o + 10 * model.n_bodies), buf.as_strided((model.n_bodies, 10), (10, 1), o), qb, qdb
 
 
 # ---------------------------------------------------------------------------
