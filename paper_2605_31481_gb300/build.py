@@ -37,7 +37,7 @@ def nvcc_path() -> str:
 # The tile kernels (level.cuh, aligned.cuh) are instantiated in several units and
 # entry points that must agree bit for bit: products and sums are fused only
 # where the source says fmaf, so the surrounding code cannot change a rounding.
-UNIT_FLAGS = {f: ["-fmad=false"] for f in ("aligned.cu", "level.cu", "multi_level.cu")}
+UNIT_FLAGS = {f: ["-fmad=false"] for f in ("aligned.cu", "level.cu", "multi_level.cu", "warpbody.cu")}
 
 # Device headers embedded into the library for run-time specialisation
 # (NVRTC compiles them again for one fixed tree; see csrc/jit.cpp).

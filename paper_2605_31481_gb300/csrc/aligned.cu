@@ -188,6 +188,18 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
                               LaneState{state, kVjpState}, o, B, e, act);
 }
 
+// Bound by the latency of two sweeps over the levels (fixed humanoid, B = 3000:
+// 46 -> 9 us; the general kernel staged 12 cotangent rows a body and swept the
+// bodies one by one), three tiles of the humanoid
+// per SM (floating humanoid, B = 65536: 305 -> 57 us, 75 MB read).
+__global__ void __launch_bounds__(256) fk_vjp_tile_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                          const float* __restrict__ pbar, float* __restrict__ qbar) {
+  FST_TILE;
+  stage_block_rows(tile, q, mv.nq, B, e);
+  const SmemModel sm = stage_model(mv, smem);
+  fk_vjp_tile(sm, tile_col(tile, 0), pbar, LaneState{tile + mv.nq * kLaneEnvs, kFkVjpState}, qbar, B, e, act);
+}
+
 // The store variant's forward: RNEA that also leaves its state on the tape.
 __global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                               const float* __restrict__ qd,
@@ -208,6 +220,10 @@ __global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int6
 // bit. Blocks of the heaviest operator come first. EXT (a kernel of its own,
 // so that the plain one keeps its registers): the RNEA adjoint beside tau, and
 // M and J in the packed layouts.
+// Bound by the ABA blocks' latency at B = 4096 (quadruped, five operators: 14.1
+// us; the specialised fused kernel that the default took before 31.3, its
+// roles' straight-line code refetched by every SM) and by shared memory, two
+// to four tiles an SM, at larger batches (humanoid, B = 16384: 164 -> 86 us).
 template <bool EXT>
 __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B, EvalArgs a, int maxw) {
   FST_TILE;
@@ -310,6 +326,18 @@ size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw) {
   else
     f += (size_t)kFkState * mv.n;
   return smem_bytes(mv.n) + floats32(f);
+}
+
+size_t fk_vjp_tile_smem(const ModelView& mv) {
+  return smem_bytes(mv.n) + floats32((size_t)mv.nq + (size_t)kFkVjpState * mv.n);
+}
+
+cudaError_t launch_fk_vjp_tile(const ModelView& mv, int64_t B, const float* q, const float* pbar, float* qbar,
+                               int block, cudaStream_t s) {
+  const size_t sh = fk_vjp_tile_smem(mv);
+  prepare(fk_vjp_tile_kernel, sh);
+  fk_vjp_tile_kernel<<<grid_for(B, kLaneEnvs), block, sh, s>>>(mv, B, q, pbar, qbar);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,

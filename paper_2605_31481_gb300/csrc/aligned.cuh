@@ -398,7 +398,8 @@ __device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, 
 // Where the cotangent comes from.
 enum VjpMode {
   VJP_GIVEN = 0,  // staged in tb
-  VJP_LOSS        // tb holds measured torques; the cotangent is 2 (tau - tb), the loss their squared difference
+  VJP_LOSS,       // tb holds measured torques; the cotangent is 2 (tau - tb), the loss their squared difference
+  VJP_TAU         // the cotangent is tau (warpbody.cuh)
 };
 
 struct VjpAligned {
@@ -683,6 +684,80 @@ __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, co
     store_if(o.qddbar, bi.vi, B, e, o.sign * dot(psi, A), true);
   }
   return loss;
+}
+
+// ---- the adjoint of forward kinematics -----------------------------------------
+// Moving joint i turns and shifts its whole subtree as one rigid body, so of
+// the poses' cotangents (Rbar_k, pbar_k) only the total force F = sum pbar_k
+// and moment T = sum (R_k's columns x Rbar_k's columns) + moments of the pbar_k
+// act on it: qbar_i = S_w . T + S_v . F, with T about body i's origin. Summing
+// six numbers up the tree replaces twelve and two matrix products per body. A
+// free root's quaternion sees the moment alone: qbar = 2 (0, T) (x) q.
+// Floats of shared state per body and environment: world pose 12 | T 3, F 3.
+__device__ __forceinline__ void fk_vjp_tile(const SmemModel& tp, const Col& q, const float* __restrict__ pbar,
+                                            const LaneState& S, float* __restrict__ qbar, int64_t B, int64_t e,
+                                            bool act) {
+  const int W = n_warps(), w = warp_id(), n = tp.n();
+  enum { P_ = 0, T_ = 12 };
+  // the cotangents' local part needs the world rotation: run the poses first
+  for (int l = 0; l < tp.depth(); ++l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const Xf X = joint_X(tp.C(i), bi, q);
+      Xf P = X;
+      if (bi.parent >= 0) {
+        const Xf Pp = S.X(bi.parent, P_);
+        compose(Pp.R, Pp.t, X, P.R, P.t);
+      }
+      S.putX(i, P_, P);
+    }
+    __syncthreads();
+  }
+  for (int i = w; i < n; i += W) {
+    float g[12];
+    const float* src = pbar + (int64_t)i * 12 * B + e;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) g[k] = act ? __ldg(src + (int64_t)k * B) : 0.f;
+    float R[9];
+    S.get_n(i, P_, R, 9);
+    SV f{f3{0.f, 0.f, 0.f}, f3{g[9], g[10], g[11]}};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.w = f.w + cross(f3{R[c], R[3 + c], R[6 + c]}, f3{g[c], g[3 + c], g[6 + c]});
+    S.put(i, T_, f);
+  }
+  __syncthreads();
+  for (int l = tp.depth() - 1; l >= 0; --l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const BodyC& c = tp.C(i);
+      const Xf P = S.X(i, P_);
+      SV f = S.sv(i, T_);
+      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
+        const float* t = S.at(tp.child(ch), P_ + 9);
+        f = f + shift_force(S.sv(tp.child(ch), T_), f3{t[0] - P.t[0], t[32] - P.t[1], t[64] - P.t[2]});
+      }
+      S.put(i, T_, f);
+      if (!act) continue;
+      if (one_dof(bi)) {
+        const SV psi = psi_of(c, P.R);
+        qbar[(int64_t)bi.qi * B + e] = dot(psi, f);
+      } else if (bi.type == FST_JOINT_FREE) {
+        const f3 F = RTmul(c.R0, f.v), T = RTmul(c.R0, f.w);
+        f3 v = f3{q[bi.qi + 3], q[bi.qi + 4], q[bi.qi + 5]};
+        float s = q[bi.qi + 6];
+        const float inv = rsqrtf(fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, s * s))));
+        v = inv * v;
+        s *= inv;
+        const f3 gv = 2.f * inv * (s * T + cross(T, v));
+        const float out[7] = {F.x, F.y, F.z, gv.x, gv.y, gv.z, -2.f * inv * dot(T, v)};
+#pragma unroll
+        for (int r = 0; r < 7; ++r) qbar[(int64_t)(bi.qi + r) * B + e] = out[r];
+      }
+    }
+    __syncthreads();
+  }
 }
 
 // ---- forward-dynamics derivatives: the tree-sparse factorisation ----------------

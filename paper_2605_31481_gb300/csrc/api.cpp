@@ -93,29 +93,73 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
          level_smem_needed(view_of(m, nullptr), level_kind, level_tiles(m, kind)) <= kLevelSmemLimit;
 }
 
-// Whether a call of this kind runs its aligned-frame kernel (aligned.cu): the
-// default unless the kind is pinned to another variant or the tree's state
-// does not fit in shared memory (`need` bytes; about 33 bodies). There is no
-// line in B: the aligned kernels were the faster ones at every size measured,
-// against the generic and the specialised kernels (us): arm7 RNEA adjoint
-// B = 32768 27 / 26-40, quadruped B = 16384 25 / 43, humanoid B = 512 14 / 66;
-// derivatives 3 to 20 times faster everywhere.
-bool aligned_fits(const fst_model* m, int kind, size_t need) {
-  return m->variant[kind] == FST_VARIANT_AUTO && need + 1024 <= kLevelSmemLimit;  // 1 KB: static shared memory
-}
-
-// Whether calls that keep the default variant run as tiles of 32 environments
-// whose warps share the bodies (level.cuh, aligned.cuh), for this model and
-// batch. The rule does not look at the operator, so every entry point that
-// computes one gives the same bits.
-bool tile_default(const fst_model* m, int64_t B) {
-  (void)m;
-  (void)B;
-  return true;
+// Whether a call that keeps the default variant runs as tiles of 32
+// environments whose warps share the bodies (level.cuh, aligned.cuh) rather
+// than one environment per thread. op: the operator's kind; spec: whether the
+// other side is a specialised kernel. The rule is the operator's, not the
+// entry point's, so the fused evaluation and the single calls give the same
+// bits. Both sides measured on GB300 (us, tiles / other):
+//  * generic other side. Tiles shorten the chain from the bodies to the
+//    levels: humanoid29 B = 4096 RNEA 9.1 / 22.8, CRBA 10.6 / 72.5, ABA 15 /
+//    53; B = 65536 FK 24 / 40, CRBA 91 / 160, ABA 117 / 200. A chain has no
+//    width to share: arm7 ABA 13 / 13 at 4096, 26 / 16 at 16384. Narrow trees
+//    (fewer than three bodies a level) at large batches are better off with
+//    more environments per SM where the sweeps are light: quadruped11 B =
+//    65536 FK 16 / 15, RNEA 31 / 24, but CRBA 29 / 38, ABA 50 / 78.
+//  * specialised other side. Its straight-line code costs an instruction
+//    fetch per body whatever the batch, so it wins on small trees (arm7 B =
+//    4096 FK 5.4 / 2.8, ABA 13.6 / 9.0; B = 65536 ABA 64 / 15) and large
+//    batches (quadruped11 B = 16384 RNEA 10 / 7.7, ABA 14 / 14.8, B = 32768
+//    ABA 26 / 16; at 4096 ABA 11 / 14.6, the step 14 / 17) and on large trees
+//    only for the light operators (humanoid29 B = 32768 FK 13 / 8.5, RNEA 38 /
+//    23; CRBA 52 / 93, ABA 67 / 149).
+bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
+  const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
+  if (spec) {
+    if (m->n <= 8) return false;
+    if (m->n <= 16) return B < 8192;
+    return !light || B < (op == JK_RNEA || op == JK_RNEA_STORE ? 24576 : 16384);
+  }
+  if (2 * m->n < 3 * m->depth) return B <= 152 * 2 * 32;
+  return !light || m->n >= 3 * m->depth || B < 32768;
 }
 
 bool use_tile(const fst_model* m, int kind, int64_t B, size_t need) {
-  return m->variant[kind] == FST_VARIANT_AUTO && need <= kLevelSmemLimit && tile_default(m, B);
+  return m->variant[kind] == FST_VARIANT_AUTO && need <= kLevelSmemLimit && tile_rule(m, kind, jit_has(m, kind), B);
+}
+
+// The same question for the adjoints, whose tiles do more per barrier: against
+// a specialised kernel they win until the batch fills the chip with one
+// environment per thread (quadruped11 B = 32768 loss and gradient 48 / 41, ABA
+// adjoint 77 / 64; 16384: 26 / 40 and 41 / 44), against the generic ones
+// always, except for long batches of a chain (arm7 B = 65536 ABA adjoint 89 /
+// 73). The FK adjoint is light: arm7 specialised 5.5 / 8.2 at every batch,
+// quadruped11 8.5 / 7.5 at 4096 and 8.6 / 10 at 16384. For the smallest trees
+// the RNEA adjoint follows the specialised fused step, whose result it must
+// equal bit for bit.
+bool adjoint_tile_rule(const fst_model* m, int kind, bool spec, int64_t B) {
+  if (kind == JK_FK_VJP) return spec ? m->n > 8 && (m->n > 16 || B < 12288) : true;
+  if (spec && m->n <= 8 && kind == JK_RNEA_VJP) return false;
+  if (spec && m->n <= 16) return B < 24576;
+  return 2 * m->n >= 3 * m->depth || B <= 24576;
+}
+
+// Whether a default call of an adjoint or of the dense derivatives runs its
+// tile kernel (`need` bytes of shared memory, about 33 bodies). The derivatives'
+// tiles were the faster ones at every size measured, 3 to 20 times.
+bool use_adjoint_tile(const fst_model* m, int kind, int64_t B, size_t need) {
+  if (m->variant[kind] != FST_VARIANT_AUTO || need + 1024 > kLevelSmemLimit) return false;  // 1 KB: static part
+  return kind == JK_RNEA_DERIVS || kind == JK_ABA_DERIVS || adjoint_tile_rule(m, kind, jit_has(m, kind), B);
+}
+
+// Trees of at most 16 bodies run their dynamics adjoints with a warp per body
+// (warpbody.cuh) while the tiles fill the SMs at most twice: quadruped11 B =
+// 4096 ABA adjoint 12.4 against 18.4 us, RNEA adjoint 10.3 against 12.5; at
+// B = 16384 42 against 40, and larger trees' registers spill (humanoid29 ABA
+// adjoint 29.6 against 26).
+bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
+  return m->variant[kind] == FST_VARIANT_AUTO && m->block[kind] == 0 && m->wt.n > 0 && B <= 152 * 2 * 32 &&
+         adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
 constexpr int kMultiTileBlock = 256;  // threads per block of the mixed-tree launch in tiles
@@ -192,6 +236,11 @@ template <typename... A>
 cudaError_t jit_go_slot(const fst_model* m, int kind, int slot, int64_t B, int rows, int P, unsigned gy,
                         cudaStream_t s, unsigned* nblk, A... args) {
   int T = block_of(m, kind, B);
+  // The fused evaluation's roles are different straight-line code: fewer,
+  // larger blocks let more warps of one SM share a role's instructions (arm7
+  // B = 4096: 19.0 us with 32 threads, 9.0 with 128, 8.8 with 256; quadruped11
+  // 31.3, 17.1, 21.6).
+  if (kind == JK_EVAL && m->block[kind] == 0) T = m->n <= 8 ? 256 : 128;
   auto smem = [&](int t) { return (size_t)rows * t * sizeof(float) + (size_t)(t / 32) * P * sizeof(float); };
   while (T > 32 && smem(T) > 96 * 1024) T /= 2;
   const dim3 grid(grid_for(B, T), gy);
@@ -668,24 +717,39 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
   if (skip || a.n_roles == 0) return FST_OK;
   if (m->nq) FST_CHECK(need(fn, io->q, "q"));
   const ModelView mv = view_of(m, theta);
-  if (m->variant[JK_EVAL] == FST_VARIANT_AUTO && tile_default(m, B)) {
-    EvalArgs t = a;  // the kinematics run in blocks of their own
-    if (t.rnea_flags & EVAL_KIN_IN_RNEA) {
-      t.rnea_flags &= ~EVAL_KIN_IN_RNEA;
-      t.roles[t.n_roles++] = ROLE_KIN;
+  if (m->variant[JK_EVAL] == FST_VARIANT_AUTO) {
+    // the operators that run as tiles in one launch, the others in another
+    const bool spec = jit_has(m, JK_EVAL);
+    auto tiled = [&](int role) {
+      const int op = role == ROLE_ABA ? JK_ABA : role == ROLE_CRBA ? JK_CRBA : role == ROLE_RNEA ? JK_RNEA
+                                                                             : (a.J ? JK_JACOBIAN : JK_FK);
+      return tile_rule(m, op, spec, B);
+    };
+    EvalArgs t = a, g = a;
+    t.n_roles = g.n_roles = 0;
+    for (int r = 0; r < a.n_roles; ++r) {
+      EvalArgs& to = tiled(a.roles[r]) ? t : g;
+      to.roles[to.n_roles++] = a.roles[r];
     }
+    if ((a.rnea_flags & EVAL_KIN_IN_RNEA) && tiled(ROLE_RNEA)) {  // in tiles the kinematics have blocks of their own
+      EvalArgs& to = tiled(ROLE_KIN) ? t : g;
+      to.roles[to.n_roles++] = ROLE_KIN;
+    }
+    (tiled(ROLE_RNEA) ? g : t).rnea_flags = 0;
+    t.rnea_flags &= ~EVAL_KIN_IN_RNEA;
     size_t sh = 0;
-    for (int r = 0; r < t.n_roles; ++r) {
-      const size_t role = eval_tile_smem(mv, t.roles[r], vjp, m->max_width);
-      if (role > sh) sh = role;
+    for (int r = 0; r < t.n_roles; ++r)
+      sh = std::max(sh, eval_tile_smem(mv, t.roles[r], (t.rnea_flags & EVAL_RNEA_VJP) != 0, m->max_width));
+    if (t.n_roles && sh <= kLevelSmemLimit) {
+      const cudaError_t err = launch_eval_tile(mv, B, t, sh, m->max_width, tile_block(m, JK_EVAL), (cudaStream_t)stream);
+      if (err != cudaSuccess || g.n_roles == 0) return finish(fn, err);
+      a = g;
     }
-    if (sh <= kLevelSmemLimit)
-      return finish(fn, launch_eval_tile(mv, B, t, sh, m->max_width, tile_block(m, JK_EVAL), (cudaStream_t)stream));
   }
   if (a.rnea_flags || a.packed) {
     // the shared sweep and the packed layouts live in the one-environment-
     // per-thread fused kernels
-    const int rows = m->nq + (vjp ? 3 : 2) * m->nv;
+    const int rows = m->nq + (a.rnea_flags & EVAL_RNEA_VJP ? 3 : 2) * m->nv;
     if (jit_has_slot(m, JK_EVAL, JK_SLOT_EVAL_EXT) && m->variant[JK_EVAL] != FST_VARIANT_GENERIC)
       return finish(fn, jit_go_slot(m, JK_EVAL, JK_SLOT_EVAL_EXT, B, rows, 0, (unsigned)a.n_roles,
                                     (cudaStream_t)stream, nullptr, mv, B, a));
@@ -778,6 +842,8 @@ fst_status fst_fk_vjp(const fst_model* m, int64_t B, const float* q, const float
   FST_CHECK(need(fn, q, "q"));
   FST_CHECK(need(fn, poses_bar, "poses_bar"));
   const ModelView mv = view_of(m, nullptr);
+  if (use_adjoint_tile(m, JK_FK_VJP, B, fk_vjp_tile_smem(mv)))
+    return finish(fn, launch_fk_vjp_tile(mv, B, q, poses_bar, q_bar, tile_block(m, JK_FK_VJP), (cudaStream_t)stream));
   if (use_jit(m, JK_FK_VJP))
     return finish(fn, jit_go(m, JK_FK_VJP, B, m->nq + 12 * m->n, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              poses_bar, q_bar));
@@ -799,7 +865,10 @@ fst_status fst_rnea_vjp(const fst_model* m, int64_t B, const float* q, const flo
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, tau_bar, "tau_bar"));
   const ModelView mv = view_of(m, theta);
-  if (aligned_fits(m, JK_RNEA_VJP, rnea_vjp_aligned_smem(mv)))
+  if (use_warp_bodies(m, JK_RNEA_VJP, B))
+    return finish(fn, launch_wb_rnea_vjp(m->wt, mv, B, q, qd, qdd, tau_bar, q_bar, qd_bar, qdd_bar, theta_bar,
+                                         (float*)scratch, (cudaStream_t)stream));
+  if (use_adjoint_tile(m, JK_RNEA_VJP, B, rnea_vjp_aligned_smem(mv)))
     return finish(fn, launch_rnea_vjp_aligned(mv, B, q, qd, qdd, tau_bar, q_bar, qd_bar, qdd_bar, theta_bar,
                                               (float*)scratch, m->block[JK_RNEA_VJP], (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_VJP)) {
@@ -926,7 +995,7 @@ fst_status fst_rnea_derivatives(const fst_model* m, int64_t B, const float* q, c
   FST_CHECK(need(fn, qd, "qd"));
   FST_CHECK(need(fn, qdd, "qdd"));
   const ModelView mv = view_of(m, theta);
-  if (aligned_fits(m, JK_RNEA_DERIVS, rnea_derivs_aligned_smem(mv)))
+  if (use_adjoint_tile(m, JK_RNEA_DERIVS, B, rnea_derivs_aligned_smem(mv)))
     return finish(fn, launch_rnea_derivs_aligned(mv, B, q, qd, qdd, dtau_dq, dtau_dqd, m->block[JK_RNEA_DERIVS],
                                                  (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_DERIVS))
@@ -947,7 +1016,7 @@ fst_status fst_aba_derivatives(const fst_model* m, int64_t B, const float* q, co
   FST_CHECK(need(fn, tau, "tau"));
   FST_CHECK(need(fn, Minv, "Minv"));
   const ModelView mv = view_of(m, theta);
-  if (aligned_fits(m, JK_ABA_DERIVS, aba_derivs_aligned_smem(mv, m->max_width, m->dof_entries)))
+  if (use_adjoint_tile(m, JK_ABA_DERIVS, B, aba_derivs_aligned_smem(mv, m->max_width, m->dof_entries)))
     return finish(fn, launch_aba_derivs_aligned(mv, B, q, qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv, m->max_width,
                                                 m->dof_entries, m->dof_depth, m->block[JK_ABA_DERIVS],
                                                 (cudaStream_t)stream));
@@ -973,7 +1042,10 @@ fst_status fst_aba_vjp(const fst_model* m, int64_t B, const float* q, const floa
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, qdd_bar, "qdd_bar"));
   const ModelView mv = view_of(m, theta);
-  if (aligned_fits(m, JK_ABA_VJP, aba_vjp_aligned_smem(mv, m->max_width)))
+  if (use_warp_bodies(m, JK_ABA_VJP, B))
+    return finish(fn, launch_wb_aba_vjp(m->wt, mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
+                                        (float*)scratch, (cudaStream_t)stream));
+  if (use_adjoint_tile(m, JK_ABA_VJP, B, aba_vjp_aligned_smem(mv, m->max_width)))
     return finish(fn, launch_aba_vjp_aligned(mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
                                              (float*)scratch, m->max_width, m->block[JK_ABA_VJP],
                                              (cudaStream_t)stream));
@@ -1006,7 +1078,10 @@ fst_status fst_rnea_loss_grad(const fst_model* m, int64_t B, const float* q, con
   FST_CHECK(need(fn, qdd, "qdd"));
   FST_CHECK(need(fn, tau_meas, "tau_meas"));
   const ModelView mv = view_of(m, theta);
-  if (aligned_fits(m, JK_LOSS_GRAD, rnea_vjp_aligned_smem(mv)))
+  if (use_warp_bodies(m, JK_LOSS_GRAD, B))
+    return finish(fn, launch_wb_loss_grad(m->wt, mv, B, q, qd, qdd, tau_meas, loss_theta_bar, q_bar, qd_bar,
+                                          (float*)scratch, (cudaStream_t)stream));
+  if (use_adjoint_tile(m, JK_LOSS_GRAD, B, rnea_vjp_aligned_smem(mv)))
     return finish(fn, launch_loss_grad_aligned(mv, B, q, qd, qdd, tau_meas, loss_theta_bar, q_bar, qd_bar,
                                                (float*)scratch, m->block[JK_LOSS_GRAD], (cudaStream_t)stream));
   if (use_jit(m, JK_LOSS_GRAD)) {
@@ -1100,7 +1175,8 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
     level = true;
     size_t most = 0;
     for (int k = 0; k < n; ++k) {
-      level = level && (io[k].B == 0 || tile_default(g->models[k], io[k].B));
+      for (int op : {JK_FK, JK_RNEA, JK_CRBA, JK_ABA})
+        level = level && (io[k].B == 0 || tile_rule(g->models[k], op, false, io[k].B));
       for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) most = std::max(most, state_of(k, r));
     }
     level = level && a.model_bytes + (size_t)a.max_rows * 32 * sizeof(float) + most <= kLevelSmemLimit;

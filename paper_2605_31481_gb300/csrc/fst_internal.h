@@ -30,6 +30,7 @@ struct fst_model {
   fst::TopoLists* dt = nullptr;      // device copy, followed by the device copy of hd
   fst::DofLists hd{};                // the tree of the degrees of freedom (host copy)
   int dof_depth = 0;                 // its depth
+  fst::WarpTree wt{};                // the tree as an argument of the warp-per-body kernels (n = 0: too many bodies)
   int dof_entries = 0;               // entries of a tree-sparse matrix (hd.anc)
   int* dpin = nullptr;               // SM-pinned launches: role table, then the counter regions
   int pin_table[256] = {};           // host copy of the role table (FST_ROLE_*, -1 none)

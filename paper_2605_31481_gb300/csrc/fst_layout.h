@@ -102,6 +102,20 @@ struct PackedJ {
   int off[FST_MAX_LINKS];
 };
 
+constexpr int kMaxWarpBodies = 16;
+
+// The tree as a kernel argument. Entry w: the body of warp w.
+struct WarpTree {
+  struct Entry {
+    unsigned char body, type, level, n_child;
+    signed char parent;       // body index, -1 for a root
+    unsigned char child0;     // first of its children in child[]
+    unsigned char qi, vi;
+  } e[kMaxWarpBodies];
+  unsigned char child[kMaxWarpBodies];
+  int n, depth;
+};
+
 // Floats of level-parallel state per body and environment (level.cuh):
 // FK X 12; RNEA X 12 | v 6 | a 6 | f 6; CRBA X 12 | Ic 10 | contribution 10;
 // ABA X 12 | va 6 | c 6 | IA 21 | pA 6 | U 6 | invD | u.
@@ -123,6 +137,7 @@ constexpr int kCrbaLeanRingFloats = 10;
 // adjoint in aligned frames (aligned.cuh).
 constexpr int kDerivState = 49;
 constexpr int kVjpState = 51;
+constexpr int kFkVjpState = 18;
 
 // Operators of the fused evaluation kernel, in launch order (longest first,
 // so the slowest role's blocks are dispatched first).

@@ -159,6 +159,9 @@ size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw);
 // its roles. The RNEA role may carry the adjoint (a.rnea_flags), M and J the
 // packed layouts; EVAL_KIN_IN_RNEA does not apply.
 size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw);
+size_t fk_vjp_tile_smem(const ModelView& mv);
+cudaError_t launch_fk_vjp_tile(const ModelView& mv, int64_t B, const float* q, const float* pbar, float* qbar,
+                               int block, cudaStream_t s);
 cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    float* tau, float* tape, int block, cudaStream_t s);
 cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, size_t smem, int maxw, int block,
@@ -177,6 +180,16 @@ cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float
 cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
                                    float* scratch, int maxw, int block, cudaStream_t s);
+// Warp-per-body kernels (warpbody.cu), for trees of at most kMaxWarpBodies.
+cudaError_t launch_wb_rnea_vjp(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,
+                               const float* qdd, const float* tbar, float* qbar, float* qdbar, float* qddbar,
+                               float* thbar, float* scratch, cudaStream_t s);
+cudaError_t launch_wb_loss_grad(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,
+                                const float* qdd, const float* tau_meas, float* loss_theta, float* qbar, float* qdbar,
+                                float* scratch, cudaStream_t s);
+cudaError_t launch_wb_aba_vjp(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,
+                              const float* qdd, const float* qddbar, float* qbar, float* qdbar, float* taubar,
+                              float* thbar, float* scratch, cudaStream_t s);
 cudaError_t launch_aba_level_pinned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                     const float* tau, float* qdd, int block, const PinArgs& p, cudaStream_t s);
 cudaError_t launch_aba_vjp(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,

@@ -237,6 +237,19 @@ fst_status build_model_host(const fst_body_desc* bodies, int32_t n, const double
       if (bodies[j].parent == i) T.child[k++] = j;
   }
   T.child_start[n] = k;
+  if (n <= kMaxWarpBodies) {
+    WarpTree& wt = m->wt;
+    wt.n = n;
+    wt.depth = depth;
+    for (int w = 0; w < n; ++w) {
+      const int i = T.level_body[w];
+      wt.e[w] = WarpTree::Entry{(unsigned char)i, (unsigned char)m->hi[i].type, (unsigned char)(m->level[i] - 1),
+                                (unsigned char)(T.child_start[i + 1] - T.child_start[i]),
+                                (signed char)m->hi[i].parent, (unsigned char)T.child_start[i],
+                                (unsigned char)m->hi[i].qi, (unsigned char)m->hi[i].vi};
+    }
+    for (int c = 0; c < T.child_start[n]; ++c) wt.child[c] = (unsigned char)T.child[c];
+  }
   // the tree of the degrees of freedom
   DofLists& D = m->hd;
   std::vector<int> par(nv, -1), last(n, -1);  // parent of each; the last one on each body's support path
