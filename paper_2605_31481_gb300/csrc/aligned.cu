@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(512) rnea_derivs_aligned_kernel(ModelView mv, 
 __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                                  const float* __restrict__ qd,
                                                                  const float* __restrict__ tau, float* qdd, float* dq,
-                                                                 float* dqd, float* Minv, int maxw, int entries,
+                                                                 float* dqd, float* Minv, int entries,
                                                                  int dof_depth, int state_floats) {
   FST_TILE;
   const int nv = mv.nv, W = n_warps(), w = warp_id();
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, i
   const Col cq = tile_col(tile, 0), cqd = tile_col(tile, mv.nq);
   float* const qcol = tile + (mv.nq + 2 * nv) * kLaneEnvs + lane;  // qdd
   aba_level_lean(sm, world_accel(mv), cq, cqd, tile_col(tile, mv.nq + nv), LaneState{state, kAbaLeanBodyFloats},
-                 LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, qdd, B, e, act,
+                 LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, qdd, B, e, act,
                  qcol);
   const TreeMat H{hbase, lists, lists + nv, anc};
   rnea_derivs_aligned<true>(sm, world_accel(mv), cq, cqd, Col{qcol, kLaneEnvs}, nv, LaneState{state, kDerivState}, H,
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
                                                               const float* __restrict__ qd,
                                                               const float* __restrict__ qdd,
                                                               const float* __restrict__ qddbar, float* qbar,
-                                                              float* qdbar, float* taubar, float* partial, int maxw) {
+                                                              float* qdbar, float* taubar, float* partial) {
   FST_TILE;
   const int nv = mv.nv;
   // rows: q | qd | qdd | qddbar | lambda | one row of zeros
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
   float* const lam = tile + (mv.nq + 3 * nv) * kLaneEnvs + lane;
   const Col cq = tile_col(tile, 0);
   aba_level_lean(sm, sv_zero(), cq, Col{zero, 0}, tile_col(tile, mv.nq + 2 * nv), LaneState{state, kAbaLeanBodyFloats},
-                 LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, taubar, B, e, act,
+                 LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, taubar, B, e, act,
                  lam);
   const VjpAligned o{qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
   rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, tile_col(tile, mv.nq), tile_col(tile, mv.nq + nv), lam,
@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int6
 // us; the specialised fused kernel that the default took before 31.3, its
 // roles' straight-line code refetched by every SM) and by shared memory, two
 // to four tiles an SM, at larger batches (humanoid, B = 16384: 164 -> 86 us).
-template <bool EXT>
-__global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B, EvalArgs a, int maxw) {
+template <bool EXT, bool LEAN>
+__global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B, EvalArgs a) {
   FST_TILE;
   const int role = a.roles[blockIdx.y], nv = mv.nv;
   const bool vjp = EXT && role == ROLE_RNEA && (a.rnea_flags & EVAL_RNEA_VJP);
@@ -244,19 +244,28 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
   switch (role) {
     case ROLE_ABA:
       aba_level_lean(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
-                     LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, maxw, a.qdd_out, B,
+                     LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, a.qdd_out, B,
                      e, act);
       break;
     case ROLE_CRBA:
-      if (EXT && a.packed)
+      if (LEAN) {
+        const LaneState S{state, kCrbaLeanBodyFloats};
+        const LaneState R{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
+        if (EXT && a.packed)
+          crba_level_lean<true>(sm, a.q, nv, S, R, a.M, B, e, act);
+        else
+          crba_level_lean(sm, a.q, nv, S, R, a.M, B, e, act);
+      } else if (EXT && a.packed) {
         crba_level<true>(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
-      else
+      } else {
         crba_level(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
+      }
       break;
     case ROLE_RNEA:
       if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
-        rnea_level(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaState}, a.tau_out, B, e, act,
-                   vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
+        rnea_level<LEAN>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
+                         a.tau_out, B, e, act,
+                         vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
       if (vjp)  // rnea_level ends with a barrier: the cotangent is complete and the state free
         rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, c1, c2, tile + (mv.nq + 2 * nv) * kLaneEnvs + lane,
                                     LaneState{state, kVjpState}, VjpAligned{a.qbar, a.qdbar, a.qddbar, nullptr, 1.f},
@@ -272,8 +281,8 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
 size_t floats32(size_t f) { return f * kLaneEnvs * sizeof(float); }
 
 // Per-body state that also holds the lean ABA's (run before it in the same space).
-size_t state_with_aba(int n, int maxw, int per_body) {
-  const size_t a = (size_t)kAbaLeanBodyFloats * n + 2 * kAbaLeanRingFloats * maxw, b = (size_t)per_body * n;
+size_t state_with_aba(int n, int slots, int per_body) {
+  const size_t a = (size_t)kAbaLeanBodyFloats * n + kAbaLeanSlotFloats * slots, b = (size_t)per_body * n;
   return a > b ? a : b;
 }
 
@@ -295,34 +304,34 @@ size_t rnea_vjp_aligned_smem(const ModelView& mv) {
   return smem_bytes(mv.n) + floats32((size_t)mv.nq + 3 * mv.nv + (size_t)kVjpState * mv.n);
 }
 
-size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw) {
-  return smem_bytes(mv.n) + floats32((size_t)mv.nq + 4 * mv.nv + 1 + state_with_aba(mv.n, maxw, kVjpState));
+size_t aba_vjp_aligned_smem(const ModelView& mv, int slots) {
+  return smem_bytes(mv.n) + floats32((size_t)mv.nq + 4 * mv.nv + 1 + state_with_aba(mv.n, slots, kVjpState));
 }
 
 // The forward-dynamics derivatives' solve phase keeps two columns per warp in
 // the state's space: the block is as large as that allows (0: not one warp).
-static int aba_derivs_threads(const ModelView& mv, int maxw, int set, int64_t tiles) {
-  const size_t st = state_with_aba(mv.n, maxw, kDerivState);
+static int aba_derivs_threads(const ModelView& mv, int slots, int set, int64_t tiles) {
+  const size_t st = state_with_aba(mv.n, slots, kDerivState);
   int t = aligned_block(set, mv.n, tiles);
   while (t >= 32 && (size_t)(t / 32) * 2 * mv.nv > st) t /= 2;
   return t >= 32 ? t : 0;
 }
 
-size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries) {
-  if (!aba_derivs_threads(mv, maxw, 32, 1)) return kLevelSmemLimit + 1;
+size_t aba_derivs_aligned_smem(const ModelView& mv, int slots, int entries) {
+  if (!aba_derivs_threads(mv, slots, 32, 1)) return kLevelSmemLimit + 1;
   return smem_bytes(mv.n) +
-         floats32((size_t)mv.nq + 3 * mv.nv + state_with_aba(mv.n, maxw, kDerivState) + entries) +
+         floats32((size_t)mv.nq + 3 * mv.nv + state_with_aba(mv.n, slots, kDerivState) + entries) +
          ((size_t)4 * mv.nv + 1 + entries) * sizeof(int);
 }
 
-size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw) {
+size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, bool lean, int slots) {
   size_t f = mv.nq;
   if (role == ROLE_ABA)
-    f += 2 * (size_t)mv.nv + (size_t)kAbaLeanBodyFloats * mv.n + (size_t)2 * kAbaLeanRingFloats * maxw;
+    f += 2 * (size_t)mv.nv + (size_t)kAbaLeanBodyFloats * mv.n + (size_t)kAbaLeanSlotFloats * slots;
   else if (role == ROLE_CRBA)
-    f += (size_t)kCrbaState * mv.n;
+    f += lean ? (size_t)kCrbaLeanBodyFloats * mv.n + (size_t)kCrbaLeanSlotFloats * slots : (size_t)kCrbaState * mv.n;
   else if (role == ROLE_RNEA)
-    f += (vjp ? 3 : 2) * (size_t)mv.nv + (size_t)(vjp ? kVjpState : kRneaState) * mv.n;
+    f += (vjp ? 3 : 2) * (size_t)mv.nv + (size_t)(vjp ? kVjpState : lean ? kRneaLeanFloats : kRneaState) * mv.n;
   else
     f += (size_t)kFkState * mv.n;
   return smem_bytes(mv.n) + floats32(f);
@@ -348,17 +357,16 @@ cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, size_t smem, int maxw, int block,
+cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, bool lean, size_t smem, int block,
                              cudaStream_t s) {
   const dim3 grid(grid_for(B, kLaneEnvs), a.n_roles);
-  if (a.rnea_flags || a.packed) {
-    prepare(eval_tile_kernel<true>, smem);
-    eval_tile_kernel<true><<<grid, block, smem, s>>>(mv, B, a, maxw);
-  } else {
-    prepare(eval_tile_kernel<false>, smem);
-    eval_tile_kernel<false><<<grid, block, smem, s>>>(mv, B, a, maxw);
-  }
-  return cudaGetLastError();
+  auto go = [&](auto* k) {
+    prepare(k, smem);
+    k<<<grid, block, smem, s>>>(mv, B, a);
+    return cudaGetLastError();
+  };
+  if (a.rnea_flags || a.packed) return lean ? go(eval_tile_kernel<true, true>) : go(eval_tile_kernel<true, false>);
+  return lean ? go(eval_tile_kernel<false, true>) : go(eval_tile_kernel<false, false>);
 }
 
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
@@ -371,13 +379,13 @@ cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const flo
 }
 
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
-                                      const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int maxw,
+                                      const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int slots,
                                       int entries, int dof_depth, int block, cudaStream_t s) {
-  const size_t sh = aba_derivs_aligned_smem(mv, maxw, entries);
+  const size_t sh = aba_derivs_aligned_smem(mv, slots, entries);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_derivs_aligned_kernel, sh);
-  aba_derivs_aligned_kernel<<<tiles, aba_derivs_threads(mv, maxw, block, tiles), sh, s>>>(
-      mv, B, q, qd, tau, qdd, dq, dqd, Minv, maxw, entries, dof_depth, (int)state_with_aba(mv.n, maxw, kDerivState));
+  aba_derivs_aligned_kernel<<<tiles, aba_derivs_threads(mv, slots, block, tiles), sh, s>>>(
+      mv, B, q, qd, tau, qdd, dq, dqd, Minv, entries, dof_depth, (int)state_with_aba(mv.n, slots, kDerivState));
   return cudaGetLastError();
 }
 
@@ -409,12 +417,12 @@ cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float
 
 cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
-                                   float* scratch, int maxw, int block, cudaStream_t s) {
-  const size_t sh = aba_vjp_aligned_smem(mv, maxw);
+                                   float* scratch, int slots, int block, cudaStream_t s) {
+  const size_t sh = aba_vjp_aligned_smem(mv, slots);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_vjp_aligned_kernel, sh);
   aba_vjp_aligned_kernel<<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(mv, B, q, qd, qdd, qddbar, qbar, qdbar,
-                                                                             taubar, thbar ? scratch : nullptr, maxw);
+                                                                             taubar, thbar ? scratch : nullptr);
   cudaError_t err = cudaGetLastError();
   if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
   return err;

@@ -101,7 +101,7 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 // bits. Both sides measured on GB300 (us, tiles / other):
 //  * generic other side. Tiles shorten the chain from the bodies to the
 //    levels: humanoid29 B = 4096 RNEA 9.1 / 22.8, CRBA 10.6 / 72.5, ABA 15 /
-//    53; B = 65536 FK 24 / 40, CRBA 91 / 160, ABA 117 / 200. A chain has no
+//    53; B = 65536 FK 24 / 40, RNEA 51 / 68, CRBA 91 / 160, ABA 94 / 200. A chain has no
 //    width to share: arm7 ABA 13 / 13 at 4096, 26 / 16 at 16384. Narrow trees
 //    (fewer than three bodies a level) at large batches are better off with
 //    more environments per SM where the sweeps are light: quadruped11 B =
@@ -111,8 +111,8 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 //    4096 FK 5.4 / 2.8, ABA 13.6 / 9.0; B = 65536 ABA 64 / 15) and large
 //    batches (quadruped11 B = 16384 RNEA 10 / 7.7, ABA 14 / 14.8, B = 32768
 //    ABA 26 / 16; at 4096 ABA 11 / 14.6, the step 14 / 17) and on large trees
-//    only for the light operators (humanoid29 B = 32768 FK 13 / 8.5, RNEA 38 /
-//    23; CRBA 52 / 93, ABA 67 / 149).
+//    only for the light operators (humanoid29 B = 32768 FK 13 / 8.5, RNEA 29 /
+//    23; CRBA 52 / 93, ABA 56 / 149).
 bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
   const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
   if (spec) {
@@ -164,9 +164,20 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
 
 constexpr int kMultiTileBlock = 256;  // threads per block of the mixed-tree launch in tiles
 
-int tile_block(const fst_model* m, int kind) {
+// Whether enough tiles wait for an SM (more than two each) that the forms
+// which keep less state, and so more tiles per SM, are the better ones.
+bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
+
+// Threads per block of a tile launch that does not set them: eight warps, but
+// four where many tiles share an SM and a level is never wider (quadruped11 B =
+// 16384 RNEA 9.8 -> 8.6 us, ABA 24.4 -> 14.1, the step 40.5 -> 38.8; legged18, six
+// bodies wide, ABA 19.0 against 27.5 with four). The adjoint's state leaves
+// room for too few tiles (the fused step with it 38.7 against 44.3 with four),
+// and CRBA's stores want the warps (B = 65536 29.1 against 31.1).
+int tile_block(const fst_model* m, int kind, int64_t B, bool vjp = false) {
   if (m->block[kind]) return m->block[kind];
-  return 256;
+  if (!many_tiles(B) || m->max_width > 4 || vjp || kind == JK_CRBA) return 256;
+  return m->n <= 16 || kind == JK_ABA ? 128 : 256;
 }
 
 // The path-parallel kernel slot a call of this kind runs (0: none): 1 for
@@ -448,7 +459,7 @@ fst_status fst_fk(const fst_model* m, int64_t B, const float* q, float* poses, v
     return finish(fn, launch_fk_level(mv, B, q, poses, level_block(m, JK_FK), level_tiles(m, JK_FK),
                         (cudaStream_t)stream));
   if (use_tile(m, JK_FK, B, level_smem_needed(mv, LEVEL_FK)))
-    return finish(fn, launch_fk_level(mv, B, q, poses, tile_block(m, JK_FK), 1, (cudaStream_t)stream));
+    return finish(fn, launch_fk_level(mv, B, q, poses, tile_block(m, JK_FK, B), 1, (cudaStream_t)stream));
   if (use_path(m, JK_FK))
     return finish(fn, path_go(m, JK_FK, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, poses));
   if (use_jit(m, JK_FK))
@@ -478,7 +489,7 @@ fst_status fst_jacobian(const fst_model* m, int64_t B, const float* q, const int
     return finish(fn, launch_jac_level(mv, B, q, L, J, level_block(m, JK_JACOBIAN), level_tiles(m, JK_JACOBIAN),
                         (cudaStream_t)stream));
   if (use_tile(m, JK_JACOBIAN, B, level_smem_needed(mv, LEVEL_JAC)))
-    return finish(fn, launch_jac_level(mv, B, q, L, J, tile_block(m, JK_JACOBIAN), 1, (cudaStream_t)stream));
+    return finish(fn, launch_jac_level(mv, B, q, L, J, tile_block(m, JK_JACOBIAN, B), 1, (cudaStream_t)stream));
   if (use_path(m, JK_JACOBIAN))
     return finish(fn, path_go(m, JK_JACOBIAN, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, L, J));
   if (use_jit(m, JK_JACOBIAN))
@@ -501,7 +512,10 @@ fst_status fst_rnea(const fst_model* m, int64_t B, const float* q, const float* 
     return finish(fn, launch_rnea_level(mv, B, q, qd, qdd, tau, level_block(m, JK_RNEA), level_tiles(m, JK_RNEA),
                         (cudaStream_t)stream));
   if (use_tile(m, JK_RNEA, B, level_smem_needed(mv, LEVEL_RNEA)))
-    return finish(fn, launch_rnea_level(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA), 1, (cudaStream_t)stream));
+    return finish(fn, many_tiles(B)
+                          ? launch_rnea_lean(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA, B), (cudaStream_t)stream)
+                          : launch_rnea_level(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA, B), 1,
+                                              (cudaStream_t)stream));
   if (use_path(m, JK_RNEA))
     return finish(fn, path_go(m, JK_RNEA, B, m->nq + 2 * m->nv, 1, (cudaStream_t)stream, mv, B, q, qd, qdd, tau));
   if (use_jit(m, JK_RNEA))
@@ -521,11 +535,11 @@ fst_status fst_crba(const fst_model* m, int64_t B, const float* q, const float* 
   if (use_level(m, JK_CRBA, LEVEL_CRBA))
     return finish(fn, launch_crba_level(mv, B, q, M, level_block(m, JK_CRBA), level_tiles(m, JK_CRBA),
                         (cudaStream_t)stream));
-  if (m->variant[JK_CRBA] == FST_VARIANT_LEVEL_LEAN && crba_lean_smem_needed(mv, m->max_width) <= kLevelSmemLimit)
-    return finish(fn, launch_crba_level_lean(mv, B, q, M, level_block(m, JK_CRBA), m->max_width,
+  if (m->variant[JK_CRBA] == FST_VARIANT_LEVEL_LEAN && crba_lean_smem_needed(mv, m->slots) <= kLevelSmemLimit)
+    return finish(fn, launch_crba_level_lean(mv, B, q, M, level_block(m, JK_CRBA), m->slots,
                                              (cudaStream_t)stream));
   if (use_tile(m, JK_CRBA, B, level_smem_needed(mv, LEVEL_CRBA)))
-    return finish(fn, launch_crba_level(mv, B, q, M, tile_block(m, JK_CRBA), 1, (cudaStream_t)stream));
+    return finish(fn, launch_crba_level(mv, B, q, M, tile_block(m, JK_CRBA, B), 1, (cudaStream_t)stream));
   if (use_path(m, JK_CRBA))
     return finish(fn, path_go(m, JK_CRBA, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, M));
   if (use_jit(m, JK_CRBA))
@@ -547,8 +561,8 @@ fst_status fst_aba(const fst_model* m, int64_t B, const float* q, const float* q
   if (use_level(m, JK_ABA, LEVEL_ABA))
     return finish(fn, launch_aba_level(mv, B, q, qd, tau, qdd, level_block(m, JK_ABA), level_tiles(m, JK_ABA),
                         (cudaStream_t)stream));
-  if (m->variant[JK_ABA] == FST_VARIANT_LEVEL_LEAN && aba_lean_smem_needed(mv, m->max_width) <= kLevelSmemLimit)
-    return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, level_block(m, JK_ABA), m->max_width,
+  if (m->variant[JK_ABA] == FST_VARIANT_LEVEL_LEAN && aba_lean_smem_needed(mv, m->slots) <= kLevelSmemLimit)
+    return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, level_block(m, JK_ABA), m->slots,
                                             (cudaStream_t)stream));
   if (m->variant[JK_ABA] == FST_VARIANT_PINNED) {
     int* counters = m->dpin + kPinTableSize + kPinAbaRegion * kPinRegion;
@@ -558,8 +572,8 @@ fst_status fst_aba(const fst_model* m, int64_t B, const float* q, const float* q
                                     PinArgs{m->dpin, counters}, (cudaStream_t)stream);
     return finish(fn, err);
   }
-  if (use_tile(m, JK_ABA, B, aba_lean_smem_needed(mv, m->max_width)))
-    return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, tile_block(m, JK_ABA), m->max_width,
+  if (use_tile(m, JK_ABA, B, aba_lean_smem_needed(mv, m->slots)))
+    return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, tile_block(m, JK_ABA, B), m->slots,
                                             (cudaStream_t)stream));
   if (use_path(m, JK_ABA))
     return finish(fn, path_go(m, JK_ABA, B, m->nq + 2 * m->nv, 1, (cudaStream_t)stream, mv, B, q, qd, tau, qdd));
@@ -739,9 +753,10 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
     t.rnea_flags &= ~EVAL_KIN_IN_RNEA;
     size_t sh = 0;
     for (int r = 0; r < t.n_roles; ++r)
-      sh = std::max(sh, eval_tile_smem(mv, t.roles[r], (t.rnea_flags & EVAL_RNEA_VJP) != 0, m->max_width));
+      sh = std::max(sh, eval_tile_smem(mv, t.roles[r], (t.rnea_flags & EVAL_RNEA_VJP) != 0, many_tiles(B), m->slots));
     if (t.n_roles && sh <= kLevelSmemLimit) {
-      const cudaError_t err = launch_eval_tile(mv, B, t, sh, m->max_width, tile_block(m, JK_EVAL), (cudaStream_t)stream);
+      const cudaError_t err = launch_eval_tile(mv, B, t, many_tiles(B), sh,
+                                               tile_block(m, JK_EVAL, B, t.rnea_flags != 0), (cudaStream_t)stream);
       if (err != cudaSuccess || g.n_roles == 0) return finish(fn, err);
       a = g;
     }
@@ -843,7 +858,7 @@ fst_status fst_fk_vjp(const fst_model* m, int64_t B, const float* q, const float
   FST_CHECK(need(fn, poses_bar, "poses_bar"));
   const ModelView mv = view_of(m, nullptr);
   if (use_adjoint_tile(m, JK_FK_VJP, B, fk_vjp_tile_smem(mv)))
-    return finish(fn, launch_fk_vjp_tile(mv, B, q, poses_bar, q_bar, tile_block(m, JK_FK_VJP), (cudaStream_t)stream));
+    return finish(fn, launch_fk_vjp_tile(mv, B, q, poses_bar, q_bar, tile_block(m, JK_FK_VJP, B), (cudaStream_t)stream));
   if (use_jit(m, JK_FK_VJP))
     return finish(fn, jit_go(m, JK_FK_VJP, B, m->nq + 12 * m->n, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              poses_bar, q_bar));
@@ -907,7 +922,7 @@ fst_status fst_rnea_store(const fst_model* m, int64_t B, const float* q, const f
   }
   const ModelView mv = view_of(m, theta);
   if (use_tile(m, JK_RNEA_STORE, B, level_smem_needed(mv, LEVEL_RNEA)))
-    return finish(fn, launch_rnea_store_tile(mv, B, q, qd, qdd, tau, tape, tile_block(m, JK_RNEA_STORE),
+    return finish(fn, launch_rnea_store_tile(mv, B, q, qd, qdd, tau, tape, tile_block(m, JK_RNEA_STORE, B),
                                              (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_STORE))
     return finish(fn, jit_go(m, JK_RNEA_STORE, B, m->nq + 2 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
@@ -1016,8 +1031,8 @@ fst_status fst_aba_derivatives(const fst_model* m, int64_t B, const float* q, co
   FST_CHECK(need(fn, tau, "tau"));
   FST_CHECK(need(fn, Minv, "Minv"));
   const ModelView mv = view_of(m, theta);
-  if (use_adjoint_tile(m, JK_ABA_DERIVS, B, aba_derivs_aligned_smem(mv, m->max_width, m->dof_entries)))
-    return finish(fn, launch_aba_derivs_aligned(mv, B, q, qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv, m->max_width,
+  if (use_adjoint_tile(m, JK_ABA_DERIVS, B, aba_derivs_aligned_smem(mv, m->slots, m->dof_entries)))
+    return finish(fn, launch_aba_derivs_aligned(mv, B, q, qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv, m->slots,
                                                 m->dof_entries, m->dof_depth, m->block[JK_ABA_DERIVS],
                                                 (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_DERIVS))
@@ -1045,9 +1060,9 @@ fst_status fst_aba_vjp(const fst_model* m, int64_t B, const float* q, const floa
   if (use_warp_bodies(m, JK_ABA_VJP, B))
     return finish(fn, launch_wb_aba_vjp(m->wt, mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
                                         (float*)scratch, (cudaStream_t)stream));
-  if (use_adjoint_tile(m, JK_ABA_VJP, B, aba_vjp_aligned_smem(mv, m->max_width)))
+  if (use_adjoint_tile(m, JK_ABA_VJP, B, aba_vjp_aligned_smem(mv, m->slots)))
     return finish(fn, launch_aba_vjp_aligned(mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
-                                             (float*)scratch, m->max_width, m->block[JK_ABA_VJP],
+                                             (float*)scratch, m->slots, m->block[JK_ABA_VJP],
                                              (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_VJP)) {
     unsigned nblk = 0;
@@ -1150,7 +1165,6 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
     a.io[k] = MultiIO{x.q, x.qd, x.qdd, x.tau, x.poses, m->nv ? x.tau_out : nullptr, m->nv ? x.M : nullptr,
                       m->nv ? x.qdd_out : nullptr, x.B};
     if (m->n > max_n) max_n = m->n;
-    a.maxw[k] = m->max_width;
     const int rows = m->nq + 2 * m->nv;
     if (rows > a.max_rows) a.max_rows = rows;
   }
@@ -1163,7 +1177,7 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
   // environments if every tree's calls do and their state fits
   auto state_of = [&](int k, int r) {  // level: bytes of per-body state of a (tree, operator) pair
     const fst_model* m = g->models[k];
-    const size_t floats = r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + 2 * kAbaLeanRingFloats * m->max_width
+    const size_t floats = r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + kAbaLeanSlotFloats * m->slots
                           : (size_t)(r == ROLE_CRBA ? kCrbaStateFloats
                                      : r == ROLE_RNEA ? kRneaStateFloats : kFkStateFloats) * m->n;
     return floats * 32 * sizeof(float);

@@ -37,7 +37,7 @@ struct BodyC {
   float S[6];
   float theta[10];
   unsigned long long anc;  // bit j set: body j is on this body's support path (itself included)
-  int32_t lpos;            // position of the body within its tree level (level_body order)
+  int32_t slot;            // where the lean CRBA and ABA leave its contribution to the parent
   float pad[9];
 };
 static_assert(sizeof(BodyC) == 256, "BodyC must stay 256 bytes");
@@ -117,21 +117,22 @@ struct WarpTree {
 };
 
 // Floats of level-parallel state per body and environment (level.cuh):
-// FK X 12; RNEA X 12 | v 6 | a 6 | f 6; CRBA X 12 | Ic 10 | contribution 10;
+// FK X 12; RNEA v 6 | a 6 | f 6 | X 12 (lean: the first two); CRBA X 12 | Ic 10 | contribution 10;
 // ABA X 12 | va 6 | c 6 | IA 21 | pA 6 | U 6 | invD | u.
 constexpr int kFkStateFloats = 12;
 constexpr int kRneaStateFloats = 30;
+constexpr int kRneaLeanFloats = 12;
 constexpr int kCrbaStateFloats = 32;
 constexpr int kAbaStateFloats = 59;
 // The lean level-parallel ABA (FST_VARIANT_LEVEL_LEAN): per body VU 6 (v,
-// then U, then a) | c 6 | invD | u; per level parity and position within the
-// level, the contribution to the parent: X^T I^a X 21 | X^T p^a 6.
+// then U, then a) | c 6 | invD | u; per contribution slot, what a body passes
+// to its parent: X^T I^a X 21 | X^T p^a 6.
 constexpr int kAbaLeanBodyFloats = 14;
-constexpr int kAbaLeanRingFloats = 27;
-// The lean level-parallel CRBA: per body X 12 | F = Ic S 6; per ring slot
-// the composite-inertia contribution to the parent (10).
+constexpr int kAbaLeanSlotFloats = 27;
+// The lean level-parallel CRBA: per body X 12 | F = Ic S 6; per slot the
+// composite-inertia contribution to the parent (10).
 constexpr int kCrbaLeanBodyFloats = 18;
-constexpr int kCrbaLeanRingFloats = 10;
+constexpr int kCrbaLeanSlotFloats = 10;
 
 // Shared state per body and environment of the dense derivatives and of the
 // adjoint in aligned frames (aligned.cuh).

@@ -114,14 +114,16 @@ cudaError_t launch_aba_level(const ModelView& mv, int64_t B, const float* q, con
                              float* qdd, int block, int tiles, cudaStream_t s);
 cudaError_t launch_eval_level(const ModelView& mv, int64_t B, const EvalArgs& a, int block, int tiles,
                               cudaStream_t s);
-// The lean level-parallel ABA (FST_VARIANT_LEVEL_LEAN); maxw = bodies of the
-// widest tree level.
-size_t aba_lean_smem_needed(const ModelView& mv, int maxw, int tiles = 1);
+// The lean level-parallel ABA (FST_VARIANT_LEVEL_LEAN); slots = fst_model::slots.
+size_t aba_lean_smem_needed(const ModelView& mv, int slots);
 cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* tau,
-                                  float* qdd, int block, int maxw, cudaStream_t s);
+                                  float* qdd, int block, int slots, cudaStream_t s);
+// RNEA with the lean state (the same bits as launch_rnea_level).
+cudaError_t launch_rnea_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                             float* tau, int block, cudaStream_t s);
 // The lean level-parallel CRBA (FST_VARIANT_LEVEL_LEAN).
-size_t crba_lean_smem_needed(const ModelView& mv, int maxw);
-cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int maxw,
+size_t crba_lean_smem_needed(const ModelView& mv, int slots);
+cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int slots,
                                    cudaStream_t s);
 
 // Adjoints (adjoint.cu). scratch: vjp_scratch_floats(n, B) floats of device
@@ -149,27 +151,27 @@ cudaError_t launch_crba_vjp(const ModelView& mv, int64_t B, const float* q, cons
                             float* thbar, float* scratch, cudaStream_t s);
 // Aligned-frame kernels (aligned.cu), one tile of 32 environments per block
 // (block = 0: built-in choice). The *_smem functions give the shared memory a
-// launch needs: above kLevelSmemLimit the kernel cannot run. maxw = bodies of
-// the widest tree level; entries, dof_depth: see fst_model.
+// launch needs: above kLevelSmemLimit the kernel cannot run. slots, entries, dof_depth: see fst_model.
 size_t rnea_derivs_aligned_smem(const ModelView& mv);
-size_t aba_derivs_aligned_smem(const ModelView& mv, int maxw, int entries);
+size_t aba_derivs_aligned_smem(const ModelView& mv, int slots, int entries);
 size_t rnea_vjp_aligned_smem(const ModelView& mv);
-size_t aba_vjp_aligned_smem(const ModelView& mv, int maxw);
+size_t aba_vjp_aligned_smem(const ModelView& mv, int slots);
 // The fused evaluation with these bodies; smem: the largest eval_tile_smem of
 // its roles. The RNEA role may carry the adjoint (a.rnea_flags), M and J the
-// packed layouts; EVAL_KIN_IN_RNEA does not apply.
-size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, int maxw);
+// packed layouts; EVAL_KIN_IN_RNEA does not apply. lean: RNEA and CRBA keep
+// their lean state (the same bits).
+size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, bool lean, int slots);
 size_t fk_vjp_tile_smem(const ModelView& mv);
 cudaError_t launch_fk_vjp_tile(const ModelView& mv, int64_t B, const float* q, const float* pbar, float* qbar,
                                int block, cudaStream_t s);
 cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    float* tau, float* tape, int block, cudaStream_t s);
-cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, size_t smem, int maxw, int block,
+cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, bool lean, size_t smem, int block,
                              cudaStream_t s);
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                        const float* qdd, float* dq, float* dqd, int block, cudaStream_t s);
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
-                                      const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int maxw,
+                                      const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int slots,
                                       int entries, int dof_depth, int block, cudaStream_t s);
 cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                     const float* tbar, float* qbar, float* qdbar, float* qddbar, float* thbar,
@@ -179,7 +181,7 @@ cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float
                                      float* scratch, int block, cudaStream_t s);
 cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
-                                   float* scratch, int maxw, int block, cudaStream_t s);
+                                   float* scratch, int slots, int block, cudaStream_t s);
 // Warp-per-body kernels (warpbody.cu), for trees of at most kMaxWarpBodies.
 cudaError_t launch_wb_rnea_vjp(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,
                                const float* qdd, const float* tbar, float* qbar, float* qdbar, float* qddbar,

@@ -55,6 +55,20 @@ __global__ void __launch_bounds__(256) rnea_level_kernel(ModelView mv, int64_t B
              Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
+// RNEA with 12 floats of state a body: four tiles of the floating humanoid per
+// SM instead of two (B = 65536: 66.6 -> 50.8 us, 16384: 20.1 -> 16.2).
+__global__ void __launch_bounds__(256) rnea_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                        const float* __restrict__ qd, const float* __restrict__ qdd,
+                                                        float* __restrict__ tau) {
+  FST_LEVEL_PROLOGUE(mv.nq + 2 * mv.nv, kRneaLeanFloats);
+  stage_block_rows(tile, q, mv.nq, B, e);
+  stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
+  stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
+  FST_LEVEL_READY;
+  rnea_level<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+                   Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
+}
+
 __global__ void __launch_bounds__(256) crba_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                          float* __restrict__ M) {
   FST_LEVEL_PROLOGUE(mv.nq, kCrbaState);
@@ -76,32 +90,38 @@ __global__ void __launch_bounds__(256) aba_level_kernel(ModelView mv, int64_t B,
 }
 
 // ABA with the lean per-tile state (FST_VARIANT_LEVEL_LEAN): per body
-// kAbaLeanBodyFloats, plus a ring of 2 x maxw contribution slots.
+// kAbaLeanBodyFloats, plus the contribution slots. Bound by the latency of its
+// level phases, so by the tiles an SM holds: with a slot per running
+// contribution instead of a ring of two levels the floating humanoid's tile
+// takes 75 KB instead of 90, three an SM instead of two (B = 65536: 118 -> 94
+// us; FP32 floor 18). Tried on top and not kept: four tiles, with qd and tau
+// read from global memory and the bias accelerations folded into the forces
+// (105 us, and 1 us more at small batches).
 __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                        const float* __restrict__ qd, const float* __restrict__ tau,
-                                                       float* __restrict__ qdd, int maxw) {
+                                                       float* __restrict__ qdd, int slots) {
   const int rows = mv.nq + 2 * mv.nv;
   FST_LEVEL_PROLOGUE_S(rows, kAbaLeanBodyFloats,
-                       (rows + kAbaLeanBodyFloats * mv.n + 2 * kAbaLeanRingFloats * maxw) * kLaneEnvs);
-  const LaneState R{tile + (rows + kAbaLeanBodyFloats * mv.n) * kLaneEnvs, kAbaLeanRingFloats};
+                       (rows + kAbaLeanBodyFloats * mv.n + kAbaLeanSlotFloats * slots) * kLaneEnvs);
+  const LaneState R{tile + (rows + kAbaLeanBodyFloats * mv.n) * kLaneEnvs, kAbaLeanSlotFloats};
   stage_block_rows(tile, q, mv.nq, B, e);
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, tau, mv.nv, B, e);
   FST_LEVEL_READY;
   aba_level_lean(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
-                 Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, maxw, qdd, B, e, act);
+                 Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, qdd, B, e, act);
 }
 
 // CRBA with the lean per-tile state (FST_VARIANT_LEVEL_LEAN): no staged
 // rows (q is read from global memory), kCrbaLeanBodyFloats per body, a ring
-// of 2 x maxw contribution slots. Up to three blocks per SM.
+// of contribution slots. Up to three blocks per SM.
 __global__ void __launch_bounds__(256, 3) crba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
-                                                           float* __restrict__ M, int maxw) {
+                                                           float* __restrict__ M, int slots) {
   FST_LEVEL_PROLOGUE_S(0, kCrbaLeanBodyFloats,
-                       (kCrbaLeanBodyFloats * mv.n + 2 * kCrbaLeanRingFloats * maxw) * kLaneEnvs);
-  const LaneState R{tile + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanRingFloats};
+                       (kCrbaLeanBodyFloats * mv.n + kCrbaLeanSlotFloats * slots) * kLaneEnvs);
+  const LaneState R{tile + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
   FST_LEVEL_READY;
-  crba_level_lean(sm, q, mv.nv, S, R, maxw, M, B, e, act);
+  crba_level_lean(sm, q, mv.nv, S, R, M, B, e, act);
 }
 
 // SM-pinned ABA (FST_VARIANT_PINNED): blocks on SMs pinned to ABA take
@@ -227,6 +247,11 @@ cudaError_t launch_rnea_level(const ModelView& mv, int64_t B, const float* q, co
                               float* tau, int block, int tiles, cudaStream_t s) {
   return go(rnea_level_kernel, mv, B, level_smem_needed(mv, LEVEL_RNEA, tiles), block, tiles, 1, s, q, qd, qdd, tau);
 }
+cudaError_t launch_rnea_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
+                             float* tau, int block, cudaStream_t s) {
+  const size_t sh = smem_bytes(mv.n) + level_tile_bytes(mv, mv.nq + 2 * mv.nv, kRneaLeanFloats);
+  return go(rnea_lean_kernel, mv, B, sh, block, 1, 1, s, q, qd, qdd, tau);
+}
 cudaError_t launch_crba_level(const ModelView& mv, int64_t B, const float* q, float* M, int block, int tiles,
                               cudaStream_t s) {
   return go(crba_level_kernel, mv, B, level_smem_needed(mv, LEVEL_CRBA, tiles), block, tiles, 1, s, q, M);
@@ -235,22 +260,21 @@ cudaError_t launch_aba_level(const ModelView& mv, int64_t B, const float* q, con
                              float* qdd, int block, int tiles, cudaStream_t s) {
   return go(aba_level_kernel, mv, B, level_smem_needed(mv, LEVEL_ABA, tiles), block, tiles, 1, s, q, qd, tau, qdd);
 }
-size_t aba_lean_smem_needed(const ModelView& mv, int maxw, int tiles) {
-  const size_t t = level_tile_bytes(mv, mv.nq + 2 * mv.nv, kAbaLeanBodyFloats) +
-                   (size_t)2 * kAbaLeanRingFloats * maxw * kLaneEnvs * sizeof(float);
-  return smem_bytes(mv.n) + (size_t)tiles * t;
+size_t aba_lean_smem_needed(const ModelView& mv, int slots) {
+  return smem_bytes(mv.n) + level_tile_bytes(mv, mv.nq + 2 * mv.nv, kAbaLeanBodyFloats) +
+         (size_t)kAbaLeanSlotFloats * slots * kLaneEnvs * sizeof(float);
 }
 cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* tau,
-                                  float* qdd, int block, int maxw, cudaStream_t s) {
-  return go(aba_lean_kernel, mv, B, aba_lean_smem_needed(mv, maxw, 1), block, 1, 1, s, q, qd, tau, qdd, maxw);
+                                  float* qdd, int block, int slots, cudaStream_t s) {
+  return go(aba_lean_kernel, mv, B, aba_lean_smem_needed(mv, slots), block, 1, 1, s, q, qd, tau, qdd, slots);
 }
-size_t crba_lean_smem_needed(const ModelView& mv, int maxw) {
+size_t crba_lean_smem_needed(const ModelView& mv, int slots) {
   return smem_bytes(mv.n) +
-         (size_t)(kCrbaLeanBodyFloats * mv.n + 2 * kCrbaLeanRingFloats * maxw) * kLaneEnvs * sizeof(float);
+         (size_t)(kCrbaLeanBodyFloats * mv.n + kCrbaLeanSlotFloats * slots) * kLaneEnvs * sizeof(float);
 }
-cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int maxw,
+cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int slots,
                                    cudaStream_t s) {
-  return go(crba_lean_kernel, mv, B, crba_lean_smem_needed(mv, maxw), block, 1, 1, s, q, M, maxw);
+  return go(crba_lean_kernel, mv, B, crba_lean_smem_needed(mv, slots), block, 1, 1, s, q, M, slots);
 }
 cudaError_t launch_aba_level_pinned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                     const float* tau, float* qdd, int block, const PinArgs& p, cudaStream_t s) {

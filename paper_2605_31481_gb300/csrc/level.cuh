@@ -100,7 +100,7 @@ struct LaneState {
 
 // floats of per-body state per environment
 constexpr int kFkState = kFkStateFloats;
-constexpr int kRneaState = kRneaStateFloats;   // X 12 | v 6 | a 6 | f 6
+constexpr int kRneaState = kRneaStateFloats;   // v 6 | a 6 | f 6 | X 12
 constexpr int kCrbaState = kCrbaStateFloats;   // X 12 | Ic 10 | contribution 10
 constexpr int kAbaState = kAbaStateFloats;    // X 12 | va 6 | c 6 | IA 21 | pA 6 | U 6 | invD | u
 
@@ -215,13 +215,21 @@ __device__ __forceinline__ void kin_level(const TP& tp, const Col& q, int nv, co
 // tau goes to global memory (may be null) and, if tau_col is not null, also to
 // that shared-memory column (rows of 32). With a tape, the forward state of
 // every body is left there for the store variant of the adjoint (tape_store's
-// layout).
-template <class TP>
+// layout). LEAN keeps 12 floats a body instead of 30: the force is formed on
+// the way back from v and a, which it then replaces, and the joint transform is
+// evaluated again instead of stored. That lengthens the chain (quadruped, B =
+// 4096: 7.4 -> 8 us) and lets twice the tiles share an SM; the arithmetic and
+// so the bits are the same.
+template <bool LEAN = false, class TP>
 __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& qdd,
                                            const LaneState& S, float* __restrict__ tau, int64_t B, int64_t e,
                                            bool act, float* tau_col = nullptr, float* tape = nullptr) {
   const int W = n_warps(), w = warp_id();
-  enum { X_ = 0, V_ = 12, A_ = 18, F_ = 24 };
+  enum { V_ = 0, A_ = 6, C_ = LEAN ? 0 : 12, X_ = 18 };  // v 6 | a 6 | force, then its contribution 6 | X 12
+  auto force = [&](int i, SV v, SV a) {
+    const In10 I = in_load(tp.theta(i));
+    return in_mul(I, a) + crf(v, in_mul(I, v));
+  };
   FST_UNROLL
   for (int l = 0; l < tp.depth(); ++l) {
     FST_FOR_MY_BODIES(tp, l, k) {
@@ -239,18 +247,19 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
         vi = X_motion(X, S.sv(bi.parent, V_)) + vJ;
         ai = X_motion(X, S.sv(bi.parent, A_)) + aJ + crm(vi, vJ);
       }
-      const In10 I = in_load(tp.theta(i));
-      S.putX(i, X_, X);
       S.put(i, V_, vi);
       S.put(i, A_, ai);
-      S.put(i, F_, in_mul(I, ai) + crf(vi, in_mul(I, vi)));
+      if (!LEAN) {
+        S.putX(i, X_, X);
+        S.put(i, C_, force(i, vi, ai));
+      }
       if (tape && act) {
         float* p = tape + (int64_t)i * 30 * B + e;
         const float r[24] = {X.R[0], X.R[1], X.R[2], X.R[3], X.R[4], X.R[5], X.R[6], X.R[7],
                              X.R[8], X.t[0], X.t[1], X.t[2], vi.w.x, vi.w.y, vi.w.z, vi.v.x,
                              vi.v.y, vi.v.z, ai.w.x, ai.w.y, ai.w.z, ai.v.x, ai.v.y, ai.v.z};
 #pragma unroll
-        for (int c = 0; c < 24; ++c) p[(int64_t)c * B] = r[c];
+        for (int c2 = 0; c2 < 24; ++c2) p[(int64_t)c2 * B] = r[c2];
       }
     }
     __syncthreads();
@@ -260,17 +269,17 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
     FST_FOR_MY_BODIES(tp, l, k) {
       const int i = tp.level_body(k);
       const BodyI bi = tp.I(i);
-      SV F = S.sv(i, F_);
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) F = F + S.sv(tp.child(ch), F_);
+      SV F = LEAN ? force(i, S.sv(i, V_), S.sv(i, A_)) : S.sv(i, C_);
+      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) F = F + S.sv(tp.child(ch), C_);
       if (act && tau) ST_store(tp.C(i), bi, F, tau, B, e);
       if (tau_col) ST_store(tp.C(i), bi, F, tau_col, kLaneEnvs, 0);
       if (tape && act) {
         float* p = tape + ((int64_t)i * 30 + 24) * B + e;
         const float r[6] = {F.w.x, F.w.y, F.w.z, F.v.x, F.v.y, F.v.z};
 #pragma unroll
-        for (int c = 0; c < 6; ++c) p[(int64_t)c * B] = r[c];
+        for (int c2 = 0; c2 < 6; ++c2) p[(int64_t)c2 * B] = r[c2];
       }
-      if (bi.parent >= 0) S.put(i, F_, XT_force(S.X(i, X_), F));
+      if (bi.parent >= 0) S.put(i, C_, XT_force(LEAN ? joint_X(tp.C(i), bi, q) : S.X(i, X_), F));
     }
     __syncthreads();
   }
@@ -381,29 +390,27 @@ __device__ __forceinline__ Xf joint_X_rows(const BodyC& c, const BodyI& bi, cons
 // The composite-rigid-body algorithm with less shared memory per tile (so
 // that three tiles of a large tree fit on one SM): per body only X and
 // F = I^c S stay (kCrbaLeanBodyFloats); a body's composite inertia moved to
-// its parent lives in ring R, slot (level parity, position within the
-// level), until the parent has added it; the root keeps its own I^c in its
-// level-0 slot for a free base's 6 x 6 block. q is read from global memory,
+// its parent lives in a slot of R (BodyC::slot) until the parent has added it;
+// the root keeps its own I^c in its slot for a free base's 6 x 6 block. q is read from global memory,
 // not staged. Same arithmetic, in the same order, as crba_level.
-template <class TP>
+template <bool PACKED = false, class TP>
 __device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __restrict__ q, int nv,
-                                                const LaneState& S, const LaneState& R, int maxw,
+                                                const LaneState& S, const LaneState& R,
                                                 float* __restrict__ M, int64_t B, int64_t e, bool act) {
   const int W = n_warps(), w = warp_id();
   enum { X_ = 0, F_ = 12 };
   const int64_t ec = act ? e : B - 1;  // lanes past B compute on the last environment and store nothing
-  if (tp.depth() > 0) m_clear_tile(M, (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
+  if (tp.depth() > 0) m_clear_tile(M, PACKED ? (int64_t)nv * (nv + 1) / 2 : (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
   FST_UNROLL
   for (int l = tp.depth() - 1; l >= 0; --l) {
     FST_FOR_MY_BODIES(tp, l, k) {
       const int i = tp.level_body(k);
       const BodyI bi = tp.I(i);
-      const int slot = (l & 1) * maxw + (k - tp.level_begin(l));
-      const int child_ring = ((l + 1) & 1) * maxw;
+      const int slot = tp.C(i).slot;
       const Xf X = joint_X_rows(tp.C(i), bi, q, B, ec);
       In10 Ic = in_load(tp.theta(i));
       for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch)
-        in_add(Ic, R.in10(child_ring + tp.C(tp.child(ch)).lpos, 0));
+        in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
       S.putX(i, X_, X);
       if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) S.put(i, F_, in_mul(Ic, S_of(tp.C(i))));
       R.putin(slot, 0, bi.parent >= 0 ? in_to_parent(X, Ic) : Ic);
@@ -411,32 +418,27 @@ __device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __res
     __syncthreads();
   }
   if (!act) return;
-  float* Me = M + e;
+  const MOut<PACKED> Me{M + e, nv, B};
   for (int i = w; i < tp.n(); i += W) {
     const BodyI bi = tp.I(i);
     if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
       SV F = S.sv(i, F_);
-      Me[((int64_t)bi.vi * nv + bi.vi) * B] = dot(S_of(tp.C(i)), F);
+      Me.one(bi.vi, bi.vi, dot(S_of(tp.C(i)), F));
       int kk = i;
       for (int j = bi.parent; j >= 0; j = tp.I(j).parent) {
         F = XT_force(S.X(kk, X_), F);
         kk = j;
         const BodyI bj = tp.I(j);
         if (bj.type == FST_JOINT_REVOLUTE || bj.type == FST_JOINT_PRISMATIC) {
-          const float mij = dot(S_of(tp.C(j)), F);
-          Me[((int64_t)bi.vi * nv + bj.vi) * B] = mij;
-          Me[((int64_t)bj.vi * nv + bi.vi) * B] = mij;
+          Me.sym(bi.vi, bj.vi, dot(S_of(tp.C(j)), F));
         } else if (bj.type == FST_JOINT_FREE) {
           const float col[6] = {F.v.x, F.v.y, F.v.z, F.w.x, F.w.y, F.w.z};
 #pragma unroll
-          for (int r = 0; r < 6; ++r) {
-            Me[((int64_t)(bj.vi + r) * nv + bi.vi) * B] = col[r];
-            Me[((int64_t)bi.vi * nv + bj.vi + r) * B] = col[r];
-          }
+          for (int r = 0; r < 6; ++r) Me.sym(bj.vi + r, bi.vi, col[r]);
         }
       }
     } else if (bi.type == FST_JOINT_FREE) {
-      const In10 I = R.in10(tp.C(i).lpos, 0);  // the root's own slot (level 0, parity 0)
+      const In10 I = R.in10(tp.C(i).slot, 0);  // the root's own slot
       const float blk[6][6] = {
           {I.m, 0.f, 0.f, 0.f, I.h.z, -I.h.y},
           {0.f, I.m, 0.f, -I.h.z, 0.f, I.h.x},
@@ -448,7 +450,7 @@ __device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __res
 #pragma unroll
       for (int r = 0; r < 6; ++r)
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) Me[((int64_t)(bi.vi + r) * nv + bi.vi + cc) * B] = blk[r][cc];
+        for (int cc = 0; cc < 6; ++cc) Me.one(bi.vi + r, bi.vi + cc, blk[r][cc]);
     }
   }
 }
@@ -560,20 +562,20 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
 // The same three passes with less state per tile, so that a large tree's
 // tiles fit two per SM: per body only VU (v in pass 1, U from pass 2, a in
 // pass 3), c, invD and u stay (kAbaLeanBodyFloats); a body's contribution to
-// its parent (X^T I^a X, X^T p^a) lives in ring R, slot (level parity,
-// position within the level), only until the parent has read it
-// (kAbaLeanRingFloats each, 2 x widest level slots); the rigid inertia and
+// its parent (X^T I^a X, X^T p^a) lives in a slot of R only until the parent
+// has read it (kAbaLeanSlotFloats each; the parent reuses its first child's,
+// BodyC::slot, so the humanoid needs 4); the rigid inertia and
 // the bias force are formed in pass 2, and the joint transforms recomputed
 // in passes 2 and 3 instead of stored. The root's I^A and p^A, which pass 3
-// needs for a free base, stay in its level-0 ring slot.
+// needs for a free base, stay in its slot.
 template <class TP>
 __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& tau,
-                                               const LaneState& S, const LaneState& R, int maxw,
+                                               const LaneState& S, const LaneState& R,
                                                float* __restrict__ qdd, int64_t B, int64_t e, bool act,
                                                float* qdd_col = nullptr) {
   const int W = n_warps(), w = warp_id();
   enum { VU_ = 0, C_ = 6, ID_ = 12, u_ = 13 };  // per body
-  enum { RI_ = 0, RP_ = 21 };                      // per ring slot
+  enum { RI_ = 0, RP_ = 21 };                      // per slot
   // 1. root to leaf: velocities and bias accelerations
   FST_UNROLL
   for (int l = 0; l < tp.depth(); ++l) {
@@ -595,21 +597,19 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
     }
     __syncthreads();
   }
-  // 2. leaf to root: articulated inertias; a body of level l leaves its
-  //    contribution in ring slot (l & 1) * maxw + its position in the level
+  // 2. leaf to root: articulated inertias
   FST_UNROLL
   for (int l = tp.depth() - 1; l >= 0; --l) {
     FST_FOR_MY_BODIES(tp, l, k) {
       const int i = tp.level_body(k);
       const BodyI bi = tp.I(i);
-      const int slot = (l & 1) * maxw + (k - tp.level_begin(l));
-      const int child_ring = ((l + 1) & 1) * maxw;
+      const int slot = tp.C(i).slot;
       const In10 I = in_load(tp.theta(i));
       const SV vi = S.sv(i, VU_);
       Sym6 IA = sym6_from_in(I);
       SV pA = crf(vi, in_mul(I, vi));
       for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
-        const int cs = child_ring + tp.C(tp.child(ch)).lpos;
+        const int cs = tp.C(tp.child(ch)).slot;
         sym6_add(IA, R.sym(cs, RI_));
         pA = pA + R.sv(cs, RP_);
       }
@@ -656,7 +656,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         if (qdd_col) qdd_col[bi.vi << 5] = qi;
         ai = sv_fma(qi, S_of(tp.C(i)), ai);
       } else if (bi.type == FST_JOINT_FREE) {
-        const int slot = k - tp.level_begin(l);  // level 0: ring parity 0
+        const int slot = tp.C(i).slot;
         const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};
         const SV anew = sym6_solve(R.sym(slot, RI_), tf - R.sv(slot, RP_));
         const SV x = anew - ai;

@@ -223,10 +223,7 @@ fst_status build_model_host(const fst_body_desc* bodies, int32_t n, const double
   for (int l = 0; l < depth; ++l) {
     T.level_start[l] = k;
     for (int i = 0; i < n; ++i)
-      if (m->level[i] == l + 1) {
-        m->hc[i].lpos = k - T.level_start[l];
-        T.level_body[k++] = i;
-      }
+      if (m->level[i] == l + 1) T.level_body[k++] = i;
     m->max_width = std::max(m->max_width, k - T.level_start[l]);
   }
   T.level_start[depth] = k;
@@ -237,6 +234,27 @@ fst_status build_model_host(const fst_body_desc* bodies, int32_t n, const double
       if (bodies[j].parent == i) T.child[k++] = j;
   }
   T.child_start[n] = k;
+  // Contribution slots, from the deepest level up: a body takes over its first
+  // child's slot (it has read it by then) and a leaf a free one; the other
+  // children's slots are free again from the next level on.
+  std::vector<int> freed, idle;
+  m->slots = 0;
+  for (int l = depth - 1; l >= 0; --l) {
+    idle.insert(idle.end(), freed.begin(), freed.end());
+    freed.clear();
+    for (int b = T.level_start[l]; b < T.level_start[l + 1]; ++b) {
+      const int i = T.level_body[b];
+      if (T.child_start[i] < T.child_start[i + 1]) {
+        m->hc[i].slot = m->hc[T.child[T.child_start[i]]].slot;
+        for (int c = T.child_start[i] + 1; c < T.child_start[i + 1]; ++c) freed.push_back(m->hc[T.child[c]].slot);
+      } else if (!idle.empty()) {
+        m->hc[i].slot = idle.back();
+        idle.pop_back();
+      } else {
+        m->hc[i].slot = m->slots++;
+      }
+    }
+  }
   if (n <= kMaxWarpBodies) {
     WarpTree& wt = m->wt;
     wt.n = n;

@@ -12,7 +12,7 @@ namespace {
 // block's warps split each of the tree's levels. Shared memory: the largest
 // tree's model, the staged input rows, then the per-body state of the
 // largest (tree, operator) pair. ABA runs in its lean form (aba_level_lean:
-// 14 floats per body and a ring of contributions instead of 59 floats per
+// 12 floats per body and a few contribution slots instead of 59 floats per
 // body), so that the block's shared memory, sized for the largest pair, is
 // not set by ABA.
 __global__ void __launch_bounds__(256) multi_level_kernel(MultiArgs a) {
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) multi_level_kernel(MultiArgs a) {
     switch (op) {
       case ROLE_ABA:
         aba_level_lean(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
-                       LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanRingFloats}, a.maxw[m],
+                       LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats},
                        io.qdd_out, B, e, act);
         break;
       case ROLE_CRBA:
