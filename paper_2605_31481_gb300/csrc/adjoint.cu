@@ -312,6 +312,8 @@ __global__ void __launch_bounds__(1024) partial_reduce_kernel(const float* __res
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
   float s = 0.f;
+  pdl_launch();
+  pdl_wait();
   if (p < P) {
 #pragma unroll 8
     for (int b = w; b < nblk; b += 32) s += partial[(int64_t)b * P + p];
@@ -334,8 +336,7 @@ int fit_block(int64_t B, int n, int rows, bool theta) {
 }
 
 cudaError_t reduce(const float* partial, int nblk, int P, float* out, cudaStream_t s) {
-  partial_reduce_kernel<<<(P + 31) / 32, 1024, 0, s>>>(partial, nblk, P, out);
-  return cudaGetLastError();
+  return launch_pdl(partial_reduce_kernel, (P + 31) / 32, 1024, 0, s, partial, nblk, P, out);
 }
 
 }  // namespace

@@ -14,7 +14,10 @@ namespace {
   float* const tile = smem_tile(smem, mv.n);                     \
   const int lane = threadIdx.x & 31;                             \
   const int64_t e = (int64_t)blockIdx.x * kLaneEnvs + lane;      \
-  const bool act = e < B
+  const bool act = e < B;                                        \
+  pdl_launch();                                                  \
+  stage_model_begin(mv, smem);                                   \
+  pdl_wait()
 
 __device__ __forceinline__ Col tile_col(float* tile, int row) {
   return Col{tile + row * kLaneEnvs + (threadIdx.x & 31), kLaneEnvs};
@@ -35,7 +38,7 @@ __global__ void __launch_bounds__(512) rnea_derivs_aligned_kernel(ModelView mv, 
   stage_block_rows(tile, q, mv.nq, B, e);
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   const LaneState S{tile + (mv.nq + 2 * mv.nv) * kLaneEnvs, kDerivState};
   rnea_derivs_aligned<false>(sm, world_accel(mv), tile_col(tile, 0), tile_col(tile, mv.nq),
                              tile_col(tile, mv.nq + mv.nv), mv.nv, S, TreeMat{}, dq, dqd, B, e, act);
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, i
   for (int k = threadIdx.x; k <= dof_depth; k += blockDim.x) cp_async4(lists + 3 * nv + k, dl->level + k);
   int* const anc = lists + 4 * nv + 1;
   for (int k = threadIdx.x; k < entries; k += blockDim.x) cp_async4(anc + k, dl->anc + k);
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   const Col cq = tile_col(tile, 0), cqd = tile_col(tile, mv.nq);
   float* const qcol = tile + (mv.nq + 2 * nv) * kLaneEnvs + lane;  // qdd
   aba_level_lean(sm, world_accel(mv), cq, cqd, tile_col(tile, mv.nq + nv), LaneState{state, kAbaLeanBodyFloats},
@@ -118,10 +121,10 @@ __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, i
 
 // The adjoint of inverse dynamics and the identification loss with its
 // gradient. Bound by latency: shared memory holds one tile of the humanoid
-// (172 KB) or two of the quadruped per SM. The one-thread-per-environment
+// (172 KB) or two of the quadruped per SM (see rnea_vjp_lean_kernel). The one-thread-per-environment
 // kernel ran all sweeps in series with their state in local memory and 50
-// shuffles per body for the parameter gradient: humanoid, B = 65536: 310 ->
-// 160 us; arm, B = 8192, loss and gradient: 16.0 -> 12.0 us (the specialised
+// shuffles per body for the parameter gradient: humanoid, B = 4096: 70 -> 16
+// us; arm, B = 8192, loss and gradient: 16.0 -> 12.0 us (the specialised
 // kernel against this one).
 template <int MODE>
 __global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, nv, B, e);
   stage_block_rows(tile + (mv.nq + nv) * kLaneEnvs, qdd, nv, B, e);
   stage_block_rows(tile + (mv.nq + 2 * nv) * kLaneEnvs, tb, nv, B, e);
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   const LaneState S{tile + (mv.nq + 3 * nv) * kLaneEnvs, kVjpState};
   float* const th = partial ? partial + (int64_t)blockIdx.x * P : nullptr;
   const VjpAligned o{qbar, qdbar, qddbar, th, 1.f};
@@ -157,6 +160,30 @@ __global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int
   }
 }
 
+// The same with the lean state, blockDim.y tiles per block over one copy of
+// the model: two tiles of the humanoid an SM instead of one, four of the
+// quadruped instead of two. Adjoint with the parameter gradient, B = 65536:
+// humanoid 320 us in one thread per environment, 161 in rnea_vjp_aligned_kernel,
+// 127 here; quadruped 80 -> 60. A short chain gains nothing (arm7 B = 16384 15.4
+// against 17.2), so trees of up to 8 bodies keep the other form.
+__global__ void __launch_bounds__(512) rnea_vjp_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+                                                            const float* __restrict__ qd,
+                                                            const float* __restrict__ qdd,
+                                                            const float* __restrict__ tb, float* qbar, float* qdbar,
+                                                            float* qddbar, float* partial) {
+  extern __shared__ float4 smem[];
+  const int64_t t = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  const int64_t e = t * kLaneEnvs + (threadIdx.x & 31);
+  pdl_launch();
+  stage_model_begin(mv, smem);
+  pdl_wait();
+  const SmemModel sm = stage_model_end(mv, smem);
+  if (t * kLaneEnvs >= B) return;  // a whole tile past the end, its warps alone share its barrier
+  const LaneState S{smem_tile(smem, mv.n) + (size_t)threadIdx.y * kVjpLeanState * mv.n * kLaneEnvs, kVjpLeanState};
+  const VjpAligned o{qbar, qdbar, qddbar, partial ? partial + t * mv.n * 10 : nullptr, 1.f};
+  rnea_vjp_lean(sm, world_accel(mv), q, qd, qdd, tb, S, o, B, e, e < B);
+}
+
 // The ABA adjoint in one launch: lambda = M^-1 qddbar by the lean
 // level-parallel ABA at rest and without gravity, then minus the adjoint of
 // inverse dynamics at (q, qd, qdd) for the cotangent lambda. Quadruped,
@@ -176,7 +203,7 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
   const int rows = mv.nq + 4 * nv + 1;
   float* const zero = tile + (rows - 1) * kLaneEnvs + lane;
   if (threadIdx.x < 32) *zero = 0.f;
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   float* const state = tile + rows * kLaneEnvs;
   float* const lam = tile + (mv.nq + 3 * nv) * kLaneEnvs + lane;
   const Col cq = tile_col(tile, 0);
@@ -196,7 +223,7 @@ __global__ void __launch_bounds__(256) fk_vjp_tile_kernel(ModelView mv, int64_t 
                                                           const float* __restrict__ pbar, float* __restrict__ qbar) {
   FST_TILE;
   stage_block_rows(tile, q, mv.nq, B, e);
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   fk_vjp_tile(sm, tile_col(tile, 0), pbar, LaneState{tile + mv.nq * kLaneEnvs, kFkVjpState}, qbar, B, e, act);
 }
 
@@ -209,7 +236,7 @@ __global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int6
   stage_block_rows(tile, q, mv.nq, B, e);
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   rnea_level(sm, world_accel(mv), tile_col(tile, 0), tile_col(tile, mv.nq), tile_col(tile, mv.nq + mv.nv),
              LaneState{tile + (mv.nq + 2 * mv.nv) * kLaneEnvs, kRneaState}, tau, B, e, act, nullptr, tape);
 }
@@ -238,7 +265,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
       stage_block_rows(tile + (rows + 2 * nv) * kLaneEnvs, a.tau_bar, nv, B, e);
     rows += (vjp ? 3 : 2) * nv;
   }
-  const SmemModel sm = stage_model(mv, smem);
+  const SmemModel sm = stage_model_end(mv, smem);
   float* const state = tile + rows * kLaneEnvs;
   const Col cq = tile_col(tile, 0), c1 = tile_col(tile, mv.nq), c2 = tile_col(tile, mv.nq + nv);
   switch (role) {
@@ -345,16 +372,14 @@ cudaError_t launch_fk_vjp_tile(const ModelView& mv, int64_t B, const float* q, c
                                int block, cudaStream_t s) {
   const size_t sh = fk_vjp_tile_smem(mv);
   prepare(fk_vjp_tile_kernel, sh);
-  fk_vjp_tile_kernel<<<grid_for(B, kLaneEnvs), block, sh, s>>>(mv, B, q, pbar, qbar);
-  return cudaGetLastError();
+  return launch_pdl(fk_vjp_tile_kernel, grid_for(B, kLaneEnvs), block, sh, s, mv, B, q, pbar, qbar);
 }
 
 cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    float* tau, float* tape, int block, cudaStream_t s) {
   const size_t sh = level_smem_needed(mv, LEVEL_RNEA);
   prepare(rnea_store_tile_kernel, sh);
-  rnea_store_tile_kernel<<<grid_for(B, kLaneEnvs), block, sh, s>>>(mv, B, q, qd, qdd, tau, tape);
-  return cudaGetLastError();
+  return launch_pdl(rnea_store_tile_kernel, grid_for(B, kLaneEnvs), block, sh, s, mv, B, q, qd, qdd, tau, tape);
 }
 
 cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, bool lean, size_t smem, int block,
@@ -362,8 +387,7 @@ cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, 
   const dim3 grid(grid_for(B, kLaneEnvs), a.n_roles);
   auto go = [&](auto* k) {
     prepare(k, smem);
-    k<<<grid, block, smem, s>>>(mv, B, a);
-    return cudaGetLastError();
+    return launch_pdl(k, grid, block, smem, s, mv, B, a);
   };
   if (a.rnea_flags || a.packed) return lean ? go(eval_tile_kernel<true, true>) : go(eval_tile_kernel<true, false>);
   return lean ? go(eval_tile_kernel<false, true>) : go(eval_tile_kernel<false, false>);
@@ -374,8 +398,8 @@ cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const flo
   const size_t sh = rnea_derivs_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(rnea_derivs_aligned_kernel, sh);
-  rnea_derivs_aligned_kernel<<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(mv, B, q, qd, qdd, dq, dqd);
-  return cudaGetLastError();
+  return launch_pdl(rnea_derivs_aligned_kernel, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd, qdd, dq,
+                    dqd);
 }
 
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
@@ -384,9 +408,8 @@ cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const floa
   const size_t sh = aba_derivs_aligned_smem(mv, slots, entries);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_derivs_aligned_kernel, sh);
-  aba_derivs_aligned_kernel<<<tiles, aba_derivs_threads(mv, slots, block, tiles), sh, s>>>(
-      mv, B, q, qd, tau, qdd, dq, dqd, Minv, entries, dof_depth, (int)state_with_aba(mv.n, slots, kDerivState));
-  return cudaGetLastError();
+  return launch_pdl(aba_derivs_aligned_kernel, tiles, aba_derivs_threads(mv, slots, block, tiles), sh, s, mv, B, q, qd,
+                    tau, qdd, dq, dqd, Minv, entries, dof_depth, (int)state_with_aba(mv.n, slots, kDerivState));
 }
 
 cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
@@ -394,10 +417,22 @@ cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float*
                                     float* scratch, int block, cudaStream_t s) {
   const size_t sh = rnea_vjp_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
-  prepare(rnea_vjp_aligned_kernel<VJP_GIVEN>, sh);
-  rnea_vjp_aligned_kernel<VJP_GIVEN><<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(
-      mv, B, q, qd, qdd, tbar, qbar, qdbar, qddbar, thbar ? scratch : nullptr);
-  cudaError_t err = cudaGetLastError();
+  float* const partial = thbar ? scratch : nullptr;
+  // Where more tiles wait than the SMs take, the lean state, in as many tiles
+  // per block as double the tiles per SM.
+  const size_t model = smem_bytes(mv.n), lean = floats32((size_t)kVjpLeanState * mv.n);
+  const int T = model + 2 * lean <= kLevelSmemLimit && 2 * (model + lean + 1024) > kLevelSmemLimit ? 2 : 1;
+  cudaError_t err;
+  if (tiles > 152 * 2 && block == 0 && mv.n > 8) {
+    const int W = mv.n > 16 ? 8 : 4;
+    prepare(rnea_vjp_lean_kernel, model + T * lean);
+    err = launch_pdl(rnea_vjp_lean_kernel, (tiles + T - 1) / T, dim3(32, T, W), model + T * lean, s, mv, B, q, qd, qdd,
+                     tbar, qbar, qdbar, qddbar, partial);
+  } else {
+    prepare(rnea_vjp_aligned_kernel<VJP_GIVEN>, sh);
+    err = launch_pdl(rnea_vjp_aligned_kernel<VJP_GIVEN>, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd,
+                     qdd, tbar, qbar, qdbar, qddbar, partial);
+  }
   if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
   return err;
 }
@@ -408,9 +443,8 @@ cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float
   const size_t sh = rnea_vjp_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(rnea_vjp_aligned_kernel<VJP_LOSS>, sh);
-  rnea_vjp_aligned_kernel<VJP_LOSS><<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(
-      mv, B, q, qd, qdd, tau_meas, qbar, qdbar, nullptr, scratch);
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err = launch_pdl(rnea_vjp_aligned_kernel<VJP_LOSS>, tiles, aligned_block(block, mv.n, tiles), sh, s, mv,
+                               B, q, qd, qdd, tau_meas, qbar, qdbar, nullptr, scratch);
   if (err == cudaSuccess) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10 + 1, loss_theta, s);
   return err;
 }
@@ -421,9 +455,8 @@ cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* 
   const size_t sh = aba_vjp_aligned_smem(mv, slots);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_vjp_aligned_kernel, sh);
-  aba_vjp_aligned_kernel<<<tiles, aligned_block(block, mv.n, tiles), sh, s>>>(mv, B, q, qd, qdd, qddbar, qbar, qdbar,
-                                                                             taubar, thbar ? scratch : nullptr);
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err = launch_pdl(aba_vjp_aligned_kernel, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd,
+                               qdd, qddbar, qbar, qdbar, taubar, thbar ? scratch : nullptr);
   if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
   return err;
 }

@@ -686,6 +686,180 @@ __device__ __forceinline__ float rnea_vjp_aligned(const SmemModel& tp, SV a0, co
   return loss;
 }
 
+// Barrier of one tile's warps in a (32, T, W) block: a named one for each
+// tile, so that its tiles drift apart and one's arithmetic fills the other's
+// waits.
+__device__ __forceinline__ void tile_barrier() {
+  asm volatile("barrier.sync %0, %1;" ::"r"((int)threadIdx.y + 1), "r"((int)(blockDim.x * blockDim.z)) : "memory");
+}
+
+// The same adjoint (VJP_GIVEN, the same arithmetic and bits) with 36 floats a
+// body, so that two tiles of the humanoid share an SM: nothing is staged (a
+// body's coordinates wait in the slots that its velocities will take), the
+// inertia and the functionals are formed on the way up instead of stored
+// between two sweeps, and a body's contribution to its parent takes the place
+// of its own v, a and w, which only its children needed.
+// psi 6 | v 6, a 6, w 6, then the force, A and H for the parent | R 9 | r 3.
+__device__ __forceinline__ void rnea_vjp_lean(const SmemModel& tp, SV a0, const float* __restrict__ q,
+                                              const float* __restrict__ qd, const float* __restrict__ qdd,
+                                              const float* __restrict__ tbar, const LaneState& S, const VjpAligned& o,
+                                              int64_t B, int64_t e, bool act) {
+  const int W = n_warps(), w = warp_id(), n = tp.n();
+  enum { PSI = 0, V_ = 6, A_ = 12, W_ = 18, R_ = 24, RR = 33 };
+  const int64_t ec = act ? e : B - 1;
+  for (int i = w; i < n; i += W) {
+    const BodyI bi = tp.I(i);
+    const int nqb = bi.type == FST_JOINT_FREE ? 7 : bi.type == FST_JOINT_FIXED ? 0 : 1, nvb = nv_of(bi.type);
+    float qb[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) qb[k] = k < nqb ? __ldg(q + (int64_t)(bi.qi + k) * B + ec) : 0.f;
+    float x[3][6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int64_t at = (int64_t)(bi.vi + k) * B + ec;
+      x[0][k] = k < nvb ? __ldg(qd + at) : 0.f;
+      x[1][k] = k < nvb ? __ldg(qdd + at) : 0.f;
+      x[2][k] = k < nvb ? __ldg(tbar + at) : 0.f;
+    }
+    BodyI b0 = bi;
+    b0.qi = 0;
+    S.putX(i, R_, joint_X(tp.C(i), b0, Col{qb, 1}));
+    if (bi.type == FST_JOINT_FREE) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        S.put(i, V_ + 6 * c, SV{f3{x[c][3], x[c][4], x[c][5]}, f3{x[c][0], x[c][1], x[c][2]}});
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) *S.at(i, V_ + 6 * c) = x[c][0];
+    }
+  }
+  tile_barrier();
+  for (int l = 0; l < tp.depth(); ++l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const Xf X = S.X(i, R_);
+      if (bi.type == FST_JOINT_FREE) {  // the root frame is this body's own; v and w are in place
+        const float Id[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
+        S.put_n(i, R_, Id, 9);
+        S.put(i, A_, S.sv(i, A_) + SV{f3{0.f, 0.f, 0.f}, RTmul(X.R, a0.v)});
+        continue;
+      }
+      SV vl = sv_zero(), al = a0, wl = sv_zero();
+      float R[9];
+      if (bi.parent < 0) {
+#pragma unroll
+        for (int c = 0; c < 9; ++c) R[c] = X.R[c];
+      } else {
+        float Rp[9], rr[3];
+        S.get_n(bi.parent, R_, Rp, 9);
+        const float zero[3] = {0.f, 0.f, 0.f};
+        compose(Rp, zero, X, R, rr);
+        const f3 r = f3{rr[0], rr[1], rr[2]};
+        S.put_n(i, RR, rr, 3);
+        S.put_n(i, R_, R, 9);
+        vl = shift_motion(S.sv(bi.parent, V_), r);
+        al = shift_motion(S.sv(bi.parent, A_), r);
+        wl = shift_motion(S.sv(bi.parent, W_), r);
+      }
+      if (one_dof(bi)) {
+        const SV psi = psi_of(tp.C(i), R);
+        S.put(i, PSI, psi);
+        const float xd = *S.at(i, V_);
+        const SV psd = crm(vl, psi);
+        al = sv_fma(*S.at(i, A_), psi, sv_fma(xd, psd, al));
+        vl = sv_fma(xd, psi, vl);
+        wl = sv_fma(*S.at(i, W_), psi, wl);
+      }
+      S.put(i, V_, vl);
+      S.put(i, A_, al);
+      S.put(i, W_, wl);
+    }
+    tile_barrier();
+  }
+  if (o.thbar) {
+    for (int i = w; i < n; i += W) {
+      float R[9];
+      S.get_n(i, R_, R, 9);
+      const SV v = S.sv(i, V_), wv = S.sv(i, W_);
+      float g[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+      inertia_contract(wv, S.sv(i, A_), g);
+      inertia_contract(crm(wv, v), v, g);
+      inertia_grad_to_body(R, g);
+#pragma unroll
+      for (int c = 0; c < 10; ++c) g[c] = act ? o.sign * g[c] : 0.f;
+      warp_sum10_store(g, o.thbar + 10 * i);
+    }
+    tile_barrier();
+  }
+  if (!o.qbar && !o.qdbar && !o.qddbar) return;  // uniform over the launch
+  for (int l = tp.depth() - 1; l >= 0; --l) {
+    FST_FOR_MY_BODIES(tp, l, k) {
+      const int i = tp.level_body(k);
+      const BodyI bi = tp.I(i);
+      const SV v = S.sv(i, V_), wv = S.sv(i, W_);
+      float R[9];
+      S.get_n(i, R_, R, 9);
+      const In10 I = in_rotate(R, in_load(tp.theta(i)));
+      const SV hv = in_mul(I, v);
+      SV f = in_mul(I, S.sv(i, A_)) + crf(v, hv);
+      SV A = in_mul(I, wv);
+      f3 H = 2.f * (second_moment_mul(I, cross(v.w, wv.w)) + (dot(I.h, v.v) * wv.w - dot(v.v, wv.w) * I.h) -
+                    cross(wv.v, hv.v));
+      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
+        const int c = tp.child(ch);
+        const float* h = S.at(c, W_);
+        A = A + S.sv(c, A_);
+        f = f + S.sv(c, V_);
+        H = H + f3{h[0], h[32], h[64]};
+      }
+      const float* t = S.at(i, RR);
+      const f3 r = f3{t[0], t[32], t[64]};
+      if (act && bi.type == FST_JOINT_FREE) {
+        const SV y = crf(v, A);
+        const f3 g1 = RTmul(tp.C(i).R0, a0.v);
+        const float G[9] = {g1.x * A.v.x, g1.x * A.v.y, g1.x * A.v.z, g1.y * A.v.x, g1.y * A.v.y,
+                            g1.y * A.v.z, g1.z * A.v.x, g1.z * A.v.y, g1.z * A.v.z};
+        const float* qq = q + (int64_t)(bi.qi + 3) * B + e;
+        float gq[4];
+        quat_grad(__ldg(qq), __ldg(qq + B), __ldg(qq + 2 * B), __ldg(qq + 3 * B), G, gq);
+        const float qo[7] = {0.f, 0.f, 0.f, gq[0], gq[1], gq[2], gq[3]};
+        const float vo[6] = {-y.v.x, -y.v.y, -y.v.z, H.x - y.w.x, H.y - y.w.y, H.z - y.w.z};
+        const float ao[6] = {A.v.x, A.v.y, A.v.z, A.w.x, A.w.y, A.w.z};
+#pragma unroll
+        for (int c = 0; c < 7; ++c) store_if(o.qbar, bi.qi + c, B, e, o.sign * qo[c], true);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          store_if(o.qdbar, bi.vi + c, B, e, o.sign * vo[c], true);
+          store_if(o.qddbar, bi.vi + c, B, e, o.sign * ao[c], true);
+        }
+      } else if (act && one_dof(bi)) {
+        SV vl = sv_zero(), al = a0, wl = sv_zero();
+        if (bi.parent >= 0) {
+          vl = shift_motion(S.sv(bi.parent, V_), r);
+          al = shift_motion(S.sv(bi.parent, A_), r);
+          wl = shift_motion(S.sv(bi.parent, W_), r);
+        }
+        const SV psi = S.sv(i, PSI);
+        const SV psd = crm(vl, psi);
+        const SV psdd = crm(al, psi) + crm(vl, psd);
+        store_if(o.qbar, bi.qi, B, e, o.sign * (dot(crm(wl, psi), f) + dot(psdd, A) + dot(psd.w, H)), true);
+        store_if(o.qdbar, bi.vi, B, e, o.sign * fmaf(2.f, dot(psd, A), dot(psi.w, H)), true);
+        store_if(o.qddbar, bi.vi, B, e, o.sign * dot(psi, A), true);
+      }
+      if (bi.parent >= 0) {
+        S.put(i, V_, shift_force(f, r));
+        S.put(i, A_, shift_force(A, r));
+        float* h = S.at(i, W_);
+        h[0] = H.x;
+        h[32] = H.y;
+        h[64] = H.z;
+      }
+    }
+    tile_barrier();
+  }
+}
+
 // ---- the adjoint of forward kinematics -----------------------------------------
 // Moving joint i turns and shifts its whole subtree as one rigid body, so of
 // the poses' cotangents (Rbar_k, pbar_k) only the total force F = sum pbar_k

@@ -340,7 +340,9 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // own earlier cp.async copies (its staged inputs). The BodyC and BodyI
 // arrays are separate device allocations (256-byte aligned) of 256- and
 // 16-byte records, so their 16-byte copies are aligned on both sides.
-__device__ __forceinline__ SmemModel stage_model(const ModelView& mv, float4* smem) {
+// In two parts, so that a kernel can issue the copies before it waits for the
+// kernel ahead of it (pdl_wait): the model is constant.
+__device__ __forceinline__ void stage_model_begin(const ModelView& mv, float4* smem) {
   BodyC* sc = reinterpret_cast<BodyC*>(smem);
   BodyI* si = reinterpret_cast<BodyI*>(sc + mv.n);
   TopoLists* st = reinterpret_cast<TopoLists*>(si + mv.n);
@@ -356,6 +358,14 @@ __device__ __forceinline__ SmemModel stage_model(const ModelView& mv, float4* sm
   const int* ts = reinterpret_cast<const int*>(mv.topo);
   int* td = reinterpret_cast<int*>(st);
   for (int k = tid; k < (int)(sizeof(TopoLists) / sizeof(int)); k += nt) cp_async4(td + k, ts + k);
+}
+
+__device__ __forceinline__ SmemModel stage_model_end(const ModelView& mv, float4* smem) {
+  BodyC* sc = reinterpret_cast<BodyC*>(smem);
+  BodyI* si = reinterpret_cast<BodyI*>(sc + mv.n);
+  TopoLists* st = reinterpret_cast<TopoLists*>(si + mv.n);
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int nt = blockDim.x * blockDim.y * blockDim.z;
   cp_async_wait_all();
   __syncthreads();
   if (mv.theta) {  // the override replaces the staged parameters, after they have landed
@@ -365,6 +375,28 @@ __device__ __forceinline__ SmemModel stage_model(const ModelView& mv, float4* sm
   }
   return SmemModel{sc, si, mv.n, st, mv.depth};
 }
+
+__device__ __forceinline__ SmemModel stage_model(const ModelView& mv, float4* smem) {
+  stage_model_begin(mv, smem);
+  return stage_model_end(mv, smem);
+}
+
+// Programmatic dependent launch (launch.h: launch_pdl). pdl_launch lets the
+// next kernel of the stream start once every block of this one has; pdl_wait
+// returns when the kernel ahead has finished and its writes are visible. A
+// kernel launched that way calls pdl_wait in every thread before it touches
+// anything that another kernel reads or writes. Both do nothing in a kernel
+// that was launched the ordinary way.
+// A grid of between half and all of the SMs does not let the next one in early:
+// its blocks would gather on the SMs that this one leaves idle and then share
+// them (humanoid29 B = 4096, 128 blocks: CRBA 10.8 -> 12.8 us; the five-operator
+// step of the quadruped, 512 blocks, 16.2 -> 13.9, and one of 2 blocks 0.9 us
+// less).
+__device__ __forceinline__ void pdl_launch() {
+  const unsigned blocks = gridDim.x * gridDim.y;
+  if (blocks <= 76 || blocks > 152) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __host__ __device__ inline size_t smem_bytes(int n) {
   return (size_t)n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;

@@ -138,6 +138,7 @@ constexpr int kCrbaLeanSlotFloats = 10;
 // adjoint in aligned frames (aligned.cuh).
 constexpr int kDerivState = 49;
 constexpr int kVjpState = 51;
+constexpr int kVjpLeanState = 36;
 constexpr int kFkVjpState = 18;
 
 // Operators of the fused evaluation kernel, in launch order (longest first,

@@ -78,6 +78,25 @@ inline void prepare(K* kernel, size_t smem) {
   done[(const void*)kernel] = Done{keep, gen};
 }
 
+// Launches a kernel that starts with pdl_launch and pdl_wait (fst_device.cuh)
+// so that its launch, its blocks' start and its copy of the model overlap the
+// end of the kernel ahead of it in the stream. The order of the two kernels'
+// effects is the stream's, as for any launch.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Kernel launchers (return the cudaGetLastError() after the launch).
 cudaError_t launch_fk(const ModelView& mv, int64_t B, const float* q, float* poses, const Launch& L);
 cudaError_t launch_jacobian(const ModelView& mv, int64_t B, const float* q, const LinkList& links, float* J,

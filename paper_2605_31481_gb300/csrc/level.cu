@@ -18,13 +18,16 @@ __device__ __forceinline__ float* level_tile(float4* smem, int n) { return smem_
   const LaneState S{tile + (rows) * kLaneEnvs, (F)};                                     \
   const int lane = threadIdx.x & 31;                                                     \
   const int64_t e = ((int64_t)blockIdx.x * blockDim.y + threadIdx.y) * kLaneEnvs + lane; \
-  const bool act = e < B
+  const bool act = e < B;                                                                \
+  pdl_launch();                                                                          \
+  stage_model_begin(mv, smem);                                                           \
+  pdl_wait()
 
 #define FST_LEVEL_PROLOGUE(rows, F) FST_LEVEL_PROLOGUE_S(rows, F, ((rows) + (F) * mv.n) * kLaneEnvs)
 
-// stage_model waits for the model and for this thread's staged rows, then
+// stage_model_end waits for the model and for this thread's staged rows, then
 // synchronises the block, so everything staged is visible to every warp.
-#define FST_LEVEL_READY const SmemModel sm = stage_model(mv, smem)
+#define FST_LEVEL_READY const SmemModel sm = stage_model_end(mv, smem)
 
 __global__ void __launch_bounds__(256) fk_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                        float* __restrict__ poses) {
@@ -198,16 +201,15 @@ size_t level_tile_bytes(const ModelView& mv, int rows, int F) {
 
 // `block` threads (a multiple of 32 T) as `tiles` tiles of block / (32 T)
 // warps each: a 1-D block for one tile, (32, T, W) for several.
-template <typename K, typename... A>
-cudaError_t go(K* kernel, const ModelView& mv, int64_t B, size_t sh, int block, int tiles, unsigned gy,
+template <typename... P, typename... A>
+cudaError_t go(void (*kernel)(P...), const ModelView& mv, int64_t B, size_t sh, int block, int tiles, unsigned gy,
                cudaStream_t s, A... args) {
   if (sh > kLevelSmemLimit || tiles < 1 || block < 32 * tiles || block % (32 * tiles))
     return cudaErrorInvalidConfiguration;
   prepare(kernel, sh);
   const int64_t envs = (int64_t)kLaneEnvs * tiles;
   const dim3 blk = tiles == 1 ? dim3(block) : dim3(32, tiles, block / (32 * tiles));
-  kernel<<<dim3((unsigned)((B + envs - 1) / envs), gy), blk, sh, s>>>(mv, B, args...);
-  return cudaGetLastError();
+  return launch_pdl(kernel, dim3((unsigned)((B + envs - 1) / envs), gy), blk, sh, s, mv, B, args...);
 }
 
 }  // namespace

@@ -18,7 +18,9 @@ namespace {
   const bool act = e < B;                                   \
   const int64_t ec = act ? e : B - 1;                       \
   const Me me(t);                                           \
-  (void)ec
+  (void)ec;                                                 \
+  pdl_launch();                                             \
+  pdl_wait()
 
 template <int T, int MINB, int MODE>
 __global__ void __launch_bounds__(T, MINB) wb_vjp_kernel(const __grid_constant__ WarpTree t, ModelView mv, int64_t B,
@@ -71,15 +73,11 @@ size_t wb_smem(int n, int floats) { return (size_t)n * floats * kLaneEnvs * size
     const size_t sh_ = wb_smem(t.n, kWbVjpFloats);                    \
     auto go_ = [&](auto* k_) {                                        \
       prepare(k_, sh_);                                               \
-      k_<<<grid_for(B, kLaneEnvs), 32 * t.n, sh_, s>>>(t, mv, B, __VA_ARGS__); \
+      return launch_pdl(k_, grid_for(B, kLaneEnvs), 32 * t.n, sh_, s, t, mv, B, __VA_ARGS__); \
     };                                                                \
-    if (t.n <= 8)                                                     \
-      go_(KERNEL(256, 2));                                            \
-    else if (t.n <= 12)                                               \
-      go_(KERNEL(384, 2));                                            \
-    else                                                              \
-      go_(KERNEL(512, 1));                                            \
-    return cudaGetLastError();                                        \
+    if (t.n <= 8) return go_(KERNEL(256, 2));                         \
+    if (t.n <= 12) return go_(KERNEL(384, 2));                        \
+    return go_(KERNEL(512, 1));                                       \
   } while (0)
 
 cudaError_t go_vjp(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,

@@ -145,3 +145,29 @@ def test_general_kernels_match_oracle(torch_cuda, name, variant):
     _check_adjoints(torch_cuda, m, tree, 33, name)
     _check_derivatives(torch_cuda, m, tree, 33, name)
     _check_forward(torch_cuda, m, tree, 33, name)
+
+
+@pytest.mark.parametrize("B", [152 * 64 + 1, 152 * 64 + 65])
+@pytest.mark.parametrize("name", ["random1", "random2", "floating_forest", "star"])
+def test_lean_forms_give_the_same_bits(torch_cuda, name, B):
+    """Past two tiles per SM the default keeps less state per tile (the RNEA
+    adjoint, RNEA, the fused evaluation's CRBA): the same arithmetic, so the
+    same bits as the small-batch forms give on the environments at both ends
+    (a tile and a tail of one; an odd number of tiles)."""
+    torch = torch_cuda
+    from paper_2605_31481_gb300 import api
+    tree = TREES[name]()
+    m = api.Model(tree)
+    _, _, _, x = _inputs(torch, tree, B, 77)
+    part = lambda lo, hi: {k: v[:, lo:hi].contiguous() for k, v in x.items() if k != "th"}  # noqa: E731
+    links = list(tree.ee) or [tree.n_bodies - 1]
+    run = lambda y: {**api.rnea_vjp(m, y["q"], y["qd"], y["qdd"], y["bar"], theta_bar=False),  # noqa: E731
+                     "tau": api.rnea(m, y["q"], y["qd"], y["qdd"]),
+                     **{"ev_" + k: v for k, v in api.eval(m, y["q"], y["qd"], y["qdd"], y["tau"], fk=True, links=links,
+                                                          rnea=True, crba=True, aba=True).items()}}
+    full = run(part(0, B))
+    for lo, hi in ((0, 33), (B - 34, B)):
+        few = run(part(lo, hi))
+        torch.cuda.synchronize()
+        for k in few:
+            assert torch.equal(full[k][..., lo:hi], few[k]), (name, B, k)
