@@ -30,7 +30,8 @@ __device__ __forceinline__ Col tile_col(float* tile, int row) {
 // through the whole tree in one thread per environment, nv times the
 // recursions' work and their state in local memory: floating humanoid,
 // B = 2048: 418 -> 21.5 us; quadruped, B = 4096: 61.6 -> 14 us.
-__global__ void __launch_bounds__(512) rnea_derivs_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+template <int T>
+__global__ void __launch_bounds__(T) rnea_derivs_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                                   const float* __restrict__ qd,
                                                                   const float* __restrict__ qdd,
                                                                   float* __restrict__ dq, float* __restrict__ dqd) {
@@ -337,9 +338,11 @@ size_t aba_vjp_aligned_smem(const ModelView& mv, int slots) {
 
 // The forward-dynamics derivatives' solve phase keeps two columns per warp in
 // the state's space: the block is as large as that allows (0: not one warp).
+// 16 warps while no SM has a second tile to run (legged12 B = 1000 30.3 -> 26.8
+// us, humanoid29 B = 2048 180 -> 146).
 static int aba_derivs_threads(const ModelView& mv, int slots, int set, int64_t tiles) {
   const size_t st = state_with_aba(mv.n, slots, kDerivState);
-  int t = aligned_block(set, mv.n, tiles);
+  int t = set ? set : tiles <= 152 ? 512 : aligned_block(set, mv.n, tiles);
   while (t >= 32 && (size_t)(t / 32) * 2 * mv.nv > st) t /= 2;
   return t >= 32 ? t : 0;
 }
@@ -397,9 +400,14 @@ cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const flo
                                        const float* qdd, float* dq, float* dqd, int block, cudaStream_t s) {
   const size_t sh = rnea_derivs_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
-  prepare(rnea_derivs_aligned_kernel, sh);
-  return launch_pdl(rnea_derivs_aligned_kernel, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd, qdd, dq,
-                    dqd);
+  auto go = [&](auto* k, int threads) {
+    prepare(k, sh);
+    return launch_pdl(k, tiles, threads, sh, s, mv, B, q, qd, qdd, dq, dqd);
+  };
+  // 24 warps where an SM has one tile and the tree work for them (humanoid29 B =
+  // 2048: 21.0 -> 19.7 us, legged18 B = 2700 11.0 -> 10.3).
+  if (block == 0 && mv.n > 16 && tiles <= 152) return go(rnea_derivs_aligned_kernel<768>, 768);
+  return go(rnea_derivs_aligned_kernel<512>, aligned_block(block, mv.n, tiles));
 }
 
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,

@@ -162,7 +162,10 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
-constexpr int kMultiTileBlock = 256;  // threads per block of the mixed-tree launch in tiles
+// Threads per block of the mixed-tree launch in tiles (five trees, 7936
+// environments: 64 threads 24.5 us, 128 22.0, 256 22.4; a group with a large
+// tree wants its warps).
+constexpr int kMultiTileBlock = 256;
 
 // Whether enough tiles wait for an SM (more than two each) that the forms
 // which keep less state, and so more tiles per SM, are the better ones.
@@ -1175,29 +1178,22 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
     for (int j = i; j > 0 && g->models[order[j]]->n > g->models[order[j - 1]]->n; --j) std::swap(order[j], order[j - 1]);
   // the default form is the one that the single-tree calls take: tiles of 32
   // environments if every tree's calls do and their state fits
-  auto state_of = [&](int k, int r) {  // level: bytes of per-body state of a (tree, operator) pair
-    const fst_model* m = g->models[k];
-    const size_t floats = r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + kAbaLeanSlotFloats * m->slots
-                          : (size_t)(r == ROLE_CRBA ? kCrbaStateFloats
-                                     : r == ROLE_RNEA ? kRneaStateFloats : kFkStateFloats) * m->n;
-    return floats * 32 * sizeof(float);
-  };
+  auto tile_smem = [&](int k, int r) { return multi_tile_smem(a.mv[k], r, g->models[k]->slots); };
   a.model_bytes = (size_t)max_n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;
   a.model_bytes = (a.model_bytes + 15) / 16 * 16;
   bool level = g->variant == FST_VARIANT_LEVEL;
   if (g->variant == FST_VARIANT_AUTO) {
     level = true;
-    size_t most = 0;
     for (int k = 0; k < n; ++k) {
       for (int op : {JK_FK, JK_RNEA, JK_CRBA, JK_ABA})
         level = level && (io[k].B == 0 || tile_rule(g->models[k], op, false, io[k].B));
-      for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) most = std::max(most, state_of(k, r));
+      for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) level = level && tile_smem(k, r) <= kLevelSmemLimit;
     }
-    level = level && a.model_bytes + (size_t)a.max_rows * 32 * sizeof(float) + most <= kLevelSmemLimit;
   }
   const int block = g->variant == FST_VARIANT_AUTO && level ? kMultiTileBlock : g->block;
   const int T = level ? 32 : block;  // environments per item
-  size_t state_bytes = 0;            // level: per-body state of the largest (tree, operator) pair
+  size_t smem = 0;                   // level: shared memory of the largest (tree, operator) pair
+  size_t full = 0;                   // and its state floats a lane with nothing taken over or re-formed
   // every block of the persistent grid draws one item past the last, so the
   // int work counter reaches n_items + grid: keep ample headroom below 2^31
   const int64_t kMaxItems = (int64_t)INT32_MAX - (1 << 24);
@@ -1211,7 +1207,14 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
                        : r == ROLE_CRBA ? (const void*)x.M
                        : r == ROLE_RNEA ? (const void*)x.tau_out : (const void*)x.poses;
       if (!outp || x.B == 0) continue;
-      if (level) state_bytes = std::max(state_bytes, state_of(k, r));
+      if (level) {
+        const fst_model* m = g->models[k];
+        smem = std::max(smem, tile_smem(k, r));
+        full = std::max(full, r == ROLE_ABA ? (size_t)kAbaLeanBodyFloats * m->n + 2 * kAbaLeanSlotFloats * m->max_width
+                              : (size_t)(r == ROLE_CRBA   ? kCrbaStateFloats
+                                         : r == ROLE_RNEA ? kRneaStateFloats
+                                                          : kFkStateFloats) * m->n);
+      }
       a.seg_start[seg] = (int)items;  // within kMaxItems: checked below on every addition
       a.seg_model[seg] = (unsigned char)k;
       a.seg_op[seg] = (unsigned char)r;
@@ -1224,11 +1227,12 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
   a.n_items = (int)items;
   if (items == 0) return FST_OK;
   if (level) {
-    const size_t sh = a.model_bytes + (size_t)a.max_rows * 32 * sizeof(float) + state_bytes;
-    if (sh > kLevelSmemLimit)
+    // the limit of an explicit choice is that of the full states, as for the single calls
+    const size_t need = a.model_bytes + ((size_t)a.max_rows + full) * 32 * sizeof(float);
+    if (smem > kLevelSmemLimit || (g->variant == FST_VARIANT_LEVEL && need > kLevelSmemLimit))
       return set_error(FST_ERR_INVALID_ARG, std::string(fn) + ": the level-parallel state of the largest tree "
                                                               "does not fit in shared memory");
-    return finish(fn, launch_multi_level(a, state_bytes, block, (cudaStream_t)stream));
+    return finish(fn, launch_multi_tiles(a, smem, block, (cudaStream_t)stream));
   }
   return finish(fn, launch_multi(a, max_n, T, (cudaStream_t)stream));
 }

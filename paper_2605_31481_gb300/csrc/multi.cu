@@ -77,6 +77,18 @@ __global__ void __launch_bounds__(256) multi_kernel(MultiArgs a) {
 
 }  // namespace
 
+// Grid = resident blocks per SM x SMs (from the occupancy calculator), but
+// never more blocks than items.
+template <typename K>
+int persistent_grid(K* kernel, int block, size_t smem, int n_items) {
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
+  const int g = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+  return g < n_items ? g : n_items;
+}
+
 cudaError_t launch_multi(const MultiArgs& a, int max_n, int block, cudaStream_t s) {
   const size_t sh = a.model_bytes + (size_t)a.max_rows * block * sizeof(float);
   cudaError_t err = cudaMemsetAsync(a.counter, 0, sizeof(int), s);

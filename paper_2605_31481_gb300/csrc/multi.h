@@ -1,4 +1,4 @@
-// Persistent multi-tree launch (multi.cu): per-call arguments.
+// One launch over several trees (multi.cu, multi_level.cu): per-call arguments.
 #pragma once
 
 #include "fst_internal.h"
@@ -31,27 +31,15 @@ struct MultiArgs {
   int n_items;
   int max_rows;          // staged input rows of the widest item
   size_t model_bytes;    // shared memory reserved for the largest tree
-  int* counter;          // device work counter (reset before each launch)
+  int* counter;          // generic form: device work counter (reset before each launch)
 };
 
-// Grid = resident blocks per SM x SMs (from the occupancy calculator), but
-// never more blocks than items.
-template <typename K>
-inline int persistent_grid(K* kernel, int block, size_t smem, int n_items) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem);
-  const int g = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-  return g < n_items ? g : n_items;
-}
-
-// Environments per item: `block` for the generic kernel (one environment per
-// thread), 32 for the level-parallel one.
+// The generic form (multi.cu): one environment per thread, `block` per item.
 cudaError_t launch_multi(const MultiArgs& a, int max_n, int block, cudaStream_t s);
-// The level-parallel form: items of 32 environments, the block's warps
-// splitting each tree level; state_bytes of per-body state per block.
-cudaError_t launch_multi_level(const MultiArgs& a, size_t state_bytes, int block, cudaStream_t s);
+// The form in tiles (multi_level.cu): one block per item of 32 environments;
+// smem: the largest multi_tile_smem of its (tree, operator) pairs.
+size_t multi_tile_smem(const ModelView& mv, int role, int slots);
+cudaError_t launch_multi_tiles(const MultiArgs& a, size_t smem, int block, cudaStream_t s);
 
 }  // namespace fst
 
