@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
   const Col cq = tile_col(tile, 0), c1 = tile_col(tile, mv.nq), c2 = tile_col(tile, mv.nq + nv);
   switch (role) {
     case ROLE_ABA:
-      aba_level_lean(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
+      aba_level_lean<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
                      LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, a.qdd_out, B,
                      e, act);
       break;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
       break;
     case ROLE_RNEA:
       if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
-        rnea_level<LEAN>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
+        rnea_level<LEAN, LEAN && !EXT>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
                          a.tau_out, B, e, act,
                          vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
       if (vjp)  // rnea_level ends with a barrier: the cotangent is complete and the state free

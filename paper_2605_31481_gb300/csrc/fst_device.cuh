@@ -437,8 +437,9 @@ struct Col {
   const float* p;
   int ld;
   __device__ __forceinline__ float operator[](int k) const { return p[k * ld]; }
+  // a staged row that its reader has done with
+  __device__ __forceinline__ float* spent(int k) const { return const_cast<float*>(p) + k * ld; }
 };
-
 
 // ---- SM-pinned tile loops ---------------------------------------------------
 // The straight-line specialised kernels run fast only while an SM keeps
@@ -514,14 +515,22 @@ __device__ __forceinline__ Col stage_rows(float* tile, const float* __restrict__
 // Pose of body i in its parent from q (paper Eq. 4-5 for revolute joints).
 // sin q and 1 - cos q come from one sincos of q/2: sin q = 2 s c,
 // 1 - cos q = 2 s^2, which keeps 1 - cos q accurate near q = 0.
-__device__ __forceinline__ Xf joint_X(const BodyC& c, const BodyI& b, const Col& q) {
+struct SinOmc {
+  float s, omc;  // sin q, 1 - cos q
+};
+__device__ __forceinline__ SinOmc sin_omc(float q) {
+  float sh, ch;
+  sincosf(0.5f * q, &sh, &ch);
+  return SinOmc{2.f * sh * ch, 2.f * sh * sh};
+}
+// TURNED: a revolute body's angle was replaced by its sine before, and its
+// 1 - cosine is at *omc_at.
+template <bool TURNED = false>
+__device__ __forceinline__ Xf joint_X(const BodyC& c, const BodyI& b, const Col& q, const float* omc_at = nullptr) {
   Xf X;
   if (b.type == FST_JOINT_REVOLUTE) {
-    const float qi = q[b.qi];
-    float sh, ch;
-    sincosf(0.5f * qi, &sh, &ch);
-    const float s = 2.f * sh * ch;
-    const float omc = 2.f * sh * sh;
+    const SinOmc t = TURNED ? SinOmc{q[b.qi], *omc_at} : sin_omc(q[b.qi]);
+    const float s = t.s, omc = t.omc;
 #pragma unroll
     for (int k = 0; k < 9; ++k) X.R[k] = fmaf(omc, c.Bm[k], fmaf(s, c.A[k], c.R0[k]));
 #pragma unroll

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(256) rnea_lean_kernel(ModelView mv, int64_t B,
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
   FST_LEVEL_READY;
-  rnea_level<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+  rnea_level<true, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
                    Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, 
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, tau, mv.nv, B, e);
   FST_LEVEL_READY;
-  aba_level_lean(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+  aba_level_lean<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
                  Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, qdd, B, e, act);
 }
 

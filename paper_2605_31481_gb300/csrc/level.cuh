@@ -220,7 +220,10 @@ __device__ __forceinline__ void kin_level(const TP& tp, const Col& q, int nv, co
 // evaluated again instead of stored. That lengthens the chain (quadruped, B =
 // 4096: 7.4 -> 8 us) and lets twice the tiles share an SM; the arithmetic and
 // so the bits are the same.
-template <bool LEAN = false, class TP>
+// SPEND (with LEAN): the staged rows are the sweep's to overwrite: a joint's sine
+// and 1 - cosine replace its q and qd until the way back has used them
+// (humanoid B = 65536: 50.2 -> 49.0 us).
+template <bool LEAN = false, bool SPEND = false, class TP>
 __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& qdd,
                                            const LaneState& S, float* __restrict__ tau, int64_t B, int64_t e,
                                            bool act, float* tau_col = nullptr, float* tape = nullptr) {
@@ -236,9 +239,16 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
       const int i = tp.level_body(k);
       const BodyC& c = tp.C(i);
       const BodyI bi = tp.I(i);
-      const Xf X = joint_X(c, bi, q);
+      float omc = 0.f;
+      if (SPEND && bi.type == FST_JOINT_REVOLUTE) {
+        const SinOmc t = sin_omc(q[bi.qi]);
+        *q.spent(bi.qi) = t.s;
+        omc = t.omc;
+      }
+      const Xf X = joint_X<SPEND>(c, bi, q, &omc);
       const SV vJ = S_times(c, bi, qd);
       const SV aJ = S_times(c, bi, qdd);
+      if (SPEND && bi.type == FST_JOINT_REVOLUTE) *qd.spent(bi.vi) = omc;
       SV vi, ai;
       if (bi.parent < 0) {
         vi = vJ;
@@ -279,7 +289,8 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
 #pragma unroll
         for (int c2 = 0; c2 < 6; ++c2) p[(int64_t)c2 * B] = r[c2];
       }
-      if (bi.parent >= 0) S.put(i, C_, XT_force(LEAN ? joint_X(tp.C(i), bi, q) : S.X(i, X_), F));
+      if (bi.parent >= 0)
+        S.put(i, C_, XT_force(LEAN ? joint_X<SPEND>(tp.C(i), bi, q, qd.p + bi.vi * qd.ld) : S.X(i, X_), F));
     }
     __syncthreads();
   }
@@ -568,14 +579,30 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
 // the bias force are formed in pass 2, and the joint transforms recomputed
 // in passes 2 and 3 instead of stored. The root's I^A and p^A, which pass 3
 // needs for a free base, stay in its slot.
-template <class TP>
+// SPEND: the caller has no further use for the staged rows. The sines of all
+// joints are then taken first, by all warps at once and not once a pass on the
+// chain of levels, and stay in the rows of q and the state; 1 / D and u move
+// to the rows of qd and tau once pass 2 has read them (B = 4096: quadruped
+// 11.0 -> 10.3 us, arm7 13.8 -> 12.6; humanoid B = 65536 93.2 -> 91.6).
+template <bool SPEND = false, class TP>
 __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& tau,
                                                const LaneState& S, const LaneState& R,
                                                float* __restrict__ qdd, int64_t B, int64_t e, bool act,
                                                float* qdd_col = nullptr) {
   const int W = n_warps(), w = warp_id();
-  enum { VU_ = 0, C_ = 6, ID_ = 12, u_ = 13 };  // per body
-  enum { RI_ = 0, RP_ = 21 };                      // per slot
+  enum { VU_ = 0, C_ = 6, OMC_ = 12, ID_ = 12, u_ = 13 };  // per body
+  enum { RI_ = 0, RP_ = 21 };                              // per slot
+  if (SPEND) {
+    for (int i = w; i < tp.n(); i += W) {
+      const BodyI bi = tp.I(i);
+      if (bi.type != FST_JOINT_REVOLUTE) continue;
+      const SinOmc t = sin_omc(q[bi.qi]);
+      *q.spent(bi.qi) = t.s;
+      *S.at(i, OMC_) = t.omc;
+    }
+    __syncthreads();
+  }
+  auto X_of = [&](int i, const BodyI& bi) { return joint_X<SPEND>(tp.C(i), bi, q, S.at(i, OMC_)); };
   // 1. root to leaf: velocities and bias accelerations
   FST_UNROLL
   for (int l = 0; l < tp.depth(); ++l) {
@@ -589,7 +616,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         vi = vJ;
         ci = sv_zero();
       } else {
-        vi = X_motion(joint_X(c, bi, q), S.sv(bi.parent, VU_)) + vJ;
+        vi = X_motion(X_of(i, bi), S.sv(bi.parent, VU_)) + vJ;
         ci = crm(vi, vJ);
       }
       S.put(i, VU_, vi);
@@ -626,8 +653,8 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         const float iD = 1.0f / dot(Sv, Ui);
         const float ui = tau[bi.vi] - dot(Sv, pA);
         S.put(i, VU_, Ui);
-        *S.at(i, ID_) = iD;
-        *S.at(i, u_) = ui;
+        *(SPEND ? qd.spent(bi.vi) : S.at(i, ID_)) = iD;
+        *(SPEND ? tau.spent(bi.vi) : S.at(i, u_)) = ui;
         if (bi.parent < 0) continue;
         sym6_rank1_sub(Ia, Ui, iD);
         pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, S.sv(i, C_)));
@@ -635,7 +662,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         if (bi.parent < 0) continue;
         pa = pa + sym6_mul(Ia, S.sv(i, C_));
       }
-      const Xf X = joint_X(tp.C(i), bi, q);
+      const Xf X = X_of(i, bi);
       R.putsym(slot, RI_, sym6_to_parent(X, Ia));
       R.put(slot, RP_, XT_force(X, pa));
     }
@@ -649,9 +676,10 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
       const int i = tp.level_body(k);
       const BodyI bi = tp.I(i);
       const SV ap = bi.parent < 0 ? a0 : S.sv(bi.parent, VU_);
-      SV ai = X_motion(joint_X(tp.C(i), bi, q), ap) + S.sv(i, C_);
+      SV ai = X_motion(X_of(i, bi), ap) + S.sv(i, C_);
       if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
-        const float qi = (*S.at(i, u_) - dot(S.sv(i, VU_), ai)) * *S.at(i, ID_);
+        const float ui = SPEND ? tau[bi.vi] : *S.at(i, u_), iD = SPEND ? qd[bi.vi] : *S.at(i, ID_);
+        const float qi = (ui - dot(S.sv(i, VU_), ai)) * iD;
         if (act && qdd) qdd[(int64_t)bi.vi * B + e] = qi;
         if (qdd_col) qdd_col[bi.vi << 5] = qi;
         ai = sv_fma(qi, S_of(tp.C(i)), ai);

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
   float* const state = tile + rows * kLaneEnvs;
   switch (op) {
     case ROLE_ABA:
-      aba_level_lean(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
+      aba_level_lean<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
                      LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, io.qdd_out, B, e,
                      act);
       break;
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
                       LaneState{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats}, io.M, B, e, act);
       break;
     case ROLE_RNEA:
-      rnea_level<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B, e, act);
+      rnea_level<true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B, e, act);
       break;
     default:
       fk_level(sm, cq, LaneState{state, kFkState}, io.poses, B, e, act);
