@@ -248,10 +248,10 @@ __global__ void __launch_bounds__(256) rnea_store_tile_kernel(ModelView mv, int6
 // bit. Blocks of the heaviest operator come first. EXT (a kernel of its own,
 // so that the plain one keeps its registers): the RNEA adjoint beside tau, and
 // M and J in the packed layouts.
-// Bound by the ABA blocks' latency at B = 4096 (quadruped, five operators: 14.1
+// Bound by the ABA blocks' latency at B = 4096 (quadruped, five operators: 13.3
 // us; the specialised fused kernel that the default took before 31.3, its
 // roles' straight-line code refetched by every SM) and by shared memory, two
-// to four tiles an SM, at larger batches (humanoid, B = 16384: 164 -> 86 us).
+// to four tiles an SM, at larger batches (humanoid, B = 16384: 164 -> 72 us).
 template <bool EXT, bool LEAN>
 __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B, EvalArgs a) {
   FST_TILE;
@@ -269,6 +269,8 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
   const SmemModel sm = stage_model_end(mv, smem);
   float* const state = tile + rows * kLaneEnvs;
   const Col cq = tile_col(tile, 0), c1 = tile_col(tile, mv.nq), c2 = tile_col(tile, mv.nq + nv);
+  auto X_of = [&](const BodyC& c, const BodyI& bi) { return joint_X(c, bi, cq); };
+  const LaneState R{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
   switch (role) {
     case ROLE_ABA:
       aba_level_lean<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
@@ -276,18 +278,10 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
                      e, act);
       break;
     case ROLE_CRBA:
-      if (LEAN) {
-        const LaneState S{state, kCrbaLeanBodyFloats};
-        const LaneState R{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
-        if (EXT && a.packed)
-          crba_level_lean<true>(sm, a.q, nv, S, R, a.M, B, e, act);
-        else
-          crba_level_lean(sm, a.q, nv, S, R, a.M, B, e, act);
-      } else if (EXT && a.packed) {
-        crba_level<true>(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
-      } else {
-        crba_level(sm, cq, nv, LaneState{state, kCrbaState}, a.M, B, e, act);
-      }
+      if (EXT && a.packed)
+        crba_level_lean<true>(sm, X_of, nv, LaneState{state, kCrbaLeanBodyFloats}, R, a.M, B, e, act);
+      else
+        crba_level_lean(sm, X_of, nv, LaneState{state, kCrbaLeanBodyFloats}, R, a.M, B, e, act);
       break;
     case ROLE_RNEA:
       if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
@@ -359,7 +353,7 @@ size_t eval_tile_smem(const ModelView& mv, int role, bool vjp, bool lean, int sl
   if (role == ROLE_ABA)
     f += 2 * (size_t)mv.nv + (size_t)kAbaLeanBodyFloats * mv.n + (size_t)kAbaLeanSlotFloats * slots;
   else if (role == ROLE_CRBA)
-    f += lean ? (size_t)kCrbaLeanBodyFloats * mv.n + (size_t)kCrbaLeanSlotFloats * slots : (size_t)kCrbaState * mv.n;
+    f += (size_t)kCrbaLeanBodyFloats * mv.n + (size_t)kCrbaLeanSlotFloats * slots;
   else if (role == ROLE_RNEA)
     f += (vjp ? 3 : 2) * (size_t)mv.nv + (size_t)(vjp ? kVjpState : lean ? kRneaLeanFloats : kRneaState) * mv.n;
   else

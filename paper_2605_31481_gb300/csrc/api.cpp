@@ -100,8 +100,8 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 // entry point's, so the fused evaluation and the single calls give the same
 // bits. Both sides measured on GB300 (us, tiles / other):
 //  * generic other side. Tiles shorten the chain from the bodies to the
-//    levels: humanoid29 B = 4096 RNEA 9.1 / 22.8, CRBA 10.6 / 72.5, ABA 15 /
-//    53; B = 65536 FK 24 / 40, RNEA 51 / 68, CRBA 91 / 160, ABA 94 / 200. A chain has no
+//    levels: humanoid29 B = 4096 RNEA 9.1 / 22.8, CRBA 10.1 / 72.5, ABA 15 /
+//    53; B = 65536 FK 24 / 40, RNEA 49 / 68, CRBA 77 / 160, ABA 92 / 200. A chain has no
 //    width to share: arm7 ABA 13 / 13 at 4096, 26 / 16 at 16384. Narrow trees
 //    (fewer than three bodies a level) at large batches are better off with
 //    more environments per SM where the sweeps are light: quadruped11 B =
@@ -542,7 +542,7 @@ fst_status fst_crba(const fst_model* m, int64_t B, const float* q, const float* 
     return finish(fn, launch_crba_level_lean(mv, B, q, M, level_block(m, JK_CRBA), m->slots,
                                              (cudaStream_t)stream));
   if (use_tile(m, JK_CRBA, B, level_smem_needed(mv, LEVEL_CRBA)))
-    return finish(fn, launch_crba_level(mv, B, q, M, tile_block(m, JK_CRBA, B), 1, (cudaStream_t)stream));
+    return finish(fn, launch_crba_level_lean(mv, B, q, M, tile_block(m, JK_CRBA, B), m->slots, (cudaStream_t)stream));
   if (use_path(m, JK_CRBA))
     return finish(fn, path_go(m, JK_CRBA, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, M));
   if (use_jit(m, JK_CRBA))

@@ -141,7 +141,7 @@ cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q
 cudaError_t launch_rnea_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                              float* tau, int block, cudaStream_t s);
 // The lean level-parallel CRBA (FST_VARIANT_LEVEL_LEAN).
-size_t crba_lean_smem_needed(const ModelView& mv, int slots);
+size_t crba_lean_smem_needed(const ModelView& mv, int slots, bool staged = false);
 cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int slots,
                                    cudaStream_t s);
 

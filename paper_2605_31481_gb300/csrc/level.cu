@@ -111,20 +111,33 @@ __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, 
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, tau, mv.nv, B, e);
   FST_LEVEL_READY;
-  aba_level_lean<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
-                 Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, qdd, B, e, act);
+  aba_level_lean<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs},
+                       Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+                       Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, qdd, B, e, act);
 }
 
-// CRBA with the lean per-tile state (FST_VARIANT_LEVEL_LEAN): no staged
-// rows (q is read from global memory), kCrbaLeanBodyFloats per body, a ring
-// of contribution slots. Up to three blocks per SM.
-__global__ void __launch_bounds__(256, 3) crba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
+// CRBA with the lean per-tile state (FST_VARIANT_LEVEL_LEAN, and the default's
+// tiles): kCrbaLeanBodyFloats per body and the contribution slots, three tiles
+// of the floating humanoid per SM where the full state has two. Bound by the
+// level phases' latency, then by the stores of M (B = 65536: 92 -> 77 us, of
+// them 33 for the bytes; 4096: 10.4 -> 10.1). q is staged where it fits (read
+// from global memory in the level loop instead: 93 us) and the bodies with the
+// longest walk to the root go first. More than 80 registers a thread would cost
+// small trees a block an SM: none is forced here (58 used).
+template <bool STAGED>
+__global__ void __launch_bounds__(256) crba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                            float* __restrict__ M, int slots) {
-  FST_LEVEL_PROLOGUE_S(0, kCrbaLeanBodyFloats,
-                       (kCrbaLeanBodyFloats * mv.n + kCrbaLeanSlotFloats * slots) * kLaneEnvs);
-  const LaneState R{tile + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
+  const int rows = STAGED ? mv.nq : 0;
+  FST_LEVEL_PROLOGUE_S(rows, kCrbaLeanBodyFloats,
+                       (rows + kCrbaLeanBodyFloats * mv.n + kCrbaLeanSlotFloats * slots) * kLaneEnvs);
+  const LaneState R{tile + (rows + kCrbaLeanBodyFloats * mv.n) * kLaneEnvs, kCrbaLeanSlotFloats};
+  if (STAGED) stage_block_rows(tile, q, mv.nq, B, e);
   FST_LEVEL_READY;
-  crba_level_lean(sm, q, mv.nv, S, R, M, B, e, act);
+  const int64_t ec = act ? e : B - 1;  // lanes past B compute on the last environment and store nothing
+  auto X_of = [&](const BodyC& c, const BodyI& bi) {
+    return STAGED ? joint_X(c, bi, Col{tile + lane, kLaneEnvs}) : joint_X_rows(c, bi, q, B, ec);
+  };
+  crba_level_lean(sm, X_of, mv.nv, S, R, M, B, e, act);
 }
 
 // SM-pinned ABA (FST_VARIANT_PINNED): blocks on SMs pinned to ABA take
@@ -270,13 +283,15 @@ cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q
                                   float* qdd, int block, int slots, cudaStream_t s) {
   return go(aba_lean_kernel, mv, B, aba_lean_smem_needed(mv, slots), block, 1, 1, s, q, qd, tau, qdd, slots);
 }
-size_t crba_lean_smem_needed(const ModelView& mv, int slots) {
-  return smem_bytes(mv.n) +
+size_t crba_lean_smem_needed(const ModelView& mv, int slots, bool staged) {
+  return smem_bytes(mv.n) + (staged ? level_tile_bytes(mv, mv.nq, 0) : 0) +
          (size_t)(kCrbaLeanBodyFloats * mv.n + kCrbaLeanSlotFloats * slots) * kLaneEnvs * sizeof(float);
 }
 cudaError_t launch_crba_level_lean(const ModelView& mv, int64_t B, const float* q, float* M, int block, int slots,
                                    cudaStream_t s) {
-  return go(crba_lean_kernel, mv, B, crba_lean_smem_needed(mv, slots), block, 1, 1, s, q, M, slots);
+  const size_t sh = crba_lean_smem_needed(mv, slots, true);
+  if (sh <= kLevelSmemLimit) return go(crba_lean_kernel<true>, mv, B, sh, block, 1, 1, s, q, M, slots);
+  return go(crba_lean_kernel<false>, mv, B, crba_lean_smem_needed(mv, slots, false), block, 1, 1, s, q, M, slots);
 }
 cudaError_t launch_aba_level_pinned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                     const float* tau, float* qdd, int block, const PinArgs& p, cudaStream_t s) {

@@ -404,13 +404,12 @@ __device__ __forceinline__ Xf joint_X_rows(const BodyC& c, const BodyI& bi, cons
 // its parent lives in a slot of R (BodyC::slot) until the parent has added it;
 // the root keeps its own I^c in its slot for a free base's 6 x 6 block. q is read from global memory,
 // not staged. Same arithmetic, in the same order, as crba_level.
-template <bool PACKED = false, class TP>
-__device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __restrict__ q, int nv,
+template <bool PACKED = false, class TP, class XF>
+__device__ __forceinline__ void crba_level_lean(const TP& tp, const XF& X_of, int nv,
                                                 const LaneState& S, const LaneState& R,
                                                 float* __restrict__ M, int64_t B, int64_t e, bool act) {
   const int W = n_warps(), w = warp_id();
   enum { X_ = 0, F_ = 12 };
-  const int64_t ec = act ? e : B - 1;  // lanes past B compute on the last environment and store nothing
   if (tp.depth() > 0) m_clear_tile(M, PACKED ? (int64_t)nv * (nv + 1) / 2 : (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
   FST_UNROLL
   for (int l = tp.depth() - 1; l >= 0; --l) {
@@ -418,7 +417,7 @@ __device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __res
       const int i = tp.level_body(k);
       const BodyI bi = tp.I(i);
       const int slot = tp.C(i).slot;
-      const Xf X = joint_X_rows(tp.C(i), bi, q, B, ec);
+      const Xf X = X_of(tp.C(i), bi);
       In10 Ic = in_load(tp.theta(i));
       for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch)
         in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
@@ -430,7 +429,9 @@ __device__ __forceinline__ void crba_level_lean(const TP& tp, const float* __res
   }
   if (!act) return;
   const MOut<PACKED> Me{M + e, nv, B};
-  for (int i = w; i < tp.n(); i += W) {
+  // deepest bodies, and so longest walks, first: the warps end together
+  for (int k = tp.n() - 1 - w; k >= 0; k -= W) {
+    const int i = tp.level_body(k);
     const BodyI bi = tp.I(i);
     if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
       SV F = S.sv(i, F_);

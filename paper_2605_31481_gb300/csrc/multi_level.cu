@@ -52,7 +52,8 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
                      act);
       break;
     case ROLE_CRBA:
-      crba_level_lean(sm, io.q, mv.nv, LaneState{state, kCrbaLeanBodyFloats},
+      crba_level_lean(sm, [&](const BodyC& c, const BodyI& bi) { return joint_X(c, bi, cq); }, mv.nv,
+                      LaneState{state, kCrbaLeanBodyFloats},
                       LaneState{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats}, io.M, B, e, act);
       break;
     case ROLE_RNEA:
