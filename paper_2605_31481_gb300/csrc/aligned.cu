@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, i
   const SmemModel sm = stage_model_end(mv, smem);
   const Col cq = tile_col(tile, 0), cqd = tile_col(tile, mv.nq);
   float* const qcol = tile + (mv.nq + 2 * nv) * kLaneEnvs + lane;  // qdd
-  aba_level_lean(sm, world_accel(mv), cq, cqd, tile_col(tile, mv.nq + nv), LaneState{state, kAbaLeanBodyFloats},
+  aba_level_lean<false, true>(sm, world_accel(mv), cq, cqd, tile_col(tile, mv.nq + nv), LaneState{state, kAbaLeanBodyFloats},
                  LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, qdd, B, e, act,
                  qcol);
   const TreeMat H{hbase, lists, lists + nv, anc};
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
   float* const state = tile + rows * kLaneEnvs;
   float* const lam = tile + (mv.nq + 3 * nv) * kLaneEnvs + lane;
   const Col cq = tile_col(tile, 0);
-  aba_level_lean(sm, sv_zero(), cq, Col{zero, 0}, tile_col(tile, mv.nq + 2 * nv), LaneState{state, kAbaLeanBodyFloats},
+  aba_level_lean<false, true>(sm, sv_zero(), cq, Col{zero, 0}, tile_col(tile, mv.nq + 2 * nv), LaneState{state, kAbaLeanBodyFloats},
                  LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, taubar, B, e, act,
                  lam);
   const VjpAligned o{qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
   const LaneState R{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats};
   switch (role) {
     case ROLE_ABA:
-      aba_level_lean<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
+      aba_level_lean<true, !LEAN>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
                      LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, a.qdd_out, B,
                      e, act);
       break;
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
       break;
     case ROLE_RNEA:
       if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
-        rnea_level<LEAN, LEAN && !EXT>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
+        rnea_level<LEAN, LEAN && !EXT, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
                          a.tau_out, B, e, act,
                          vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
       if (vjp)  // rnea_level ends with a barrier: the cotangent is complete and the state free
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
                                     B, e, act);
       break;
     default:
-      kin_level(sm, cq, nv, a.links, LaneState{state, kFkState}, a.poses, a.J, B, e, act,
+      kin_level<!LEAN>(sm, cq, nv, a.links, LaneState{state, kFkState}, a.poses, a.J, B, e, act,
                 EXT && a.packed ? &a.pj : nullptr);
       break;
   }

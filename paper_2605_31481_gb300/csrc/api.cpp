@@ -100,7 +100,7 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 // entry point's, so the fused evaluation and the single calls give the same
 // bits. Both sides measured on GB300 (us, tiles / other):
 //  * generic other side. Tiles shorten the chain from the bodies to the
-//    levels: humanoid29 B = 4096 RNEA 9.1 / 22.8, CRBA 10.1 / 72.5, ABA 15 /
+//    levels: humanoid29 B = 4096 RNEA 8.3 / 22.8, CRBA 9.8 / 72.5, ABA 13.7 /
 //    53; B = 65536 FK 24 / 40, RNEA 49 / 68, CRBA 77 / 160, ABA 92 / 200. A chain has no
 //    width to share: arm7 ABA 13 / 13 at 4096, 26 / 16 at 16384. Narrow trees
 //    (fewer than three bodies a level) at large batches are better off with
@@ -120,12 +120,34 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
     if (m->n <= 16) return B < 8192;
     return !light || B < (op == JK_RNEA || op == JK_RNEA_STORE ? 24576 : 16384);
   }
-  if (2 * m->n < 3 * m->depth) return B <= 152 * 2 * 32;
+  if (2 * m->n < 3 * m->depth) {
+    const int64_t most = op != JK_RNEA || m->n <= 8 ? 152 * 2 * 32 : m->n <= 16 ? 152 * 32 : 0;
+    return B <= most;
+  }
   return !light || m->n >= 3 * m->depth || B < 32768;
 }
 
-bool use_tile(const fst_model* m, int kind, int64_t B, size_t need) {
-  return m->variant[kind] == FST_VARIANT_AUTO && need <= kLevelSmemLimit && tile_rule(m, kind, jit_has(m, kind), B);
+// Shared memory of one tile of an operator's state in full. Where that does not
+// fit the operator does not run as tiles, though a leaner form of it might: all
+// entry points ask the same question.
+size_t tile_need(const fst_model* m, int kind) {
+  const ModelView mv = view_of(m, nullptr);
+  switch (kind) {
+    case JK_ABA:
+      return aba_lean_smem_needed(mv, m->slots);
+    case JK_CRBA:
+      return level_smem_needed(mv, LEVEL_CRBA);
+    case JK_RNEA:
+    case JK_RNEA_STORE:
+      return level_smem_needed(mv, LEVEL_RNEA);
+    default:
+      return level_smem_needed(mv, LEVEL_FK);
+  }
+}
+
+bool use_tile(const fst_model* m, int kind, int64_t B) {
+  return m->variant[kind] == FST_VARIANT_AUTO && tile_need(m, kind) <= kLevelSmemLimit &&
+         tile_rule(m, kind, jit_has(m, kind), B);
 }
 
 // The same question for the adjoints, whose tiles do more per barrier: against
@@ -136,11 +158,12 @@ bool use_tile(const fst_model* m, int kind, int64_t B, size_t need) {
 // 73). The FK adjoint is light: arm7 specialised 5.5 / 8.2 at every batch,
 // quadruped11 8.5 / 7.5 at 4096 and 8.6 / 10 at 16384. For the smallest trees
 // the RNEA adjoint follows the specialised fused step, whose result it must
-// equal bit for bit.
+// equal bit for bit (where the step is better off with it: quadruped11 B = 8192 30.8
+// us in one launch, 43 as step and adjoint).
 bool adjoint_tile_rule(const fst_model* m, int kind, bool spec, int64_t B) {
   if (kind == JK_FK_VJP) return spec ? m->n > 8 && (m->n > 16 || B < 12288) : true;
   if (spec && m->n <= 8 && kind == JK_RNEA_VJP) return false;
-  if (spec && m->n <= 16) return B < 24576;
+  if (spec && m->n <= 16) return B < (kind == JK_RNEA_VJP ? 8192 : 24576);
   return 2 * m->n >= 3 * m->depth || B <= 24576;
 }
 
@@ -162,10 +185,11 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
-// Threads per block of the mixed-tree launch in tiles (five trees, 7936
-// environments: 64 threads 24.5 us, 128 22.0, 256 22.4; a group with a large
-// tree wants its warps).
-constexpr int kMultiTileBlock = 256;
+// Threads per block of the mixed-tree launch in tiles: four warps let four
+// blocks share an SM (110 registers a thread), eight are the faster ones while
+// all items run at once (five trees, 8192 environments: 19.3 / 23.9 us; 4096: 15.0 /
+// 13.5; 64: 12.4 / 10.8).
+int multi_tile_block(int items) { return items <= 152 * 2 ? 256 : 128; }
 
 // Whether enough tiles wait for an SM (more than two each) that the forms
 // which keep less state, and so more tiles per SM, are the better ones.
@@ -176,9 +200,13 @@ bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
 // 16384 RNEA 9.8 -> 8.6 us, ABA 24.4 -> 14.1, the step 40.5 -> 38.8; legged18, six
 // bodies wide, ABA 19.0 against 27.5 with four). The adjoint's state leaves
 // room for too few tiles (the fused step with it 38.7 against 44.3 with four),
-// and CRBA's stores want the warps (B = 65536 29.1 against 31.1).
+// and CRBA's stores want the warps (B = 65536 29.1 against 31.1). The step of a
+// small narrow tree takes four warps from half a tile per SM on: at 110 registers a
+// thread four such blocks share an SM (quadruped11 B = 4096 13.2 against 15.5 us,
+// 8192 20.9 against 26.7; but 9.9 against 9.0 at 64).
 int tile_block(const fst_model* m, int kind, int64_t B, bool vjp = false) {
   if (m->block[kind]) return m->block[kind];
+  if (kind == JK_EVAL && !vjp && m->max_width <= 4 && m->n <= 16 && B > 152 * 32 / 2) return 128;
   if (!many_tiles(B) || m->max_width > 4 || vjp || kind == JK_CRBA) return 256;
   return m->n <= 16 || kind == JK_ABA ? 128 : 256;
 }
@@ -461,7 +489,7 @@ fst_status fst_fk(const fst_model* m, int64_t B, const float* q, float* poses, v
   if (use_level(m, JK_FK, LEVEL_FK))
     return finish(fn, launch_fk_level(mv, B, q, poses, level_block(m, JK_FK), level_tiles(m, JK_FK),
                         (cudaStream_t)stream));
-  if (use_tile(m, JK_FK, B, level_smem_needed(mv, LEVEL_FK)))
+  if (use_tile(m, JK_FK, B))
     return finish(fn, launch_fk_level(mv, B, q, poses, tile_block(m, JK_FK, B), 1, (cudaStream_t)stream));
   if (use_path(m, JK_FK))
     return finish(fn, path_go(m, JK_FK, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, poses));
@@ -491,7 +519,7 @@ fst_status fst_jacobian(const fst_model* m, int64_t B, const float* q, const int
   if (use_level(m, JK_JACOBIAN, LEVEL_JAC))
     return finish(fn, launch_jac_level(mv, B, q, L, J, level_block(m, JK_JACOBIAN), level_tiles(m, JK_JACOBIAN),
                         (cudaStream_t)stream));
-  if (use_tile(m, JK_JACOBIAN, B, level_smem_needed(mv, LEVEL_JAC)))
+  if (use_tile(m, JK_JACOBIAN, B))
     return finish(fn, launch_jac_level(mv, B, q, L, J, tile_block(m, JK_JACOBIAN, B), 1, (cudaStream_t)stream));
   if (use_path(m, JK_JACOBIAN))
     return finish(fn, path_go(m, JK_JACOBIAN, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, L, J));
@@ -514,7 +542,7 @@ fst_status fst_rnea(const fst_model* m, int64_t B, const float* q, const float* 
   if (use_level(m, JK_RNEA, LEVEL_RNEA))
     return finish(fn, launch_rnea_level(mv, B, q, qd, qdd, tau, level_block(m, JK_RNEA), level_tiles(m, JK_RNEA),
                         (cudaStream_t)stream));
-  if (use_tile(m, JK_RNEA, B, level_smem_needed(mv, LEVEL_RNEA)))
+  if (use_tile(m, JK_RNEA, B))
     return finish(fn, many_tiles(B)
                           ? launch_rnea_lean(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA, B), (cudaStream_t)stream)
                           : launch_rnea_level(mv, B, q, qd, qdd, tau, tile_block(m, JK_RNEA, B), 1,
@@ -541,7 +569,7 @@ fst_status fst_crba(const fst_model* m, int64_t B, const float* q, const float* 
   if (m->variant[JK_CRBA] == FST_VARIANT_LEVEL_LEAN && crba_lean_smem_needed(mv, m->slots) <= kLevelSmemLimit)
     return finish(fn, launch_crba_level_lean(mv, B, q, M, level_block(m, JK_CRBA), m->slots,
                                              (cudaStream_t)stream));
-  if (use_tile(m, JK_CRBA, B, level_smem_needed(mv, LEVEL_CRBA)))
+  if (use_tile(m, JK_CRBA, B))
     return finish(fn, launch_crba_level_lean(mv, B, q, M, tile_block(m, JK_CRBA, B), m->slots, (cudaStream_t)stream));
   if (use_path(m, JK_CRBA))
     return finish(fn, path_go(m, JK_CRBA, B, m->nq, 1, (cudaStream_t)stream, mv, B, q, M));
@@ -575,7 +603,7 @@ fst_status fst_aba(const fst_model* m, int64_t B, const float* q, const float* q
                                     PinArgs{m->dpin, counters}, (cudaStream_t)stream);
     return finish(fn, err);
   }
-  if (use_tile(m, JK_ABA, B, aba_lean_smem_needed(mv, m->slots)))
+  if (use_tile(m, JK_ABA, B))
     return finish(fn, launch_aba_level_lean(mv, B, q, qd, tau, qdd, tile_block(m, JK_ABA, B), m->slots,
                                             (cudaStream_t)stream));
   if (use_path(m, JK_ABA))
@@ -740,8 +768,20 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
     auto tiled = [&](int role) {
       const int op = role == ROLE_ABA ? JK_ABA : role == ROLE_CRBA ? JK_CRBA : role == ROLE_RNEA ? JK_RNEA
                                                                              : (a.J ? JK_JACOBIAN : JK_FK);
-      return tile_rule(m, op, spec, B);
+      return tile_need(m, op) <= kLevelSmemLimit && tile_rule(m, op, spec, B);
     };
+    const bool adjoint_tiled =
+        vjp && rnea_vjp_aligned_smem(mv) + 1024 <= kLevelSmemLimit && adjoint_tile_rule(m, JK_RNEA_VJP, spec, B);
+    if (vjp && adjoint_tiled != tiled(ROLE_RNEA)) {
+      // the adjoint's own call takes another form than RNEA's: it follows as that
+      // call, so that its values are that call's
+      fst_eval_io rest = *io;
+      rest.tau_bar = nullptr;
+      rest.q_bar = rest.qd_bar = rest.qdd_bar = nullptr;
+      FST_CHECK(fst_eval(m, B, &rest, theta, stream));
+      return fst_rnea_vjp(m, B, io->q, io->qd, io->qdd, theta, io->tau_bar, io->q_bar, io->qd_bar, io->qdd_bar, nullptr,
+                          nullptr, 0, stream);
+    }
     EvalArgs t = a, g = a;
     t.n_roles = g.n_roles = 0;
     for (int r = 0; r < a.n_roles; ++r) {
@@ -924,7 +964,7 @@ fst_status fst_rnea_store(const fst_model* m, int64_t B, const float* q, const f
     FST_CHECK(need(fn, qdd, "qdd"));
   }
   const ModelView mv = view_of(m, theta);
-  if (use_tile(m, JK_RNEA_STORE, B, level_smem_needed(mv, LEVEL_RNEA)))
+  if (use_tile(m, JK_RNEA_STORE, B))
     return finish(fn, launch_rnea_store_tile(mv, B, q, qd, qdd, tau, tape, tile_block(m, JK_RNEA_STORE, B),
                                              (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_STORE))
@@ -1190,8 +1230,7 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
       for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) level = level && tile_smem(k, r) <= kLevelSmemLimit;
     }
   }
-  const int block = g->variant == FST_VARIANT_AUTO && level ? kMultiTileBlock : g->block;
-  const int T = level ? 32 : block;  // environments per item
+  const int T = level ? 32 : g->block;  // environments per item
   size_t smem = 0;                   // level: shared memory of the largest (tree, operator) pair
   size_t full = 0;                   // and its state floats a lane with nothing taken over or re-formed
   // every block of the persistent grid draws one item past the last, so the
@@ -1232,6 +1271,7 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
     if (smem > kLevelSmemLimit || (g->variant == FST_VARIANT_LEVEL && need > kLevelSmemLimit))
       return set_error(FST_ERR_INVALID_ARG, std::string(fn) + ": the level-parallel state of the largest tree "
                                                               "does not fit in shared memory");
+    const int block = g->variant == FST_VARIANT_AUTO ? multi_tile_block((int)items) : g->block;
     return finish(fn, launch_multi_tiles(a, smem, block, (cudaStream_t)stream));
   }
   return finish(fn, launch_multi(a, max_n, T, (cudaStream_t)stream));

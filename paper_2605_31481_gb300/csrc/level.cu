@@ -29,21 +29,23 @@ __device__ __forceinline__ float* level_tile(float4* smem, int n) { return smem_
 // synchronises the block, so everything staged is visible to every warp.
 #define FST_LEVEL_READY const SmemModel sm = stage_model_end(mv, smem)
 
+template <bool AHEAD>
 __global__ void __launch_bounds__(256) fk_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                        float* __restrict__ poses) {
   FST_LEVEL_PROLOGUE(mv.nq, kFkState);
   stage_block_rows(tile, q, mv.nq, B, e);
   FST_LEVEL_READY;
-  fk_level(sm, Col{tile + lane, kLaneEnvs}, S, poses, B, e, act);
+  fk_level<AHEAD>(sm, Col{tile + lane, kLaneEnvs}, S, poses, B, e, act);
 }
 
+template <bool AHEAD>
 __global__ void __launch_bounds__(256) jac_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                         LinkList links, float* __restrict__ poses,
                                                         float* __restrict__ J) {
   FST_LEVEL_PROLOGUE(mv.nq, kFkState);
   stage_block_rows(tile, q, mv.nq, B, e);
   FST_LEVEL_READY;
-  kin_level(sm, Col{tile + lane, kLaneEnvs}, mv.nv, links, S, poses, J, B, e, act);
+  kin_level<AHEAD>(sm, Col{tile + lane, kLaneEnvs}, mv.nv, links, S, poses, J, B, e, act);
 }
 
 __global__ void __launch_bounds__(256) rnea_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
@@ -54,12 +56,12 @@ __global__ void __launch_bounds__(256) rnea_level_kernel(ModelView mv, int64_t B
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
   FST_LEVEL_READY;
-  rnea_level(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+  rnea_level<false, false, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
              Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
 // RNEA with 12 floats of state a body: four tiles of the floating humanoid per
-// SM instead of two (B = 65536: 66.6 -> 50.8 us, 16384: 20.1 -> 16.2).
+// SM instead of two (B = 65536: 66.6 -> 47.3 us, 16384: 20.1 -> 15.0).
 __global__ void __launch_bounds__(256) rnea_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                         const float* __restrict__ qd, const float* __restrict__ qdd,
                                                         float* __restrict__ tau) {
@@ -68,7 +70,7 @@ __global__ void __launch_bounds__(256) rnea_lean_kernel(ModelView mv, int64_t B,
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
   FST_LEVEL_READY;
-  rnea_level<true, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+  rnea_level<true, true, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
                    Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(256) aba_level_kernel(ModelView mv, int64_t B,
 // us; FP32 floor 18). Tried on top and not kept: four tiles, with qd and tau
 // read from global memory and the bias accelerations folded into the forces
 // (105 us, and 1 us more at small batches).
+template <bool AHEAD>
 __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                        const float* __restrict__ qd, const float* __restrict__ tau,
                                                        float* __restrict__ qdd, int slots) {
@@ -111,7 +114,7 @@ __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, 
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, tau, mv.nv, B, e);
   FST_LEVEL_READY;
-  aba_level_lean<true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs},
+  aba_level_lean<true, AHEAD>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs},
                        Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
                        Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, R, qdd, B, e, act);
 }
@@ -120,10 +123,10 @@ __global__ void __launch_bounds__(256) aba_lean_kernel(ModelView mv, int64_t B, 
 // tiles): kCrbaLeanBodyFloats per body and the contribution slots, three tiles
 // of the floating humanoid per SM where the full state has two. Bound by the
 // level phases' latency, then by the stores of M (B = 65536: 92 -> 77 us, of
-// them 33 for the bytes; 4096: 10.4 -> 10.1). q is staged where it fits (read
+// them 33 for the bytes; 4096: 10.4 -> 9.8). q is staged where it fits (read
 // from global memory in the level loop instead: 93 us) and the bodies with the
 // longest walk to the root go first. More than 80 registers a thread would cost
-// small trees a block an SM: none is forced here (58 used).
+// small trees a block an SM: none is forced here (64 used).
 template <bool STAGED>
 __global__ void __launch_bounds__(256) crba_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                            float* __restrict__ M, int slots) {
@@ -225,6 +228,10 @@ cudaError_t go(void (*kernel)(P...), const ModelView& mv, int64_t B, size_t sh, 
   return launch_pdl(kernel, dim3((unsigned)((B + envs - 1) / envs), gy), blk, sh, s, mv, B, args...);
 }
 
+// Whether the warps of a tile do their next bodies' own work ahead of its level
+// (level_pass) in FK and ABA: up to two tiles an SM, see there for both sides.
+bool few_tiles(int64_t B) { return B <= 152 * 2 * 32; }
+
 }  // namespace
 
 size_t model_smem_bytes(int n) { return smem_bytes(n); }
@@ -251,12 +258,13 @@ size_t level_smem_needed(const ModelView& mv, int kind, int tiles) {
 
 cudaError_t launch_fk_level(const ModelView& mv, int64_t B, const float* q, float* poses, int block, int tiles,
                             cudaStream_t s) {
-  return go(fk_level_kernel, mv, B, level_smem_needed(mv, LEVEL_FK, tiles), block, tiles, 1, s, q, poses);
+  return go(few_tiles(B) ? fk_level_kernel<true> : fk_level_kernel<false>, mv, B,
+            level_smem_needed(mv, LEVEL_FK, tiles), block, tiles, 1, s, q, poses);
 }
 cudaError_t launch_jac_level(const ModelView& mv, int64_t B, const float* q, const LinkList& links, float* J,
                              int block, int tiles, cudaStream_t s) {
-  return go(jac_level_kernel, mv, B, level_smem_needed(mv, LEVEL_JAC, tiles), block, tiles, 1, s, q, links,
-            (float*)nullptr, J);
+  return go(few_tiles(B) ? jac_level_kernel<true> : jac_level_kernel<false>, mv, B,
+            level_smem_needed(mv, LEVEL_JAC, tiles), block, tiles, 1, s, q, links, (float*)nullptr, J);
 }
 cudaError_t launch_rnea_level(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                               float* tau, int block, int tiles, cudaStream_t s) {
@@ -281,7 +289,7 @@ size_t aba_lean_smem_needed(const ModelView& mv, int slots) {
 }
 cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* tau,
                                   float* qdd, int block, int slots, cudaStream_t s) {
-  return go(aba_lean_kernel, mv, B, aba_lean_smem_needed(mv, slots), block, 1, 1, s, q, qd, tau, qdd, slots);
+  return go(few_tiles(B) ? aba_lean_kernel<true> : aba_lean_kernel<false>, mv, B, aba_lean_smem_needed(mv, slots), block, 1, 1, s, q, qd, tau, qdd, slots);
 }
 size_t crba_lean_smem_needed(const ModelView& mv, int slots, bool staged) {
   return smem_bytes(mv.n) + (staged ? level_tile_bytes(mv, mv.nq, 0) : 0) +

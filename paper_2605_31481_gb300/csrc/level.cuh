@@ -139,36 +139,85 @@ __device__ __forceinline__ void stage_block_rows(float* tile, const float* __res
 #define FST_FOR_MY_BODIES(tp, l, k) for (int k = (tp).level_begin(l) + w; k < (tp).level_begin((l) + 1); k += W)
 #endif
 
+// A pass over the levels, root to leaf or (UP) leaf to root, with a barrier
+// after each: dep(o) with o = loc(i) for each body i, where loc reads only what
+// is known before the pass. With AHEAD body k of the level order is warp k mod
+// W's, so that the bodies of neighbouring levels are different warps', and a warp
+// whose level has not come yet does the loc of its next body meanwhile: what is
+// left on the chain of levels is dep. Without it each level starts at warp 0.
+// A tile's time is that chain's as long as an SM has few tiles (us without ->
+// with, humanoid29 B = 4096: FK 5.0 -> 4.6, RNEA 9.0 -> 8.3, CRBA 10.6 -> 9.8, ABA
+// 14.6 -> 13.6; arm7 ABA 12.6 -> 11.1; legged12 B = 1000 d qdd 26.7 -> 23.6). Where
+// many tiles wait it still pays for CRBA and the lean RNEA (humanoid29 B = 65536
+// 79.8 -> 76.8 and 49.0 -> 47.3), but the lean ABA's registers (109 instead of 77)
+// then cost more than the shorter chain saves (91.6 -> 96).
+struct BlockBarrier {
+  __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+template <bool UP, bool AHEAD, class TP, class Loc, class Dep, class Bar = BlockBarrier>
+__device__ __forceinline__ void level_pass(const TP& tp, const Loc& loc, const Dep& dep, const Bar& barrier = Bar()) {
+  const int W = n_warps(), w = warp_id(), D = tp.depth();
+  if (!AHEAD) {
+    FST_UNROLL
+    for (int s = 0; s < D; ++s) {
+      FST_FOR_MY_BODIES(tp, UP ? D - 1 - s : s, k) dep(loc(tp.level_body(k)));
+      barrier();
+    }
+    return;
+  }
+  const int n = tp.n();
+  decltype(loc(0)) mine;
+  bool have = false;
+  int j = w;  // position in the order of the pass
+  int end = UP ? n - tp.level_begin(D - 1) : tp.level_begin(1);
+  for (int s = 0; s < D; ++s) {
+    for (;;) {
+      if (!have && j < n) {
+        mine = loc(tp.level_body(UP ? n - 1 - j : j));
+        have = true;
+      }
+      if (j >= end) break;
+      dep(mine);
+      have = false;
+      j += W;
+      if (j >= end) break;
+    }
+    const int next = s + 1 < D ? s + 1 : s;
+    end = UP ? n - tp.level_begin(D - 1 - next) : tp.level_begin(next + 1);
+    barrier();
+  }
+}
+
 
 // ---- forward kinematics -------------------------------------------------------
-template <class TP>
+template <bool AHEAD = false, class TP>
 __device__ __forceinline__ void fk_level(const TP& tp, const Col& q, const LaneState& S, float* __restrict__ poses,
                                          int64_t B, int64_t e, bool act) {
-  const int W = n_warps(), w = warp_id();
-  FST_UNROLL
-  for (int l = 0; l < tp.depth(); ++l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const Xf X = joint_X(tp.C(i), bi, q);
-      Xf P;
-      if (bi.parent < 0) {
-        P = X;
-      } else {
-        const Xf Pp = S.X(bi.parent, 0);
-        compose(Pp.R, Pp.t, X, P.R, P.t);
-      }
-      S.putX(i, 0, P);
-      if (poses && act) {
-        float* out = poses + (int64_t)i * 12 * B + e;
+  struct Own {
+    int i, parent;
+    Xf X;
+  };
+  level_pass<false, AHEAD>(
+      tp,
+      [&](int i) {
+        const BodyI bi = tp.I(i);
+        return Own{i, bi.parent, joint_X(tp.C(i), bi, q)};
+      },
+      [&](const Own& o) {
+        Xf P = o.X;
+        if (o.parent >= 0) {
+          const Xf Pp = S.X(o.parent, 0);
+          compose(Pp.R, Pp.t, o.X, P.R, P.t);
+        }
+        S.putX(o.i, 0, P);
+        if (poses && act) {
+          float* out = poses + (int64_t)o.i * 12 * B + e;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) out[(int64_t)c * B] = P.R[c];
+          for (int c = 0; c < 9; ++c) out[(int64_t)c * B] = P.R[c];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) out[(int64_t)(9 + c) * B] = P.t[c];
-      }
-    }
-    __syncthreads();
-  }
+          for (int c = 0; c < 3; ++c) out[(int64_t)(9 + c) * B] = P.t[c];
+        }
+      });
 }
 
 // Jacobians after fk_level: one (link, body) column per work item; columns
@@ -203,11 +252,11 @@ __device__ __forceinline__ void jac_columns(const TP& tp, int nv, const LinkList
 }
 
 // FK, then the Jacobian columns of `links` when J is given.
-template <class TP>
+template <bool AHEAD = false, class TP>
 __device__ __forceinline__ void kin_level(const TP& tp, const Col& q, int nv, const LinkList& links,
                                           const LaneState& S, float* __restrict__ poses, float* __restrict__ J,
                                           int64_t B, int64_t e, bool act, const PackedJ* PK = nullptr) {
-  fk_level(tp, q, S, poses, B, e, act);
+  fk_level<AHEAD>(tp, q, S, poses, B, e, act);
   if (J) jac_columns(tp, nv, links, S, J, B, e, act, PK);
 }
 
@@ -223,7 +272,7 @@ __device__ __forceinline__ void kin_level(const TP& tp, const Col& q, int nv, co
 // SPEND (with LEAN): the staged rows are the sweep's to overwrite: a joint's sine
 // and 1 - cosine replace its q and qd until the way back has used them
 // (humanoid B = 65536: 50.2 -> 49.0 us).
-template <bool LEAN = false, bool SPEND = false, class TP>
+template <bool LEAN = false, bool SPEND = false, bool AHEAD = false, class TP>
 __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& qdd,
                                            const LaneState& S, float* __restrict__ tau, int64_t B, int64_t e,
                                            bool act, float* tau_col = nullptr, float* tape = nullptr) {
@@ -233,67 +282,86 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
     const In10 I = in_load(tp.theta(i));
     return in_mul(I, a) + crf(v, in_mul(I, v));
   };
-  FST_UNROLL
-  for (int l = 0; l < tp.depth(); ++l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyC& c = tp.C(i);
-      const BodyI bi = tp.I(i);
-      float omc = 0.f;
-      if (SPEND && bi.type == FST_JOINT_REVOLUTE) {
-        const SinOmc t = sin_omc(q[bi.qi]);
-        *q.spent(bi.qi) = t.s;
-        omc = t.omc;
-      }
-      const Xf X = joint_X<SPEND>(c, bi, q, &omc);
-      const SV vJ = S_times(c, bi, qd);
-      const SV aJ = S_times(c, bi, qdd);
-      if (SPEND && bi.type == FST_JOINT_REVOLUTE) *qd.spent(bi.vi) = omc;
-      SV vi, ai;
-      if (bi.parent < 0) {
-        vi = vJ;
-        ai = X_motion(X, a0) + aJ;
-      } else {
-        vi = X_motion(X, S.sv(bi.parent, V_)) + vJ;
-        ai = X_motion(X, S.sv(bi.parent, A_)) + aJ + crm(vi, vJ);
-      }
-      S.put(i, V_, vi);
-      S.put(i, A_, ai);
-      if (!LEAN) {
-        S.putX(i, X_, X);
-        S.put(i, C_, force(i, vi, ai));
-      }
-      if (tape && act) {
-        float* p = tape + (int64_t)i * 30 * B + e;
-        const float r[24] = {X.R[0], X.R[1], X.R[2], X.R[3], X.R[4], X.R[5], X.R[6], X.R[7],
-                             X.R[8], X.t[0], X.t[1], X.t[2], vi.w.x, vi.w.y, vi.w.z, vi.v.x,
-                             vi.v.y, vi.v.z, ai.w.x, ai.w.y, ai.w.z, ai.v.x, ai.v.y, ai.v.z};
+  struct Moved {
+    int i, parent;
+    Xf X;
+    SV vJ, aJ;
+  };
+  level_pass<false, AHEAD>(
+      tp,
+      [&](int i) {
+        const BodyC& c = tp.C(i);
+        const BodyI bi = tp.I(i);
+        float omc = 0.f;
+        if (SPEND && bi.type == FST_JOINT_REVOLUTE) {
+          const SinOmc t = sin_omc(q[bi.qi]);
+          *q.spent(bi.qi) = t.s;
+          omc = t.omc;
+        }
+        Moved m;
+        m.i = i;
+        m.parent = bi.parent;
+        m.X = joint_X<SPEND>(c, bi, q, &omc);
+        m.vJ = S_times(c, bi, qd);
+        m.aJ = S_times(c, bi, qdd);
+        if (SPEND && bi.type == FST_JOINT_REVOLUTE) *qd.spent(bi.vi) = omc;
+        return m;
+      },
+      [&](const Moved& m) {
+        const int i = m.i;
+        const Xf& X = m.X;
+        SV vi, ai;
+        if (m.parent < 0) {
+          vi = m.vJ;
+          ai = X_motion(X, a0) + m.aJ;
+        } else {
+          vi = X_motion(X, S.sv(m.parent, V_)) + m.vJ;
+          ai = X_motion(X, S.sv(m.parent, A_)) + m.aJ + crm(vi, m.vJ);
+        }
+        S.put(i, V_, vi);
+        S.put(i, A_, ai);
+        if (!LEAN) S.putX(i, X_, X);
+        if (!LEAN && !AHEAD) S.put(i, C_, force(i, vi, ai));
+        if (tape && act) {
+          float* p = tape + (int64_t)i * 30 * B + e;
+          const float r[24] = {X.R[0], X.R[1], X.R[2], X.R[3], X.R[4], X.R[5], X.R[6], X.R[7],
+                               X.R[8], X.t[0], X.t[1], X.t[2], vi.w.x, vi.w.y, vi.w.z, vi.v.x,
+                               vi.v.y, vi.v.z, ai.w.x, ai.w.y, ai.w.z, ai.v.x, ai.v.y, ai.v.z};
 #pragma unroll
-        for (int c2 = 0; c2 < 24; ++c2) p[(int64_t)c2 * B] = r[c2];
-      }
-    }
-    __syncthreads();
-  }
-  FST_UNROLL
-  for (int l = tp.depth() - 1; l >= 0; --l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      SV F = LEAN ? force(i, S.sv(i, V_), S.sv(i, A_)) : S.sv(i, C_);
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) F = F + S.sv(tp.child(ch), C_);
-      if (act && tau) ST_store(tp.C(i), bi, F, tau, B, e);
-      if (tau_col) ST_store(tp.C(i), bi, F, tau_col, kLaneEnvs, 0);
-      if (tape && act) {
-        float* p = tape + ((int64_t)i * 30 + 24) * B + e;
-        const float r[6] = {F.w.x, F.w.y, F.w.z, F.v.x, F.v.y, F.v.z};
+          for (int c2 = 0; c2 < 24; ++c2) p[(int64_t)c2 * B] = r[c2];
+        }
+      });
+  struct Own {
+    int i, ch, ch_end;
+    BodyI b;
+    SV F;
+    Xf X;
+  };
+  level_pass<true, AHEAD>(
+      tp,
+      [&](int i) {
+        Own o;
+        o.i = i;
+        o.b = tp.I(i);
+        o.ch = tp.child_begin(i);
+        o.ch_end = tp.child_begin(i + 1);
+        o.F = LEAN || AHEAD ? force(i, S.sv(i, V_), S.sv(i, A_)) : S.sv(i, C_);
+        if (o.b.parent >= 0) o.X = LEAN ? joint_X<SPEND>(tp.C(i), o.b, q, qd.p + o.b.vi * qd.ld) : S.X(i, X_);
+        return o;
+      },
+      [&](const Own& o) {
+        SV F = o.F;
+        for (int ch = o.ch; ch < o.ch_end; ++ch) F = F + S.sv(tp.child(ch), C_);
+        if (act && tau) ST_store(tp.C(o.i), o.b, F, tau, B, e);
+        if (tau_col) ST_store(tp.C(o.i), o.b, F, tau_col, kLaneEnvs, 0);
+        if (tape && act) {
+          float* p = tape + ((int64_t)o.i * 30 + 24) * B + e;
+          const float r[6] = {F.w.x, F.w.y, F.w.z, F.v.x, F.v.y, F.v.z};
 #pragma unroll
-        for (int c2 = 0; c2 < 6; ++c2) p[(int64_t)c2 * B] = r[c2];
-      }
-      if (bi.parent >= 0)
-        S.put(i, C_, XT_force(LEAN ? joint_X<SPEND>(tp.C(i), bi, q, qd.p + bi.vi * qd.ld) : S.X(i, X_), F));
-    }
-    __syncthreads();
-  }
+          for (int c2 = 0; c2 < 6; ++c2) p[(int64_t)c2 * B] = r[c2];
+        }
+        if (o.b.parent >= 0) S.put(o.i, C_, XT_force(o.X, F));
+      });
 }
 
 // ---- CRBA -----------------------------------------------------------------------
@@ -404,29 +472,41 @@ __device__ __forceinline__ Xf joint_X_rows(const BodyC& c, const BodyI& bi, cons
 // its parent lives in a slot of R (BodyC::slot) until the parent has added it;
 // the root keeps its own I^c in its slot for a free base's 6 x 6 block. q is read from global memory,
 // not staged. Same arithmetic, in the same order, as crba_level.
-template <bool PACKED = false, class TP, class XF>
+template <bool PACKED = false, bool AHEAD = true, class TP, class XF>
 __device__ __forceinline__ void crba_level_lean(const TP& tp, const XF& X_of, int nv,
                                                 const LaneState& S, const LaneState& R,
                                                 float* __restrict__ M, int64_t B, int64_t e, bool act) {
   const int W = n_warps(), w = warp_id();
   enum { X_ = 0, F_ = 12 };
   if (tp.depth() > 0) m_clear_tile(M, PACKED ? (int64_t)nv * (nv + 1) / 2 : (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
-  FST_UNROLL
-  for (int l = tp.depth() - 1; l >= 0; --l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const int slot = tp.C(i).slot;
-      const Xf X = X_of(tp.C(i), bi);
-      In10 Ic = in_load(tp.theta(i));
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch)
-        in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
-      S.putX(i, X_, X);
-      if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) S.put(i, F_, in_mul(Ic, S_of(tp.C(i))));
-      R.putin(slot, 0, bi.parent >= 0 ? in_to_parent(X, Ic) : Ic);
-    }
-    __syncthreads();
-  }
+  struct Own {
+    int i, type, parent, slot, ch, ch_end;
+    Xf X;
+    In10 I;
+  };
+  level_pass<true, AHEAD>(
+      tp,
+      [&](int i) {
+        const BodyI bi = tp.I(i);
+        Own o;
+        o.i = i;
+        o.type = bi.type;
+        o.parent = bi.parent;
+        o.slot = tp.C(i).slot;
+        o.ch = tp.child_begin(i);
+        o.ch_end = tp.child_begin(i + 1);
+        o.X = X_of(tp.C(i), bi);
+        o.I = in_load(tp.theta(i));
+        S.putX(i, X_, o.X);
+        return o;
+      },
+      [&](const Own& o) {
+        In10 Ic = o.I;
+        for (int ch = o.ch; ch < o.ch_end; ++ch) in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
+        if (o.type == FST_JOINT_REVOLUTE || o.type == FST_JOINT_PRISMATIC)
+          S.put(o.i, F_, in_mul(Ic, S_of(tp.C(o.i))));
+        R.putin(o.slot, 0, o.parent >= 0 ? in_to_parent(o.X, Ic) : Ic);
+      });
   if (!act) return;
   const MOut<PACKED> Me{M + e, nv, B};
   // deepest bodies, and so longest walks, first: the warps end together
@@ -585,7 +665,7 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
 // chain of levels, and stay in the rows of q and the state; 1 / D and u move
 // to the rows of qd and tau once pass 2 has read them (B = 4096: quadruped
 // 11.0 -> 10.3 us, arm7 13.8 -> 12.6; humanoid B = 65536 93.2 -> 91.6).
-template <bool SPEND = false, class TP>
+template <bool SPEND = false, bool AHEAD = false, class TP>
 __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q, const Col& qd, const Col& tau,
                                                const LaneState& S, const LaneState& R,
                                                float* __restrict__ qdd, int64_t B, int64_t e, bool act,
@@ -605,102 +685,135 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
   }
   auto X_of = [&](int i, const BodyI& bi) { return joint_X<SPEND>(tp.C(i), bi, q, S.at(i, OMC_)); };
   // 1. root to leaf: velocities and bias accelerations
-  FST_UNROLL
-  for (int l = 0; l < tp.depth(); ++l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyC& c = tp.C(i);
-      const BodyI bi = tp.I(i);
-      const SV vJ = S_times(c, bi, qd);
-      SV vi, ci;
-      if (bi.parent < 0) {
-        vi = vJ;
-        ci = sv_zero();
-      } else {
-        vi = X_motion(X_of(i, bi), S.sv(bi.parent, VU_)) + vJ;
-        ci = crm(vi, vJ);
-      }
-      S.put(i, VU_, vi);
-      S.put(i, C_, ci);
-    }
-    __syncthreads();
-  }
+  struct Moved {
+    int i, parent;
+    Xf X;
+    SV vJ;
+  };
+  level_pass<false, AHEAD>(
+      tp,
+      [&](int i) {
+        const BodyI bi = tp.I(i);
+        Moved m;
+        m.i = i;
+        m.parent = bi.parent;
+        m.vJ = S_times(tp.C(i), bi, qd);
+        if (bi.parent >= 0) m.X = X_of(i, bi);
+        return m;
+      },
+      [&](const Moved& m) {
+        SV vi = m.vJ, ci = sv_zero();
+        if (m.parent >= 0) {
+          vi = X_motion(m.X, S.sv(m.parent, VU_)) + m.vJ;
+          ci = crm(vi, m.vJ);
+        }
+        S.put(m.i, VU_, vi);
+        S.put(m.i, C_, ci);
+      });
   // 2. leaf to root: articulated inertias
-  FST_UNROLL
-  for (int l = tp.depth() - 1; l >= 0; --l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const int slot = tp.C(i).slot;
-      const In10 I = in_load(tp.theta(i));
-      const SV vi = S.sv(i, VU_);
-      Sym6 IA = sym6_from_in(I);
-      SV pA = crf(vi, in_mul(I, vi));
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
-        const int cs = tp.C(tp.child(ch)).slot;
-        sym6_add(IA, R.sym(cs, RI_));
-        pA = pA + R.sv(cs, RP_);
-      }
-      if (bi.type == FST_JOINT_FREE) {
-        R.putsym(slot, RI_, IA);
-        R.put(slot, RP_, pA);
-        continue;
-      }
-      Sym6 Ia = IA;
-      SV pa = pA;
-      if (bi.type != FST_JOINT_FIXED) {
-        const SV Sv = S_of(tp.C(i));
-        const SV Ui = sym6_mul(IA, Sv);
-        const float iD = 1.0f / dot(Sv, Ui);
-        const float ui = tau[bi.vi] - dot(Sv, pA);
-        S.put(i, VU_, Ui);
-        *(SPEND ? qd.spent(bi.vi) : S.at(i, ID_)) = iD;
-        *(SPEND ? tau.spent(bi.vi) : S.at(i, u_)) = ui;
-        if (bi.parent < 0) continue;
-        sym6_rank1_sub(Ia, Ui, iD);
-        pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, S.sv(i, C_)));
-      } else {
-        if (bi.parent < 0) continue;
-        pa = pa + sym6_mul(Ia, S.sv(i, C_));
-      }
-      const Xf X = X_of(i, bi);
-      R.putsym(slot, RI_, sym6_to_parent(X, Ia));
-      R.put(slot, RP_, XT_force(X, pa));
-    }
-    __syncthreads();
-  }
+  struct Own {
+    int i, slot, ch, ch_end, ch_slot;
+    BodyI b;
+    In10 I;
+    SV p;
+    Xf X;
+  };
+  level_pass<true, AHEAD>(
+      tp,
+      [&](int i) {
+        const BodyI bi = tp.I(i);
+        Own o;
+        o.i = i;
+        o.b = bi;
+        o.slot = tp.C(i).slot;
+        o.ch = tp.child_begin(i);
+        o.ch_end = tp.child_begin(i + 1);
+        o.ch_slot = AHEAD && o.ch < o.ch_end ? tp.C(tp.child(o.ch)).slot : 0;
+        o.I = in_load(tp.theta(i));
+        const SV vi = S.sv(i, VU_);
+        o.p = crf(vi, in_mul(o.I, vi));
+        if (AHEAD && bi.parent >= 0) o.X = X_of(i, bi);
+        return o;
+      },
+      [&](const Own& o) {
+        Sym6 IA = sym6_from_in(o.I);
+        SV pA = o.p;
+        for (int ch = o.ch; ch < o.ch_end; ++ch) {
+          const int cs = AHEAD && ch == o.ch ? o.ch_slot : tp.C(tp.child(ch)).slot;
+          sym6_add(IA, R.sym(cs, RI_));
+          pA = pA + R.sv(cs, RP_);
+        }
+        if (o.b.type == FST_JOINT_FREE) {
+          R.putsym(o.slot, RI_, IA);
+          R.put(o.slot, RP_, pA);
+          return;
+        }
+        Sym6 Ia = IA;
+        SV pa = pA;
+        if (o.b.type != FST_JOINT_FIXED) {
+          const SV Sv = S_of(tp.C(o.i));
+          const SV Ui = sym6_mul(IA, Sv);
+          const float iD = 1.0f / dot(Sv, Ui);
+          const float ui = tau[o.b.vi] - dot(Sv, pA);
+          S.put(o.i, VU_, Ui);
+          *(SPEND ? qd.spent(o.b.vi) : S.at(o.i, ID_)) = iD;
+          *(SPEND ? tau.spent(o.b.vi) : S.at(o.i, u_)) = ui;
+          if (o.b.parent < 0) return;
+          sym6_rank1_sub(Ia, Ui, iD);
+          pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, S.sv(o.i, C_)));
+        } else {
+          if (o.b.parent < 0) return;
+          pa = pa + sym6_mul(Ia, S.sv(o.i, C_));
+        }
+        const Xf X = AHEAD ? o.X : X_of(o.i, o.b);
+        R.putsym(o.slot, RI_, sym6_to_parent(X, Ia));
+        R.put(o.slot, RP_, XT_force(X, pa));
+      });
   // 3. root to leaf: accelerations (each body reads its U before it
   //    overwrites VU with its acceleration)
-  FST_UNROLL
-  for (int l = 0; l < tp.depth(); ++l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const SV ap = bi.parent < 0 ? a0 : S.sv(bi.parent, VU_);
-      SV ai = X_motion(X_of(i, bi), ap) + S.sv(i, C_);
-      if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
-        const float ui = SPEND ? tau[bi.vi] : *S.at(i, u_), iD = SPEND ? qd[bi.vi] : *S.at(i, ID_);
-        const float qi = (ui - dot(S.sv(i, VU_), ai)) * iD;
-        if (act && qdd) qdd[(int64_t)bi.vi * B + e] = qi;
-        if (qdd_col) qdd_col[bi.vi << 5] = qi;
-        ai = sv_fma(qi, S_of(tp.C(i)), ai);
-      } else if (bi.type == FST_JOINT_FREE) {
-        const int slot = tp.C(i).slot;
-        const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};
-        const SV anew = sym6_solve(R.sym(slot, RI_), tf - R.sv(slot, RP_));
-        const SV x = anew - ai;
-        const float xo[6] = {x.v.x, x.v.y, x.v.z, x.w.x, x.w.y, x.w.z};
-#pragma unroll
-        for (int r = 0; r < 6; ++r) {
-          if (act && qdd) qdd[(int64_t)(bi.vi + r) * B + e] = xo[r];
-          if (qdd_col) qdd_col[(bi.vi + r) << 5] = xo[r];
+  struct Joint {
+    int i;
+    BodyI b;
+    Xf X;
+    SV c, U;
+  };
+  level_pass<false, AHEAD>(
+      tp,
+      [&](int i) {
+        Joint m;
+        m.i = i;
+        m.b = tp.I(i);
+        if (AHEAD) {
+          m.X = X_of(i, m.b);
+          m.c = S.sv(i, C_);
+          m.U = S.sv(i, VU_);
         }
-        ai = anew;
-      }
-      S.put(i, VU_, ai);
-    }
-    __syncthreads();
-  }
+        return m;
+      },
+      [&](const Joint& m) {
+        const SV ap = m.b.parent < 0 ? a0 : S.sv(m.b.parent, VU_);
+        SV ai = X_motion(AHEAD ? m.X : X_of(m.i, m.b), ap) + (AHEAD ? m.c : S.sv(m.i, C_));
+        if (m.b.type == FST_JOINT_REVOLUTE || m.b.type == FST_JOINT_PRISMATIC) {
+          const float u = SPEND ? tau[m.b.vi] : *S.at(m.i, u_), iD = SPEND ? qd[m.b.vi] : *S.at(m.i, ID_);
+          const float qi = (u - dot(AHEAD ? m.U : S.sv(m.i, VU_), ai)) * iD;
+          if (act && qdd) qdd[(int64_t)m.b.vi * B + e] = qi;
+          if (qdd_col) qdd_col[m.b.vi << 5] = qi;
+          ai = sv_fma(qi, S_of(tp.C(m.i)), ai);
+        } else if (m.b.type == FST_JOINT_FREE) {
+          const int slot = tp.C(m.i).slot, vi = m.b.vi;
+          const SV tf = SV{f3{tau[vi + 3], tau[vi + 4], tau[vi + 5]}, f3{tau[vi], tau[vi + 1], tau[vi + 2]}};
+          const SV anew = sym6_solve(R.sym(slot, RI_), tf - R.sv(slot, RP_));
+          const SV x = anew - ai;
+          const float xo[6] = {x.v.x, x.v.y, x.v.z, x.w.x, x.w.y, x.w.z};
+#pragma unroll
+          for (int r = 0; r < 6; ++r) {
+            if (act && qdd) qdd[(int64_t)(vi + r) * B + e] = xo[r];
+            if (qdd_col) qdd_col[(vi + r) << 5] = xo[r];
+          }
+          ai = anew;
+        }
+        S.put(m.i, VU_, ai);
+      });
 }
 
 }  // namespace fst

@@ -9,8 +9,8 @@
 // the largest (tree, operator) pair, all in their lean forms: 65 KB for the
 // 23-body tree, so three blocks an SM. Bound by the latency of the longest
 // items (that tree's ABA, 11 levels three times over). Five trees, 7936
-// environments: 70 us in the generic form, 22 here; a whole call 70.7 -> 31.8
-// us, of which the host's part is now the larger one.
+// environments: 70 us in the generic form, 19 here; a whole call 70.7 -> 30 us,
+// which is the host's part.
 #include "launch.h"
 #include "level.cuh"
 #include "multi.h"
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
   float* const state = tile + rows * kLaneEnvs;
   switch (op) {
     case ROLE_ABA:
-      aba_level_lean<true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
+      aba_level_lean<true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kAbaLeanBodyFloats},
                      LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, io.qdd_out, B, e,
                      act);
       break;
@@ -57,10 +57,10 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
                       LaneState{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats}, io.M, B, e, act);
       break;
     case ROLE_RNEA:
-      rnea_level<true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B, e, act);
+      rnea_level<true, true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B, e, act);
       break;
     default:
-      fk_level(sm, cq, LaneState{state, kFkState}, io.poses, B, e, act);
+      fk_level<true>(sm, cq, LaneState{state, kFkState}, io.poses, B, e, act);
       break;
   }
 }

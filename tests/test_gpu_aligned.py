@@ -171,3 +171,31 @@ def test_lean_forms_give_the_same_bits(torch_cuda, name, B):
         torch.cuda.synchronize()
         for k in few:
             assert torch.equal(full[k][..., lo:hi], few[k]), (name, B, k)
+
+
+@pytest.mark.parametrize("name,B,specialize", [
+    ("chain7", 9728, False), ("chain7", 9729, False),      # RNEA leaves the tiles before its adjoint does
+    ("chain12", 4865, False), ("chain30", 40, False), ("wide36", 40, False),  # wide36: only the adjoint does not fit
+    ("quadruped11", 8191, True), ("quadruped11", 8192, True),
+])
+def test_fused_evaluation_equals_separate_calls_at_the_rules_edges(torch_cuda, name, B, specialize):
+    torch = torch_cuda
+    from paper_2605_31481_gb300 import api
+    tree = {"quadruped11": w.spined_quadruped, "wide36": lambda: w.random_tree([-1] + [i // 3 for i in range(35)],
+                                                                          [w.REVOLUTE] * 36, 6),
+            }.get(name, lambda: w.chain(int(name[5:]), seed=5))()
+    m = api.Model(tree, specialize=specialize)
+    _, _, _, x = _inputs(torch, tree, B, 83)
+    q, qd, qdd, tau = (x[k] for k in ("q", "qd", "qdd", "tau"))
+    links = [tree.n_bodies - 1]
+    want = {"poses": api.fk(m, q), "J": api.jacobian(m, q, links), "tau": api.rnea(m, q, qd, qdd),
+            "M": api.crba(m, q), "qdd": api.aba(m, q, qd, tau)}
+    for bar in ("tau", x["bar"]):
+        res = api.eval(m, q, qd, qdd, tau, fk=True, links=links, rnea=True, crba=True, aba=True, tau_bar=bar,
+                       q_bar=True, qd_bar=True, qdd_bar=True)
+        vjp = api.rnea_vjp(m, q, qd, qdd, want["tau"] if isinstance(bar, str) else bar, theta_bar=False)
+        torch.cuda.synchronize()
+        for k, v in want.items():
+            assert torch.equal(res[k], v), (name, B, k)
+        for k in ("q", "qd", "qdd"):
+            assert torch.equal(res[k + "_bar"], vjp[k]), (name, B, k + "_bar")
