@@ -165,8 +165,10 @@ __global__ void __launch_bounds__(512) rnea_vjp_aligned_kernel(ModelView mv, int
 // the model: two tiles of the humanoid an SM instead of one, four of the
 // quadruped instead of two. Adjoint with the parameter gradient, B = 65536:
 // humanoid 320 us in one thread per environment, 161 in rnea_vjp_aligned_kernel,
-// 127 here; quadruped 80 -> 60. A short chain gains nothing (arm7 B = 16384 15.4
-// against 17.2), so trees of up to 8 bodies keep the other form.
+// 123 here (133 before a body's own terms and its sums for theta's gradient were
+// formed ahead of its level; 16384 39.1 -> 36.2); quadruped 80 -> 60. A short
+// chain gains nothing (arm7 B = 16384 15.4 against 17.2), so trees of up to 8
+// bodies keep the other form.
 __global__ void __launch_bounds__(512) rnea_vjp_lean_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                             const float* __restrict__ qd,
                                                             const float* __restrict__ qdd,

@@ -399,7 +399,6 @@ __device__ __forceinline__ void rnea_derivs_aligned(const SmemModel& tp, SV a0, 
 enum VjpMode {
   VJP_GIVEN = 0,  // staged in tb
   VJP_LOSS,       // tb holds measured torques; the cotangent is 2 (tau - tb), the loss their squared difference
-  VJP_TAU         // the cotangent is tau (warpbody.cuh)
 };
 
 struct VjpAligned {
@@ -734,130 +733,160 @@ __device__ __forceinline__ void rnea_vjp_lean(const SmemModel& tp, SV a0, const 
     }
   }
   tile_barrier();
-  for (int l = 0; l < tp.depth(); ++l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const Xf X = S.X(i, R_);
-      if (bi.type == FST_JOINT_FREE) {  // the root frame is this body's own; v and w are in place
-        const float Id[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
-        S.put_n(i, R_, Id, 9);
-        S.put(i, A_, S.sv(i, A_) + SV{f3{0.f, 0.f, 0.f}, RTmul(X.R, a0.v)});
-        continue;
-      }
-      SV vl = sv_zero(), al = a0, wl = sv_zero();
-      float R[9];
-      if (bi.parent < 0) {
-#pragma unroll
-        for (int c = 0; c < 9; ++c) R[c] = X.R[c];
-      } else {
-        float Rp[9], rr[3];
-        S.get_n(bi.parent, R_, Rp, 9);
-        const float zero[3] = {0.f, 0.f, 0.f};
-        compose(Rp, zero, X, R, rr);
-        const f3 r = f3{rr[0], rr[1], rr[2]};
-        S.put_n(i, RR, rr, 3);
-        S.put_n(i, R_, R, 9);
-        vl = shift_motion(S.sv(bi.parent, V_), r);
-        al = shift_motion(S.sv(bi.parent, A_), r);
-        wl = shift_motion(S.sv(bi.parent, W_), r);
-      }
-      if (one_dof(bi)) {
-        const SV psi = psi_of(tp.C(i), R);
-        S.put(i, PSI, psi);
-        const float xd = *S.at(i, V_);
-        const SV psd = crm(vl, psi);
-        al = sv_fma(*S.at(i, A_), psi, sv_fma(xd, psd, al));
-        vl = sv_fma(xd, psi, vl);
-        wl = sv_fma(*S.at(i, W_), psi, wl);
-      }
-      S.put(i, V_, vl);
-      S.put(i, A_, al);
-      S.put(i, W_, wl);
-    }
-    tile_barrier();
-  }
-  if (o.thbar) {
-    for (int i = w; i < n; i += W) {
-      float R[9];
-      S.get_n(i, R_, R, 9);
-      const SV v = S.sv(i, V_), wv = S.sv(i, W_);
-      float g[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-      inertia_contract(wv, S.sv(i, A_), g);
-      inertia_contract(crm(wv, v), v, g);
-      inertia_grad_to_body(R, g);
-#pragma unroll
-      for (int c = 0; c < 10; ++c) g[c] = act ? o.sign * g[c] : 0.f;
-      warp_sum10_store(g, o.thbar + 10 * i);
-    }
-    tile_barrier();
-  }
-  if (!o.qbar && !o.qdbar && !o.qddbar) return;  // uniform over the launch
-  for (int l = tp.depth() - 1; l >= 0; --l) {
-    FST_FOR_MY_BODIES(tp, l, k) {
-      const int i = tp.level_body(k);
-      const BodyI bi = tp.I(i);
-      const SV v = S.sv(i, V_), wv = S.sv(i, W_);
-      float R[9];
-      S.get_n(i, R_, R, 9);
-      const In10 I = in_rotate(R, in_load(tp.theta(i)));
-      const SV hv = in_mul(I, v);
-      SV f = in_mul(I, S.sv(i, A_)) + crf(v, hv);
-      SV A = in_mul(I, wv);
-      f3 H = 2.f * (second_moment_mul(I, cross(v.w, wv.w)) + (dot(I.h, v.v) * wv.w - dot(v.v, wv.w) * I.h) -
-                    cross(wv.v, hv.v));
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
-        const int c = tp.child(ch);
-        const float* h = S.at(c, W_);
-        A = A + S.sv(c, A_);
-        f = f + S.sv(c, V_);
-        H = H + f3{h[0], h[32], h[64]};
-      }
-      const float* t = S.at(i, RR);
-      const f3 r = f3{t[0], t[32], t[64]};
-      if (act && bi.type == FST_JOINT_FREE) {
-        const SV y = crf(v, A);
-        const f3 g1 = RTmul(tp.C(i).R0, a0.v);
-        const float G[9] = {g1.x * A.v.x, g1.x * A.v.y, g1.x * A.v.z, g1.y * A.v.x, g1.y * A.v.y,
-                            g1.y * A.v.z, g1.z * A.v.x, g1.z * A.v.y, g1.z * A.v.z};
-        const float* qq = q + (int64_t)(bi.qi + 3) * B + e;
-        float gq[4];
-        quat_grad(__ldg(qq), __ldg(qq + B), __ldg(qq + 2 * B), __ldg(qq + 3 * B), G, gq);
-        const float qo[7] = {0.f, 0.f, 0.f, gq[0], gq[1], gq[2], gq[3]};
-        const float vo[6] = {-y.v.x, -y.v.y, -y.v.z, H.x - y.w.x, H.y - y.w.y, H.z - y.w.z};
-        const float ao[6] = {A.v.x, A.v.y, A.v.z, A.w.x, A.w.y, A.w.z};
-#pragma unroll
-        for (int c = 0; c < 7; ++c) store_if(o.qbar, bi.qi + c, B, e, o.sign * qo[c], true);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          store_if(o.qdbar, bi.vi + c, B, e, o.sign * vo[c], true);
-          store_if(o.qddbar, bi.vi + c, B, e, o.sign * ao[c], true);
+  auto barrier = [] { tile_barrier(); };
+  struct Joint {
+    int i;
+    BodyI b;
+    Xf X;
+  };
+  level_pass<false, true>(
+      tp,
+      [&](int i) { return Joint{i, tp.I(i), S.X(i, R_)}; },
+      [&](const Joint& j) {
+        const int i = j.i;
+        const BodyI& bi = j.b;
+        if (bi.type == FST_JOINT_FREE) {  // the root frame is this body's own; v and w are in place
+          const float Id[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f};
+          S.put_n(i, R_, Id, 9);
+          S.put(i, A_, S.sv(i, A_) + SV{f3{0.f, 0.f, 0.f}, RTmul(j.X.R, a0.v)});
+          return;
         }
-      } else if (act && one_dof(bi)) {
         SV vl = sv_zero(), al = a0, wl = sv_zero();
-        if (bi.parent >= 0) {
+        float R[9];
+        if (bi.parent < 0) {
+#pragma unroll
+          for (int c = 0; c < 9; ++c) R[c] = j.X.R[c];
+        } else {
+          float Rp[9], rr[3];
+          S.get_n(bi.parent, R_, Rp, 9);
+          const float zero[3] = {0.f, 0.f, 0.f};
+          compose(Rp, zero, j.X, R, rr);
+          const f3 r = f3{rr[0], rr[1], rr[2]};
+          S.put_n(i, RR, rr, 3);
+          S.put_n(i, R_, R, 9);
           vl = shift_motion(S.sv(bi.parent, V_), r);
           al = shift_motion(S.sv(bi.parent, A_), r);
           wl = shift_motion(S.sv(bi.parent, W_), r);
         }
-        const SV psi = S.sv(i, PSI);
-        const SV psd = crm(vl, psi);
-        const SV psdd = crm(al, psi) + crm(vl, psd);
-        store_if(o.qbar, bi.qi, B, e, o.sign * (dot(crm(wl, psi), f) + dot(psdd, A) + dot(psd.w, H)), true);
-        store_if(o.qdbar, bi.vi, B, e, o.sign * fmaf(2.f, dot(psd, A), dot(psi.w, H)), true);
-        store_if(o.qddbar, bi.vi, B, e, o.sign * dot(psi, A), true);
-      }
-      if (bi.parent >= 0) {
-        S.put(i, V_, shift_force(f, r));
-        S.put(i, A_, shift_force(A, r));
-        float* h = S.at(i, W_);
-        h[0] = H.x;
-        h[32] = H.y;
-        h[64] = H.z;
-      }
+        if (one_dof(bi)) {
+          const SV psi = psi_of(tp.C(i), R);
+          S.put(i, PSI, psi);
+          const float xd = *S.at(i, V_);
+          const SV psd = crm(vl, psi);
+          al = sv_fma(*S.at(i, A_), psi, sv_fma(xd, psd, al));
+          vl = sv_fma(xd, psi, vl);
+          wl = sv_fma(*S.at(i, W_), psi, wl);
+        }
+        S.put(i, V_, vl);
+        S.put(i, A_, al);
+        S.put(i, W_, wl);
+      },
+      barrier);
+  auto contract = [&](int i, const float* R, SV v, SV acc, SV wv) {
+    float g[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    inertia_contract(wv, acc, g);
+    inertia_contract(crm(wv, v), v, g);
+    inertia_grad_to_body(R, g);
+#pragma unroll
+    for (int c = 0; c < 10; ++c) g[c] = act ? o.sign * g[c] : 0.f;
+    warp_sum10_store(g, o.thbar + 10 * i);
+  };
+  if (!o.qbar && !o.qdbar && !o.qddbar) {  // uniform over the launch
+    for (int i = w; o.thbar && i < n; i += W) {
+      float R[9];
+      S.get_n(i, R_, R, 9);
+      contract(i, R, S.sv(i, V_), S.sv(i, A_), S.sv(i, W_));
     }
-    tile_barrier();
+    return;
   }
+  // A body's own force and functionals, its part of theta's gradient and what
+  // its outputs take from its parent's velocities are formed before its level:
+  // only the sums over the children and the outputs wait for it.
+  struct Own {
+    int i, ch, ch_end;
+    BodyI b;
+    SV f, A, psi, psd, psdd, cwp;
+    f3 H, r;
+  };
+  level_pass<true, true>(
+      tp,
+      [&](int i) {
+        Own s;
+        s.i = i;
+        s.b = tp.I(i);
+        s.ch = tp.child_begin(i);
+        s.ch_end = tp.child_begin(i + 1);
+        const SV v = S.sv(i, V_), wv = S.sv(i, W_);
+        float R[9];
+        S.get_n(i, R_, R, 9);
+        const In10 I = in_rotate(R, in_load(tp.theta(i)));
+        const SV hv = in_mul(I, v), acc = S.sv(i, A_);
+        if (o.thbar) contract(i, R, v, acc, wv);
+        s.f = in_mul(I, acc) + crf(v, hv);
+        s.A = in_mul(I, wv);
+        s.H = 2.f * (second_moment_mul(I, cross(v.w, wv.w)) + (dot(I.h, v.v) * wv.w - dot(v.v, wv.w) * I.h) -
+                     cross(wv.v, hv.v));
+        const float* t = S.at(i, RR);
+        s.r = f3{t[0], t[32], t[64]};
+        if (one_dof(s.b)) {
+          SV vl = sv_zero(), al = a0, wl = sv_zero();
+          if (s.b.parent >= 0) {
+            vl = shift_motion(S.sv(s.b.parent, V_), s.r);
+            al = shift_motion(S.sv(s.b.parent, A_), s.r);
+            wl = shift_motion(S.sv(s.b.parent, W_), s.r);
+          }
+          s.psi = S.sv(i, PSI);
+          s.psd = crm(vl, s.psi);
+          s.psdd = crm(al, s.psi) + crm(vl, s.psd);
+          s.cwp = crm(wl, s.psi);
+        }
+        return s;
+      },
+      [&](const Own& s) {
+        const int i = s.i;
+        const BodyI& bi = s.b;
+        SV f = s.f, A = s.A;
+        f3 H = s.H;
+        for (int ch = s.ch; ch < s.ch_end; ++ch) {
+          const int c = tp.child(ch);
+          const float* h = S.at(c, W_);
+          A = A + S.sv(c, A_);
+          f = f + S.sv(c, V_);
+          H = H + f3{h[0], h[32], h[64]};
+        }
+        if (act && bi.type == FST_JOINT_FREE) {
+          const SV y = crf(S.sv(i, V_), A);
+          const f3 g1 = RTmul(tp.C(i).R0, a0.v);
+          const float G[9] = {g1.x * A.v.x, g1.x * A.v.y, g1.x * A.v.z, g1.y * A.v.x, g1.y * A.v.y,
+                              g1.y * A.v.z, g1.z * A.v.x, g1.z * A.v.y, g1.z * A.v.z};
+          const float* qq = q + (int64_t)(bi.qi + 3) * B + e;
+          float gq[4];
+          quat_grad(__ldg(qq), __ldg(qq + B), __ldg(qq + 2 * B), __ldg(qq + 3 * B), G, gq);
+          const float qo[7] = {0.f, 0.f, 0.f, gq[0], gq[1], gq[2], gq[3]};
+          const float vo[6] = {-y.v.x, -y.v.y, -y.v.z, H.x - y.w.x, H.y - y.w.y, H.z - y.w.z};
+          const float ao[6] = {A.v.x, A.v.y, A.v.z, A.w.x, A.w.y, A.w.z};
+#pragma unroll
+          for (int c = 0; c < 7; ++c) store_if(o.qbar, bi.qi + c, B, e, o.sign * qo[c], true);
+#pragma unroll
+          for (int c = 0; c < 6; ++c) {
+            store_if(o.qdbar, bi.vi + c, B, e, o.sign * vo[c], true);
+            store_if(o.qddbar, bi.vi + c, B, e, o.sign * ao[c], true);
+          }
+        } else if (act && one_dof(bi)) {
+          store_if(o.qbar, bi.qi, B, e, o.sign * (dot(s.cwp, f) + dot(s.psdd, A) + dot(s.psd.w, H)), true);
+          store_if(o.qdbar, bi.vi, B, e, o.sign * fmaf(2.f, dot(s.psd, A), dot(s.psi.w, H)), true);
+          store_if(o.qddbar, bi.vi, B, e, o.sign * dot(s.psi, A), true);
+        }
+        if (bi.parent >= 0) {
+          S.put(i, V_, shift_force(f, s.r));
+          S.put(i, A_, shift_force(A, s.r));
+          float* h = S.at(i, W_);
+          h[0] = H.x;
+          h[32] = H.y;
+          h[64] = H.z;
+        }
+      },
+      barrier);
 }
 
 // ---- the adjoint of forward kinematics -----------------------------------------
