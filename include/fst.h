@@ -155,7 +155,9 @@ FST_API fst_status fst_model_specialize(fst_model* model, uint32_t kinds);
 /* Launch configuration of the selected kinds (FST_SPEC_* mask, 0 = all) on
  * this model: threads per block (32, 64, 128 or 256; 0 = built-in heuristic)
  * and which kernel variant runs:
- *   AUTO        the specialised kernel when compiled, else the generic one;
+ *   AUTO        the built-in choice by operator, tree and B: tiles of 32
+ *               environments whose warps share the bodies (below), the
+ *               specialised kernel when compiled, or the generic one;
  *   GENERIC     one environment per thread, tree from shared memory;
  *   SPECIALIZED one environment per thread, kernel compiled for this tree;
  *   LEVEL       level-parallel (paper Sec. 3.3 on warps): 32 environments per
@@ -225,10 +227,11 @@ FST_API fst_status fst_model_specialize(fst_model* model, uint32_t kinds);
  * ABA only; "all kinds" means those two). ABA: per body 14 floats per
  * environment (v, then U, then a; c; 1/D; u) instead of 59; each body's
  * contribution to its parent (X^T I^a X, X^T p^a: 27 floats) sits in a
- * ring of two levels' slots only until the parent reads it; the joint
- * transforms are recomputed in passes 2 and 3. CRBA: per body X and
- * F = I^c S (18 floats) instead of 32, the composite-inertia contributions
- * in the same kind of ring, q read from global memory instead of staged.
+ * slot only until the parent reads it, and the parent's takes the slot of
+ * its first child; the joint transforms are recomputed in passes 2 and 3.
+ * CRBA: per body X and F = I^c S (18 floats) instead of 32, the
+ * composite-inertia contributions in the same kind of slots (q is read from
+ * global memory where its staged rows do not fit).
  * Same recursions (Sec. 3.3 level-parallel form); results agree with
  * FST_VARIANT_LEVEL within FP32 rounding. Where even the lean tile does not
  * fit in shared memory, the generic kernel runs. */
@@ -371,7 +374,8 @@ typedef struct fst_eval_io {
 FST_API fst_status fst_packed_layout(const fst_model* model, const int32_t* links, int32_t n_links,
                                      int32_t* cols, int32_t* j_rows, int32_t* m_rows);
 
-/* Every requested operator of one batch in ONE launch. The paper computes
+/* Every requested operator of one batch in one launch (two or three where the
+ * default variant's rules part the operators, see below). The paper computes
  * only the kinematic tiers a query needs (Sec. 3.1); here the operators
  * whose outputs are NULL are skipped and the others run side by side on the
  * GPU, one group of thread blocks per operator. Results are bit-identical
@@ -382,12 +386,18 @@ FST_API fst_status fst_packed_layout(const fst_model* model, const int32_t* link
  * Jacobians and inverse dynamics, here with RNEA's gradient). With
  * FST_EVAL_ONE_SWEEP and the RNEA operator requested, poses and J are also
  * computed by those blocks from the same joint transforms (paper Eq. 4-5
- * evaluated once per joint) instead of by blocks of their own. Both run the
- * one-environment-per-thread fused kernel: the one specialised for the tree
- * when it is compiled (FST_SPEC_EVAL) and the eval kind is not set to
- * FST_VARIANT_GENERIC, else the generic one. FST_EVAL_PACKED writes M and J
- * in the layouts of fst_packed_layout (M then has nv*(nv+1)/2 rows), on the
- * same kernels; values are bit-identical to the full layouts' entries. */
+ * evaluated once per joint) instead of by blocks of their own. Where the
+ * operators run as tiles (FST_VARIANT_AUTO) the kinematics keep blocks of
+ * their own in the same launch (the flag then changes nothing: one sweep would
+ * lengthen the tile's chain); otherwise both run the one-environment-per-thread
+ * fused kernel: the one specialised for the tree when it is compiled
+ * (FST_SPEC_EVAL) and the eval kind is not set to FST_VARIANT_GENERIC, else
+ * the generic one. FST_EVAL_PACKED writes M and J in the layouts of
+ * fst_packed_layout (M then has nv*(nv+1)/2 rows), on the same kernels; values
+ * are bit-identical to the full layouts' entries. With the default variant the
+ * operators that run as tiles are one launch and those that do not another,
+ * and an adjoint whose own call would take another form than RNEA's follows
+ * as that call, so that every output is its operator's own call's. */
 FST_API fst_status fst_eval(const fst_model* model, int64_t B, const fst_eval_io* io,
                             const float* theta, void* stream);
 
@@ -577,23 +587,26 @@ FST_API fst_status fst_multi_create(const fst_model* const* models, int32_t n_mo
 FST_API fst_status fst_multi_destroy(fst_multi* multi);
 
 /* Evaluates the requested operators (FK Sec. 3.1, RNEA Sec. 3.3, CRBA
- * Sec. 3.5, ABA Sec. 4.1) of every tree in one persistent launch
- * (plus a 4-byte memset that resets the work counter; both are ordered on
- * `stream` and can be captured into a CUDA graph). io has n_models entries,
+ * Sec. 3.5, ABA Sec. 4.1) of every tree in one launch, which is ordered on
+ * `stream` and can be captured into a CUDA graph (the generic form is a
+ * persistent launch behind a 4-byte memset that resets its work counter). io has n_models entries,
  * in the order given to fst_multi_create. Overlapping calls on the same
  * group (unordered streams) race on its counter; create one group per
- * stream for that. Results are bit-identical to the per-tree generic calls
- * (with the default launch form; see fst_multi_set_launch). */
+ * stream for that. Results are bit-identical to the per-tree calls with their
+ * default variant and no specialised kernels (with the default launch form;
+ * see fst_multi_set_launch). */
 FST_API fst_status fst_multi_eval(fst_multi* multi, const fst_multi_io* io, void* stream);
 
 /* Launch form of a group's fst_multi_eval (not in the paper; a tuning knob).
- * FST_VARIANT_GENERIC (the default, block 64): one environment per thread,
- * items of `block` environments. FST_VARIANT_LEVEL: the level-parallel
+ * The default until this is called: tiles of 32 environments if every tree's
+ * own calls run as tiles at that batch size and its state fits in shared
+ * memory, else the generic form at block 64. FST_VARIANT_GENERIC: one
+ * environment per thread, items of `block` environments. FST_VARIANT_LEVEL: the level-parallel
  * bodies of paper Sec. 3.3, items of 32 environments with the block's
  * block/32 warps splitting each tree level, ABA in its lean form (results
  * then bit-identical to the per-tree calls at that block with
  * FST_VARIANT_LEVEL, and FST_VARIANT_LEVEL_LEAN for ABA); a group whose largest
- * tree's state does not fit in shared memory then returns
+ * tree's full level-parallel state does not fit in shared memory then returns
  * FST_ERR_INVALID_ARG from fst_multi_eval. block: 32, 64, 128 or 256. */
 FST_API fst_status fst_multi_set_launch(fst_multi* multi, int32_t block, int32_t variant);
 
