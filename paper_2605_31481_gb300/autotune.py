@@ -382,8 +382,11 @@ class StepPlan:
         for carveout in (-1, 100):
             api.set_smem_carveout(carveout)
             for mode in modes:
-                cfgs = {"hybrid": hybrid_cfgs, "split": hybrid_cfgs, "pinned": pinned_cfgs,
-                        "partitioned": part_cfgs}.get(
+                # one launch: the tuned variant, and the library's own choice, which
+                # the eval tuning does not time (quadruped11 B = 4096 17.1
+                # against 13.9 us, the best plan before it 16.0)
+                cfgs = {"fused": [f"{best_eval}|{best_aba}", f"auto/0|{best_aba}"], "hybrid": hybrid_cfgs,
+                        "split": hybrid_cfgs, "pinned": pinned_cfgs, "partitioned": part_cfgs}.get(
                     mode, [f"{best_eval}|{best_aba}"])
                 for ev in cfgs:
                     try:
@@ -591,9 +594,15 @@ class StepPlan:
     def describe(self):
         kinds = {k: f"{v['variant']}/{v['block']}" for k, v in self.tuned.items()}
         kinds["eval"], kinds["aba"] = self.eval_config.split("|")
+
+        tuned_eval = self.times.keys() - {k for k in self.times if k[0] != "fused" or k[3].startswith("auto/")}
+
+        def named(k):                        # the launch configurations are part of the plan's name
+            return k[0] in ("hybrid", "split", "pinned", "partitioned") or \
+                (k[0] == "fused" and k not in tuned_eval and bool(tuned_eval))
         return {"mode": self.mode, "carveout": self.carveout, "priorities": self.prio,
                 "fused_forked_first": self.alt and self.mode != "concurrent",
-                "us": {f"{k[0]}{'[' + k[3] + ']' if k[0] in ('hybrid', 'split', 'pinned', 'partitioned') else ''}"
+                "us": {f"{k[0]}{'[' + k[3] + ']' if named(k) else ''}"
                        f"{'' if k[1] < 0 else f'@{k[1]}%'}"
                        f"{('+prio' if k[0] == 'concurrent' else '+fusedfirst') if k[2] else ''}": None if v is None else round(v, 3)
                        for k, v in self.times.items()},
