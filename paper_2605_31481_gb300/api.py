@@ -555,7 +555,7 @@ def rnea_loss_grad(model: Model, q, qd, qdd, tau_meas, theta=None, *, q_bar=Fals
 # ---------------------------------------------------------------------------
 
 class MultiBatch:
-    """Several models evaluated in one persistent launch (fst_multi_eval)."""
+    """Several models evaluated in one launch (fst_multi_eval)."""
 
     def __init__(self, models):
         self.models = list(models)
@@ -565,8 +565,8 @@ class MultiBatch:
         self._h = h
 
     def set_launch(self, block=64, variant="generic"):
-        """Launch form of eval() (fst_multi_set_launch): "generic" (one
-        environment per thread) or "level" (level-parallel, 32 environments
+        """Launch form of eval() (fst_multi_set_launch), in place of the
+        library's own choice: "generic" (one environment per thread) or "level" (level-parallel, 32 environments
         per item), with `block` threads per block."""
         check(_ffi.lib().fst_multi_set_launch(self._h, int(block), _ffi.VARIANTS[variant]))
 
