@@ -287,9 +287,9 @@ __global__ void __launch_bounds__(256) eval_tile_kernel(ModelView mv, int64_t B,
       break;
     case ROLE_RNEA:
       if (!vjp || a.tau_out || (a.rnea_flags & EVAL_TBAR_IS_TAU))
-        rnea_level<LEAN, LEAN && !EXT, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState},
-                         a.tau_out, B, e, act,
-                         vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
+        rnea_level<LEAN, LEAN && !EXT, true>(
+            sm, world_accel(mv), cq, c1, c2, LaneState{state, LEAN ? kRneaLeanFloats : kRneaState}, a.tau_out, B, e, act,
+            vjp && (a.rnea_flags & EVAL_TBAR_IS_TAU) ? tile + (mv.nq + 2 * nv) * kLaneEnvs + lane : nullptr);
       if (vjp)  // rnea_level ends with a barrier: the cotangent is complete and the state free
         rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, c1, c2, tile + (mv.nq + 2 * nv) * kLaneEnvs + lane,
                                     LaneState{state, kVjpState}, VjpAligned{a.qbar, a.qdbar, a.qddbar, nullptr, 1.f},

@@ -56,8 +56,9 @@ __global__ void __launch_bounds__(256) rnea_level_kernel(ModelView mv, int64_t B
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
   FST_LEVEL_READY;
-  rnea_level<false, false, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
-             Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
+  rnea_level<false, false, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs},
+                                 Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+                                 Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
 // RNEA with 12 floats of state a body: four tiles of the floating humanoid per
@@ -70,8 +71,9 @@ __global__ void __launch_bounds__(256) rnea_lean_kernel(ModelView mv, int64_t B,
   stage_block_rows(tile + mv.nq * kLaneEnvs, qd, mv.nv, B, e);
   stage_block_rows(tile + (mv.nq + mv.nv) * kLaneEnvs, qdd, mv.nv, B, e);
   FST_LEVEL_READY;
-  rnea_level<true, true, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs}, Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
-                   Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
+  rnea_level<true, true, true>(sm, world_accel(mv), Col{tile + lane, kLaneEnvs},
+                               Col{tile + mv.nq * kLaneEnvs + lane, kLaneEnvs},
+                               Col{tile + (mv.nq + mv.nv) * kLaneEnvs + lane, kLaneEnvs}, S, tau, B, e, act);
 }
 
 __global__ void __launch_bounds__(256) crba_level_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
@@ -289,7 +291,8 @@ size_t aba_lean_smem_needed(const ModelView& mv, int slots) {
 }
 cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* tau,
                                   float* qdd, int block, int slots, cudaStream_t s) {
-  return go(few_tiles(B) ? aba_lean_kernel<true> : aba_lean_kernel<false>, mv, B, aba_lean_smem_needed(mv, slots), block, 1, 1, s, q, qd, tau, qdd, slots);
+  return go(few_tiles(B) ? aba_lean_kernel<true> : aba_lean_kernel<false>, mv, B, aba_lean_smem_needed(mv, slots),
+            block, 1, 1, s, q, qd, tau, qdd, slots);
 }
 size_t crba_lean_smem_needed(const ModelView& mv, int slots, bool staged) {
   return smem_bytes(mv.n) + (staged ? level_tile_bytes(mv, mv.nq, 0) : 0) +

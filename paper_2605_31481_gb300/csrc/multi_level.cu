@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(256) multi_tile_kernel(const __grid_constant__
                       LaneState{state + kCrbaLeanBodyFloats * mv.n * kLaneEnvs, kCrbaLeanSlotFloats}, io.M, B, e, act);
       break;
     case ROLE_RNEA:
-      rnea_level<true, true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B, e, act);
+      rnea_level<true, true, true>(sm, world_accel(mv), cq, c1, c2, LaneState{state, kRneaLeanFloats}, io.tau_out, B,
+                                   e, act);
       break;
     default:
       fk_level<true>(sm, cq, LaneState{state, kFkState}, io.poses, B, e, act);
