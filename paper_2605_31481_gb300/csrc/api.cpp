@@ -109,15 +109,17 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
 //  * specialised other side. Its straight-line code costs an instruction
 //    fetch per body whatever the batch, so it wins on small trees (arm7 B =
 //    4096 FK 5.4 / 2.8, ABA 13.6 / 9.0; B = 65536 ABA 64 / 15) and large
-//    batches (quadruped11 B = 16384 RNEA 10 / 7.7, ABA 14 / 14.8, B = 32768
-//    ABA 26 / 16; at 4096 ABA 11 / 14.6, the step 14 / 17) and on large trees
+//    batches (quadruped11 B = 16384 RNEA 9.8 / 7.7, ABA 12.8 / 14.6, the step 36.7 /
+//    36.8, B = 32768 ABA 26 / 16; up to two tiles an SM the tiles' shorter chain
+//    wins: 9700 ABA 10.5 / 14.6, the step 21.2 / 27.0, the step of RNEA and its adjoint
+//    20.2 / 30.1, though the Jacobians alone 6.7 / 5.9) and on large trees
 //    only for the light operators (humanoid29 B = 32768 FK 13 / 8.5, RNEA 29 /
 //    23; CRBA 52 / 93, ABA 56 / 149).
 bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
   const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
   if (spec) {
     if (m->n <= 8) return false;
-    if (m->n <= 16) return B < 8192;
+    if (m->n <= 16) return B <= 152 * 2 * 32;
     return !light || B < (op == JK_RNEA || op == JK_RNEA_STORE ? 24576 : 16384);
   }
   if (2 * m->n < 3 * m->depth) {
@@ -158,12 +160,12 @@ bool use_tile(const fst_model* m, int kind, int64_t B) {
 // 73). The FK adjoint is light: arm7 specialised 5.5 / 8.2 at every batch,
 // quadruped11 8.5 / 7.5 at 4096 and 8.6 / 10 at 16384. For the smallest trees
 // the RNEA adjoint follows the specialised fused step, whose result it must
-// equal bit for bit (where the step is better off with it: quadruped11 B = 8192 30.8
-// us in one launch, 43 as step and adjoint).
+// equal bit for bit (where the step is better off with it: quadruped11 B = 16384 31
+// us in one launch, 38 as tiles and more as step and adjoint).
 bool adjoint_tile_rule(const fst_model* m, int kind, bool spec, int64_t B) {
   if (kind == JK_FK_VJP) return spec ? m->n > 8 && (m->n > 16 || B < 12288) : true;
   if (spec && m->n <= 8 && kind == JK_RNEA_VJP) return false;
-  if (spec && m->n <= 16) return B < (kind == JK_RNEA_VJP ? 8192 : 24576);
+  if (spec && m->n <= 16) return kind == JK_RNEA_VJP ? B <= 152 * 2 * 32 : B < 24576;
   return 2 * m->n >= 3 * m->depth || B <= 24576;
 }
 

@@ -176,7 +176,7 @@ def test_lean_forms_give_the_same_bits(torch_cuda, name, B):
 @pytest.mark.parametrize("name,B,specialize", [
     ("chain7", 9728, False), ("chain7", 9729, False),      # RNEA leaves the tiles before its adjoint does
     ("chain12", 4865, False), ("chain30", 40, False), ("wide36", 40, False),  # wide36: only the adjoint does not fit
-    ("quadruped11", 8191, True), ("quadruped11", 8192, True),
+    ("quadruped11", 8191, True), ("quadruped11", 8192, True), ("quadruped11", 9728, True), ("quadruped11", 9729, True),
 ])
 def test_fused_evaluation_equals_separate_calls_at_the_rules_edges(torch_cuda, name, B, specialize):
     torch = torch_cuda
