@@ -306,8 +306,7 @@ __global__ void __launch_bounds__(256) crba_vjp_kernel(ModelView mv, int64_t B, 
 // sums are added in warp order: the order is fixed, so the result is the same
 // run to run. (One thread per column read nblk rows one after the other: 5.0 us
 // for 256 rows of 71 values.)
-__global__ void __launch_bounds__(1024) partial_reduce_kernel(const float* __restrict__ partial, int nblk, int P,
-                                                              float* __restrict__ out) {
+__global__ void __launch_bounds__(1024) partial_reduce_kernel(const float* partial, int nblk, int P, float* out) {
   __shared__ float part[32][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int p = blockIdx.x * 32 + lane;
@@ -316,7 +315,7 @@ __global__ void __launch_bounds__(1024) partial_reduce_kernel(const float* __res
   pdl_wait();
   if (p < P) {
 #pragma unroll 8
-    for (int b = w; b < nblk; b += 32) s += partial[(int64_t)b * P + p];
+    for (int b = w; b < nblk; b += 32) s += ld_input(partial + (int64_t)b * P + p);
   }
   part[w][lane] = s;
   __syncthreads();

@@ -711,14 +711,14 @@ __device__ __forceinline__ void rnea_vjp_lean(const SmemModel& tp, SV a0, const 
     const int nqb = bi.type == FST_JOINT_FREE ? 7 : bi.type == FST_JOINT_FIXED ? 0 : 1, nvb = nv_of(bi.type);
     float qb[7];
 #pragma unroll
-    for (int k = 0; k < 7; ++k) qb[k] = k < nqb ? __ldg(q + (int64_t)(bi.qi + k) * B + ec) : 0.f;
+    for (int k = 0; k < 7; ++k) qb[k] = k < nqb ? ld_input(q + (int64_t)(bi.qi + k) * B + ec) : 0.f;
     float x[3][6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
       const int64_t at = (int64_t)(bi.vi + k) * B + ec;
-      x[0][k] = k < nvb ? __ldg(qd + at) : 0.f;
-      x[1][k] = k < nvb ? __ldg(qdd + at) : 0.f;
-      x[2][k] = k < nvb ? __ldg(tbar + at) : 0.f;
+      x[0][k] = k < nvb ? ld_input(qd + at) : 0.f;
+      x[1][k] = k < nvb ? ld_input(qdd + at) : 0.f;
+      x[2][k] = k < nvb ? ld_input(tbar + at) : 0.f;
     }
     BodyI b0 = bi;
     b0.qi = 0;
@@ -861,7 +861,7 @@ __device__ __forceinline__ void rnea_vjp_lean(const SmemModel& tp, SV a0, const 
                               g1.y * A.v.z, g1.z * A.v.x, g1.z * A.v.y, g1.z * A.v.z};
           const float* qq = q + (int64_t)(bi.qi + 3) * B + e;
           float gq[4];
-          quat_grad(__ldg(qq), __ldg(qq + B), __ldg(qq + 2 * B), __ldg(qq + 3 * B), G, gq);
+          quat_grad(ld_input(qq), ld_input(qq + B), ld_input(qq + 2 * B), ld_input(qq + 3 * B), G, gq);
           const float qo[7] = {0.f, 0.f, 0.f, gq[0], gq[1], gq[2], gq[3]};
           const float vo[6] = {-y.v.x, -y.v.y, -y.v.z, H.x - y.w.x, H.y - y.w.y, H.z - y.w.z};
           const float ao[6] = {A.v.x, A.v.y, A.v.z, A.w.x, A.w.y, A.w.z};
@@ -921,7 +921,7 @@ __device__ __forceinline__ void fk_vjp_tile(const SmemModel& tp, const Col& q, c
     float g[12];
     const float* src = pbar + (int64_t)i * 12 * B + e;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) g[k] = act ? __ldg(src + (int64_t)k * B) : 0.f;
+    for (int k = 0; k < 12; ++k) g[k] = act ? ld_input(src + (int64_t)k * B) : 0.f;
     float R[9];
     S.get_n(i, P_, R, 9);
     SV f{f3{0.f, 0.f, 0.f}, f3{g[9], g[10], g[11]}};

@@ -398,6 +398,20 @@ __device__ __forceinline__ void pdl_launch() {
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A load of anything that a kernel ahead in the stream may have written, for
+// kernels launched that way. Such a kernel is resident while its inputs are
+// still being written (and while an older kernel still reads the memory that
+// they reuse), so the read-only path, __ldg or what the compiler makes of a
+// const __restrict__ pointer, is not open to it: that path is defined for data
+// which nothing writes during the kernel's life, and may be served from a line
+// fetched before the wait. This one is an ordinary coherent load, and, volatile
+// like pdl_wait, stays behind it.
+__device__ __forceinline__ float ld_input(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+
 __host__ __device__ inline size_t smem_bytes(int n) {
   return (size_t)n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;
 }

@@ -460,7 +460,7 @@ __device__ __forceinline__ Xf joint_X_rows(const BodyC& c, const BodyI& bi, cons
   const int nqb = bi.type == FST_JOINT_FREE ? 7 : bi.type == FST_JOINT_FIXED ? 0 : 1;
   float qb[7];
 #pragma unroll
-  for (int k = 0; k < 7; ++k) qb[k] = k < nqb ? __ldg(q + (int64_t)(bi.qi + k) * B + ec) : 0.f;
+  for (int k = 0; k < 7; ++k) qb[k] = k < nqb ? ld_input(q + (int64_t)(bi.qi + k) * B + ec) : 0.f;
   BodyI b0 = bi;
   b0.qi = 0;
   return joint_X(c, b0, Col{qb, 1});

@@ -60,7 +60,7 @@ struct Own {
 __device__ __forceinline__ Own own_rows(const float* __restrict__ src, int first, int count, int64_t B, int64_t ec) {
   Own o;
 #pragma unroll
-  for (int k = 0; k < 7; ++k) o.x[k] = k < count ? __ldg(src + (int64_t)(first + k) * B + ec) : 0.f;
+  for (int k = 0; k < 7; ++k) o.x[k] = k < count ? ld_input(src + (int64_t)(first + k) * B + ec) : 0.f;
   return o;
 }
 __device__ __forceinline__ Own own_q(const Me& me, const float* __restrict__ q, int64_t B, int64_t ec) {
@@ -81,7 +81,7 @@ __device__ __forceinline__ In10 own_inertia(const Me& me, const ModelView& mv) {
   const float* th = own_theta(me, mv);
   float t[10];
 #pragma unroll
-  for (int k = 0; k < 10; ++k) t[k] = __ldg(th + k);
+  for (int k = 0; k < 10; ++k) t[k] = ld_input(th + k);
   return in_load(t);
 }
 
