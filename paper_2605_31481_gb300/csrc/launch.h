@@ -81,7 +81,9 @@ inline void prepare(K* kernel, size_t smem) {
 // Launches a kernel that starts with pdl_launch and pdl_wait (fst_device.cuh)
 // so that its launch, its blocks' start and its copy of the model overlap the
 // end of the kernel ahead of it in the stream. The order of the two kernels'
-// effects is the stream's, as for any launch.
+// effects is the stream's, as for any launch. Returns the last error and clears
+// it, as every launcher here does: a refused launch is this call's to report,
+// not that of the next launch or check of the program around it.
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
   cudaLaunchAttribute attr{};
@@ -94,7 +96,8 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  return cudaGetLastError();
 }
 
 // Kernel launchers (return the cudaGetLastError() after the launch).

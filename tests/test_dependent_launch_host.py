@@ -6,6 +6,10 @@ __restrict__ pointer, which the compiler may turn into one), and it must wait
 before it reads them."""
 import os
 import re
+import shutil
+import subprocess
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_31481_gb300", "csrc")
 
@@ -81,3 +85,18 @@ def test_every_kernel_waits_before_it_stages_inputs():
         first = re.search(r"stage_block_rows|ld_input|vjp_warp|minv_warp|rnea_vjp_lean\(", body)
         wait = min((body.index(w) for w in _waits(_read(unit)) if w in body))
         assert first is None or wait < first.start(), (unit, name)
+
+
+def test_a_refused_launch_leaves_no_error_behind(tmp_path):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("needs nvcc")
+    root = os.path.dirname(os.path.dirname(CSRC))
+    exe = tmp_path / "launch_errors"
+    host = os.path.join(root, "tests", "host", "launch_errors")
+    cmd = [nvcc, "-std=c++17", "-cudart", "none", "-I", CSRC, "-I", os.path.join(root, "include"), host + ".cu",
+           host + ".cpp", "-o", str(exe)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
