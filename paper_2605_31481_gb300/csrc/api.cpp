@@ -130,8 +130,9 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
 }
 
 // Shared memory of one tile of an operator's state in full. Where that does not
-// fit the operator does not run as tiles, though a leaner form of it might: all
-// entry points ask the same question.
+// fit the operator's call and the fused evaluation do not run as tiles, though a
+// leaner form of it might (the mixed-tree launch, which keeps every state lean,
+// takes it): a large tile leaves an SM one block.
 size_t tile_need(const fst_model* m, int kind) {
   const ModelView mv = view_of(m, nullptr);
   switch (kind) {

@@ -433,15 +433,16 @@ __device__ __forceinline__ void quat_R(float x, float y, float z, float w, float
   y *= s;
   z *= s;
   w *= s;
-  R[0] = 1.f - 2.f * (y * y + z * z);
-  R[1] = 2.f * (x * y - w * z);
-  R[2] = 2.f * (x * z + w * y);
-  R[3] = 2.f * (x * y + w * z);
-  R[4] = 1.f - 2.f * (x * x + z * z);
-  R[5] = 2.f * (y * z - w * x);
-  R[6] = 2.f * (x * z - w * y);
-  R[7] = 2.f * (y * z + w * x);
-  R[8] = 1.f - 2.f * (x * x + y * y);
+  // fused by hand: the units are compiled with different rules for fusing
+  R[0] = fmaf(-2.f, fmaf(y, y, z * z), 1.f);
+  R[1] = 2.f * fmaf(x, y, -(w * z));
+  R[2] = 2.f * fmaf(x, z, w * y);
+  R[3] = 2.f * fmaf(x, y, w * z);
+  R[4] = fmaf(-2.f, fmaf(x, x, z * z), 1.f);
+  R[5] = 2.f * fmaf(y, z, -(w * x));
+  R[6] = 2.f * fmaf(x, z, -(w * y));
+  R[7] = 2.f * fmaf(y, z, w * x);
+  R[8] = fmaf(-2.f, fmaf(x, x, y * y), 1.f);
 }
 
 // One environment's column of a staged [field][envs-per-block] tile in

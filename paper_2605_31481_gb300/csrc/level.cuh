@@ -11,7 +11,10 @@
 // gathers, not scatters: each body leaves its contribution to the parent in
 // its own slots and the parent adds its children's after the level barrier,
 // so no atomics are needed (the paper keeps these passes sequential for the
-// same reason, Sec. 3.3).
+// same reason, Sec. 3.3). A body adds its children's from the last to the
+// first, the order in which a single thread's sweep from the last body to the
+// first meets them: the two forms then round alike, and a call gives the same
+// bits in either.
 //
 // Every warp runs the same loops with the same trip counts, so all warps
 // meet every __syncthreads(); padding lanes (environments past B) compute on
@@ -351,7 +354,7 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
       },
       [&](const Own& o) {
         SV F = o.F;
-        for (int ch = o.ch; ch < o.ch_end; ++ch) F = F + S.sv(tp.child(ch), C_);
+        for (int ch = o.ch_end - 1; ch >= o.ch; --ch) F = F + S.sv(tp.child(ch), C_);
         if (act && tau) ST_store(tp.C(o.i), o.b, F, tau, B, e);
         if (tau_col) ST_store(tp.C(o.i), o.b, F, tau_col, kLaneEnvs, 0);
         if (tape && act) {
@@ -404,7 +407,7 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
       const BodyI bi = tp.I(i);
       const Xf X = joint_X(tp.C(i), bi, q);
       In10 Ic = in_load(tp.theta(i));
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) in_add(Ic, S.in10(tp.child(ch), CT_));
+      for (int ch = tp.child_begin(i + 1) - 1; ch >= tp.child_begin(i); --ch) in_add(Ic, S.in10(tp.child(ch), CT_));
       S.putX(i, X_, X);
       S.putin(i, IC_, Ic);
       if (bi.parent >= 0) S.putin(i, CT_, in_to_parent(X, Ic));
@@ -502,7 +505,7 @@ __device__ __forceinline__ void crba_level_lean(const TP& tp, const XF& X_of, in
       },
       [&](const Own& o) {
         In10 Ic = o.I;
-        for (int ch = o.ch; ch < o.ch_end; ++ch) in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
+        for (int ch = o.ch_end - 1; ch >= o.ch; --ch) in_add(Ic, R.in10(tp.C(tp.child(ch)).slot, 0));
         if (o.type == FST_JOINT_REVOLUTE || o.type == FST_JOINT_PRISMATIC)
           S.put(o.i, F_, in_mul(Ic, S_of(tp.C(o.i))));
         R.putin(o.slot, 0, o.parent >= 0 ? in_to_parent(o.X, Ic) : Ic);
@@ -589,7 +592,7 @@ __device__ __forceinline__ void aba_level(const TP& tp, SV a0, const Col& q, con
       const BodyI bi = tp.I(i);
       Sym6 IA = S.sym(i, IA_);
       SV pA = S.sv(i, PA_);
-      for (int ch = tp.child_begin(i); ch < tp.child_begin(i + 1); ++ch) {
+      for (int ch = tp.child_begin(i + 1) - 1; ch >= tp.child_begin(i); --ch) {
         sym6_add(IA, S.sym(tp.child(ch), IA_));
         pA = pA + S.sv(tp.child(ch), PA_);
       }
@@ -728,7 +731,7 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
         o.slot = tp.C(i).slot;
         o.ch = tp.child_begin(i);
         o.ch_end = tp.child_begin(i + 1);
-        o.ch_slot = AHEAD && o.ch < o.ch_end ? tp.C(tp.child(o.ch)).slot : 0;
+        o.ch_slot = AHEAD && o.ch < o.ch_end ? tp.C(tp.child(o.ch_end - 1)).slot : 0;
         o.I = in_load(tp.theta(i));
         const SV vi = S.sv(i, VU_);
         o.p = crf(vi, in_mul(o.I, vi));
@@ -738,8 +741,8 @@ __device__ __forceinline__ void aba_level_lean(const TP& tp, SV a0, const Col& q
       [&](const Own& o) {
         Sym6 IA = sym6_from_in(o.I);
         SV pA = o.p;
-        for (int ch = o.ch; ch < o.ch_end; ++ch) {
-          const int cs = AHEAD && ch == o.ch ? o.ch_slot : tp.C(tp.child(ch)).slot;
+        for (int ch = o.ch_end - 1; ch >= o.ch; --ch) {
+          const int cs = AHEAD && ch == o.ch_end - 1 ? o.ch_slot : tp.C(tp.child(ch)).slot;
           sym6_add(IA, R.sym(cs, RI_));
           pA = pA + R.sv(cs, RP_);
         }

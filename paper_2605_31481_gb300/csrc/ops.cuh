@@ -445,7 +445,7 @@ __device__ __forceinline__ void aba_env(const TP& tp, SV a0, const Col& q, const
       u[i] = ui;
       if (bi.parent < 0) continue;
       sym6_rank1_sub(Ia, Ui, iD);
-      pa = pa + sym6_mul(Ia, cb[i]) + (ui * iD) * Ui;
+      pa = sv_fma(ui * iD, Ui, pa + sym6_mul(Ia, cb[i]));
     } else {
       if (bi.parent < 0) continue;
       pa = pa + sym6_mul(Ia, cb[i]);
@@ -462,7 +462,7 @@ __device__ __forceinline__ void aba_env(const TP& tp, SV a0, const Col& q, const
       const float qi = (u[i] - dot(U[i], ai)) * invD[i];
       if (qdd) qdd[(int64_t)bi.vi * B + e] = qi;
       if (qdd_col) qdd_col[bi.vi * qdd_ld] = qi;
-      ai = ai + qi * S_of(tp.C(i));
+      ai = sv_fma(qi, S_of(tp.C(i)), ai);
     } else if (bi.type == FST_JOINT_FREE) {
       const SV tf = SV{f3{tau[bi.vi + 3], tau[bi.vi + 4], tau[bi.vi + 5]}, f3{tau[bi.vi], tau[bi.vi + 1], tau[bi.vi + 2]}};
       const SV anew = sym6_solve(IA[i], tf - pA[i]);
