@@ -374,8 +374,8 @@ typedef struct fst_eval_io {
 FST_API fst_status fst_packed_layout(const fst_model* model, const int32_t* links, int32_t n_links,
                                      int32_t* cols, int32_t* j_rows, int32_t* m_rows);
 
-/* Every requested operator of one batch in one launch (two or three where the
- * default variant's rules part the operators, see below). The paper computes
+/* Every requested operator of one batch in one launch (two or three in some
+ * cases of the default variant, see below). The paper computes
  * only the kinematic tiers a query needs (Sec. 3.1); here the operators
  * whose outputs are NULL are skipped and the others run side by side on the
  * GPU, one group of thread blocks per operator. Results are bit-identical
@@ -394,9 +394,9 @@ FST_API fst_status fst_packed_layout(const fst_model* model, const int32_t* link
  * (FST_SPEC_EVAL) and the eval kind is not set to FST_VARIANT_GENERIC, else
  * the generic one. FST_EVAL_PACKED writes M and J in the layouts of
  * fst_packed_layout (M then has nv*(nv+1)/2 rows), on the same kernels; values
- * are bit-identical to the full layouts' entries. With the default variant the
- * operators that run as tiles are one launch and those that do not another,
- * and an adjoint whose own call would take another form than RNEA's follows
+ * are bit-identical to the full layouts' entries. With the default variant an
+ * operator of a large tree whose state does not fit a tile has a launch of its
+ * own, and an adjoint whose own call would take another form than RNEA's follows
  * as that call, so that every output is its operator's own call's. */
 FST_API fst_status fst_eval(const fst_model* model, int64_t B, const fst_eval_io* io,
                             const float* theta, void* stream);
@@ -599,7 +599,7 @@ FST_API fst_status fst_multi_eval(fst_multi* multi, const fst_multi_io* io, void
 
 /* Launch form of a group's fst_multi_eval (not in the paper; a tuning knob).
  * The default until this is called: tiles of 32 environments if every tree's
- * own calls run as tiles at that batch size and its state fits in shared
+ * fused evaluation runs as tiles at that batch size and its state fits in shared
  * memory, else the generic form at block 64. FST_VARIANT_GENERIC: one
  * environment per thread, items of `block` environments. FST_VARIANT_LEVEL: the level-parallel
  * bodies of paper Sec. 3.3, items of 32 environments with the block's

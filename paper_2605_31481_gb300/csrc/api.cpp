@@ -93,40 +93,87 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
          level_smem_needed(view_of(m, nullptr), level_kind, level_tiles(m, kind)) <= kLevelSmemLimit;
 }
 
-// Whether a call that keeps the default variant runs as tiles of 32
-// environments whose warps share the bodies (level.cuh, aligned.cuh) rather
-// than one environment per thread. op: the operator's kind; spec: whether the
-// other side is a specialised kernel. The rule is the operator's, not the
-// entry point's, so the fused evaluation and the single calls give the same
-// bits. Both sides measured on GB300 (us, tiles / other):
+// Environments of one tile on every SM, k times.
+int64_t tiles_an_sm(int k) { return (int64_t)k * 152 * 32; }
+
+// A tree with fewer than 1.5 bodies a level has no width to share.
+bool is_chain(const fst_model* m) { return 2 * m->n < 3 * m->depth; }
+
+// Whether an operator's own call that keeps the default variant runs as tiles of
+// 32 environments whose warps share the bodies (level.cuh) rather than one
+// environment per thread. The forms give the same bits (one exception: the
+// specialised ABA of a tree with prismatic joints), so that the fused evaluation
+// can follow a rule of its own: its roles share the chip, and what is best for
+// one alone is not what is best for it there. Both sides measured on GB300 (us
+// in the kernel, tiles / other):
 //  * generic other side. Tiles shorten the chain from the bodies to the
-//    levels: humanoid29 B = 4096 RNEA 8.3 / 22.8, CRBA 9.8 / 72.5, ABA 13.7 /
-//    53; B = 65536 FK 24 / 40, RNEA 49 / 68, CRBA 77 / 160, ABA 92 / 200. A chain has no
-//    width to share: arm7 ABA 13 / 13 at 4096, 26 / 16 at 16384. Narrow trees
-//    (fewer than three bodies a level) at large batches are better off with
-//    more environments per SM where the sweeps are light: quadruped11 B =
-//    65536 FK 16 / 15, RNEA 31 / 24, but CRBA 29 / 38, ABA 50 / 78.
-//  * specialised other side. Its straight-line code costs an instruction
-//    fetch per body whatever the batch, so it wins on small trees (arm7 B =
-//    4096 FK 5.4 / 2.8, ABA 13.6 / 9.0; B = 65536 ABA 64 / 15) and large
-//    batches (quadruped11 B = 16384 RNEA 9.8 / 7.7, ABA 12.8 / 14.6, the step 36.7 /
-//    36.8, B = 32768 ABA 26 / 16; up to two tiles an SM the tiles' shorter chain
-//    wins: 9700 ABA 10.5 / 14.6, the step 21.2 / 27.0, the step of RNEA and its adjoint
-//    20.2 / 30.1, though the Jacobians alone 6.7 / 5.9) and on large trees
-//    only for the light operators (humanoid29 B = 32768 FK 13 / 8.5, RNEA 29 /
-//    23; CRBA 52 / 93, ABA 56 / 149).
+//    levels: humanoid29 B = 4096 RNEA 8.2 / 21.2, CRBA 9.7 / 61.9, ABA 13.4 /
+//    48.3; B = 65536 FK 24 / 37, RNEA 47 / 69, CRBA 77 / 161, ABA 92 / 203. A
+//    chain's RNEA is better off in one thread (7 bodies, B = 1024 6.6 / 6.2, 4096 7.2 /
+//    6.2; 24 bodies 20.1 / 19.3; with the tape 9.7 / 7.2 and 30 / 24), its FK and
+//    CRBA are not (7 bodies 4.3 / 5.7 and 6.2 / 9.1), and ABA of few bodies only
+//    from a second tile on (4096 10.7 / 9.3, 6000 10.6 / 11.5). Narrow trees (fewer
+//    than three bodies a level) at large batches keep more environments per SM
+//    where the sweeps are light.
+//  * specialised other side. Its straight-line code costs an instruction fetch
+//    per body whatever the batch, so it wins on small trees (arm7 B = 4096 FK 5.4
+//    / 2.8, ABA 13.6 / 9.0) and, for light operators, as soon as an SM has a
+//    second tile (B = 8192: quadruped11 FK 4.3 / 3.7, Jacobians 7.8 / 5.6, RNEA 8.1 /
+//    7.4; but ABA 10.2 / 14.6, and legged12, four bodies a level, FK 3.7 / 4.2, RNEA
+//    6.6 / 7.6, Jacobians 7.5 / 6.0). Above 16 bodies later: FK 16384 (humanoid29 6.6 /
+//    8.0, at 20000 10.0 / 8.2), RNEA four tiles an SM (legged18 19456 9.9 / 10.9, 20000
+//    13.7 / 10.9) or 24576 (humanoid29 21.8 / 21.7), CRBA of up to 20 bodies three
+//    (legged18 14592 8.4 / 11.1, 16384 12.3 / 11.1), the others never (humanoid29
+//    B = 32768 CRBA 41 / 93, ABA 56 / 149, RNEA with the tape 49 / 150).
 bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
-  const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
+  const bool wide = m->n >= 3 * m->depth;
   if (spec) {
     if (m->n <= 8) return false;
-    if (m->n <= 16) return B <= 152 * 2 * 32;
-    return !light || B < (op == JK_RNEA || op == JK_RNEA_STORE ? 24576 : 16384);
+    if (m->n <= 16) {
+      const bool one = op == JK_JACOBIAN || (!wide && (op == JK_FK || op == JK_RNEA));
+      return B <= tiles_an_sm(one ? 1 : 2);
+    }
+    switch (op) {
+      case JK_FK:
+        return B < 16384;
+      case JK_JACOBIAN:
+        return B <= tiles_an_sm(1);
+      case JK_RNEA:
+        return m->n <= 20 ? B <= tiles_an_sm(4) : B < 24576;
+      case JK_CRBA:
+        return m->n > 20 || B <= tiles_an_sm(3);
+      default:
+        return true;
+    }
   }
-  if (2 * m->n < 3 * m->depth) {
-    const int64_t most = op != JK_RNEA || m->n <= 8 ? 152 * 2 * 32 : m->n <= 16 ? 152 * 32 : 0;
-    return B <= most;
+  if (is_chain(m)) {
+    if (op == JK_RNEA || op == JK_RNEA_STORE) return false;
+    return B <= tiles_an_sm(2) && !(op == JK_ABA && m->n <= 8 && B <= tiles_an_sm(1));
   }
-  return !light || m->n >= 3 * m->depth || B < 32768;
+  const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
+  return !light || wide || B < 32768;
+}
+
+// The same question for the operators of a fused evaluation together (us, tiles /
+// other). aba: whether ABA is among them; kin: whether FK and the Jacobians are
+// all there is.
+//  * generic other side: the whole step of every tree but a chain is the faster
+//    one in tiles (quadruped11 B = 65536 111 / 153). A chain up to two tiles an SM
+//    (7 bodies, FK, J, RNEA and CRBA B = 4096 7.8 / 9.7, 9728 11.6 / 11.9), of few
+//    bodies with ABA only with the second (1024 10.7 / 9.8, 6000 13.4 / 15.6).
+//  * specialised other side: up to two tiles an SM for trees of 9 to 16 bodies
+//    (quadruped11 B = 8192 the step 21.5 / 23.0, at 9728 21.0 / 26.8); above 16 the
+//    roles' straight-line code no longer fits beside each other (humanoid29 B =
+//    16384 70 / 200, 65536 262 / 548; legged18 45 / 86 and 170 / 252). The kinematics
+//    alone as above (quadruped11 B = 4864 6.4 / 7.2, 8192 8.2 / 7.4; legged18 12288
+//    12.6 / 15.5, 16384 17.1 / 15.4; humanoid29 16384 19.8 / 47).
+bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin) {
+  if (spec) {
+    if (m->n <= 8) return false;
+    if (m->n <= 16) return B <= tiles_an_sm(kin ? 1 : 2);
+    return !kin || m->n > 20 || B <= tiles_an_sm(3);
+  }
+  return !is_chain(m) || (B <= tiles_an_sm(2) && !(aba && m->n <= 8 && B <= tiles_an_sm(1)));
 }
 
 // Shared memory of one tile of an operator's state in full. Where that does not
@@ -283,9 +330,12 @@ cudaError_t jit_go_slot(const fst_model* m, int kind, int slot, int64_t B, int r
   int T = block_of(m, kind, B);
   // The fused evaluation's roles are different straight-line code: fewer,
   // larger blocks let more warps of one SM share a role's instructions (arm7
-  // B = 4096: 19.0 us with 32 threads, 9.0 with 128, 8.8 with 256; quadruped11
-  // 31.3, 17.1, 21.6).
-  if (kind == JK_EVAL && m->block[kind] == 0) T = m->n <= 8 ? 256 : 128;
+  // B = 4096, the step: 18.5 us with 32 threads, 8.8 with 128, 8.4 with 256;
+  // quadruped11, B = 10000, 35.5, 27.1, 20.7). A single role has nothing to share
+  // (arm7's kinematics at every B to 16384 3.3 us with 32 threads, 4.2 with 256;
+  // quadruped11 B = 32768 8.8 and 10.2), nor has a batch of a few blocks
+  // (B = 256: FK, J, RNEA and CRBA 4.3 with 32 and 8.8 with 256, the step 7.8 and 11.9).
+  if (kind == JK_EVAL && m->block[kind] == 0 && gy > 1 && B >= 1024) T = m->n <= 8 ? 256 : 128;
   auto smem = [&](int t) { return (size_t)rows * t * sizeof(float) + (size_t)(t / 32) * P * sizeof(float); };
   while (T > 32 && smem(T) > 96 * 1024) T /= 2;
   const dim3 grid(grid_for(B, T), gy);
@@ -766,12 +816,13 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
   if (m->nq) FST_CHECK(need(fn, io->q, "q"));
   const ModelView mv = view_of(m, theta);
   if (m->variant[JK_EVAL] == FST_VARIANT_AUTO) {
-    // the operators that run as tiles in one launch, the others in another
+    // an operator whose state in full does not fit a tile has a launch of its own
     const bool spec = jit_has(m, JK_EVAL);
+    const bool kin = a.n_roles == 1 && a.roles[0] == ROLE_KIN;
+    const bool as_tiles = eval_tile_rule(m, spec, B, a.roles[0] == ROLE_ABA && !vjp, kin);
     auto tiled = [&](int role) {
-      const int op = role == ROLE_ABA ? JK_ABA : role == ROLE_CRBA ? JK_CRBA : role == ROLE_RNEA ? JK_RNEA
-                                                                             : (a.J ? JK_JACOBIAN : JK_FK);
-      return tile_need(m, op) <= kLevelSmemLimit && tile_rule(m, op, spec, B);
+      const int op = role == ROLE_ABA ? JK_ABA : role == ROLE_CRBA ? JK_CRBA : role == ROLE_RNEA ? JK_RNEA : JK_FK;
+      return as_tiles && tile_need(m, op) <= kLevelSmemLimit;
     };
     const bool adjoint_tiled =
         vjp && rnea_vjp_aligned_smem(mv) + 1024 <= kLevelSmemLimit && adjoint_tile_rule(m, JK_RNEA_VJP, spec, B);
@@ -1219,8 +1270,9 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
   for (int k = 0; k < n; ++k) order[k] = k;
   for (int i = 1; i < n; ++i)
     for (int j = i; j > 0 && g->models[order[j]]->n > g->models[order[j - 1]]->n; --j) std::swap(order[j], order[j - 1]);
-  // the default form is the one that the single-tree calls take: tiles of 32
-  // environments if every tree's calls do and their state fits
+  // the default form is tiles of 32 environments, if every tree's fused evaluation
+  // takes them (a short chain's from one tile an SM on: beside larger trees its
+  // tiles are the shorter ones) and their state fits
   auto tile_smem = [&](int k, int r) { return multi_tile_smem(a.mv[k], r, g->models[k]->slots); };
   a.model_bytes = (size_t)max_n * (sizeof(BodyC) + sizeof(BodyI)) + (sizeof(TopoLists) + 15) / 16 * 16;
   a.model_bytes = (a.model_bytes + 15) / 16 * 16;
@@ -1228,8 +1280,7 @@ fst_status fst_multi_eval(fst_multi* g, const fst_multi_io* io, void* stream) {
   if (g->variant == FST_VARIANT_AUTO) {
     level = true;
     for (int k = 0; k < n; ++k) {
-      for (int op : {JK_FK, JK_RNEA, JK_CRBA, JK_ABA})
-        level = level && (io[k].B == 0 || tile_rule(g->models[k], op, false, io[k].B));
+      level = level && (io[k].B == 0 || !is_chain(g->models[k]) || io[k].B <= tiles_an_sm(2));
       for (int r : {ROLE_ABA, ROLE_CRBA, ROLE_RNEA, ROLE_KIN}) level = level && tile_smem(k, r) <= kLevelSmemLimit;
     }
   }

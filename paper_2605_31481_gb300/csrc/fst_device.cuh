@@ -580,12 +580,31 @@ __device__ __forceinline__ Xf joint_X(const BodyC& c, const BodyI& b, const Col&
 __device__ __forceinline__ SV S_of(const BodyC& c) { return SV{f3{c.S[0], c.S[1], c.S[2]}, f3{c.S[3], c.S[4], c.S[5]}}; }
 
 // S_i x_i for a joint-space column x; the free joint maps its velocity
-// coordinates [v; w] to spatial (w, v).
+// coordinates [v; w] to spatial (w, v). The products are rounded by themselves:
+// where a compiler sees the joint's type it would fuse them into the sum that
+// follows, and a specialised kernel would round differently from the others.
 __device__ __forceinline__ SV S_times(const BodyC& c, const BodyI& b, const Col& x) {
-  if (b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC) return x[b.vi] * S_of(c);
+  if (b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC) {
+    const float y = x[b.vi];
+    const SV s = S_of(c);
+    return SV{f3{__fmul_rn(y, s.w.x), __fmul_rn(y, s.w.y), __fmul_rn(y, s.w.z)},
+              f3{__fmul_rn(y, s.v.x), __fmul_rn(y, s.v.y), __fmul_rn(y, s.v.z)}};
+  }
   if (b.type == FST_JOINT_FREE)
     return SV{f3{x[b.vi + 3], x[b.vi + 4], x[b.vi + 5]}, f3{x[b.vi], x[b.vi + 1], x[b.vi + 2]}};
   return sv_zero();
+}
+
+// a + S_i x_i with the product fused into the sum, as one scaled vector: a
+// caller can form it before it knows a.
+struct ScaledSV {
+  float x;
+  SV s;
+  __device__ __forceinline__ SV add_to(SV a) const { return sv_fma(x, s, a); }
+};
+__device__ __forceinline__ ScaledSV S_scaled(const BodyC& c, const BodyI& b, const Col& x) {
+  if (b.type == FST_JOINT_REVOLUTE || b.type == FST_JOINT_PRISMATIC) return ScaledSV{x[b.vi], S_of(c)};
+  return ScaledSV{1.f, S_times(c, b, x)};
 }
 
 // out_i = S_i^T f

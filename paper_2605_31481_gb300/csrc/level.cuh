@@ -288,7 +288,8 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
   struct Moved {
     int i, parent;
     Xf X;
-    SV vJ, aJ;
+    SV vJ;
+    ScaledSV aJ;
   };
   level_pass<false, AHEAD>(
       tp,
@@ -306,7 +307,7 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
         m.parent = bi.parent;
         m.X = joint_X<SPEND>(c, bi, q, &omc);
         m.vJ = S_times(c, bi, qd);
-        m.aJ = S_times(c, bi, qdd);
+        m.aJ = S_scaled(c, bi, qdd);
         if (SPEND && bi.type == FST_JOINT_REVOLUTE) *qd.spent(bi.vi) = omc;
         return m;
       },
@@ -316,10 +317,10 @@ __device__ __forceinline__ void rnea_level(const TP& tp, SV a0, const Col& q, co
         SV vi, ai;
         if (m.parent < 0) {
           vi = m.vJ;
-          ai = X_motion(X, a0) + m.aJ;
+          ai = m.aJ.add_to(X_motion(X, a0));
         } else {
           vi = X_motion(X, S.sv(m.parent, V_)) + m.vJ;
-          ai = X_motion(X, S.sv(m.parent, A_)) + m.aJ + crm(vi, m.vJ);
+          ai = m.aJ.add_to(X_motion(X, S.sv(m.parent, A_))) + crm(vi, m.vJ);
         }
         S.put(i, V_, vi);
         S.put(i, A_, ai);

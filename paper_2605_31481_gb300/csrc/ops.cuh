@@ -192,14 +192,14 @@ __device__ __forceinline__ void rnea_forward(const TP& tp, SV a0, const Col& q, 
     const BodyI bi = tp.I(i);
     X[i] = joint_X(c, bi, q);
     const SV vJ = S_times(c, bi, qd);
-    const SV aJ = S_times(c, bi, qdd);
+    const ScaledSV aJ = S_scaled(c, bi, qdd);
     SV vi, ai;
     if (bi.parent < 0) {
       vi = vJ;
-      ai = X_motion(X[i], a0) + aJ;
+      ai = aJ.add_to(X_motion(X[i], a0));
     } else {
       vi = X_motion(X[i], v[bi.parent]) + vJ;
-      ai = X_motion(X[i], a[bi.parent]) + aJ + crm(vi, vJ);
+      ai = aJ.add_to(X_motion(X[i], a[bi.parent])) + crm(vi, vJ);
     }
     const In10 I = in_load(tp.theta(i));
     v[i] = vi;

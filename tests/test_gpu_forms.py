@@ -83,6 +83,43 @@ def test_mixed_batch_of_a_tree_near_the_body_limit(torch_cuda):
     _compare_mixed(torch, api, [wide, w.legged(4, seed=0)], (300, 500))
 
 
+@pytest.mark.parametrize("name", list(TREES))
+def test_specialised_kernels_give_the_same_bits(torch_cuda, name):
+    """The operators whose own call and fused evaluation may take different forms at one batch size."""
+    torch = torch_cuda
+    from paper_2605_31481_gb300 import api
+    tree = TREES[name]()
+    ee = _ee(tree)
+    m = api.Model(tree, specialize=["fk", "jacobian", "rnea", "crba"])
+    q, qd, qdd, _ = _inputs(tree, 197, torch)
+    out = {}
+    for form in ("generic", "specialized"):
+        m.set_launch(["fk", "jacobian", "rnea", "crba"], 0, form)
+        out[form] = {"poses": api.fk(m, q), "J": api.jacobian(m, q, ee), "tau": api.rnea(m, q, qd, qdd),
+                     "M": api.crba(m, q)}
+    for k, want in out["generic"].items():
+        assert torch.equal(out["specialized"][k], want), (name, k)
+
+
+@pytest.mark.parametrize("name,B,specialize", [
+    ("chain7", 4000, False), ("chain7", 6000, False), ("chain12", 2000, False), ("quadruped11", 40000, False),
+    ("chain7", 4000, True), ("quadruped11", 6000, True), ("quadruped11", 12000, True), ("humanoid23", 12000, True),
+    ("humanoid29", 26000, True)])
+def test_fused_evaluation_gives_the_calls_bits_where_their_forms_differ(torch_cuda, name, B, specialize):
+    torch = torch_cuda
+    from paper_2605_31481_gb300 import api
+    tree = w.chain(12, seed=0) if name == "chain12" else TREES[name]()
+    ee = _ee(tree)
+    m = api.Model(tree, specialize=["fk", "jacobian", "rnea", "crba", "aba", "eval"] if specialize else None)
+    x = _inputs(tree, B, torch)
+    want = _run(api, m, x, ee)
+    got = api.eval(m, *x, fk=True, links=ee, rnea=True, crba=True, aba=True)
+    alone = api.eval(m, x[0], fk=True, links=ee)
+    for k in want:
+        assert torch.equal(got[k], want[k]), (name, k)
+        assert k not in alone or torch.equal(alone[k], want[k]), (name, k, "alone")
+
+
 def _compare_mixed(torch, api, trees, counts):
     models = [api.Model(t) for t in trees]
     xs = [_inputs(t, B, torch, seed=20 + k) for k, (t, B) in enumerate(zip(trees, counts))]
