@@ -157,7 +157,9 @@ FST_API fst_status fst_model_specialize(fst_model* model, uint32_t kinds);
  * and which kernel variant runs:
  *   AUTO        the built-in choice by operator, tree and B: tiles of 32
  *               environments whose warps share the bodies (below), the
- *               specialised kernel when compiled, or the generic one;
+ *               specialised kernel when compiled, or the generic one
+ *               (tiles choose their own block; a given one is for the
+ *               one-environment-per-thread kernels);
  *   GENERIC     one environment per thread, tree from shared memory;
  *   SPECIALIZED one environment per thread, kernel compiled for this tree;
  *   LEVEL       level-parallel (paper Sec. 3.3 on warps): 32 environments per

@@ -310,10 +310,9 @@ size_t state_with_aba(int n, int slots, int per_body) {
   return a > b ? a : b;
 }
 
-// Threads per block: a caller's setting, else one warp per two or three
-// bodies while the tiles fill the SMs, more when they do not.
-int aligned_block(int set, int n, int64_t tiles) {
-  if (set) return set;
+// Threads per block: one warp per two or three bodies while the tiles fill the
+// SMs, more when they do not.
+int aligned_block(int n, int64_t tiles) {
   if (n >= 16) return tiles <= 304 ? 512 : 256;
   return tiles <= 304 ? 256 : 128;
 }
@@ -336,15 +335,15 @@ size_t aba_vjp_aligned_smem(const ModelView& mv, int slots) {
 // the state's space: the block is as large as that allows (0: not one warp).
 // 16 warps while no SM has a second tile to run (legged12 B = 1000 30.3 -> 26.8
 // us, humanoid29 B = 2048 180 -> 146).
-static int aba_derivs_threads(const ModelView& mv, int slots, int set, int64_t tiles) {
+static int aba_derivs_threads(const ModelView& mv, int slots, int64_t tiles) {
   const size_t st = state_with_aba(mv.n, slots, kDerivState);
-  int t = set ? set : tiles <= 152 ? 512 : aligned_block(set, mv.n, tiles);
+  int t = tiles <= 152 ? 512 : aligned_block(mv.n, tiles);
   while (t >= 32 && (size_t)(t / 32) * 2 * mv.nv > st) t /= 2;
   return t >= 32 ? t : 0;
 }
 
 size_t aba_derivs_aligned_smem(const ModelView& mv, int slots, int entries) {
-  if (!aba_derivs_threads(mv, slots, 32, 1)) return kLevelSmemLimit + 1;
+  if (!aba_derivs_threads(mv, slots, 1)) return kLevelSmemLimit + 1;
   return smem_bytes(mv.n) +
          floats32((size_t)mv.nq + 3 * mv.nv + state_with_aba(mv.n, slots, kDerivState) + entries) +
          ((size_t)4 * mv.nv + 1 + entries) * sizeof(int);
@@ -393,7 +392,7 @@ cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, 
 }
 
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
-                                       const float* qdd, float* dq, float* dqd, int block, cudaStream_t s) {
+                                       const float* qdd, float* dq, float* dqd, cudaStream_t s) {
   const size_t sh = rnea_derivs_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   auto go = [&](auto* k, int threads) {
@@ -402,23 +401,23 @@ cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const flo
   };
   // 24 warps where an SM has one tile and the tree work for them (humanoid29 B =
   // 2048: 21.0 -> 19.7 us, legged18 B = 2700 11.0 -> 10.3).
-  if (block == 0 && mv.n > 16 && tiles <= 152) return go(rnea_derivs_aligned_kernel<768>, 768);
-  return go(rnea_derivs_aligned_kernel<512>, aligned_block(block, mv.n, tiles));
+  if (mv.n > 16 && tiles <= 152) return go(rnea_derivs_aligned_kernel<768>, 768);
+  return go(rnea_derivs_aligned_kernel<512>, aligned_block(mv.n, tiles));
 }
 
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                       const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int slots,
-                                      int entries, int dof_depth, int block, cudaStream_t s) {
+                                      int entries, int dof_depth, cudaStream_t s) {
   const size_t sh = aba_derivs_aligned_smem(mv, slots, entries);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_derivs_aligned_kernel, sh);
-  return launch_pdl(aba_derivs_aligned_kernel, tiles, aba_derivs_threads(mv, slots, block, tiles), sh, s, mv, B, q, qd,
+  return launch_pdl(aba_derivs_aligned_kernel, tiles, aba_derivs_threads(mv, slots, tiles), sh, s, mv, B, q, qd,
                     tau, qdd, dq, dqd, Minv, entries, dof_depth, (int)state_with_aba(mv.n, slots, kDerivState));
 }
 
 cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                     const float* tbar, float* qbar, float* qdbar, float* qddbar, float* thbar,
-                                    float* scratch, int block, cudaStream_t s) {
+                                    float* scratch, cudaStream_t s) {
   const size_t sh = rnea_vjp_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   float* const partial = thbar ? scratch : nullptr;
@@ -427,14 +426,14 @@ cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float*
   const size_t model = smem_bytes(mv.n), lean = floats32((size_t)kVjpLeanState * mv.n);
   const int T = model + 2 * lean <= kLevelSmemLimit && 2 * (model + lean + 1024) > kLevelSmemLimit ? 2 : 1;
   cudaError_t err;
-  if (tiles > 152 * 2 && block == 0 && mv.n > 8) {
+  if (tiles > 152 * 2 && mv.n > 8) {
     const int W = mv.n > 16 ? 8 : 4;
     prepare(rnea_vjp_lean_kernel, model + T * lean);
     err = launch_pdl(rnea_vjp_lean_kernel, (tiles + T - 1) / T, dim3(32, T, W), model + T * lean, s, mv, B, q, qd, qdd,
                      tbar, qbar, qdbar, qddbar, partial);
   } else {
     prepare(rnea_vjp_aligned_kernel<VJP_GIVEN>, sh);
-    err = launch_pdl(rnea_vjp_aligned_kernel<VJP_GIVEN>, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd,
+    err = launch_pdl(rnea_vjp_aligned_kernel<VJP_GIVEN>, tiles, aligned_block(mv.n, tiles), sh, s, mv, B, q, qd,
                      qdd, tbar, qbar, qdbar, qddbar, partial);
   }
   if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
@@ -443,11 +442,11 @@ cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float*
 
 cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                      const float* tau_meas, float* loss_theta, float* qbar, float* qdbar,
-                                     float* scratch, int block, cudaStream_t s) {
+                                     float* scratch, cudaStream_t s) {
   const size_t sh = rnea_vjp_aligned_smem(mv);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(rnea_vjp_aligned_kernel<VJP_LOSS>, sh);
-  cudaError_t err = launch_pdl(rnea_vjp_aligned_kernel<VJP_LOSS>, tiles, aligned_block(block, mv.n, tiles), sh, s, mv,
+  cudaError_t err = launch_pdl(rnea_vjp_aligned_kernel<VJP_LOSS>, tiles, aligned_block(mv.n, tiles), sh, s, mv,
                                B, q, qd, qdd, tau_meas, qbar, qdbar, nullptr, scratch);
   if (err == cudaSuccess) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10 + 1, loss_theta, s);
   return err;
@@ -455,11 +454,11 @@ cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float
 
 cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
-                                   float* scratch, int slots, int block, cudaStream_t s) {
+                                   float* scratch, int slots, cudaStream_t s) {
   const size_t sh = aba_vjp_aligned_smem(mv, slots);
   const unsigned tiles = grid_for(B, kLaneEnvs);
   prepare(aba_vjp_aligned_kernel, sh);
-  cudaError_t err = launch_pdl(aba_vjp_aligned_kernel, tiles, aligned_block(block, mv.n, tiles), sh, s, mv, B, q, qd,
+  cudaError_t err = launch_pdl(aba_vjp_aligned_kernel, tiles, aligned_block(mv.n, tiles), sh, s, mv, B, q, qd,
                                qdd, qddbar, qbar, qdbar, taubar, thbar ? scratch : nullptr);
   if (err == cudaSuccess && thbar) err = launch_partial_reduce(scratch, (int)tiles, mv.n * 10, thbar, s);
   return err;

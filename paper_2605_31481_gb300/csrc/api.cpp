@@ -231,7 +231,7 @@ bool use_adjoint_tile(const fst_model* m, int kind, int64_t B, size_t need) {
 // B = 16384 42 against 40, and larger trees' registers spill (humanoid29 ABA
 // adjoint 29.6 against 26).
 bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
-  return m->variant[kind] == FST_VARIANT_AUTO && m->block[kind] == 0 && m->wt.n > 0 && B <= 152 * 2 * 32 &&
+  return m->variant[kind] == FST_VARIANT_AUTO && m->wt.n > 0 && B <= 152 * 2 * 32 &&
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
@@ -245,7 +245,8 @@ int multi_tile_block(int items) { return items <= 152 * 2 ? 256 : 128; }
 // which keep less state, and so more tiles per SM, are the better ones.
 bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
 
-// Threads per block of a tile launch that does not set them: eight warps, but
+// Threads per block of a default call's tiles (a block that the caller set is
+// meant for one environment per thread): eight warps, but
 // four where many tiles share an SM and a level is never wider (quadruped11 B =
 // 16384 RNEA 9.8 -> 8.6 us, ABA 24.4 -> 14.1, the step 40.5 -> 38.8; legged18, six
 // bodies wide, ABA 19.0 against 27.5 with four). The adjoint's state leaves
@@ -255,7 +256,6 @@ bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
 // thread four such blocks share an SM (quadruped11 B = 4096 13.2 against 15.5 us,
 // 8192 20.9 against 26.7; but 9.9 against 9.0 at 64).
 int tile_block(const fst_model* m, int kind, int64_t B, bool vjp = false) {
-  if (m->block[kind]) return m->block[kind];
   if (kind == JK_EVAL && !vjp && m->max_width <= 4 && m->n <= 16 && B > 152 * 32 / 2) return 128;
   if (!many_tiles(B) || m->max_width > 4 || vjp || kind == JK_CRBA) return 256;
   return m->n <= 16 || kind == JK_ABA ? 128 : 256;
@@ -982,7 +982,7 @@ fst_status fst_rnea_vjp(const fst_model* m, int64_t B, const float* q, const flo
                                          (float*)scratch, (cudaStream_t)stream));
   if (use_adjoint_tile(m, JK_RNEA_VJP, B, rnea_vjp_aligned_smem(mv)))
     return finish(fn, launch_rnea_vjp_aligned(mv, B, q, qd, qdd, tau_bar, q_bar, qd_bar, qdd_bar, theta_bar,
-                                              (float*)scratch, m->block[JK_RNEA_VJP], (cudaStream_t)stream));
+                                              (float*)scratch, (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_VJP)) {
     unsigned nblk = 0;
     float* partial = theta_bar ? (float*)scratch : nullptr;
@@ -1108,8 +1108,7 @@ fst_status fst_rnea_derivatives(const fst_model* m, int64_t B, const float* q, c
   FST_CHECK(need(fn, qdd, "qdd"));
   const ModelView mv = view_of(m, theta);
   if (use_adjoint_tile(m, JK_RNEA_DERIVS, B, rnea_derivs_aligned_smem(mv)))
-    return finish(fn, launch_rnea_derivs_aligned(mv, B, q, qd, qdd, dtau_dq, dtau_dqd, m->block[JK_RNEA_DERIVS],
-                                                 (cudaStream_t)stream));
+    return finish(fn, launch_rnea_derivs_aligned(mv, B, q, qd, qdd, dtau_dq, dtau_dqd, (cudaStream_t)stream));
   if (use_jit(m, JK_RNEA_DERIVS))
     return finish(fn, jit_go(m, JK_RNEA_DERIVS, B, m->nq + 2 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              qd, qdd, dtau_dq, dtau_dqd));
@@ -1130,8 +1129,7 @@ fst_status fst_aba_derivatives(const fst_model* m, int64_t B, const float* q, co
   const ModelView mv = view_of(m, theta);
   if (use_adjoint_tile(m, JK_ABA_DERIVS, B, aba_derivs_aligned_smem(mv, m->slots, m->dof_entries)))
     return finish(fn, launch_aba_derivs_aligned(mv, B, q, qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv, m->slots,
-                                                m->dof_entries, m->dof_depth, m->block[JK_ABA_DERIVS],
-                                                (cudaStream_t)stream));
+                                                m->dof_entries, m->dof_depth, (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_DERIVS))
     return finish(fn, jit_go(m, JK_ABA_DERIVS, B, m->nq + 3 * m->nv, 0, 1, (cudaStream_t)stream, nullptr, mv, B, q,
                              qd, tau, qdd, dqdd_dq, dqdd_dqd, Minv));
@@ -1159,8 +1157,7 @@ fst_status fst_aba_vjp(const fst_model* m, int64_t B, const float* q, const floa
                                         (float*)scratch, (cudaStream_t)stream));
   if (use_adjoint_tile(m, JK_ABA_VJP, B, aba_vjp_aligned_smem(mv, m->slots)))
     return finish(fn, launch_aba_vjp_aligned(mv, B, q, qd, qdd, qdd_bar, q_bar, qd_bar, tau_bar, theta_bar,
-                                             (float*)scratch, m->slots, m->block[JK_ABA_VJP],
-                                             (cudaStream_t)stream));
+                                             (float*)scratch, m->slots, (cudaStream_t)stream));
   if (use_jit(m, JK_ABA_VJP)) {
     unsigned nblk = 0;
     float* partial = theta_bar ? (float*)scratch : nullptr;
@@ -1195,7 +1192,7 @@ fst_status fst_rnea_loss_grad(const fst_model* m, int64_t B, const float* q, con
                                           (float*)scratch, (cudaStream_t)stream));
   if (use_adjoint_tile(m, JK_LOSS_GRAD, B, rnea_vjp_aligned_smem(mv)))
     return finish(fn, launch_loss_grad_aligned(mv, B, q, qd, qdd, tau_meas, loss_theta_bar, q_bar, qd_bar,
-                                               (float*)scratch, m->block[JK_LOSS_GRAD], (cudaStream_t)stream));
+                                               (float*)scratch, (cudaStream_t)stream));
   if (use_jit(m, JK_LOSS_GRAD)) {
     unsigned nblk = 0;
     const int P = m->n * 10 + 1;

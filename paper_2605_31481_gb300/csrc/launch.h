@@ -171,9 +171,9 @@ cudaError_t launch_jac_vjp(const ModelView& mv, int64_t B, const float* q, const
                            float* qbar, cudaStream_t s);
 cudaError_t launch_crba_vjp(const ModelView& mv, int64_t B, const float* q, const float* Mbar, float* qbar,
                             float* thbar, float* scratch, cudaStream_t s);
-// Aligned-frame kernels (aligned.cu), one tile of 32 environments per block
-// (block = 0: built-in choice). The *_smem functions give the shared memory a
-// launch needs: above kLevelSmemLimit the kernel cannot run. slots, entries, dof_depth: see fst_model.
+// Aligned-frame kernels (aligned.cu), one tile of 32 environments per block.
+// The *_smem functions give the shared memory a launch needs: above
+// kLevelSmemLimit the kernel cannot run. slots, entries, dof_depth: see fst_model.
 size_t rnea_derivs_aligned_smem(const ModelView& mv);
 size_t aba_derivs_aligned_smem(const ModelView& mv, int slots, int entries);
 size_t rnea_vjp_aligned_smem(const ModelView& mv);
@@ -191,19 +191,19 @@ cudaError_t launch_rnea_store_tile(const ModelView& mv, int64_t B, const float* 
 cudaError_t launch_eval_tile(const ModelView& mv, int64_t B, const EvalArgs& a, bool lean, size_t smem, int block,
                              cudaStream_t s);
 cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
-                                       const float* qdd, float* dq, float* dqd, int block, cudaStream_t s);
+                                       const float* qdd, float* dq, float* dqd, cudaStream_t s);
 cudaError_t launch_aba_derivs_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd,
                                       const float* tau, float* qdd, float* dq, float* dqd, float* Minv, int slots,
-                                      int entries, int dof_depth, int block, cudaStream_t s);
+                                      int entries, int dof_depth, cudaStream_t s);
 cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                     const float* tbar, float* qbar, float* qdbar, float* qddbar, float* thbar,
-                                    float* scratch, int block, cudaStream_t s);
+                                    float* scratch, cudaStream_t s);
 cudaError_t launch_loss_grad_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                      const float* tau_meas, float* loss_theta, float* qbar, float* qdbar,
-                                     float* scratch, int block, cudaStream_t s);
+                                     float* scratch, cudaStream_t s);
 cudaError_t launch_aba_vjp_aligned(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
                                    const float* qddbar, float* qbar, float* qdbar, float* taubar, float* thbar,
-                                   float* scratch, int slots, int block, cudaStream_t s);
+                                   float* scratch, int slots, cudaStream_t s);
 // Warp-per-body kernels (warpbody.cu), for trees of at most kMaxWarpBodies.
 cudaError_t launch_wb_rnea_vjp(const WarpTree& t, const ModelView& mv, int64_t B, const float* q, const float* qd,
                                const float* qdd, const float* tbar, float* qbar, float* qdbar, float* qddbar,

@@ -61,3 +61,12 @@ def test_default_is_not_slower_than_the_form_it_replaces(torch_cuda, name, B, ki
     default, other = _times(api, torch_cuda, name, B, kind, specialize,
                             [("auto", 0), (other, 32 if kind == "eval" else 0)])
     assert default <= 1.08 * other, (default, other)
+
+
+@pytest.mark.parametrize("name,B,kind", [("humanoid29", 64, "rnea"), ("quadruped11", 4096, "rnea_store"),
+                                         ("quadruped11", 64, "aba")])
+def test_a_block_set_with_the_default_variant_does_not_slow_the_tiles(torch_cuda, name, B, kind):
+    """A block is one of environments, one per thread: 32 of them are one warp, and a tile wants eight."""
+    from paper_2605_31481_gb300 import api
+    default, other = _times(api, torch_cuda, name, B, kind, False, [("auto", 32), ("generic", 32)])
+    assert default <= 1.08 * other, (default, other)
