@@ -3,14 +3,18 @@
 `tune(model, B)` measures, on the current GPU, every candidate configuration
 of each kernel kind and keeps the fastest via fst_model_set_launch. A
 candidate is an environment-to-thread mapping with a block size (32 to 256
-threads):
+threads), or the library's own choice, so that a tuned call is never slower
+than an untuned one:
+  auto         what an untuned model runs (variant auto, block 0), some of whose
+               kernels have no other name: the adjoints and the loss in
+               aligned frames, a warp per body, the lean RNEA and fused step;
   generic      one environment per thread, the tree from shared memory;
   specialized  one environment per thread, a kernel compiled for the tree;
   level        32 environments per block, the block's warps splitting each
                tree level;
   level2       the same with two such tiles per block (half the blocks);
   levellean    (CRBA, ABA) the level-parallel kernel with less state per
-               body and a two-level ring of contributions to the parent, so
+               body and a few slots for contributions to the parent, so
                that more tiles of a large tree fit on one SM;
   mixed        (eval) the specialised fused kernel with each role mapped as
                its own operator is set;
@@ -218,8 +222,7 @@ def _key(model, kind, B):
 
 def autotune_enabled():
     """False when FST_AUTOTUNE=0: then nothing is measured. tune() keeps the
-    library's built-in launch heuristics (variant auto: the specialised
-    kernel where compiled, else the generic one; block 0) and StepPlan runs
+    library's own choice of form (variant auto, block 0) and StepPlan runs
     the step as one fused launch."""
     return os.environ.get("FST_AUTOTUNE", "1").strip() != "0"
 
@@ -260,8 +263,9 @@ def tune(model, B, kinds=FORWARD_KINDS + ("eval",), links=None, use_cache=True, 
             variants.append("mixed")       # specialised fused kernel, roles mapped as their operators
         if kind in spec and kind in LEVEL_KINDS:
             variants += ["path", "pathwarp"]   # path-parallel, where the tree has at most 8 leaves
+        variants.append("auto")                # the library's own choice: what tuning must not fall behind
         for variant in variants:
-            blocks = (0,) if variant == "pathwarp" else CANDIDATE_BLOCKS[1:] if variant == "level2" else \
+            blocks = (0,) if variant in ("pathwarp", "auto") else CANDIDATE_BLOCKS[1:] if variant == "level2" else \
                 CANDIDATE_BLOCKS[2:] if variant == "levellean" else CANDIDATE_BLOCKS
             for block in blocks:
                 try:
@@ -383,9 +387,10 @@ class StepPlan:
             api.set_smem_carveout(carveout)
             for mode in modes:
                 # one launch: the tuned variant, and the library's own choice, which
-                # the eval tuning does not time (quadruped11 B = 4096 17.1
-                # against 13.9 us, the best plan before it 16.0)
-                cfgs = {"fused": [f"{best_eval}|{best_aba}", f"auto/0|{best_aba}"], "hybrid": hybrid_cfgs,
+                # on cold inputs can be the faster one all the same (quadruped11
+                # B = 4096 13.9 us, the best other plan 16.0)
+                cfgs = {"fused": list(dict.fromkeys((f"{best_eval}|{best_aba}", f"auto/0|{best_aba}"))),
+                        "hybrid": hybrid_cfgs,
                         "split": hybrid_cfgs, "pinned": pinned_cfgs, "partitioned": part_cfgs}.get(
                     mode, [f"{best_eval}|{best_aba}"])
                 for ev in cfgs:
