@@ -30,11 +30,14 @@ shared-memory carveouts and with its fork-order or stream-priority option.
 Timings replay a CUDA graph of repeated launches, so host launch overhead is
 excluded. Choices are cached in a JSON file (FST_TUNE_CACHE, default
 ~/.cache/fst_tune.json) keyed by the tree's fingerprint, the kind, B, the
-GPU name and the library version. FST_AUTOTUNE=0 turns all measurement off
+GPU name and a digest of the library's and the tuner's sources, so that a
+choice among kernels that have changed is made again. FST_AUTOTUNE=0 turns all measurement off
 (autotune_enabled()): built-in launch heuristics and one fused launch.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import re
@@ -44,6 +47,7 @@ import torch
 
 from . import api
 from . import _ffi
+from . import build
 
 CANDIDATE_BLOCKS = (32, 64, 128, 256)
 FORWARD_KINDS = ("fk", "jacobian", "rnea", "crba", "aba")
@@ -216,8 +220,15 @@ def _op(model, kind, buf):
     raise ValueError(kind)
 
 
+@functools.lru_cache(maxsize=None)
+def _code():
+    """Names the kernels and the candidates that a choice was made among."""
+    with open(__file__, "rb") as fh:
+        return hashlib.sha256(build.sources_digest().encode() + fh.read()).hexdigest()[:16]
+
+
 def _key(model, kind, B):
-    return f"{model.fingerprint}|{kind}|{B}|{torch.cuda.get_device_name(model.device)}|{_ffi.lib().fst_version().decode()}"
+    return f"{model.fingerprint}|{kind}|{B}|{torch.cuda.get_device_name(model.device)}|{_code()}"
 
 
 def autotune_enabled():

@@ -79,6 +79,15 @@ def _headers_digest() -> str:
     return h.hexdigest()
 
 
+def sources_digest() -> str:
+    """Names the code that the library is built from: its sources, headers and flags."""
+    h = hashlib.sha256(repr((ARCH, NVCC_FLAGS, sorted(UNIT_FLAGS.items()))).encode() + _headers_digest().encode())
+    for f in _sources():
+        with open(os.path.join(CSRC, f), "rb") as fh:
+            h.update(f.encode() + fh.read())
+    return h.hexdigest()
+
+
 def _compile(nvcc, src, flags, hdr, force):
     path = os.path.join(BUILD if src == EMBED else CSRC, src)
     flags = flags + UNIT_FLAGS.get(src, [])

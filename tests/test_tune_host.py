@@ -1,8 +1,11 @@
 """The tuner's candidates and its cache on the host, with the model, the timer
 and the kernels replaced by fakes (no GPU)."""
+import os
+import shutil
+
 import pytest
 
-from paper_2605_31481_gb300 import autotune
+from paper_2605_31481_gb300 import autotune, build
 
 KINDS = autotune.FORWARD_KINDS + ("eval", "fk_vjp", "rnea_vjp", "loss_grad", "aba_vjp", "rnea_store", "rnea_vjp_stored")
 
@@ -58,3 +61,24 @@ def test_a_faster_explicit_form_is_still_chosen(fakes):
     tuned = autotune.tune(model, 4096, kinds=("rnea", "rnea_vjp"), use_cache=False)
     assert model.launch == {"rnea": ("level", 128), "rnea_vjp": ("auto", 0)}
     assert all(t["us"] <= t["candidates"]["auto/0"] for t in tuned.values())
+
+
+def test_a_choice_among_other_kernels_is_not_read_back(fakes, monkeypatch, tmp_path):
+    """The cache's key follows the sources that the library is built from."""
+    model = FakeModel()
+    csrc = tmp_path / "csrc"
+    shutil.copytree(build.CSRC, csrc)
+    monkeypatch.setattr(build, "CSRC", str(csrc))
+
+    def choice():
+        autotune._code.cache_clear()
+        return autotune.tune(model, 64, kinds=("aba",))["aba"]["variant"]
+
+    fakes[("level", 128)] = 4.0
+    assert choice() == "level"
+    fakes[("auto", 0)] = 3.0
+    assert choice() == "level"                  # nothing changed: from the cache
+    with open(os.path.join(csrc, "level.cuh"), "a") as fh:
+        fh.write("// changed\n")
+    assert choice() == "auto"
+    autotune._code.cache_clear()
