@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int6
                  LaneState{state + kAbaLeanBodyFloats * mv.n * kLaneEnvs, kAbaLeanSlotFloats}, taubar, B, e, act,
                  lam);
   const VjpAligned o{qbar, qdbar, nullptr, partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr, -1.f};
-  rnea_vjp_aligned<VJP_GIVEN>(sm, world_accel(mv), cq, tile_col(tile, mv.nq), tile_col(tile, mv.nq + nv), lam,
+  rnea_vjp_aligned<VJP_GIVEN, true>(sm, world_accel(mv), cq, tile_col(tile, mv.nq), tile_col(tile, mv.nq + nv), lam,
                               LaneState{state, kVjpState}, o, B, e, act);
 }
 

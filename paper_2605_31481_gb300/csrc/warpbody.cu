@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(T, MINB) wb_aba_vjp_kernel(const __grid_consta
   const Own lam = minv_warp(me, t, mv, q, qddbar, S, taubar, B, e, act);
   __syncthreads();  // the last level has read its parents' accelerations
   float* const th = partial ? partial + (int64_t)blockIdx.x * mv.n * 10 : nullptr;
-  vjp_warp<VJP_GIVEN>(me, t, mv, q, qd, qdd, lam, S, VjpAligned{qbar, qdbar, nullptr, th, -1.f}, B, e, act);
+  vjp_warp<VJP_GIVEN, true>(me, t, mv, q, qd, qdd, lam, S, VjpAligned{qbar, qdbar, nullptr, th, -1.f}, B, e, act);
 }
 
 size_t wb_smem(int n, int floats) { return (size_t)n * floats * kLaneEnvs * sizeof(float); }

@@ -1,5 +1,5 @@
 // One warp per body: a block is one tile of 32 environments (one per lane) of
-// a tree of at most 32 bodies, and warp w owns body level_body[w] for the
+// a tree of at most 16 bodies, and warp w owns body level_body[w] for the
 // whole call.
 //
 // Everything of a body that nobody else reads stays in its warp's registers:
@@ -18,9 +18,8 @@
 // warp per body all joint transforms, inertias and forces of the tree are
 // formed at once, and a level phase is what really depends on the parent.
 //
-// Quantities are in body-origin frames with root-aligned axes (aligned.cuh):
-// towards the root an articulated inertia is shifted (60 products) instead of
-// rotated and shifted (200).
+// The adjoint's quantities are in body-origin frames with root-aligned axes
+// (aligned.cuh).
 //
 // Every warp of a block meets every barrier (phases are loops over the tree's
 // levels with a warp-uniform test inside); lanes past B work on the last
@@ -130,7 +129,7 @@ struct Sweep {
   SV v, a, vl, al, psd;
 };
 
-template <bool WITH_W>
+template <bool WITH_W, bool BODY>
 __device__ __forceinline__ void sweep_down(const Me& me, const ModelView& mv, const Xf& X, const Own& qd, const Own& qdd,
                                            const Own& tb, const LaneState& S, Sweep& s, SV& wl, SV& wv) {
   const BodyC& c = mv.c[me.i];
@@ -141,7 +140,10 @@ __device__ __forceinline__ void sweep_down(const Me& me, const ModelView& mv, co
   wv = sv_zero();
   for (int l = 0; l < me.depth; ++l) {
     if (me.lev == l) {
-      own_rotation(me, c, X, S, s.d);
+      if (BODY)
+        s.d.psi = me.one_dof() ? S_of(c) : sv_zero();
+      else
+        own_rotation(me, c, X, S, s.d);
       if (me.free_joint()) {
         s.al = SV{f3{0.f, 0.f, 0.f}, RTmul(X.R, a0.v)};
         s.v = free_motion(qd);
@@ -149,10 +151,13 @@ __device__ __forceinline__ void sweep_down(const Me& me, const ModelView& mv, co
         s.psd = sv_zero();
         if (WITH_W) wv = free_motion(tb);
       } else {
+        auto to_child = [&](SV m) { return BODY ? X_motion(X, m) : shift_motion(m, s.d.r); };
         if (me.par >= 0) {
-          s.vl = shift_motion(S.sv(me.par, 9), s.d.r);
-          s.al = shift_motion(S.sv(me.par, 15), s.d.r);
-          if (WITH_W) wl = shift_motion(S.sv(me.par, 21), s.d.r);
+          s.vl = to_child(S.sv(me.par, 9));
+          s.al = to_child(S.sv(me.par, 15));
+          if (WITH_W) wl = to_child(S.sv(me.par, 21));
+        } else if (BODY) {
+          s.al = X_motion(X, a0);
         }
         s.v = s.vl;
         s.a = s.al;
@@ -166,7 +171,7 @@ __device__ __forceinline__ void sweep_down(const Me& me, const ModelView& mv, co
         }
       }
       if (me.nch) {
-        S.put_n(me.i, 0, s.d.R, 9);
+        if (!BODY) S.put_n(me.i, 0, s.d.R, 9);
         S.put(me.i, 9, s.v);
         S.put(me.i, 15, s.a);
         if (WITH_W) S.put(me.i, 21, wv);
@@ -189,19 +194,21 @@ __device__ __forceinline__ void force_up(const Me& me, const WarpTree& t, const 
 
 // The adjoint; formulas, modes and results as in rnea_vjp_aligned, whose sums
 // run in the same order (the two give the same bits). tb: this body's rows of
-// the cotangent or of the measured torques.
-template <int MODE>
+// the cotangent or of the measured torques. BODY: in body axes, as there.
+template <int MODE, bool BODY = false>
 __device__ __forceinline__ float vjp_warp(const Me& me, const WarpTree& t, const ModelView& mv,
                                           const float* __restrict__ q, const float* __restrict__ qd,
                                           const float* __restrict__ qdd, Own tb, const LaneState& S,
                                           const VjpAligned& o, int64_t B, int64_t e, bool act) {
+  static_assert(!BODY || MODE == VJP_GIVEN, "the loss runs in root axes");
   const int64_t ec = act ? e : B - 1;
   const Own xq = own_q(me, q, B, ec), xd = own_v(me, qd, B, ec), xdd = own_v(me, qdd, B, ec);
   Sweep s;
   SV wl, wv;
   float loss = 0.f;
-  sweep_down<MODE == VJP_GIVEN>(me, mv, own_joint(me, mv, xq), xd, xdd, tb, S, s, wl, wv);
-  const In10 I = in_rotate(s.d.R, own_inertia(me, mv));
+  const Xf X = own_joint(me, mv, xq);
+  sweep_down<MODE == VJP_GIVEN, BODY>(me, mv, X, xd, xdd, tb, S, s, wl, wv);
+  const In10 I = BODY ? own_inertia(me, mv) : in_rotate(s.d.R, own_inertia(me, mv));
   const SV hv = in_mul(I, s.v);
   SV f = in_mul(I, s.a) + crf(s.v, hv);
   if (MODE != VJP_GIVEN) {
@@ -237,7 +244,7 @@ __device__ __forceinline__ float vjp_warp(const Me& me, const WarpTree& t, const
     float g[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     inertia_contract(wv, s.a, g);
     inertia_contract(crm(wv, s.v), s.v, g);
-    inertia_grad_to_body(s.d.R, g);
+    if (!BODY) inertia_grad_to_body(s.d.R, g);
 #pragma unroll
     for (int c = 0; c < 10; ++c) g[c] = act ? o.sign * g[c] : 0.f;
     warp_sum10_store(g, o.thbar + 10 * me.i);
@@ -253,12 +260,13 @@ __device__ __forceinline__ float vjp_warp(const Me& me, const WarpTree& t, const
         H = H + f3{h[0], h[32], h[64]};
       }
       if (me.par >= 0) {
-        if (MODE == VJP_GIVEN) S.put(me.i, 0, shift_force(f, s.d.r));
-        S.put(me.i, 6, shift_force(A, s.d.r));
+        if (MODE == VJP_GIVEN) S.put(me.i, 0, BODY ? XT_force(X, f) : shift_force(f, s.d.r));
+        S.put(me.i, 6, BODY ? XT_force(X, A) : shift_force(A, s.d.r));
+        const f3 hp = BODY ? Rmul(X.R, H) : H;
         float* h = S.at(me.i, 12);
-        h[0] = H.x;
-        h[32] = H.y;
-        h[64] = H.z;
+        h[0] = hp.x;
+        h[32] = hp.y;
+        h[64] = hp.z;
       }
     }
     if (l > 0) __syncthreads();
@@ -293,44 +301,15 @@ __device__ __forceinline__ float vjp_warp(const Me& me, const WarpTree& t, const
 }
 
 // ---- M^-1 ---------------------------------------------------------------
-// Shared floats per body: R 9 going down, the articulated inertia and bias
-// force about the parent's origin (21 | 6) going up, the acceleration 6 going
-// down again.
+// In body frames, unlike the adjoint above: D = S . I^A S of a joint then holds
+// the rounding of the rotations below it, not that of the product of all those
+// up to the root, which turning inertia and subspace to the root's axes would
+// put into every D and so into the result (tau_bar of the ABA adjoint against 64
+// bits, relative 2-norm: quadruped11 1.3e-7 and 3.7e-7 in root axes, arm7 2.1e-7
+// and 4.6e-7). There is no sweep of rotations down the tree before it, either.
+// Shared floats per body: the articulated inertia and bias force about the
+// parent's origin (21 | 6) going up, the acceleration 6 going down.
 static_assert(kWbVjpFloats == 27, "M^-1 and the adjoint share one layout");
-
-// X^T s X for a pure shift r = child - parent (sym6_to_parent without the rotation).
-__device__ __forceinline__ Sym6 sym6_shift(const Sym6& s, f3 t) {
-  Sym6 o;
-  const float* C = s.C;
-  const float Cf[9] = {C[0], C[1], C[3], C[1], C[2], C[4], C[3], C[4], C[5]};
-  float W[9], Z[9], Y[9];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    W[c] = fmaf(-t.z, Cf[3 + c], t.y * Cf[6 + c]);
-    W[3 + c] = fmaf(t.z, Cf[c], -t.x * Cf[6 + c]);
-    W[6 + c] = fmaf(-t.y, Cf[c], t.x * Cf[3 + c]);
-  }
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    o.Bk[k] = s.Bk[k] + W[k];
-    Z[k] = fmaf(0.5f, W[k], s.Bk[k]);
-  }
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    Y[3 * r + 0] = fmaf(Z[3 * r + 1], t.z, -Z[3 * r + 2] * t.y);
-    Y[3 * r + 1] = fmaf(-Z[3 * r + 0], t.z, Z[3 * r + 2] * t.x);
-    Y[3 * r + 2] = fmaf(Z[3 * r + 0], t.y, -Z[3 * r + 1] * t.x);
-  }
-#pragma unroll
-  for (int k = 0; k < 6; ++k) o.C[k] = s.C[k];
-  o.A[0] = fmaf(-2.0f, Y[0], s.A[0]);
-  o.A[1] = s.A[1] - (Y[1] + Y[3]);
-  o.A[2] = fmaf(-2.0f, Y[4], s.A[2]);
-  o.A[3] = s.A[3] - (Y[2] + Y[6]);
-  o.A[4] = s.A[4] - (Y[5] + Y[7]);
-  o.A[5] = fmaf(-2.0f, Y[8], s.A[5]);
-  return o;
-}
 
 // M^-1 applied to tau: the articulated-body sweep at rest and without gravity.
 // The result goes to out (may be null) and is returned for this body.
@@ -340,36 +319,29 @@ __device__ __forceinline__ Own minv_warp(const Me& me, const WarpTree& t, const 
   const int64_t ec = act ? e : B - 1;
   const Own xt = own_v(me, tau, B, ec);
   const Xf X = own_joint(me, mv, own_q(me, q, B, ec));
-  Down d;
-  for (int l = 0; l < me.depth; ++l) {
-    if (me.lev == l) {
-      own_rotation(me, mv.c[me.i], X, S, d);
-      if (me.nch) S.put_n(me.i, 0, d.R, 9);
-    }
-    __syncthreads();
-  }
-  Sym6 IA = sym6_from_in(in_rotate(d.R, own_inertia(me, mv)));
+  Sym6 IA = sym6_from_in(own_inertia(me, mv));
   SV pA = sv_zero(), U = sv_zero();
   float invD = 0.f, u = 0.f;
   for (int l = me.depth - 1; l >= 0; --l) {
     if (me.lev == l) {
-      for (int k = 0; k < me.nch; ++k) {
+      for (int k = me.nch - 1; k >= 0; --k) {  // as in the other forms of ABA
         const int ch = t.child[me.c0 + k];
         sym6_add(IA, S.sym(ch, 0));
         pA = pA + S.sv(ch, 21);
       }
       if (me.one_dof()) {
-        U = sym6_mul(IA, d.psi);
-        invD = 1.0f / dot(d.psi, U);
-        u = xt.x[0] - dot(d.psi, pA);
+        const SV s = S_of(mv.c[me.i]);
+        U = sym6_mul(IA, s);
+        invD = 1.0f / dot(s, U);
+        u = xt.x[0] - dot(s, pA);
       }
       if (me.par >= 0) {
         if (me.one_dof()) {
           sym6_rank1_sub(IA, U, invD);
           pA = sv_fma(u * invD, U, pA);
         }
-        S.putsym(me.i, 0, sym6_shift(IA, d.r));
-        S.put(me.i, 21, shift_force(pA, d.r));
+        S.putsym(me.i, 0, sym6_to_parent(X, IA));
+        S.put(me.i, 21, XT_force(X, pA));
       }
     }
     __syncthreads();
@@ -377,7 +349,7 @@ __device__ __forceinline__ Own minv_warp(const Me& me, const WarpTree& t, const 
   Own x{};
   for (int l = 0; l < me.depth; ++l) {
     if (me.lev == l) {
-      SV a = me.par < 0 ? sv_zero() : shift_motion(S.sv(me.par, 0), d.r);
+      SV a = me.par < 0 ? sv_zero() : X_motion(X, S.sv(me.par, 0));
       if (me.free_joint()) {
         a = sym6_solve(IA, free_motion(xt) - pA);
         const float xo[6] = {a.v.x, a.v.y, a.v.z, a.w.x, a.w.y, a.w.z};
@@ -385,7 +357,7 @@ __device__ __forceinline__ Own minv_warp(const Me& me, const WarpTree& t, const 
         for (int r = 0; r < 6; ++r) x.x[r] = xo[r];
       } else if (me.one_dof()) {
         x.x[0] = (u - dot(U, a)) * invD;
-        a = sv_fma(x.x[0], d.psi, a);
+        a = sv_fma(x.x[0], S_of(mv.c[me.i]), a);
       }
       if (me.nch) S.put(me.i, 0, a);
       if (out && act)

@@ -101,6 +101,21 @@ def test_specialised_kernels_give_the_same_bits(torch_cuda, name):
         assert torch.equal(out["specialized"][k], want), (name, k)
 
 
+@pytest.mark.parametrize("name", list(TREES))
+def test_the_aba_adjoint_solves_with_m_in_every_form_alike(torch_cuda, name):
+    """tau_bar = M^-1 qdd_bar: the adjoint's sweep at rest rounds as the general kernel's does, no worse."""
+    torch = torch_cuda
+    from paper_2605_31481_gb300 import api
+    tree = TREES[name]()
+    m = api.Model(tree)
+    q, qd, qdd, bar = _inputs(tree, 197, torch)
+    out = {}
+    for form in ("generic", "auto"):
+        m.set_launch(["aba_vjp"], 0, form)
+        out[form] = api.aba_vjp(m, q, qd, qdd, bar)["tau"]
+    assert torch.equal(out["auto"], out["generic"]), name
+
+
 @pytest.mark.parametrize("name,B,specialize", [
     ("chain7", 4000, False), ("chain7", 6000, False), ("chain12", 2000, False), ("quadruped11", 40000, False),
     ("chain7", 4000, True), ("quadruped11", 6000, True), ("quadruped11", 12000, True), ("humanoid23", 12000, True),
