@@ -313,8 +313,8 @@ size_t state_with_aba(int n, int slots, int per_body) {
 // Threads per block: one warp per two or three bodies while the tiles fill the
 // SMs, more when they do not.
 int aligned_block(int n, int64_t tiles) {
-  if (n >= 16) return tiles <= 304 ? 512 : 256;
-  return tiles <= 304 ? 256 : 128;
+  if (n >= 16) return tiles <= 2 * kSms ? 512 : 256;
+  return tiles <= 2 * kSms ? 256 : 128;
 }
 
 }  // namespace
@@ -337,7 +337,7 @@ size_t aba_vjp_aligned_smem(const ModelView& mv, int slots) {
 // us, humanoid29 B = 2048 180 -> 146).
 static int aba_derivs_threads(const ModelView& mv, int slots, int64_t tiles) {
   const size_t st = state_with_aba(mv.n, slots, kDerivState);
-  int t = tiles <= 152 ? 512 : aligned_block(mv.n, tiles);
+  int t = tiles <= kSms ? 512 : aligned_block(mv.n, tiles);
   while (t >= 32 && (size_t)(t / 32) * 2 * mv.nv > st) t /= 2;
   return t >= 32 ? t : 0;
 }
@@ -401,7 +401,7 @@ cudaError_t launch_rnea_derivs_aligned(const ModelView& mv, int64_t B, const flo
   };
   // 24 warps where an SM has one tile and the tree work for them (humanoid29 B =
   // 2048: 21.0 -> 19.7 us, legged18 B = 2700 11.0 -> 10.3).
-  if (mv.n > 16 && tiles <= 152) return go(rnea_derivs_aligned_kernel<768>, 768);
+  if (mv.n > 16 && tiles <= kSms) return go(rnea_derivs_aligned_kernel<768>, 768);
   return go(rnea_derivs_aligned_kernel<512>, aligned_block(mv.n, tiles));
 }
 
@@ -426,7 +426,7 @@ cudaError_t launch_rnea_vjp_aligned(const ModelView& mv, int64_t B, const float*
   const size_t model = smem_bytes(mv.n), lean = floats32((size_t)kVjpLeanState * mv.n);
   const int T = model + 2 * lean <= kLevelSmemLimit && 2 * (model + lean + 1024) > kLevelSmemLimit ? 2 : 1;
   cudaError_t err;
-  if (tiles > 152 * 2 && mv.n > 8) {
+  if (tiles > 2 * kSms && mv.n > 8) {
     const int W = mv.n > 16 ? 8 : 4;
     prepare(rnea_vjp_lean_kernel, model + T * lean);
     err = launch_pdl(rnea_vjp_lean_kernel, (tiles + T - 1) / T, dim3(32, T, W), model + T * lean, s, mv, B, q, qd, qdd,

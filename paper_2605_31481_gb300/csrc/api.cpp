@@ -93,9 +93,6 @@ bool use_level(const fst_model* m, int kind, int level_kind) {
          level_smem_needed(view_of(m, nullptr), level_kind, level_tiles(m, kind)) <= kLevelSmemLimit;
 }
 
-// Environments of one tile on every SM, k times.
-int64_t tiles_an_sm(int k) { return (int64_t)k * 152 * 32; }
-
 // A tree with fewer than 1.5 bodies a level has no width to share.
 bool is_chain(const fst_model* m) { return 2 * m->n < 3 * m->depth; }
 
@@ -213,7 +210,7 @@ bool use_tile(const fst_model* m, int kind, int64_t B) {
 bool adjoint_tile_rule(const fst_model* m, int kind, bool spec, int64_t B) {
   if (kind == JK_FK_VJP) return spec ? m->n > 8 && (m->n > 16 || B < 12288) : true;
   if (spec && m->n <= 8 && kind == JK_RNEA_VJP) return false;
-  if (spec && m->n <= 16) return kind == JK_RNEA_VJP ? B <= 152 * 2 * 32 : B < 24576;
+  if (spec && m->n <= 16) return kind == JK_RNEA_VJP ? B <= tiles_an_sm(2) : B < 24576;
   return 2 * m->n >= 3 * m->depth || B <= 24576;
 }
 
@@ -231,7 +228,7 @@ bool use_adjoint_tile(const fst_model* m, int kind, int64_t B, size_t need) {
 // B = 16384 42 against 40, and larger trees' registers spill (humanoid29 ABA
 // adjoint 29.6 against 26).
 bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
-  return m->variant[kind] == FST_VARIANT_AUTO && m->wt.n > 0 && B <= 152 * 2 * 32 &&
+  return m->variant[kind] == FST_VARIANT_AUTO && m->wt.n > 0 && B <= tiles_an_sm(2) &&
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
@@ -239,11 +236,7 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
 // blocks share an SM (110 registers a thread), eight are the faster ones while
 // all items run at once (five trees, 8192 environments: 19.3 / 23.9 us; 4096: 15.0 /
 // 13.5; 64: 12.4 / 10.8).
-int multi_tile_block(int items) { return items <= 152 * 2 ? 256 : 128; }
-
-// Whether enough tiles wait for an SM (more than two each) that the forms
-// which keep less state, and so more tiles per SM, are the better ones.
-bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
+int multi_tile_block(int items) { return items <= 2 * kSms ? 256 : 128; }
 
 // Threads per block of a default call's tiles (a block that the caller set is
 // meant for one environment per thread): eight warps, but
@@ -256,7 +249,7 @@ bool many_tiles(int64_t B) { return B > 152 * 2 * 32; }
 // thread four such blocks share an SM (quadruped11 B = 4096 13.2 against 15.5 us,
 // 8192 20.9 against 26.7; but 9.9 against 9.0 at 64).
 int tile_block(const fst_model* m, int kind, int64_t B, bool vjp = false) {
-  if (kind == JK_EVAL && !vjp && m->max_width <= 4 && m->n <= 16 && B > 152 * 32 / 2) return 128;
+  if (kind == JK_EVAL && !vjp && m->max_width <= 4 && m->n <= 16 && B > tiles_an_sm(1) / 2) return 128;
   if (!many_tiles(B) || m->max_width > 4 || vjp || kind == JK_CRBA) return 256;
   return m->n <= 16 || kind == JK_ABA ? 128 : 256;
 }

@@ -394,7 +394,7 @@ __device__ __forceinline__ SmemModel stage_model(const ModelView& mv, float4* sm
 // less).
 __device__ __forceinline__ void pdl_launch() {
   const unsigned blocks = gridDim.x * gridDim.y;
-  if (blocks <= 76 || blocks > 152) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (blocks <= kSms / 2 || blocks > kSms) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -102,6 +102,11 @@ struct PackedJ {
   int off[FST_MAX_LINKS];
 };
 
+// Streaming multiprocessors of the target (GB300). The lines between kernel forms
+// and block sizes were measured on all of them and are counted in tiles of 32
+// environments an SM; a stream confined to some of the SMs keeps the same lines.
+constexpr int kSms = 152;
+
 constexpr int kMaxWarpBodies = 16;
 
 // The tree as a kernel argument. Entry w: the body of warp w.

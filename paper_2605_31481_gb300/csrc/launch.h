@@ -17,12 +17,19 @@ struct Launch {
 };
 
 // Threads per block for B environments, one environment per thread. Small
-// batches use 32-thread blocks so the blocks spread over all 152 SMs.
+// batches use 32-thread blocks so the blocks spread over all SMs.
 inline int default_block(int64_t B) {
-  if (B <= 152 * 32) return 32;
-  if (B <= 152 * 64 * 2) return 64;
+  if (B <= kSms * 32) return 32;
+  if (B <= kSms * 64 * 2) return 64;
   return 128;
 }
+
+// Environments of k tiles of 32 on every SM.
+inline int64_t tiles_an_sm(int k) { return (int64_t)k * kSms * 32; }
+
+// Whether enough tiles wait for an SM (more than two each) that the forms
+// which keep less state, and so more tiles per SM, are the better ones.
+inline bool many_tiles(int64_t B) { return B > tiles_an_sm(2); }
 
 // Instantiates a kernel template for the smallest per-thread body capacity
 // NB in {16, 32, 64} that holds n bodies.

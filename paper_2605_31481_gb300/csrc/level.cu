@@ -230,9 +230,8 @@ cudaError_t go(void (*kernel)(P...), const ModelView& mv, int64_t B, size_t sh, 
   return launch_pdl(kernel, dim3((unsigned)((B + envs - 1) / envs), gy), blk, sh, s, mv, B, args...);
 }
 
-// Whether the warps of a tile do their next bodies' own work ahead of its level
-// (level_pass) in FK and ABA: up to two tiles an SM, see there for both sides.
-bool few_tiles(int64_t B) { return B <= 152 * 2 * 32; }
+// The warps of a tile do their next bodies' own work ahead of its level
+// (level_pass) in FK and ABA up to two tiles an SM, see there for both sides.
 
 }  // namespace
 
@@ -260,12 +259,12 @@ size_t level_smem_needed(const ModelView& mv, int kind, int tiles) {
 
 cudaError_t launch_fk_level(const ModelView& mv, int64_t B, const float* q, float* poses, int block, int tiles,
                             cudaStream_t s) {
-  return go(few_tiles(B) ? fk_level_kernel<true> : fk_level_kernel<false>, mv, B,
+  return go(many_tiles(B) ? fk_level_kernel<false> : fk_level_kernel<true>, mv, B,
             level_smem_needed(mv, LEVEL_FK, tiles), block, tiles, 1, s, q, poses);
 }
 cudaError_t launch_jac_level(const ModelView& mv, int64_t B, const float* q, const LinkList& links, float* J,
                              int block, int tiles, cudaStream_t s) {
-  return go(few_tiles(B) ? jac_level_kernel<true> : jac_level_kernel<false>, mv, B,
+  return go(many_tiles(B) ? jac_level_kernel<false> : jac_level_kernel<true>, mv, B,
             level_smem_needed(mv, LEVEL_JAC, tiles), block, tiles, 1, s, q, links, (float*)nullptr, J);
 }
 cudaError_t launch_rnea_level(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* qdd,
@@ -291,7 +290,7 @@ size_t aba_lean_smem_needed(const ModelView& mv, int slots) {
 }
 cudaError_t launch_aba_level_lean(const ModelView& mv, int64_t B, const float* q, const float* qd, const float* tau,
                                   float* qdd, int block, int slots, cudaStream_t s) {
-  return go(few_tiles(B) ? aba_lean_kernel<true> : aba_lean_kernel<false>, mv, B, aba_lean_smem_needed(mv, slots),
+  return go(many_tiles(B) ? aba_lean_kernel<false> : aba_lean_kernel<true>, mv, B, aba_lean_smem_needed(mv, slots),
             block, 1, 1, s, q, qd, tau, qdd, slots);
 }
 size_t crba_lean_smem_needed(const ModelView& mv, int slots, bool staged) {
