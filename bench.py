@@ -576,7 +576,10 @@ def run_fst(args):
             "parity_detail": parity_detail,
             **extras,
         }
-        print(json.dumps(line))
+        # everything beyond the contract goes to stderr: a reader that keeps only the
+        # end of a long output still finds the whole line on stdout
+        print("detail: " + json.dumps({k: v for k, v in line.items() if k not in short_line(line)}), file=sys.stderr)
+        print(json.dumps(short_line(line)))
     if world > 1:
         dist.destroy_process_group()
 
@@ -1142,6 +1145,21 @@ def cpu_baseline(tree, links, args, st=None, gpu_first=None, budget_s=12.0, Bs=5
                                          "p99_9": float(f"{np.quantile(bwd, 0.999):.2e}")},
                   "cond2_M": {"max": float(f"{cond.max():.3g}"), "median": float(f"{np.median(cond):.3g}")}}
     return cpu, parity, detail
+
+
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline",
+             "per_op_ms", "parity_vs_oracle")
+
+
+def short_line(line):
+    """What the one line on stdout holds; the plan by the name of the one that ran."""
+    out = {k: line[k] for k in LINE_KEYS if k in line}
+    plan = line.get("plan")
+    if plan:
+        ran = {k: us for k, us in plan["us"].items() if us is not None}
+        out["plan_ran"] = {"mode": plan["mode"], "name": min(ran, key=ran.get) if ran else plan["mode"]}
+    return out
 
 
 def run_reference(args, budget_s=120.0):
