@@ -13,7 +13,9 @@
 // joint transforms, inertias, forces and every derivative below are per-body
 // work that all warps of a block share between two barriers.
 //
-// Derivatives. With psi_j the motion subspace of degree of freedom j in this
+// Derivatives, in the manner of Singh, Russell and Wensing (Efficient Analytical
+// Derivatives of Rigid-Body Dynamics using Spatial Vector Algebra, IEEE RA-L 7(2),
+// 2022). With psi_j the motion subspace of degree of freedom j in this
 // form, v, a the velocity and acceleration (gravity included) of j's parent
 // at j's origin,
 //     psid_j = v x psi_j,   psidd_j = a x psi_j + v x psid_j,

@@ -232,9 +232,9 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
-// Threads per block of the mixed-tree launch in tiles: four warps let four
-// blocks share an SM (110 registers a thread), eight are the faster ones while
-// all items run at once (five trees, 8192 environments: 19.3 / 23.9 us; 4096: 15.0 /
+// Threads per block of the mixed-tree launch in tiles: at 110 registers a thread
+// two blocks of eight warps share an SM, and three of four warps (shared memory
+// then allows no fourth); eight are the faster ones while all items run at once (five trees, 8192 environments: 19.3 / 23.9 us; 4096: 15.0 /
 // 13.5; 64: 12.4 / 10.8).
 int multi_tile_block(int items) { return items <= 2 * kSms ? 256 : 128; }
 

@@ -390,7 +390,7 @@ __device__ __forceinline__ void m_clear_tile(float* __restrict__ M, int64_t rows
   for (int64_t r = t >> 5; r < rows; r += W, p += (int64_t)W * B) *p = 0.f;
 }
 
-template <bool PACKED = false, class TP>
+template <class TP>
 __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, const LaneState& S,
                                            float* __restrict__ M, int64_t B, int64_t e, bool act) {
   const int W = n_warps(), w = warp_id();
@@ -400,7 +400,7 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
   // The block barriers of the composite pass order the two sets of stores.
   // Nothing is read back, so DRAM sees each line once; the clear costs L2
   // writes, not a per-entry ancestry test.
-  if (tp.depth() > 0) m_clear_tile(M, PACKED ? (int64_t)nv * (nv + 1) / 2 : (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
+  if (tp.depth() > 0) m_clear_tile(M, (int64_t)nv * nv, B, e - (threadIdx.x & 31), W, w);
   FST_UNROLL
   for (int l = tp.depth() - 1; l >= 0; --l) {
     FST_FOR_MY_BODIES(tp, l, k) {
@@ -416,7 +416,7 @@ __device__ __forceinline__ void crba_level(const TP& tp, const Col& q, int nv, c
     __syncthreads();
   }
   if (!act) return;
-  const MOut<PACKED> Me{M + e, nv, B};
+  const MOut<false> Me{M + e, nv, B};
   for (int i = w; i < tp.n(); i += W) {
     const BodyI bi = tp.I(i);
     if (bi.type == FST_JOINT_REVOLUTE || bi.type == FST_JOINT_PRISMATIC) {
@@ -474,8 +474,9 @@ __device__ __forceinline__ Xf joint_X_rows(const BodyC& c, const BodyI& bi, cons
 // that three tiles of a large tree fit on one SM): per body only X and
 // F = I^c S stay (kCrbaLeanBodyFloats); a body's composite inertia moved to
 // its parent lives in a slot of R (BodyC::slot) until the parent has added it;
-// the root keeps its own I^c in its slot for a free base's 6 x 6 block. q is read from global memory,
-// not staged. Same arithmetic, in the same order, as crba_level.
+// the root keeps its own I^c in its slot for a free base's 6 x 6 block. X_of(c, b)
+// gives a joint's transform, from staged rows of q or, where those do not fit,
+// from global memory. Same arithmetic, in the same order, as crba_level.
 template <bool PACKED = false, bool AHEAD = true, class TP, class XF>
 __device__ __forceinline__ void crba_level_lean(const TP& tp, const XF& X_of, int nv,
                                                 const LaneState& S, const LaneState& R,

@@ -6,8 +6,8 @@
 // that order, which balances the SMs as the generic form's persistent grid
 // does with its atomic work counter, but needs no counter to reset, no
 // occupancy query and no second barrier per item. Shared memory is sized for
-// the largest (tree, operator) pair, all in their lean forms: 65 KB for the
-// 23-body tree, so three blocks an SM. Bound by the latency of the longest
+// the largest (tree, operator) pair, all in their lean forms: 71 KB for the
+// 23-body tree's ABA, so three blocks an SM. Bound by the latency of the longest
 // items (that tree's ABA, 11 levels three times over). Five trees, 7936
 // environments: 70 us in the generic form, 19 here; a whole call 70.7 -> 30 us,
 // which is the host's part.
