@@ -3,11 +3,11 @@
 `tune(model, B)` measures, on the current GPU, every candidate configuration
 of each kernel kind and keeps the fastest via fst_model_set_launch. A
 candidate is an environment-to-thread mapping with a block size (32 to 256
-threads), or the library's own choice, so that a tuned call is never slower
-than an untuned one:
-  auto         what an untuned model runs (variant auto, block 0), some of whose
-               kernels have no other name: the adjoints and the loss in
-               aligned frames, a warp per body, the lean RNEA and fused step;
+threads), or the library's own choice where that runs a kernel which has no
+other name, so that a tuned call is never slower than an untuned one:
+  auto         what an untuned model runs (variant auto, block 0): the adjoints
+               and the loss as tiles or with a warp per body, the store forward
+               and the fused step as tiles, RNEA with the lean state;
   generic      one environment per thread, the tree from shared memory;
   specialized  one environment per thread, a kernel compiled for the tree;
   level        32 environments per block, the block's warps splitting each
@@ -231,6 +231,13 @@ def _key(model, kind, B):
     return f"{model.fingerprint}|{kind}|{B}|{torch.cuda.get_device_name(model.device)}|{_code()}"
 
 
+def _unnamed(model, kind, B):
+    """Whether the library's own choice for this kind can be a kernel that no other candidate names."""
+    if kind == "rnea":                           # the lean state, from more than two tiles an SM on
+        return B > 2 * 32 * sm_count(model.device)
+    return kind in ("eval", "fk_vjp", "rnea_vjp", "aba_vjp", "loss_grad", "rnea_store")
+
+
 def autotune_enabled():
     """False when FST_AUTOTUNE=0: then nothing is measured. tune() keeps the
     library's own choice of form (variant auto, block 0) and StepPlan runs
@@ -274,7 +281,8 @@ def tune(model, B, kinds=FORWARD_KINDS + ("eval",), links=None, use_cache=True, 
             variants.append("mixed")       # specialised fused kernel, roles mapped as their operators
         if kind in spec and kind in LEVEL_KINDS:
             variants += ["path", "pathwarp"]   # path-parallel, where the tree has at most 8 leaves
-        variants.append("auto")                # the library's own choice: what tuning must not fall behind
+        if _unnamed(model, kind, B):
+            variants.append("auto")            # the library's own choice: what tuning must not fall behind
         for variant in variants:
             blocks = (0,) if variant in ("pathwarp", "auto") else CANDIDATE_BLOCKS[1:] if variant == "level2" else \
                 CANDIDATE_BLOCKS[2:] if variant == "levellean" else CANDIDATE_BLOCKS
