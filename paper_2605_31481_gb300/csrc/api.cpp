@@ -118,10 +118,12 @@ bool is_chain(const fst_model* m) { return 2 * m->n < 3 * m->depth; }
 //    second tile (B = 8192: quadruped11 FK 4.3 / 3.7, Jacobians 7.8 / 5.6, RNEA 8.1 /
 //    7.4; but ABA 10.2 / 14.6, and legged12, four bodies a level, FK 3.7 / 4.2, RNEA
 //    6.6 / 7.6, Jacobians 7.5 / 6.0). Above 16 bodies later: FK 16384 (humanoid29 6.6 /
-//    8.0, at 20000 10.0 / 8.2), RNEA four tiles an SM (legged18 19456 9.9 / 10.9, 20000
-//    13.7 / 10.9) or 24576 (humanoid29 21.8 / 21.7), CRBA of up to 20 bodies three
-//    (legged18 14592 8.4 / 11.1, 16384 12.3 / 11.1), the others never (humanoid29
-//    B = 32768 CRBA 41 / 93, ABA 56 / 149, RNEA with the tape 49 / 150).
+//    8.0, at 20000 10.0 / 8.2); RNEA four tiles an SM (legged18 19456 9.9 / 10.9, 20000
+//    13.7 / 10.9), or 24576 (humanoid29 21.8 / 21.7) and again once one environment per
+//    thread no longer fits the chip at once (36864 27.7 / 23.4, 40960 32.0 / 48.6, 65536
+//    46.8 / 50.6); CRBA of up to 20 bodies three tiles (legged18 14592 8.4 / 11.1, 16384
+//    12.3 / 11.1); the others never (humanoid29 B = 32768 CRBA 41 / 93, ABA 56 / 149,
+//    RNEA with the tape 49 / 150).
 bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
   const bool wide = m->n >= 3 * m->depth;
   if (spec) {
@@ -136,7 +138,7 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
       case JK_JACOBIAN:
         return B <= tiles_an_sm(1);
       case JK_RNEA:
-        return m->n <= 20 ? B <= tiles_an_sm(4) : B < 24576;
+        return m->n <= 20 ? B <= tiles_an_sm(4) : B < 24576 || B > tiles_an_sm(8);
       case JK_CRBA:
         return m->n > 20 || B <= tiles_an_sm(3);
       default:
@@ -144,8 +146,11 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
     }
   }
   if (is_chain(m)) {
-    if (op == JK_RNEA || op == JK_RNEA_STORE) return false;
-    return B <= tiles_an_sm(2) && !(op == JK_ABA && m->n <= 8 && B <= tiles_an_sm(1));
+    // (in blocks near the built-in size: 256 threads that a caller asks for gather on
+    // few SMs, ABA B = 4096 10.7 / 19.9, RNEA 7.4 / 8.8, but with the tape B = 64 9.6 / 7.0)
+    const int block = m->block[op];
+    if (op == JK_RNEA || op == JK_RNEA_STORE) return block > 128 && B > tiles_an_sm(1) / 4 && B <= tiles_an_sm(2);
+    return B <= tiles_an_sm(2) && !(op == JK_ABA && m->n <= 8 && block <= 64 && B <= tiles_an_sm(1));
   }
   const bool light = op == JK_FK || op == JK_JACOBIAN || op == JK_RNEA || op == JK_RNEA_STORE;
   return !light || wide || B < 32768;
@@ -170,7 +175,8 @@ bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin
     if (m->n <= 16) return B <= tiles_an_sm(kin ? 1 : 2);
     return !kin || m->n > 20 || B <= tiles_an_sm(3);
   }
-  return !is_chain(m) || (B <= tiles_an_sm(2) && !(aba && m->n <= 8 && B <= tiles_an_sm(1)));
+  return !is_chain(m) ||
+         (B <= tiles_an_sm(2) && !(aba && m->n <= 8 && m->block[JK_EVAL] <= 64 && B <= tiles_an_sm(1)));
 }
 
 // Shared memory of one tile of an operator's state in full. Where that does not
@@ -228,14 +234,15 @@ bool use_adjoint_tile(const fst_model* m, int kind, int64_t B, size_t need) {
 // B = 16384 42 against 40, and larger trees' registers spill (humanoid29 ABA
 // adjoint 29.6 against 26).
 bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
-  return m->variant[kind] == FST_VARIANT_AUTO && m->wt.n > 0 && B <= tiles_an_sm(2) &&
+  return m->variant[kind] == FST_VARIANT_AUTO && m->block[kind] == 0 && m->wt.n > 0 && B <= tiles_an_sm(2) &&
          adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
 // Threads per block of the mixed-tree launch in tiles: at 110 registers a thread
 // two blocks of eight warps share an SM, and three of four warps (shared memory
-// then allows no fourth); eight are the faster ones while all items run at once (five trees, 8192 environments: 19.3 / 23.9 us; 4096: 15.0 /
-// 13.5; 64: 12.4 / 10.8).
+// then allows no fourth); eight are the faster ones while all items run at once
+// (five trees, 8192 environments, four / eight: 19.3 / 23.9 us; 4096: 15.0 / 13.5;
+// 64: 12.4 / 10.8).
 int multi_tile_block(int items) { return items <= 2 * kSms ? 256 : 128; }
 
 // Threads per block of a default call's tiles (a block that the caller set is
