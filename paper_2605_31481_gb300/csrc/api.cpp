@@ -117,7 +117,10 @@ bool is_chain(const fst_model* m) { return 2 * m->n < 3 * m->depth; }
 //    / 2.8, ABA 13.6 / 9.0) and, for light operators, as soon as an SM has a
 //    second tile (B = 8192: quadruped11 FK 4.3 / 3.7, Jacobians 7.8 / 5.6, RNEA 8.1 /
 //    7.4; but ABA 10.2 / 14.6, and legged12, four bodies a level, FK 3.7 / 4.2, RNEA
-//    6.6 / 7.6, Jacobians 7.5 / 6.0). Above 16 bodies later: FK 16384 (humanoid29 6.6 /
+//    6.6 / 7.6, Jacobians 7.5 / 6.0), and for a chain until its registers spill (12 bodies,
+//    B = 4096 FK 6.0 / 4.5, RNEA 11.1 / 7.8, with the tape 16.2 / 11.3, CRBA 9.7 / 10.1 and at
+//    6000 11.7 / 10.1; 16 bodies 7.0 / 6.0, 14.0 / 10.5, 20.8 / 36, 12.8 / 22.6; ABA of 10
+//    14.4 / 12.5, of 12 16.7 / 21.1). Above 16 bodies later: FK 16384 (humanoid29 6.6 /
 //    8.0, at 20000 10.0 / 8.2); RNEA four tiles an SM (legged18 19456 9.9 / 10.9, 20000
 //    13.7 / 10.9), or 24576 (humanoid29 21.8 / 21.7) and again once one environment per
 //    thread no longer fits the chip at once (36864 27.7 / 23.4, 40960 32.0 / 48.6, 65536
@@ -128,6 +131,11 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
   const bool wide = m->n >= 3 * m->depth;
   if (spec) {
     if (m->n <= 8) return false;
+    if (is_chain(m)) {
+      if (op == JK_FK || op == JK_JACOBIAN) return false;
+      if (m->n <= (op == JK_ABA ? 10 : op == JK_RNEA ? 16 : 12)) return false;
+      if (m->n <= 16) return B <= tiles_an_sm(2);
+    }
     if (m->n <= 16) {
       const bool one = op == JK_JACOBIAN || (!wide && (op == JK_FK || op == JK_RNEA));
       return B <= tiles_an_sm(one ? 1 : 2);
@@ -168,10 +176,13 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
 //    roles' straight-line code no longer fits beside each other (humanoid29 B =
 //    16384 70 / 200, 65536 262 / 548; legged18 45 / 86 and 170 / 252). The kinematics
 //    alone as above (quadruped11 B = 4864 6.4 / 7.2, 8192 8.2 / 7.4; legged18 12288
-//    12.6 / 15.5, 16384 17.1 / 15.4; humanoid29 16384 19.8 / 47).
+//    12.6 / 15.5, 16384 17.1 / 15.4; humanoid29 16384 19.8 / 47). A chain's step follows
+//    its ABA's own call, whose last bits can differ there (10 bodies, B = 64 13.6 / 18.1,
+//    1024 14.4 / 11.5, 4096 16.5 / 13.3), and of up to 12 bodies its kinematics do.
 bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin) {
   if (spec) {
     if (m->n <= 8) return false;
+    if (is_chain(m) && m->n <= (aba ? 10 : kin ? 12 : 0)) return false;
     if (m->n <= 16) return B <= tiles_an_sm(kin ? 1 : 2);
     return !kin || m->n > 20 || B <= tiles_an_sm(3);
   }
@@ -203,21 +214,34 @@ bool use_tile(const fst_model* m, int kind, int64_t B) {
          tile_rule(m, kind, jit_has(m, kind), B);
 }
 
-// The same question for the adjoints, whose tiles do more per barrier: against
-// a specialised kernel they win until the batch fills the chip with one
-// environment per thread (quadruped11 B = 32768 loss and gradient 48 / 41, ABA
-// adjoint 77 / 64; 16384: 26 / 40 and 41 / 44), against the generic ones
-// always, except for long batches of a chain (arm7 B = 65536 ABA adjoint 89 /
-// 73). The FK adjoint is light: arm7 specialised 5.5 / 8.2 at every batch,
-// quadruped11 8.5 / 7.5 at 4096 and 8.6 / 10 at 16384. For the smallest trees
-// the RNEA adjoint follows the specialised fused step, whose result it must
-// equal bit for bit (where the step is better off with it: quadruped11 B = 16384 31
-// us in one launch, 38 as tiles and more as step and adjoint).
+// The same question for the adjoints, whose tiles do more per barrier (us, tiles /
+// other). Against a specialised kernel they win until a third wave of tiles:
+// four an SM for the ABA adjoint (quadruped11 B = 19456 36.9 / 43.5, 20000 52.3 / 43.4;
+// arm7 19.7 / 24.4 and 36.3 / 24.4) and for the loss of small trees (arm7 15.6 / 20.0,
+// 20000 26.1 / 20.3; quadruped11 only from 24576 on: 35.0 / 41.2, 32768 42 / 41), two
+// for a long chain, whose state leaves one tile an SM (12 bodies, ABA adjoint 9728
+// 33.2 / 58.7, 10000 55 / 49, loss 19456 36.9 / 44.7). Against the generic ones always,
+// except for a chain at large batches (12 bodies, ABA adjoint 10000 55 / 52.5, 16
+// bodies 20000 172 / 115; arm7 65536 89 / 72). The FK adjoint is light: arm7 specialised
+// 4.9 / 5.8, a chain of 12 9.4 / 11.7, of 16 19.9 / 15.0; quadruped11 9728 7.0 / 7.8, 10000
+// 8.6 / 8.0. For the smallest trees the RNEA adjoint follows the specialised fused step,
+// whose result it must equal bit for bit (where the step is better off with it:
+// quadruped11 B = 16384 31 us in one launch, 38 as tiles and more as step and adjoint).
 bool adjoint_tile_rule(const fst_model* m, int kind, bool spec, int64_t B) {
-  if (kind == JK_FK_VJP) return spec ? m->n > 8 && (m->n > 16 || B < 12288) : true;
-  if (spec && m->n <= 8 && kind == JK_RNEA_VJP) return false;
-  if (spec && m->n <= 16) return kind == JK_RNEA_VJP ? B <= tiles_an_sm(2) : B < 24576;
-  return 2 * m->n >= 3 * m->depth || B <= 24576;
+  const bool chain = is_chain(m), wide = m->n >= 3 * m->depth;
+  if (kind == JK_FK_VJP) {
+    if (!spec) return true;
+    if (m->n <= (chain ? 12 : 8)) return false;
+    return m->n > 16 || B <= tiles_an_sm(2) || (wide && B < 12288);
+  }
+  if (kind == JK_RNEA_VJP) {
+    if (spec && m->n <= 16) return m->n > 8 && B <= tiles_an_sm(2);
+    return !chain || spec || B <= 24576;
+  }
+  if (m->n > 16 && spec) return true;
+  if (chain && m->n > 8) return B <= tiles_an_sm(kind == JK_LOSS_GRAD && m->n <= 12 ? 4 : 2);
+  if (spec) return kind == JK_ABA_VJP || m->n <= 8 ? B <= tiles_an_sm(4) : B < 24576;
+  return !chain || B <= 24576;
 }
 
 // Whether a default call of an adjoint or of the dense derivatives runs its
