@@ -52,8 +52,8 @@ __global__ void __launch_bounds__(T) rnea_derivs_aligned_kernel(ModelView mv, in
 // output arrays (L2); a warp solves two columns at a time in shared memory
 // that the per-body state no longer needs. Latency-bound: a chain of about 60
 // short phases per tile. One thread per environment with a dense Cholesky and
-// its solves in global memory took 364 us for legged12 at B = 1000 (now 31)
-// and 2300 us for the floating humanoid at B = 2048 (now 147).
+// its solves in global memory took 364 us for legged12 at B = 1000 (now 25)
+// and 2300 us for the floating humanoid at B = 2048 (now 139).
 __global__ void __launch_bounds__(512) aba_derivs_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                                  const float* __restrict__ qd,
                                                                  const float* __restrict__ tau, float* qdd, float* dq,
@@ -189,8 +189,9 @@ __global__ void __launch_bounds__(512) rnea_vjp_lean_kernel(ModelView mv, int64_
 
 // The ABA adjoint in one launch: lambda = M^-1 qddbar by the lean
 // level-parallel ABA at rest and without gravity, then minus the adjoint of
-// inverse dynamics at (q, qd, qdd) for the cotangent lambda. Quadruped,
-// B = 5001: 20.2 us, the specialised one-thread-per-environment kernel 41.9.
+// inverse dynamics at (q, qd, qdd) for the cotangent lambda, in body axes (see
+// rnea_vjp_aligned). Quadruped, B = 5001: 17.0 us (19.9 in root axes), the
+// specialised one-thread-per-environment kernel 41.9; humanoid, 65536: 288.
 __global__ void __launch_bounds__(512) aba_vjp_aligned_kernel(ModelView mv, int64_t B, const float* __restrict__ q,
                                                               const float* __restrict__ qd,
                                                               const float* __restrict__ qdd,

@@ -252,14 +252,15 @@ bool use_adjoint_tile(const fst_model* m, int kind, int64_t B, size_t need) {
   return kind == JK_RNEA_DERIVS || kind == JK_ABA_DERIVS || adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
-// Trees of at most 16 bodies run their dynamics adjoints with a warp per body
-// (warpbody.cuh) while the tiles fill the SMs at most twice: quadruped11 B =
-// 4096 ABA adjoint 12.4 against 18.4 us, RNEA adjoint 10.3 against 12.5; at
-// B = 16384 42 against 40, and larger trees' registers spill (humanoid29 ABA
-// adjoint 29.6 against 26).
+// Trees of at most 16 bodies run the ABA adjoint and the loss with a warp per body
+// (warpbody.cuh) while the tiles fill the SMs at most twice, and those of at most 8
+// the RNEA adjoint (B = 4096, us, a warp per body / the tiles of aligned.cuh: ABA
+// adjoint arm7 11.9 / 17.0, quadruped11 14.2 / 15.2, legged12 9.9 / 11.3; loss 11.1 /
+// 12.3, 11.9 / 11.6, 9.1 / 9.6; RNEA adjoint 7.6 / 8.4, 8.6 / 8.0, 7.2 / 6.6). Beyond two
+// tiles an SM registers leave room for too few, and larger trees' spill.
 bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
   return m->variant[kind] == FST_VARIANT_AUTO && m->block[kind] == 0 && m->wt.n > 0 && B <= tiles_an_sm(2) &&
-         adjoint_tile_rule(m, kind, jit_has(m, kind), B);
+         (kind != JK_RNEA_VJP || m->n <= 8) && adjoint_tile_rule(m, kind, jit_has(m, kind), B);
 }
 
 // Threads per block of the mixed-tree launch in tiles: at 110 registers a thread
@@ -270,8 +271,7 @@ bool use_warp_bodies(const fst_model* m, int kind, int64_t B) {
 int multi_tile_block(int items) { return items <= 2 * kSms ? 256 : 128; }
 
 // Threads per block of a default call's tiles (a block that the caller set is
-// meant for one environment per thread): eight warps, but
-// four where many tiles share an SM and a level is never wider (quadruped11 B =
+// meant for one environment per thread): eight warps, but four where many tiles share an SM and a level is never wider (quadruped11 B =
 // 16384 RNEA 9.8 -> 8.6 us, ABA 24.4 -> 14.1, the step 40.5 -> 38.8; legged18, six
 // bodies wide, ABA 19.0 against 27.5 with four). The adjoint's state leaves
 // room for too few tiles (the fused step with it 38.7 against 44.3 with four),

@@ -3,8 +3,8 @@
 //
 // Bound by the chain of levels at 3 to 4 cycles an instruction of one warp;
 // registers hold one or two tiles an SM, so the tile kernels of aligned.cu take
-// over once a third tile waits. Quadruped, B = 4096: RNEA adjoint 12.5 -> 10.3
-// us, ABA adjoint 18.4 -> 12.4 us against those.
+// over once a third tile waits. ABA adjoint, B = 4096, against those: arm 17.0 ->
+// 11.9 us, quadruped 15.2 -> 14.2 (15.8 with M^-1 and the sweep in root axes).
 #include "launch.h"
 #include "warpbody.cuh"
 
