@@ -166,7 +166,7 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
 
 // The same question for the operators of a fused evaluation together (us, tiles /
 // other). aba: whether ABA is among them; kin: whether FK and the Jacobians are
-// all there is.
+// all there is; vjp: whether RNEA carries its adjoint, which is in tiles there.
 //  * generic other side: the whole step of every tree but a chain is the faster
 //    one in tiles (quadruped11 B = 65536 111 / 153). A chain up to two tiles an SM
 //    (7 bodies, FK, J, RNEA and CRBA B = 4096 7.8 / 9.7, 9728 11.6 / 11.9), of few
@@ -179,7 +179,7 @@ bool tile_rule(const fst_model* m, int op, bool spec, int64_t B) {
 //    12.6 / 15.5, 16384 17.1 / 15.4; humanoid29 16384 19.8 / 47). A chain's step follows
 //    its ABA's own call, whose last bits can differ there (10 bodies, B = 64 13.6 / 18.1,
 //    1024 14.4 / 11.5, 4096 16.5 / 13.3), and of up to 12 bodies its kinematics do.
-bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin) {
+bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin, bool vjp) {
   if (spec) {
     if (m->n <= 8) return false;
     if (is_chain(m) && m->n <= (aba ? 10 : kin ? 12 : 0)) return false;
@@ -187,7 +187,7 @@ bool eval_tile_rule(const fst_model* m, bool spec, int64_t B, bool aba, bool kin
     return !kin || m->n > 20 || B <= tiles_an_sm(3);
   }
   return !is_chain(m) ||
-         (B <= tiles_an_sm(2) && !(aba && m->n <= 8 && m->block[JK_EVAL] <= 64 && B <= tiles_an_sm(1)));
+         (B <= tiles_an_sm(2) && !(aba && !vjp && m->n <= 8 && m->block[JK_EVAL] <= 64 && B <= tiles_an_sm(1)));
 }
 
 // Shared memory of one tile of an operator's state in full. Where that does not
@@ -843,7 +843,7 @@ fst_status fst_eval(const fst_model* m, int64_t B, const fst_eval_io* io, const 
     // an operator whose state in full does not fit a tile has a launch of its own
     const bool spec = jit_has(m, JK_EVAL);
     const bool kin = a.n_roles == 1 && a.roles[0] == ROLE_KIN;
-    const bool as_tiles = eval_tile_rule(m, spec, B, a.roles[0] == ROLE_ABA && !vjp, kin);
+    const bool as_tiles = eval_tile_rule(m, spec, B, a.roles[0] == ROLE_ABA, kin, vjp);
     auto tiled = [&](int role) {
       const int op = role == ROLE_ABA ? JK_ABA : role == ROLE_CRBA ? JK_CRBA : role == ROLE_RNEA ? JK_RNEA : JK_FK;
       return as_tiles && tile_need(m, op) <= kLevelSmemLimit;
