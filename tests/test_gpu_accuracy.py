@@ -14,8 +14,7 @@ from tests._helpers import from_soa, to_soa_cuda
 pytestmark = pytest.mark.gpu
 
 TREES = {"chain7": lambda: w.chain(7, seed=0), "quadruped11": lambda: w.spined_quadruped(seed=0),
-         "legged18": lambda: w.legged(6, seed=0), "humanoid23": lambda: w.humanoid(seed=0, floating=False),
-         "humanoid29": lambda: w.humanoid(seed=0)}
+         "legged18": lambda: w.legged(6, seed=0), "humanoid29": lambda: w.humanoid(seed=0)}
 BAR = 1.2
 
 
